@@ -146,8 +146,7 @@ struct Extra {
   int limb_nmax = 0, wpb_factor = 1, wpb_back = 1;  // limb kernels: rows, warps per block
   int asm_chunks = 0;  // assembly blocks per system (the largest system's targets)
   size_t smem_factor = 0, smem_back = 0;
-  int solve_blocks = 1;
-  size_t solve_smem = 0;
+  int solve_blocks = 1, solve_lanes = 8;  // rod solver: blocks, lanes per chain
   int sms = 1;
   int wpb_factor_max = 1, wpb_back_max = 1;
   // launch shapes (dm_autotune): threads per block and work per thread of
@@ -180,6 +179,7 @@ struct Extra {
   int32_t *d_dof_rod = nullptr, *d_rod_dof0 = nullptr, *d_rod_ndof = nullptr,
           *d_rod_st0 = nullptr, *d_rod_edge0 = nullptr;
   double *d_damp = nullptr;
+  double *d_rec = nullptr;      // rod solver: [nd][12] column records
   double *d_scratch = nullptr;  // layout-sized staging for state copies
   size_t scratch_n = 0;
 };
@@ -191,15 +191,20 @@ struct dm_system_ext : dm_system {
   Extra x;
 };
 
-// Persistent rod solver shape: `warps` warps of two rods each per block,
-// `bps` blocks per SM, no more blocks than the batch needs.
-static void set_solve_shape(dm_system_ext *s, int warps, int bps) {
+// Largest rod solver shape: resident warps per SM (warps x blocks).
+constexpr int kMaxSolveWarps = 9;
+
+// Persistent rod solver shape: `warps` warps per block, `bps` blocks per SM
+// (no more than are resident at once), no more blocks than the batch needs.
+static cudaError_t set_solve_shape(dm_system_ext *s, int warps, int bps) {
   s->x.tune.solve_warps = warps;
   s->x.tune.solve_bps = bps;
-  s->x.solve_smem = (size_t)warps * kSolveRodsPerWarp * kSolveRodDoubles * sizeof(double);
-  const int rods_per_block = kSolveRodsPerWarp * warps;
+  int per_sm = 1;
+  const cudaError_t e = rod_solve_occupancy(s->x.solve_lanes, true, warps, &per_sm);
+  const int rods_per_block = rod_solve_rods_per_warp(s->x.solve_lanes) * warps;
   const int want = (s->x.n_rod_sys + rods_per_block - 1) / rods_per_block;
-  s->x.solve_blocks = std::max(1, std::min(want, bps * s->x.sms));
+  s->x.solve_blocks = std::max(1, std::min(want, std::max(1, std::min(bps, per_sm)) * s->x.sms));
+  return e;
 }
 
 static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
@@ -360,6 +365,7 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return T.sys_ndof[a] > T.sys_ndof[b]; });
   s->x.n_rod_sys = (int)order.size();
+  if (s->x.n_rod_sys > 0) DM_TRY(dalloc(s, &s->x.d_rec, 12 * (size_t)nd));
   DM_TRY(upload(s, &d.solve_order, order));
   DM_TRY(upload(s, &s->x.d_sys_kind, T.sys_kind));
   if (prm->self_contact) {
@@ -555,22 +561,17 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
   DM_TRY(dalloc(s, &s->x.d_bad, 1));
   for (int k = 0; k < 2 * DM_NUM_KERNELS; ++k) DM_CK(cudaEventCreate(&s->x.ev[k]));
   DM_CK(cudaMallocHost(&s->h_ctrl, 8 * sizeof(int32_t)));
-  // persistent banded solver: 8 rods per 128-thread block, enough blocks
-  // to cover the batch but no more than fit at once
-  s->x.solve_smem = 4 * kSolveRodsPerWarp * kSolveRodDoubles * sizeof(double);  // 4 warps
-  DM_CK(cudaFuncSetAttribute(k_solve_rod, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)s->x.solve_smem));
   {
-    int dev = 0, sms = 0, per_sm = 0;
+    // persistent rod solver: the warps take rods from the size-sorted queue
+    // (largest first); a small batch spreads its warps over the SMs (one or
+    // two per block), a large one keeps two warps per SM partition, so that
+    // one warp's loads and exchanges hide behind the other's FP64 work
+    int dev = 0;
     DM_CK(cudaGetDevice(&dev));
-    DM_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    DM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_rod, 128,
-                                                        s->x.solve_smem));
-    // persistent: one block of four warps per SM, so that each SM partition
-    // runs one warp; the warps take rod pairs from the size-sorted queue
-    // (largest first), which balances the FP64 work across partitions
-    s->x.sms = sms;
-    set_solve_shape(s, 4, 1);
+    DM_CK(cudaDeviceGetAttribute(&s->x.sms, cudaDevAttrMultiProcessorCount, dev));
+    s->x.solve_lanes = rod_solve_lanes(s->x.n_rod_sys, s->x.sms);
+    const int warps = s->x.n_rod_sys <= s->x.sms ? 1 : s->x.n_rod_sys <= 2 * s->x.sms ? 2 : 4;
+    DM_CK(set_solve_shape(s, warps, 2));
   }
   DM_CK(cudaDeviceSynchronize());
   return DM_OK;
@@ -750,7 +751,8 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
   ra.units = s->x.prof ? s->x.d_units + K_ROWS : nullptr;
   SolveArgs va{s->x.n_rod_sys, nd, s->p.tol, s->p.max_iter, d.solve_order, d.sys_dof0, d.sys_ndof, d.fixed, d.f,
                d.band, d.q, d.dq, d.sys_active, d.sys_iters, d.sys_status, d.sys_res, d.ctrl,
-               s->x.prof ? s->x.d_units + K_SOLVE : nullptr, s->x.ls_action, s->x.ls_trial};
+               s->x.prof ? s->x.d_units + K_SOLVE : nullptr, s->x.ls_action, s->x.ls_trial,
+               s->x.d_rec, 0};
   const int nn = (int)T.n_nodes;
   NodeArgs na{nn, s->p.dt, s->prm.ground_z, s->prm.delta, s->prm.slip_nu, d.q, d.qn,
               d.node_dof_arr, d.node_sys, d.node_h, d.node_mu, d.node_kc, d.sys_active, d.nt,
@@ -911,7 +913,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     if (rod_on) {
       {
         Timed t(s, K_SOLVE, rs);
-        k_solve_rod<<<s->x.solve_blocks, 32 * s->x.tune.solve_warps, s->x.solve_smem, rs>>>(va);
+        DM_CK(rod_solve_launch(va, s->x.solve_lanes, true, s->x.solve_blocks, s->x.tune.solve_warps, rs));
       }
     }
     if (long_on) {
@@ -1356,13 +1358,9 @@ dm_status dm_set_tuning(dm_system *sys, const dm_tuning *t) {
       if (v == x) return true;
     return false;
   };
-  int per_sm = 0;
-  const bool solve_ok =
-      in(t->solve_warps, {1, 2, 4}) && t->solve_blocks_per_sm >= 1 &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, k_solve_rod, 32 * t->solve_warps,
-          (size_t)t->solve_warps * kSolveRodsPerWarp * kSolveRodDoubles * 8) == cudaSuccess &&
-      per_sm >= t->solve_blocks_per_sm;
+  // a shape beyond the solver's occupancy runs with as many blocks as fit
+  const bool solve_ok = in(t->solve_warps, {1, 2, 4}) && t->solve_blocks_per_sm >= 1 &&
+                        t->solve_blocks_per_sm <= kMaxSolveWarps / t->solve_warps;
   // limb shapes beyond this system's shared-memory limit matter only if it
   // has condensation-path limbs
   const bool limb_ok = in(t->limb_factor_warps, {1, 2, 4}) && in(t->limb_back_warps, {1, 2, 4}) &&
@@ -1379,7 +1377,7 @@ dm_status dm_set_tuning(dm_system *sys, const dm_tuning *t) {
   tu.stencil_threads = t->stencil_threads;
   tu.stencil_per_thread = t->stencil_per_thread;
   tu.rows_threads = t->rows_threads;
-  set_solve_shape(s, t->solve_warps, t->solve_blocks_per_sm);
+  DM_CK(set_solve_shape(s, t->solve_warps, t->solve_blocks_per_sm));
   if (s->x.n_fast) {
     s->x.wpb_factor = t->limb_factor_warps;
     s->x.wpb_back = t->limb_back_warps;
@@ -1495,18 +1493,13 @@ dm_status dm_autotune(dm_system *sys, int32_t steps, dm_tuning *out) {
       us[2] = 1e3 * pick(K_ROWS, 3, [&](int c) { tu.rows_threads = r_thr[c]; return true; });
     }
     if (s->x.n_rod_sys > 0) {
-      const int w[] = {4, 2, 1, 4, 2, 4};
-      const int b[] = {1, 2, 4, 2, 1, 3};
+      const int w[] = {s->x.tune.solve_warps, 4, 2, 1, 4, 2};
+      const int b[] = {s->x.tune.solve_bps, 1, 2, 4, 2, 1};
       us[3] = 1e3 * pick(K_SOLVE, 6, [&](int c) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &per_sm, k_solve_rod, 32 * w[c],
-                (size_t)w[c] * kSolveRodsPerWarp * kSolveRodDoubles * 8) !=
-                cudaSuccess ||
-            per_sm < b[c])
+        if (rod_solve_occupancy(s->x.solve_lanes, true, w[c], &per_sm) != cudaSuccess || per_sm < b[c])
           return false;
-        set_solve_shape(s, w[c], b[c]);
-        return true;
+        return set_solve_shape(s, w[c], b[c]) == cudaSuccess;
       });
     }
     if (s->x.n_fast > 0 && !T.lb_n.empty()) {

@@ -1,5 +1,5 @@
 // Public batched banded solve (dm_solve_band): the twisted LDL^T kernel of
-// the Newton step (k_solve_rod) applied to caller-provided systems.
+// the Newton step (dm_rod_solve.cu) applied to caller-provided systems.
 #include <algorithm>
 #include <climits>
 #include <string>
@@ -12,13 +12,10 @@ namespace dm {
 
 namespace {
 
-__global__ void k_band_prepare(int nsys, int64_t ntot, const double *rhs, double *f,
-                               int32_t *order, int32_t *active, int32_t *iters,
-                               int32_t *status, unsigned long long *res, int32_t *ctrl) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ntot) f[i] = -rhs[i];  // the kernel solves J dq = -f
+__global__ void k_band_prepare(int nsys, int32_t *active, int32_t *iters, int32_t *status,
+                               unsigned long long *res, int32_t *ctrl) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nsys) {
-    order[i] = (int32_t)i;
     active[i] = 1;
     iters[i] = 0;
     status[i] = 0;
@@ -38,7 +35,7 @@ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Bytes of scratch the banded solve needs for a batch.
 size_t band_scratch_bytes(int32_t nsys, int64_t ntot) {
-  size_t b = align256(13 * (size_t)ntot * sizeof(double));  // band copy, f, dq
+  size_t b = align256(12 * (size_t)ntot * sizeof(double));  // column records
   b += align256(6 * (size_t)nsys * sizeof(int32_t));        // per-system ints
   b += align256((size_t)nsys * sizeof(unsigned long long)); // residual slots
   b += align256(4 * sizeof(int32_t));                       // queue / counters
@@ -93,10 +90,7 @@ dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof,
                          const double *band, const double *rhs, double *x, char *scr,
                          cudaStream_t st) {
   if (nsys == 0 || ntot == 0) return DM_OK;
-  double *bcopy = (double *)scr;  // [11][ntot] band copy (becomes L)
-  double *f = bcopy + 11 * ntot;  // [ntot] -rhs
-  double *dq = f + ntot;          // [ntot] y / D
-  char *q = scr + align256(13 * (size_t)ntot * sizeof(double));
+  char *q = scr + align256(12 * (size_t)ntot * sizeof(double));
   int32_t *ib = (int32_t *)q;
   int32_t *d_dof0 = ib, *d_ndof = ib + nsys, *order = ib + 2 * nsys;
   int32_t *active = ib + 3 * nsys, *iters = ib + 4 * nsys, *status = ib + 5 * nsys;
@@ -112,13 +106,20 @@ dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof,
       return DM_ERR_CUDA;                                                     \
     }                                                                         \
   } while (0)
-  BS_CK(cudaMemcpyAsync(bcopy, band, 11 * ntot * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  BS_CK(cudaMemcpyAsync(d_dof0, dof0, nsys * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  BS_CK(cudaMemcpyAsync(d_ndof, ndof, nsys * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-  BS_CK(cudaMemsetAsync(x, 0, ntot * sizeof(double), st));
-  const int64_t nthr = ntot > nsys ? ntot : nsys;
-  k_band_prepare<<<(unsigned)((nthr + 255) / 256), 256, 0, st>>>(nsys, ntot, rhs, f, order,
-                                                                  active, iters, status, res, ctrl);
+  // offsets, sizes and the queue's order: the largest systems first
+  std::vector<int32_t> h(3 * (size_t)nsys);
+  int64_t covered = 0;
+  for (int k = 0; k < nsys; ++k) {
+    h[k] = dof0[k];
+    h[nsys + k] = ndof[k];
+    h[2 * (size_t)nsys + k] = k;
+    covered += ndof[k];
+  }
+  std::stable_sort(h.begin() + 2 * (size_t)nsys, h.end(),
+                   [&](int32_t u, int32_t v) { return ndof[u] > ndof[v]; });
+  BS_CK(cudaMemcpyAsync(ib, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  if (covered < ntot) BS_CK(cudaMemsetAsync(x, 0, ntot * sizeof(double), st));
+  k_band_prepare<<<(unsigned)((nsys + 255) / 256), 256, 0, st>>>(nsys, active, iters, status, res, ctrl);
   BS_CK(cudaGetLastError());
   SolveArgs va{};
   va.nsys = nsys;
@@ -129,35 +130,33 @@ dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof,
   va.sys_dof0 = d_dof0;
   va.sys_ndof = d_ndof;
   va.fixed = nullptr;
-  va.f = f;
-  va.band = bcopy;
+  va.f = rhs;
+  va.band = const_cast<double *>(band);  // only read
   va.q = x;
-  va.dq = dq;
+  va.rec = (double *)scr;
+  va.direct = 1;
   va.sys_active = active;
   va.sys_iters = iters;
   va.sys_status = status;
   va.sys_res = res;
   va.ctrl = ctrl;
   va.units = nullptr;
-  const int rods_per_block = 4 * kSolveRodsPerWarp;  // four warps
-  const size_t smem = rods_per_block * kSolveRodDoubles * sizeof(double);
   int dev = 0, sms = 1, per_sm = 1;
   BS_CK(cudaGetDevice(&dev));
   BS_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  BS_CK(cudaFuncSetAttribute(k_solve_rod, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  BS_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_rod, 128, smem));
-  int nblk = (nsys + rods_per_block - 1) / rods_per_block;
-  if (nblk > per_sm * sms) nblk = per_sm * sms;
-  if (nblk > sms) nblk = sms;  // one block of four warps per SM, as in dm_step
-  if (nblk < 1) nblk = 1;
-  k_solve_rod<<<nblk, 128, smem, st>>>(va);
-  BS_CK(cudaGetLastError());
-  int32_t h[4] = {0, 0, 0, 0};
-  BS_CK(cudaMemcpyAsync(h, ctrl, sizeof(h), cudaMemcpyDeviceToHost, st));
+  const int lanes = rod_solve_lanes(nsys, sms);
+  const int warps = nsys <= sms ? 1 : nsys <= 2 * sms ? 2 : 4;  // as in dm_step
+  const int rods_per_block = warps * rod_solve_rods_per_warp(lanes);
+  BS_CK(rod_solve_occupancy(lanes, false, warps, &per_sm));
+  const int nblk = std::max(1, std::min((nsys + rods_per_block - 1) / rods_per_block,
+                                        std::max(1, std::min(per_sm, 2)) * sms));
+  BS_CK(rod_solve_launch(va, lanes, false, nblk, warps, st));
+  int32_t hc[4] = {0, 0, 0, 0};
+  BS_CK(cudaMemcpyAsync(hc, ctrl, sizeof(hc), cudaMemcpyDeviceToHost, st));
   BS_CK(cudaStreamSynchronize(st));
 #undef BS_CK
-  if (h[1] > 0) {
-    set_error("dm_solve_band: zero or non-finite pivot in system " + std::to_string(h[2]));
+  if (hc[1] > 0) {
+    set_error("dm_solve_band: zero or non-finite pivot in system " + std::to_string(hc[2]));
     return DM_ERR_DEGENERATE;
   }
   return DM_OK;

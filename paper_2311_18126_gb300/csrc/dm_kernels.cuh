@@ -68,13 +68,19 @@ struct SolveArgs {
   unsigned long long *units;
   const int32_t *ls_action;  // NULL without line search; 1 = backtracking
   int32_t *ls_trial;
+  double *rec;     // rod solver: a record of 12 doubles per DOF (z and the column's multipliers)
+  int32_t direct;  // rod solver: q = J^-1 f is written, instead of q -= J^-1 f
 };
 
-// shared memory (doubles) per rod of k_solve_rod: two chain windows and the
-// separator scratch
-constexpr int kSolveRodDoubles = 2 * (22 * 12 + 2) + 32;
-// rods per warp of k_solve_rod (two chains of eight lanes each per rod)
-constexpr int kSolveRodsPerWarp = 2;
+// Rod solver (dm_rod_solve.cu): lanes per chain for a batch of `nrods` rods
+// on `sms` SMs, shared memory of a block, resident blocks per SM, launch.
+// env: the matrices have the envelope of a rod's Jacobian.
+int rod_solve_lanes(int nrods, int sms);
+inline int rod_solve_rods_per_warp(int lanes) { return 16 / lanes; }
+size_t rod_solve_smem(int lanes, int warps);
+cudaError_t rod_solve_occupancy(int lanes, bool env, int warps, int *per_sm);
+cudaError_t rod_solve_launch(const SolveArgs &a, int lanes, bool env, int blocks, int warps,
+                             cudaStream_t st);
 
 struct NodeArgs {
   int nn;
@@ -140,6 +146,35 @@ __device__ __forceinline__ double rcp64(double d) {
   const double r = rcp64_seed(d);
   const double e = fma(-d, r, 1.0);
   return fma(r, fma(e, e, e), r);
+}
+
+// 1/d on the integer pipe, for normal d with a normal reciprocal: with the
+// mantissa D in [1, 2) as a 64-bit fixed-point number, S its approximate FP32
+// reciprocal (relative error ~2^-22) and e = 1 - D S formed exactly enough
+// (to 2^-63), the series S (1 + e + e^2) leaves e^3 ~ 2^-66, rounded to 53
+// bits: within 1.01 * 2^-53 of the exact reciprocal.  A warp's FP64
+// instruction occupies its SM partition for 64 cycles, so the three dependent
+// ones of rcp64 cost more than these integer ones.
+__device__ __forceinline__ double rcp_int(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned Dh = 0x80000000u | (hi << 11) | (lo >> 21), Dl = lo << 11;
+  float sf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(sf) : "f"(__uint_as_float(0x3F800000u | ((Dh >> 8) & 0x7FFFFFu))));
+  const unsigned sb = __float_as_uint(sf);  // in [1/2, 1]
+  const unsigned S = sb >= 0x3F800000u ? 0xFFFFFFFFu : sb < 0x3F000000u ? 0x80000000u : (sb << 8) | 0x80000000u;
+  // P = D S 2^63, e 2^63 = 2^63 - P
+  const unsigned long long P = (unsigned long long)Dh * S + __umulhi(Dl, S);
+  const long long e = (long long)(0x8000000000000000ull - P);
+  const int es = (int)(e >> 20);
+  const long long t = e + (((long long)es * es) >> 23);  // (e + e^2) 2^63
+  // r 2^64 = S 2^32 (1 + t)
+  const unsigned long long r = ((unsigned long long)S << 32) +
+                               (unsigned long long)(((long long)(int)(t >> 32) * (long long)S) * 2) +
+                               (((unsigned long long)(unsigned)t * S) >> 31);
+  const unsigned long long m = (r >> 11) + ((r >> 10) & 1);  // rounded; 2^53 carries into the exponent
+  const unsigned ex = (hi >> 20) & 0x7FFu;
+  const unsigned long long b = ((unsigned long long)(2044u - ex) << 52) + m;
+  return __hiloint2double((int)((unsigned)(b >> 32) | (hi & 0x80000000u)), (int)(unsigned)b);
 }
 
 // Asynchronous 8-byte copy global -> shared (both 8-byte aligned), and the
@@ -296,7 +331,6 @@ __global__ void k_stencil_hess(StencilArgs a);  // Hessian of systems still to b
 __global__ void k_rows_rod(RowArgs a);       // residual and band rows
 __global__ void k_rows_rod_res(RowArgs a);   // residual rows
 __global__ void k_rows_rod_band(RowArgs a);  // band rows of systems still to be solved
-__global__ void k_solve_rod(SolveArgs a);
 
 struct StepArgs {
   int nd, ne, ns, nsys;
