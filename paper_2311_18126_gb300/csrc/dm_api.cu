@@ -117,11 +117,14 @@ struct Extra {
     int table = 0, pair_cap = 0, n_contact = 0;
     double inv_cell = 0.0;
     double *edge_h = nullptr, *fc = nullptr, *dense = nullptr;
-    int32_t *edge_idx = nullptr, *contact_sys = nullptr, *sys_bw = nullptr;
+    int32_t *edge_idx = nullptr, *contact_sys = nullptr;
     int32_t *bucket_count = nullptr, *bucket_start = nullptr, *bucket_fill = nullptr,
             *bucket_edges = nullptr, *pairs = nullptr, *npairs = nullptr;
     int32_t *cgo = nullptr, *cbad = nullptr;
-    int64_t *sys_dense0 = nullptr;
+    int64_t *sys_dense0 = nullptr, *sys_nz0 = nullptr;
+    uint8_t *nz = nullptr;
+    double *lud = nullptr;
+    int max_n = 0;  // DOFs of the largest contact system
     unsigned long long *edge_key = nullptr;
   } cc;  // edge-edge contact
   struct {
@@ -376,11 +379,15 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     // excluded pairs of reading C16); edges of different rods never match
     for (int r = 0; r < T.n_rods; ++r)
       for (int64_t e = T.rod_edge0[r]; e < T.rod_edge0[r + 1]; ++e) eidx[e] = (int32_t)(e + 3 * r);
-    std::vector<int64_t> dense0(S, 0);
-    int64_t tot = 0;
+    std::vector<int64_t> dense0(S, 0), nz0(S, 0);
+    int64_t tot = 0, tiles = 0;
     for (int k = 0; k < S; ++k) {
       dense0[k] = tot;
       tot += (int64_t)T.sys_ndof[k] * T.sys_ndof[k];
+      nz0[k] = tiles;
+      const int64_t nt = (T.sys_ndof[k] + kNB - 1) / kNB;
+      tiles += nt * nt;
+      c.max_n = std::max(c.max_n, T.sys_ndof[k]);
       csys.push_back(k);
     }
     double lmax = 0.0, hmax = 0.0;
@@ -407,13 +414,14 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     DM_TRY(dalloc(s, &c.npairs, 1));
     DM_TRY(dalloc(s, &c.fc, nd));
     DM_TRY(dalloc(s, &c.dense, tot));
-    DM_TRY(dalloc(s, &c.sys_bw, S));
+    DM_TRY(upload(s, &c.sys_nz0, nz0));
+    DM_TRY(dalloc(s, &c.nz, tiles));
+    DM_TRY(dalloc(s, &c.lud, kNB * nd));
     DM_TRY(dalloc(s, &c.cgo, S));
     DM_TRY(dalloc(s, &c.cbad, S));
     DM_CK(cudaMemset(c.dense, 0, tot * sizeof(double)));
     DM_CK(cudaMemset(c.npairs, 0, sizeof(int32_t)));
-    std::vector<int32_t> bw10(S, 10);
-    DM_CK(cudaMemcpy(c.sys_bw, bw10.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice));
+    DM_CK(cudaMemset(c.nz, 0, tiles));
   }
   if (prm->line_search) {
     DM_TRY(dalloc(s, &s->x.ls_action, S));
@@ -721,7 +729,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     ca.sys_dof0 = d.sys_dof0; ca.sys_ndof = d.sys_ndof; ca.contact_sys = c.contact_sys;
     ca.ls_action = s->prm.line_search ? s->x.ls_action : nullptr;
     ca.fixed = d.fixed; ca.sys_dense0 = c.sys_dense0; ca.sys_status = d.sys_status;
-    ca.sys_bw = c.sys_bw; ca.edge_key = c.edge_key; ca.bucket_count = c.bucket_count;
+    ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud; ca.edge_key = c.edge_key; ca.bucket_count = c.bucket_count;
     ca.bucket_start = c.bucket_start; ca.bucket_fill = c.bucket_fill;
     ca.bucket_edges = c.bucket_edges; ca.pairs = c.pairs; ca.npairs = c.npairs;
     ca.fc = c.fc; ca.dense = c.dense;
@@ -868,13 +876,12 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       DM_CK(cudaMemsetAsync(c.fc, 0, nd * sizeof(double), rs));
       DM_CK(cudaMemsetAsync(c.npairs, 0, sizeof(int32_t), rs));
       DM_CK(cudaMemsetAsync(c.bucket_count, 0, c.table * sizeof(int32_t), rs));
-      k_cc_clear<<<blocks((int64_t)nd * 32, 256), 256, 0, rs>>>(ca);
-      k_cc_reset_bw<<<blocks(S, 256), 256, 0, rs>>>(ca);
+      k_cc_clear<<<dim3(blocks(c.max_n, kNB), c.n_contact), 256, 0, rs>>>(ca);
       k_cc_cells<<<blocks(ne, 256), 256, 0, rs>>>(ca);
       k_cc_scan<<<1, 1024, 0, rs>>>(ca);
       k_cc_fill<<<blocks(ne, 256), 256, 0, rs>>>(ca);
-      k_cc_pairs<<<blocks(ne, 128), 128, 0, rs>>>(ca);
-      k_cc_terms<<<blocks(c.pair_cap, 64), 64, 0, rs>>>(ca);
+      k_cc_pairs<<<blocks((int64_t)ne * 32, 128), 128, 0, rs>>>(ca);
+      k_cc_terms<<<std::min(blocks(c.pair_cap, 2), 4 * s->x.sms), 64, 0, rs>>>(ca);
       if (T.ground) k_cc_ground<<<blocks(nn, 128), 128, 0, rs>>>(ca, na.node_dof, d.node_sys, d.nt);
     }
     const bool rows_on = rod_on || contact_on || long_on;
@@ -922,22 +929,9 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     }
     if (contact_on) {
       Timed t(s, K_SOLVE_CONTACT, rs);
-      k_cc_band<<<blocks(nd, 256), 256, 0, rs>>>(ca);
-      const int nc = s->x.cc.n_contact;
-      k_cc_decide<<<blocks(nc, 128), 128, 0, rs>>>(ca, va);
-      for (int c = 0; c < nc; ++c) {
-        const int n = T.sys_ndof[c];  // contact systems are systems 0..nc-1 in order
-        for (int k = 0; k < n; k += kNB) {
-          const int rest = n - k - std::min(kNB, n - k);
-          k_lu_diag<<<1, 256, 0, rs>>>(ca, c, k);
-          if (rest > 0) {
-            k_lu_trsm<<<blocks(2 * rest, 32), 32, 0, rs>>>(ca, c, k);
-            const int t = (rest + 63) / 64;
-            k_lu_gemm<<<dim3(t, t), 256, 0, rs>>>(ca, c, k);
-          }
-        }
-      }
-      k_cc_subst<<<nc, 1024, 0, rs>>>(ca, va);
+      k_cc_band<<<blocks(nd, 256), 256, 0, rs>>>(ca, d.f, d.dq);
+      k_cc_decide<<<blocks(s->x.cc.n_contact, 128), 128, 0, rs>>>(ca, va);
+      DM_CK(lu_solve(ca, va, s->x.cc.max_n, s->x.sms, rs));
     }
     if (gen_on) {
       {
@@ -1745,7 +1739,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     ca.sys_kind = s->x.d_sys_kind; ca.sys_active = d.sys_active; ca.dof_sys = s->x.d_dof_sys;
     ca.sys_dof0 = d.sys_dof0; ca.sys_ndof = d.sys_ndof; ca.contact_sys = c.contact_sys;
     ca.ls_action = nullptr; ca.fixed = d.fixed; ca.sys_dense0 = c.sys_dense0;
-    ca.sys_status = d.sys_status; ca.sys_bw = c.sys_bw; ca.edge_key = c.edge_key;
+    ca.sys_status = d.sys_status; ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud; ca.edge_key = c.edge_key;
     ca.bucket_count = c.bucket_count; ca.bucket_start = c.bucket_start;
     ca.bucket_fill = c.bucket_fill; ca.bucket_edges = c.bucket_edges; ca.pairs = c.pairs;
     ca.npairs = c.npairs; ca.fc = c.fc; ca.dense = c.dense;
@@ -1754,13 +1748,12 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     DM_CK(cudaMemsetAsync(c.fc, 0, nd * sizeof(double), st));
     DM_CK(cudaMemsetAsync(c.npairs, 0, sizeof(int32_t), st));
     DM_CK(cudaMemsetAsync(c.bucket_count, 0, c.table * sizeof(int32_t), st));
-    k_cc_clear<<<blocks((int64_t)nd * 32, 256), 256, 0, st>>>(ca);
-    k_cc_reset_bw<<<blocks(S, 256), 256, 0, st>>>(ca);
+    k_cc_clear<<<dim3(blocks(c.max_n, kNB), c.n_contact), 256, 0, st>>>(ca);
     k_cc_cells<<<blocks(ne, 256), 256, 0, st>>>(ca);
     k_cc_scan<<<1, 1024, 0, st>>>(ca);
     k_cc_fill<<<blocks(ne, 256), 256, 0, st>>>(ca);
-    k_cc_pairs<<<blocks(ne, 128), 128, 0, st>>>(ca);
-    k_cc_terms<<<blocks(c.pair_cap, 64), 64, 0, st>>>(ca);
+    k_cc_pairs<<<blocks((int64_t)ne * 32, 128), 128, 0, st>>>(ca);
+    k_cc_terms<<<std::min(blocks(c.pair_cap, 2), 4 * s->x.sms), 64, 0, st>>>(ca);
     if (T.ground) k_cc_ground<<<blocks(nn, 128), 128, 0, st>>>(ca, d.node_dof_arr, d.node_sys, d.nt);
   }
   if (!rod_d0.empty() || contact_on) {
@@ -1852,7 +1845,6 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     // contact rods: J^T lambda = gbar with the blocked LU of the transposed
     // dense matrix (the contact kernels solve J dq = -f and add dq to q)
     const int nc = s->x.cc.n_contact;
-    k_cc_band<<<blocks(nd, 256), 256, 0, st>>>(ca);
     AdjArgs an = aa;
     an.rhs = nrhs;
     an.rhs_sign = -1.0;
@@ -1861,19 +1853,8 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     std::vector<int32_t> onec(nc, 1);
     DM_CK(cudaMemcpyAsync(ca.cgo, onec.data(), nc * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     DM_CK(cudaMemsetAsync(ca.cbad, 0, nc * sizeof(int32_t), st));
-    for (int c = 0; c < nc; ++c) {
-      const int nc_n = T.sys_ndof[c];
-      k_cc_transpose<<<blocks((int64_t)nc_n * std::max(10, nc_n), 256), 256, 0, st>>>(ca, c);
-      for (int k = 0; k < nc_n; k += kNB) {
-        const int rest = nc_n - k - std::min(kNB, nc_n - k);
-        k_lu_diag<<<1, 256, 0, st>>>(ca, c, k);
-        if (rest > 0) {
-          k_lu_trsm<<<blocks(2 * rest, 32), 32, 0, st>>>(ca, c, k);
-          const int t = (rest + 63) / 64;
-          k_lu_gemm<<<dim3(t, t), 256, 0, st>>>(ca, c, k);
-        }
-      }
-    }
+    k_cc_band<<<blocks(nd, 256), 256, 0, st>>>(ca, nrhs, d.dq);
+    k_cc_transpose<<<dim3(blocks(s->x.cc.max_n, kNB), nc), 256, 0, st>>>(ca);
     if (!A.ints) DM_TRY(dalloc(s, &A.ints, 6 * (size_t)S + 2 * (size_t)std::max(ngen, 1) + 8));
     int32_t *its = A.ints, *sts = its + S, *ctl = sts + S;
     DM_CK(cudaMemsetAsync(its, 0, 2 * S * sizeof(int32_t), st));
@@ -1883,8 +1864,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     vs.nd = nd; vs.sys_dof0 = d.sys_dof0; vs.sys_ndof = d.sys_ndof; vs.f = nrhs;
     vs.q = lam; vs.dq = d.dq; vs.sys_active = d.sys_active; vs.sys_iters = its;
     vs.sys_status = sts; vs.ctrl = ctl;
-    k_cc_subst<<<nc, 1024, 0, st>>>(ca, vs);
-    DM_CK(cudaGetLastError());
+    DM_CK(lu_solve(ca, vs, s->x.cc.max_n, s->x.sms, st));
     int32_t h[4] = {0, 0, 0, 0};
     DM_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
     DM_CK(cudaStreamSynchronize(st));

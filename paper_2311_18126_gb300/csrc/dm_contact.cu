@@ -5,23 +5,26 @@
 //                             table; cell size >= longest edge + C + delta,
 //                             so two edges closer than C + delta lie in
 //                             neighbouring cells.
-//  k_cc_pairs              -- one thread per edge: the edges of the 27
-//                             neighbouring cells, minus the excluded pairs
-//                             (sharing a node or at most two edges apart
+//  k_cc_pairs              -- a warp per edge, a lane per candidate: the edges
+//                             of the 27 neighbouring cells, minus the excluded
+//                             pairs (sharing a node or at most two edges apart
 //                             along the rod), whose segment distance D is
 //                             below C + delta (C = sum of the radii).
-//  k_cc_terms              -- one thread per active pair: D and its first
-//                             and second derivatives with respect to the 12
+//  k_cc_terms              -- a warp per active pair: D and its first and
+//                             second derivatives with respect to the 12
 //                             node coordinates (second-order forward-mode
 //                             dual numbers through the closest-point
-//                             computation), k_c E(D) of Eq. 10 by the chain
+//                             computation, their 78 second derivatives spread
+//                             over the lanes), k_c E(D) of Eq. 10 by the chain
 //                             rule; -grad into the contact force vector,
 //                             the Hessian into the system's dense matrix.
 //  k_cc_band               -- adds the rod's own band (11 lower diagonals of
 //                             the symmetric Jacobian) to the dense matrix.
-//  k_lu_* / k_cc_subst     -- blocked LU without pivoting restricted to the
-//                             current bandwidth (the rod band widened by the
-//                             contacts) over all SMs, then the solve, q += dq.
+//  k_lu_* / k_cc_subst     -- blocked LU without pivoting over the nonzero
+//                             32 x 32 tiles of the matrix (the rod band, the
+//                             contacts and their fill), all systems at once,
+//                             then the solve, q += dq.
+#include <algorithm>
 #include <cmath>
 
 #include "dm_internal.h"
@@ -32,125 +35,121 @@ namespace dm {
 namespace {
 
 constexpr int kNH = 78;  // packed upper 12x12
+constexpr int kHP = 3;   // entries of it per lane
 
-__device__ __forceinline__ int hidx(int i, int j) {  // i <= j
-  return i * 12 - i * (i - 1) / 2 + (j - i);
-}
-
-// Second-order dual number in the 12 coordinates of a pair: value,
-// gradient and Hessian (packed upper triangle).
+// Second-order dual number in the 12 coordinates x[0..11] of a pair (p0, p1,
+// q0, q1), spread over a warp: every lane has the value; lane l has the
+// second derivatives of the packed upper entries l, l + 32 and l + 64 (below
+// 78) and the first derivatives at their rows and columns, and lanes 0-11 the
+// first derivative of their own coordinate.  An operation touches 14 first
+// derivatives, 3 second ones and the value per lane instead of 12 + 78 + 1 by
+// one thread, whose numbers did not fit its registers (11 KB of local memory).
 struct HD {
-  double v;
-  double g[12];
-  double h[kNH];
+  double v, own;
+  double gi[kHP], gj[kHP], h[kHP];
 };
 
-__device__ void hd_zero(HD &o, double v) {
+// The lane's entries: coordinates (i, j) of each, and its own coordinate.
+struct HLane {
+  int i[kHP], j[kHP], own;
+  bool on[kHP];
+  __device__ __forceinline__ void load(int lane) {
+#pragma unroll
+    for (int k = 0; k < kHP; ++k) {
+      const int e = lane + 32 * k;
+      on[k] = e < kNH;
+      int r = 0, left = on[k] ? e : 0;
+      while (left >= 12 - r) left -= 12 - r++;
+      i[k] = r;
+      j[k] = r + left;
+    }
+    own = lane < 12 ? lane : 0;
+  }
+};
+
+__device__ __forceinline__ HD hd_const(double v) {
+  HD o;
   o.v = v;
+  o.own = 0.0;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = 0.0;
-#pragma unroll
-  for (int i = 0; i < kNH; ++i) o.h[i] = 0.0;
+  for (int k = 0; k < kHP; ++k) o.gi[k] = o.gj[k] = o.h[k] = 0.0;
+  return o;
 }
 
-// o = a * b (o may alias neither)
-__device__ void hd_mul(const HD &a, const HD &b, HD &o) {
+__device__ __forceinline__ HD hd_mul(const HD &a, const HD &b) {
+  HD o;
   o.v = a.v * b.v;
-  for (int i = 0; i < 12; ++i) o.g[i] = a.v * b.g[i] + b.v * a.g[i];
-  for (int i = 0; i < 12; ++i)
-    for (int j = i; j < 12; ++j) {
-      const int k = hidx(i, j);
-      o.h[k] = a.v * b.h[k] + b.v * a.h[k] + a.g[i] * b.g[j] + a.g[j] * b.g[i];
-    }
-}
-
-// o = ca * a + cb * b (o may alias a or b)
-__device__ void hd_axpby(double ca, const HD &a, double cb, const HD &b, HD &o) {
-  o.v = ca * a.v + cb * b.v;
-  for (int i = 0; i < 12; ++i) o.g[i] = ca * a.g[i] + cb * b.g[i];
-  for (int i = 0; i < kNH; ++i) o.h[i] = ca * a.h[i] + cb * b.h[i];
-}
-
-// o = f(a) for a scalar function with f(a.v) = f0, f' = f1, f'' = f2
-// (o may alias a)
-__device__ void hd_apply(const HD &a, double f0, double f1, double f2, HD &o) {
-  for (int i = 0; i < 12; ++i)
-    for (int j = i; j < 12; ++j) {
-      const int k = hidx(i, j);
-      o.h[k] = f1 * a.h[k] + f2 * a.g[i] * a.g[j];
-    }
-  for (int i = 0; i < 12; ++i) o.g[i] = f1 * a.g[i];
-  o.v = f0;
-}
-
-// o = a / b
-__device__ void hd_div(const HD &a, const HD &b, HD &tmp, HD &o) {
-  const double r = 1.0 / b.v;
-  hd_apply(b, r, -r * r, 2.0 * r * r * r, tmp);
-  hd_mul(a, tmp, o);
-}
-
-// First-order dual number in the 12 coordinates of a pair (value and
-// gradient), for the friction force whose Jacobian is not a Hessian.
-struct D1 {
-  double v;
-  double g[12];
-};
-__device__ __forceinline__ D1 d1_of(const HD &a) {
-  D1 o;
-  o.v = a.v;
+  o.own = a.v * b.own + b.v * a.own;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = a.g[i];
+  for (int k = 0; k < kHP; ++k) {
+    o.gi[k] = a.v * b.gi[k] + b.v * a.gi[k];
+    o.gj[k] = a.v * b.gj[k] + b.v * a.gj[k];
+    o.h[k] = a.v * b.h[k] + b.v * a.h[k] + a.gi[k] * b.gj[k] + a.gj[k] * b.gi[k];
+  }
   return o;
 }
-__device__ __forceinline__ D1 d1_const(double v) {
-  D1 o;
-  o.v = v;
-#pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = 0.0;
-  return o;
-}
-__device__ __forceinline__ D1 d1_var(double v, int k) {
-  D1 o = d1_const(v);
-  o.g[k] = 1.0;
-  return o;
-}
-__device__ __forceinline__ D1 operator+(const D1 &a, const D1 &b) {
-  D1 o;
+
+__device__ __forceinline__ HD hd_add(const HD &a, const HD &b) {
+  HD o;
   o.v = a.v + b.v;
+  o.own = a.own + b.own;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = a.g[i] + b.g[i];
+  for (int k = 0; k < kHP; ++k) {
+    o.gi[k] = a.gi[k] + b.gi[k];
+    o.gj[k] = a.gj[k] + b.gj[k];
+    o.h[k] = a.h[k] + b.h[k];
+  }
   return o;
 }
-__device__ __forceinline__ D1 operator-(const D1 &a, const D1 &b) {
-  D1 o;
+
+__device__ __forceinline__ HD hd_sub(const HD &a, const HD &b) {
+  HD o;
   o.v = a.v - b.v;
+  o.own = a.own - b.own;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = a.g[i] - b.g[i];
+  for (int k = 0; k < kHP; ++k) {
+    o.gi[k] = a.gi[k] - b.gi[k];
+    o.gj[k] = a.gj[k] - b.gj[k];
+    o.h[k] = a.h[k] - b.h[k];
+  }
   return o;
 }
-__device__ __forceinline__ D1 operator*(const D1 &a, const D1 &b) {
-  D1 o;
-  o.v = a.v * b.v;
-#pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = fma(a.v, b.g[i], b.v * a.g[i]);
-  return o;
-}
-__device__ __forceinline__ D1 operator*(double c, const D1 &a) {
-  D1 o;
-  o.v = c * a.v;
-#pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = c * a.g[i];
-  return o;
-}
-// f(a) with f(a.v) = f0, f'(a.v) = f1
-__device__ __forceinline__ D1 d1_apply(const D1 &a, double f0, double f1) {
-  D1 o;
+
+// f(a) for a scalar function with f(a.v) = f0, f' = f1, f'' = f2
+__device__ __forceinline__ HD hd_apply(const HD &a, double f0, double f1, double f2) {
+  HD o;
   o.v = f0;
+  o.own = f1 * a.own;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) o.g[i] = f1 * a.g[i];
+  for (int k = 0; k < kHP; ++k) {
+    o.h[k] = f1 * a.h[k] + f2 * (a.gi[k] * a.gj[k]);
+    o.gi[k] = f1 * a.gi[k];
+    o.gj[k] = f1 * a.gj[k];
+  }
   return o;
 }
+
+__device__ __forceinline__ HD hd_div(const HD &a, const HD &b) {
+  const double r = 1.0 / b.v;
+  return hd_mul(a, hd_apply(b, r, -r * r, 2.0 * r * r * r));
+}
+
+// First-order dual number in the 12 coordinates of a pair (value in every
+// lane, the derivative in coordinate l in lane l < 12), for the friction force
+// whose Jacobian is not a Hessian.
+struct D1 {
+  double v, g;
+};
+__device__ __forceinline__ D1 d1_of(const HD &a) { return {a.v, a.own}; }
+__device__ __forceinline__ D1 d1_const(double v) { return {v, 0.0}; }
+__device__ __forceinline__ D1 operator+(const D1 &a, const D1 &b) { return {a.v + b.v, a.g + b.g}; }
+__device__ __forceinline__ D1 operator-(const D1 &a, const D1 &b) { return {a.v - b.v, a.g - b.g}; }
+__device__ __forceinline__ D1 operator*(const D1 &a, const D1 &b) {
+  return {a.v * b.v, fma(a.v, b.g, b.v * a.g)};
+}
+__device__ __forceinline__ D1 operator*(double c, const D1 &a) { return {c * a.v, c * a.g}; }
+// f(a) with f(a.v) = f0, f'(a.v) = f1
+__device__ __forceinline__ D1 d1_apply(const D1 &a, double f0, double f1) { return {f0, f1 * a.g}; }
 
 // Coordinates of a pair: x[0..2] = p0, x[3..5] = p1, x[6..8] = q0,
 // x[9..11] = q1.  The vectors a = p1 - p0, b = q1 - q0, r = p0 - q0 are
@@ -158,65 +157,66 @@ __device__ __forceinline__ D1 d1_apply(const D1 &a, double f0, double f1) {
 struct Lin {
   double v[3];
   int P, N;
+  // derivative of component c in coordinate x
+  __device__ __forceinline__ double at(int x, int c) const {
+    return x == P + c ? 1.0 : x == N + c ? -1.0 : 0.0;
+  }
 };
 
-// o = u . w for linear vectors
-__device__ void hd_lindot(const Lin &u, const Lin &w, HD &o) {
-  hd_zero(o, u.v[0] * w.v[0] + u.v[1] * w.v[1] + u.v[2] * w.v[2]);
-  for (int c = 0; c < 3; ++c) {
-    o.g[u.P + c] += w.v[c];
-    o.g[u.N + c] -= w.v[c];
-    o.g[w.P + c] += u.v[c];
-    o.g[w.N + c] -= u.v[c];
-    const int ui[2] = {u.P + c, u.N + c}, wi[2] = {w.P + c, w.N + c};
-    const double sg[2] = {1.0, -1.0};
-    for (int x = 0; x < 2; ++x)
-      for (int y = 0; y < 2; ++y) {
-        const int i = ui[x], j = wi[y];
-        const double val = sg[x] * sg[y];
-        if (i == j) o.h[hidx(i, i)] += 2.0 * val;
-        else o.h[hidx(min(i, j), max(i, j))] += val;
-      }
-  }
+__device__ __forceinline__ double lin_dot_grad(const Lin &u, const Lin &w, int x) {
+  double g = 0.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) g += u.at(x, c) * w.v[c] + w.at(x, c) * u.v[c];
+  return g;
 }
 
-// o += s * L_c (scalar dual times component c of a linear vector)
-__device__ void hd_add_scaled_lin(const HD &s, const Lin &L, int c, double sign, HD &o) {
-  const double lv = L.v[c];
-  o.v += sign * s.v * lv;
-  for (int i = 0; i < 12; ++i) o.g[i] += sign * lv * s.g[i];
-  o.g[L.P + c] += sign * s.v;
-  o.g[L.N + c] -= sign * s.v;
-  for (int k = 0; k < kNH; ++k) o.h[k] += sign * lv * s.h[k];
-  // cross terms s.g (x) dL + dL (x) s.g
-  const int li[2] = {L.P + c, L.N + c};
-  const double ls[2] = {sign, -sign};
-  for (int x = 0; x < 2; ++x) {
-    const int j = li[x];
-    for (int i = 0; i < 12; ++i) {
-      const double val = ls[x] * s.g[i];
-      if (i == j) o.h[hidx(i, i)] += 2.0 * val;
-      else o.h[hidx(min(i, j), max(i, j))] += val;
-    }
+// u . w for linear vectors
+__device__ __forceinline__ HD hd_lindot(const Lin &u, const Lin &w, const HLane &ln) {
+  HD o;
+  o.v = u.v[0] * w.v[0] + u.v[1] * w.v[1] + u.v[2] * w.v[2];
+  o.own = lin_dot_grad(u, w, ln.own);
+#pragma unroll
+  for (int k = 0; k < kHP; ++k) {
+    const int x = ln.i[k], y = ln.j[k];
+    o.gi[k] = lin_dot_grad(u, w, x);
+    o.gj[k] = lin_dot_grad(u, w, y);
+    double h = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h += u.at(x, c) * w.at(y, c) + u.at(y, c) * w.at(x, c);
+    o.h[k] = h;
+  }
+  return o;
+}
+
+// o += sign * s * L_c (scalar dual times component c of a linear vector)
+__device__ __forceinline__ void hd_add_scaled_lin(const HD &s, const Lin &L, int c, double sign, const HLane &ln,
+                                                  HD &o) {
+  const double lv = sign * L.v[c], sv = sign * s.v;
+  o.v += s.v * lv;
+  o.own += lv * s.own + sv * L.at(ln.own, c);
+#pragma unroll
+  for (int k = 0; k < kHP; ++k) {
+    const double li = L.at(ln.i[k], c), lj = L.at(ln.j[k], c);
+    o.gi[k] += lv * s.gi[k] + sv * li;
+    o.gj[k] += lv * s.gj[k] + sv * lj;
+    o.h[k] += lv * s.h[k] + sign * (lj * s.gi[k] + li * s.gj[k]);
   }
 }
 
 // clamp to [0, 1]: outside the interval the result is a constant
-__device__ void hd_clamp01(HD &a) {
-  if (a.v < 0.0) hd_zero(a, 0.0);
-  else if (a.v > 1.0) hd_zero(a, 1.0);
+__device__ __forceinline__ HD hd_clamp01(const HD &a) {
+  if (a.v < 0.0) return hd_const(0.0);
+  if (a.v > 1.0) return hd_const(1.0);
+  return a;
 }
 
 // Segment distance with its derivatives, by the same closest-point rule
 // as the definition it follows: s from the unconstrained minimiser clamped
 // to [0, 1] (s = 0 for near-parallel segments), t for that s clamped, then s
 // again for the clamped t, clamped.
-struct DistWork {
-  HD A, B, Cc, Dd, Ee, den, s, t, u, w, tmp, d[3];
-};
-
-__device__ void segment_distance_hd(const double *x, DistWork &W, HD &D) {
+__device__ __forceinline__ HD segment_distance_hd(const double *x, const HLane &ln, HD &s, HD &t, HD (&d)[3]) {
   Lin a, b, r;
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
     a.v[c] = x[3 + c] - x[c];
     b.v[c] = x[9 + c] - x[6 + c];
@@ -225,50 +225,32 @@ __device__ void segment_distance_hd(const double *x, DistWork &W, HD &D) {
   a.P = 3; a.N = 0;
   b.P = 9; b.N = 6;
   r.P = 0; r.N = 6;
-  hd_lindot(a, a, W.A);
-  hd_lindot(a, b, W.B);
-  hd_lindot(b, b, W.Cc);
-  hd_lindot(a, r, W.Dd);
-  hd_lindot(b, r, W.Ee);
-  // den = A Cc - B^2
-  hd_mul(W.A, W.Cc, W.u);
-  hd_mul(W.B, W.B, W.w);
-  hd_axpby(1.0, W.u, -1.0, W.w, W.den);
-  const bool par = W.den.v < 1e-12 * W.A.v * W.Cc.v;
-  if (par) {
-    hd_zero(W.s, 0.0);
+  const HD A = hd_lindot(a, a, ln), B = hd_lindot(a, b, ln), Cc = hd_lindot(b, b, ln);
+  const HD Dd = hd_lindot(a, r, ln), Ee = hd_lindot(b, r, ln);
+  const HD den = hd_sub(hd_mul(A, Cc), hd_mul(B, B));
+  if (den.v < 1e-12 * A.v * Cc.v) {
+    s = hd_const(0.0);
   } else {
-    hd_mul(W.B, W.Ee, W.u);
-    hd_mul(W.Cc, W.Dd, W.w);
-    hd_axpby(1.0, W.u, -1.0, W.w, W.u);
-    hd_div(W.u, W.den, W.tmp, W.s);
-    hd_clamp01(W.s);
+    s = hd_clamp01(hd_div(hd_sub(hd_mul(B, Ee), hd_mul(Cc, Dd)), den));
   }
-  // t = clamp((B s + Ee) / Cc)
-  hd_mul(W.B, W.s, W.u);
-  hd_axpby(1.0, W.u, 1.0, W.Ee, W.u);
-  hd_div(W.u, W.Cc, W.tmp, W.t);
-  hd_clamp01(W.t);
-  // s = clamp((B t - Dd) / A)
-  hd_mul(W.B, W.t, W.u);
-  hd_axpby(1.0, W.u, -1.0, W.Dd, W.u);
-  hd_div(W.u, W.A, W.tmp, W.s);
-  hd_clamp01(W.s);
+  t = hd_clamp01(hd_div(hd_add(hd_mul(B, s), Ee), Cc));
+  s = hd_clamp01(hd_div(hd_sub(hd_mul(B, t), Dd), A));
   // d = r + s a - t b; D = |d|
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
-    hd_zero(W.d[c], r.v[c]);
-    W.d[c].g[r.P + c] = 1.0;
-    W.d[c].g[r.N + c] = -1.0;
-    hd_add_scaled_lin(W.s, a, c, 1.0, W.d[c]);
-    hd_add_scaled_lin(W.t, b, c, -1.0, W.d[c]);
+    d[c] = hd_const(r.v[c]);
+    d[c].own = r.at(ln.own, c);
+#pragma unroll
+    for (int k = 0; k < kHP; ++k) {
+      d[c].gi[k] = r.at(ln.i[k], c);
+      d[c].gj[k] = r.at(ln.j[k], c);
+    }
+    hd_add_scaled_lin(s, a, c, 1.0, ln, d[c]);
+    hd_add_scaled_lin(t, b, c, -1.0, ln, d[c]);
   }
-  hd_mul(W.d[0], W.d[0], W.u);
-  hd_mul(W.d[1], W.d[1], W.w);
-  hd_axpby(1.0, W.u, 1.0, W.w, W.u);
-  hd_mul(W.d[2], W.d[2], W.w);
-  hd_axpby(1.0, W.u, 1.0, W.w, W.u);
-  const double sq = sqrt(W.u.v);
-  hd_apply(W.u, sq, 0.5 / sq, -0.25 / (sq * W.u.v), D);
+  const HD u = hd_add(hd_add(hd_mul(d[0], d[0]), hd_mul(d[1], d[1])), hd_mul(d[2], d[2]));
+  const double sq = sqrt(u.v);
+  return hd_apply(u, sq, 0.5 / sq, -0.25 / (sq * u.v));
 }
 
 // Plain segment distance (same rule), for the candidate filter.
@@ -345,27 +327,35 @@ __global__ void k_cc_cells(ContactArgs a) {
   atomicAdd(a.bucket_count + hash_key(k, a.table_mask), 1);
 }
 
-// exclusive prefix sum of the bucket counts (one block)
-__global__ void k_cc_scan(ContactArgs a) {
-  __shared__ int part[1024];
-  const int T = a.table_mask + 1, tid = threadIdx.x;
+// exclusive prefix sum of the bucket counts (one block of 1024 threads: a
+// serial sum per thread, then a scan over the warps)
+__global__ void __launch_bounds__(1024) k_cc_scan(ContactArgs a) {
+  __shared__ int part[32];
+  const int T = a.table_mask + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (T + blockDim.x - 1) / blockDim.x;
-  const int b0 = tid * per, b1 = min(T, b0 + per);
+  const int b0 = min(T, tid * per), b1 = min(T, b0 + per);
   int sum = 0;
   for (int b = b0; b < b1; ++b) sum += a.bucket_count[b];
-  part[tid] = sum;
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) part[warp] = incl;
   __syncthreads();
-  if (tid == 0) {
-    int run = 0;
-    for (int k = 0; k < (int)blockDim.x; ++k) {
-      const int v = part[k];
-      part[k] = run;
-      run += v;
+  if (warp == 0) {
+    int w = part[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += v;
     }
-    a.bucket_start[T] = run;
+    part[lane] = w;
   }
   __syncthreads();
-  int run = part[tid];
+  int run = incl - sum + (warp ? part[warp - 1] : 0);
+  if (tid == (int)blockDim.x - 1) a.bucket_start[T] = run + sum;
   for (int b = b0; b < b1; ++b) {
     a.bucket_start[b] = run;
     a.bucket_fill[b] = run;
@@ -381,151 +371,176 @@ __global__ void k_cc_fill(ContactArgs a) {
   a.bucket_edges[atomicAdd(a.bucket_fill + h, 1)] = e;
 }
 
-__global__ void k_cc_pairs(ContactArgs a) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per edge: lanes 0-26 look up the neighbouring cells' buckets, then
+// every lane takes candidates of the joint list (a segment distance is some
+// 150 dependent FP64 instructions, so candidates side by side, not in turn).
+__global__ void __launch_bounds__(128) k_cc_pairs(ContactArgs a) {
+  const int e = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (e >= a.ne) return;
   const int s = a.edge_sys[e];
   if (!a.sys_active[s] || a.sys_kind[s] != SOLVE_CONTACT) return;
+  const unsigned full = 0xffffffffu;
   int c[3];
   edge_cell(a, e, c);
   double x[12];
   const int ia = a.edge_a[e], ib = a.edge_b[e];
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
     x[k] = a.q[ia + k];
     x[3 + k] = a.q[ib + k];
   }
-  for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        const unsigned long long key = cell_key(c[0] + dx, c[1] + dy, c[2] + dz);
-        const unsigned h = hash_key(key, a.table_mask);
-        for (int k = a.bucket_start[h]; k < a.bucket_start[h + 1]; ++k) {
-          const int f = a.bucket_edges[k];
-          if (f <= e || a.edge_key[f] != key || a.edge_sys[f] != s) continue;
-          if (abs(a.edge_idx[f] - a.edge_idx[e]) <= 2) continue;  // excluded pairs
-          const int ja = a.edge_a[f], jb = a.edge_b[f];
-          for (int k2 = 0; k2 < 3; ++k2) {
-            x[6 + k2] = a.q[ja + k2];
-            x[9 + k2] = a.q[jb + k2];
-          }
-          const double C = a.edge_h[e] + a.edge_h[f];
-          const double D = segment_distance(x);
-          if (!(D > 0.0)) {  // Eq. 10 undefined: interpenetration
-            atomicCAS(a.sys_status + s, 0, (int)DM_ERR_PENETRATION);
-            continue;
-          }
-          if (D < C + a.delta) {
-            const int p = atomicAdd(a.npairs, 1);
-            if (p < a.pair_cap) {
-              a.pairs[2 * p] = e;
-              a.pairs[2 * p + 1] = f;
-            } else {
-              atomicCAS(a.sys_status + s, 0, (int)DM_ERR_DEGENERATE);
-            }
-          }
-        }
+  unsigned long long key = 0;
+  int start = 0, cnt = 0;
+  if (lane < 27) {
+    key = cell_key(c[0] + lane % 3 - 1, c[1] + (lane / 3) % 3 - 1, c[2] + lane / 9 - 1);
+    const unsigned h = hash_key(key, a.table_mask);
+    start = a.bucket_start[h];
+    cnt = a.bucket_start[h + 1] - start;
+  }
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int total = __shfl_sync(full, incl, 31), excl = incl - cnt;
+  for (int base = 0; base < total; base += 32) {
+    // candidate base + lane: the cell whose range of the joint list holds it
+    const int m = base + lane;
+    int cell = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const int v = __shfl_sync(full, excl, min(cell + o, 31));
+      if (cell + o < 32 && v <= m) cell += o;
+    }
+    const unsigned long long ck = __shfl_sync(full, key, cell);
+    const int at = __shfl_sync(full, start, cell) + m - __shfl_sync(full, excl, cell);
+    if (m >= total) continue;
+    const int f = a.bucket_edges[at];
+    if (f <= e || a.edge_key[f] != ck || a.edge_sys[f] != s) continue;
+    if (abs(a.edge_idx[f] - a.edge_idx[e]) <= 2) continue;  // excluded pairs
+    const int ja = a.edge_a[f], jb = a.edge_b[f];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      x[6 + k] = a.q[ja + k];
+      x[9 + k] = a.q[jb + k];
+    }
+    const double C = a.edge_h[e] + a.edge_h[f];
+    const double D = segment_distance(x);
+    if (!(D > 0.0)) {  // Eq. 10 undefined: interpenetration
+      atomicCAS(a.sys_status + s, 0, (int)DM_ERR_PENETRATION);
+      continue;
+    }
+    if (D < C + a.delta) {
+      const int p = atomicAdd(a.npairs, 1);
+      if (p < a.pair_cap) {
+        a.pairs[2 * p] = e;
+        a.pairs[2 * p + 1] = f;
+      } else {
+        atomicCAS(a.sys_status + s, 0, (int)DM_ERR_DEGENERATE);
       }
+    }
+  }
 }
 
+// The tiles of entries (r, c) and (c, r) of a contact system's matrix are in use.
+__device__ __forceinline__ void mark_tile(const ContactArgs &a, int s, int n, int r, int c) {
+  const int nt = (n + kNB - 1) / kNB, I = r / kNB, J = c / kNB;
+  uint8_t *nz = a.nz + a.sys_nz0[s];
+  nz[(size_t)I * nt + J] = 1;
+  nz[(size_t)J * nt + I] = 1;
+}
+
+// A warp per pair; the launch's warps stride over the pairs found.
 __global__ void __launch_bounds__(64) k_cc_terms(ContactArgs a) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  const int np = min(*a.npairs, a.pair_cap);
-  if (p >= np) return;
-  const int e = a.pairs[2 * p], f = a.pairs[2 * p + 1];
-  const int s = a.edge_sys[e];
-  int dof[12];
-  const int nodes[4] = {a.edge_a[e], a.edge_b[e], a.edge_a[f], a.edge_b[f]};
-  double x[12];
-  for (int n = 0; n < 4; ++n)
-    for (int k = 0; k < 3; ++k) {
-      dof[3 * n + k] = nodes[n] + k;
-      x[3 * n + k] = a.q[nodes[n] + k];
-    }
-  DistWork W;
-  HD D;
-  segment_distance_hd(x, W, D);
-  const double C = a.edge_h[e] + a.edge_h[f];
-  double e0, e1, e2;
-  imc(D.v, C, a.delta, e0, e1, e2);
-  const double kc = a.kc;
-  const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
-  double *M = a.dense + a.sys_dense0[s];
-  int bw = 0;
-  for (int i = 0; i < 12; ++i) {
-    if (a.fixed[dof[i]]) continue;
-    atomicAdd(a.fc + dof[i], -kc * e1 * D.g[i]);  // F = -dE/dq (Eq. 11)
-    for (int j = 0; j < 12; ++j) {
-      if (a.fixed[dof[j]]) continue;
-      const int lo = min(i, j), hi = max(i, j);
-      const double hv = kc * (e1 * D.h[hidx(lo, hi)] + e2 * D.g[i] * D.g[j]);
-      const int r = dof[i] - d0, c = dof[j] - d0;
+  const int np = min(*a.npairs, a.pair_cap), lane = threadIdx.x & 31;
+  const int nwarp = (int)(gridDim.x * (blockDim.x >> 5));
+  HLane ln;
+  ln.load(lane);
+  for (int p = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); p < np; p += nwarp) {
+    const int e = a.pairs[2 * p], f = a.pairs[2 * p + 1];
+    const int s = a.edge_sys[e];
+    const int nodes[4] = {a.edge_a[e], a.edge_b[e], a.edge_a[f], a.edge_b[f]};
+    double x[12];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) x[3 * n + k] = a.q[nodes[n] + k];
+    auto dof = [&](int i) { return (i < 6 ? (i < 3 ? nodes[0] : nodes[1]) : (i < 9 ? nodes[2] : nodes[3])) + i % 3; };
+    HD st, tt, d[3];
+    const HD D = segment_distance_hd(x, ln, st, tt, d);
+    const double C = a.edge_h[e] + a.edge_h[f];
+    double e0, e1, e2;
+    imc(D.v, C, a.delta, e0, e1, e2);
+    const double kc = a.kc;
+    const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
+    double *M = a.dense + a.sys_dense0[s];
+    const bool mine = lane < 12 && !a.fixed[dof(ln.own)];
+    if (mine) atomicAdd(a.fc + dof(ln.own), -kc * e1 * D.own);  // F = -dE/dq (Eq. 11)
+#pragma unroll
+    for (int k = 0; k < kHP; ++k) {
+      const int di = dof(ln.i[k]), dj = dof(ln.j[k]);
+      if (!ln.on[k] || a.fixed[di] || a.fixed[dj]) continue;
+      const double hv = kc * (e1 * D.h[k] + e2 * D.gi[k] * D.gj[k]);
+      const int r = di - d0, c = dj - d0;
       atomicAdd(M + (size_t)r * n + c, hv);
-      bw = max(bw, abs(r - c));
+      if (r != c) atomicAdd(M + (size_t)c * n + r, hv);
+      mark_tile(a, s, n, r, c);
     }
-  }
-  atomicMax(a.sys_bw + s, bw);
-  if (a.mu == 0.0) return;
-  // Friction at the closest points (Eq. 12-13): u = tangential relative
-  // velocity of the closest points with the implicit velocities
-  // (x - x_n)/dt; F_a = -mu gamma(|u|) u/|u| |F_con| on edge a, -F_a on
-  // edge b, spread by the closest-point weights; |F_con| = k_c |dE/dD|.
-  // Derivatives by first-order dual numbers; at |u| = 0 the limit
-  // gamma/|u| -> K2/2 of the smooth law.
-  const D1 sD = d1_of(W.s), tD = d1_of(W.t), Dd = d1_of(D);
-  D1 nrm[3];
-  const D1 iD = d1_apply(Dd, 1.0 / Dd.v, -1.0 / (Dd.v * Dd.v));
-#pragma unroll
-  for (int c = 0; c < 3; ++c) nrm[c] = d1_of(W.d[c]) * iD;
-  const double idt = 1.0 / a.dt;
-  D1 ur[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const D1 v0 = idt * (d1_var(x[c], c) - d1_const(a.qn[dof[c]]));
-    const D1 v1 = idt * (d1_var(x[3 + c], 3 + c) - d1_const(a.qn[dof[3 + c]]));
-    const D1 v2 = idt * (d1_var(x[6 + c], 6 + c) - d1_const(a.qn[dof[6 + c]]));
-    const D1 v3 = idt * (d1_var(x[9 + c], 9 + c) - d1_const(a.qn[dof[9 + c]]));
-    const D1 one = d1_const(1.0);
-    ur[c] = ((one - sD) * v0 + sD * v1) - ((one - tD) * v2 + tD * v3);
-  }
-  const D1 vn = ur[0] * nrm[0] + ur[1] * nrm[1] + ur[2] * nrm[2];
-  D1 u[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) u[c] = ur[c] - vn * nrm[c];
-  const D1 s2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  // |F_con| = -k_c e1 (e1 <= 0 in contact), derivative -k_c e2 grad D
-  const D1 fn = d1_apply(Dd, -kc * e1, -kc * e2);
-  D1 coef;
-  if (s2.v > 0.0) {
-    const double sg = sqrt(s2.v);
-    const D1 sig = d1_apply(s2, sg, 0.5 / sg);
-    const double ex = exp(-a.K2 * sg);
-    const double gam = 2.0 / (1.0 + ex) - 1.0;
-    const double dgam = 2.0 * a.K2 * ex / ((1.0 + ex) * (1.0 + ex));
-    // gamma(sigma) / sigma
-    const D1 gs = d1_apply(sig, gam / sg, (dgam * sg - gam) / (sg * sg));
-    coef = (-a.mu) * (fn * gs);
-  } else {
-    coef = (-0.5 * a.mu * a.K2) * fn;
-  }
-  D1 Fa[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) Fa[c] = coef * u[c];
-  const D1 one = d1_const(1.0);
-  const D1 wgt[4] = {one - sD, sD, tD - one, d1_const(0.0) - tD};
-#pragma unroll
-  for (int nd = 0; nd < 4; ++nd)
+    if (a.mu == 0.0) continue;
+    // Friction at the closest points (Eq. 12-13): u = tangential relative
+    // velocity of the closest points with the implicit velocities
+    // (x - x_n)/dt; F_a = -mu gamma(|u|) u/|u| |F_con| on edge a, -F_a on
+    // edge b, spread by the closest-point weights; |F_con| = k_c |dE/dD|.
+    // Derivatives by first-order dual numbers; at |u| = 0 the limit
+    // gamma/|u| -> K2/2 of the smooth law.
+    const D1 sD = d1_of(st), tD = d1_of(tt), Dd = d1_of(D), one = d1_const(1.0);
+    const D1 iD = d1_apply(Dd, 1.0 / Dd.v, -1.0 / (Dd.v * Dd.v));
+    const double idt = 1.0 / a.dt;
+    D1 nrm[3], ur[3], u[3], Fa[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const int i = 3 * nd + c;
-      if (a.fixed[dof[i]]) continue;
-      const D1 F = wgt[nd] * Fa[c];
-      atomicAdd(a.fc + dof[i], F.v);
-      for (int j = 0; j < 12; ++j) {
-        if (a.fixed[dof[j]] || F.g[j] == 0.0) continue;
-        const int r = dof[i] - d0, cc = dof[j] - d0;
-        atomicAdd(M + (size_t)r * n + cc, -F.g[j]);  // J = -dF/dq
-      }
+      nrm[c] = d1_of(d[c]) * iD;
+      D1 v[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        v[m] = {idt * (x[3 * m + c] - a.qn[nodes[m] + c]), ln.own == 3 * m + c ? idt : 0.0};
+      ur[c] = ((one - sD) * v[0] + sD * v[1]) - ((one - tD) * v[2] + tD * v[3]);
     }
+    const D1 vn = ur[0] * nrm[0] + ur[1] * nrm[1] + ur[2] * nrm[2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) u[c] = ur[c] - vn * nrm[c];
+    const D1 s2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    // |F_con| = -k_c e1 (e1 <= 0 in contact), derivative -k_c e2 grad D
+    const D1 fn = d1_apply(Dd, -kc * e1, -kc * e2);
+    D1 coef;
+    if (s2.v > 0.0) {
+      const double sg = sqrt(s2.v);
+      const D1 sig = d1_apply(s2, sg, 0.5 / sg);
+      const double ex = exp(-a.K2 * sg);
+      const double gam = 2.0 / (1.0 + ex) - 1.0;
+      const double dgam = 2.0 * a.K2 * ex / ((1.0 + ex) * (1.0 + ex));
+      // gamma(sigma) / sigma
+      const D1 gs = d1_apply(sig, gam / sg, (dgam * sg - gam) / (sg * sg));
+      coef = (-a.mu) * (fn * gs);
+    } else {
+      coef = (-0.5 * a.mu * a.K2) * fn;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Fa[c] = coef * u[c];
+    const D1 wgt[4] = {one - sD, sD, tD - one, d1_const(0.0) - tD};
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int i = nodes[m] + c;
+        if (a.fixed[i]) continue;
+        const D1 F = wgt[m] * Fa[c];
+        if (lane == 0) atomicAdd(a.fc + i, F.v);
+        // J = -dF/dq, one column per lane (its tile is marked above)
+        if (mine && F.g != 0.0) atomicAdd(M + (size_t)(i - d0) * n + (dof(ln.own) - d0), -F.g);
+      }
+  }
 }
 
 // Ground contact and friction of the nodes of contact systems (Eq. 10-13,
@@ -548,13 +563,16 @@ __global__ void k_cc_ground(ContactArgs a, const int32_t *node_dof, const int32_
     a.fc[d + r] += nt[r * NN + v];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      if (!a.fixed[d + c]) M[(size_t)(d + r - d0) * n + (d + c - d0)] += nt[(3 + 3 * r + c) * NN + v];
+      if (!a.fixed[d + c]) {
+        M[(size_t)(d + r - d0) * n + (d + c - d0)] += nt[(3 + 3 * r + c) * NN + v];
+        mark_tile(a, s, n, d + r - d0, d + c - d0);
+      }
   }
 }
 
 // The rod's band (lower, symmetric) into the dense matrix of each contact
-// system, one thread per DOF row.
-__global__ void k_cc_band(ContactArgs a) {
+// system, one thread per DOF row, and the right-hand side y = -f.
+__global__ void k_cc_band(ContactArgs a, const double *f, double *y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.nd) return;
   const int s = a.dof_sys[i];
@@ -562,44 +580,63 @@ __global__ void k_cc_band(ContactArgs a) {
   if (a.ls_action && a.ls_action[s] == 1) return;
   const int d0 = a.sys_dof0[s], n = a.sys_ndof[s], r = i - d0;
   double *M = a.dense + a.sys_dense0[s];
+  y[i] = -f[i];
+  int reach = 0;  // the farthest nonzero diagonal: no tile is marked beyond it
   for (int d = 0; d <= 10 && d <= r; ++d) {
     const double v = a.band[(size_t)d * a.nd + i];
+    if (d > 0 && v == 0.0) continue;
     M[(size_t)r * n + (r - d)] += v;
     if (d > 0) M[(size_t)(r - d) * n + r] += v;
+    reach = d;
   }
+  mark_tile(a, s, n, r, r);
+  if ((r - reach) / kNB != r / kNB) mark_tile(a, s, n, r, r - reach);
 }
 
-// Clears the band (of the last bandwidth) of each active contact system.
-// A warp per matrix row, lanes striding along it (coalesced stores).
-__global__ void k_cc_clear(ContactArgs a) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = (int)(t >> 5), lane = (int)(t & 31);
-  if (i >= a.nd) return;
-  const int s = a.dof_sys[i];
-  if (a.sys_kind[s] != SOLVE_CONTACT) return;
-  const int d0 = a.sys_dof0[s], n = a.sys_ndof[s], r = i - d0;
-  const int bw = max(10, a.sys_bw[s]);
-  double *M = a.dense + a.sys_dense0[s] + (size_t)r * n;
-  for (int c = max(0, r - bw) + lane; c <= min(n - 1, r + bw); c += 32) M[c] = 0.0;
+// Zeroes the tiles that the last factorisation of each contact system used,
+// and their marks: a block per tile row.
+__global__ void __launch_bounds__(256) k_cc_clear(ContactArgs a) {
+  const int s = a.contact_sys[blockIdx.y];
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.x;
+  if (I >= nt) return;
+  uint8_t *nz = a.nz + a.sys_nz0[s] + (size_t)I * nt;
+  double *M = a.dense + a.sys_dense0[s];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int J = 0; J < nt; ++J) {
+    if (!nz[J]) continue;
+    const int c = J * kNB + tx;
+#pragma unroll
+    for (int r = ty; r < kNB; r += 8)
+      if (I * kNB + r < n && c < n) M[(size_t)(I * kNB + r) * n + c] = 0.0;
+  }
+  __syncthreads();
+  for (int J = threadIdx.x; J < nt; J += blockDim.x) nz[J] = 0;
 }
 
-__global__ void k_cc_reset_bw(ContactArgs a) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < a.nsys) a.sys_bw[s] = 10;
-}
-
-// --- blocked LU of a contact system (no pivoting), spread over the GPU ---
+// --- blocked LU of the contact systems (no pivoting), spread over the GPU ---
 //
-// The rod's Jacobian widened by the contact blocks, within its current
-// bandwidth bw, is factored in panels of kNB columns: the kNB x kNB
-// diagonal block by one block (k_lu_diag), the panel's L (rows below) and
-// U (columns right) by triangular solves with one thread per row or column
-// (k_lu_trsm), and the trailing update A22 -= L21 U12 by 64 x 64 FP64 tiles
-// over all SMs (k_lu_gemm).  Nothing outside |i - j| <= bw is touched: the
-// LU of a band matrix without pivoting has no fill outside the band.
+// The rods' Jacobian with the contact blocks is sparse in 32 x 32 tiles: the
+// band along each rod, the tiles that touching edges couple, and the fill
+// between them (its pattern is symmetric).  `nz` marks the tiles in use; for
+// each tile column k in turn, all systems at once:
+//   k_lu_panel   factors the diagonal tile (in every block, which saves a
+//                launch; block 0 keeps it in `lud`) and solves the tiles below
+//                (L = A U^-1) and right of it (U = L^-1 A) and the right-hand
+//                side, a warp per row or column: 32 steps of a shuffle and one
+//                FMA, the pivots' reciprocals moved out of the chain into
+//                the rows of U;
+//   k_lu_update  subtracts L(I,k) U(k,J) from the tiles (I, J) of the column's
+//                nonzero rows, in quarters of 16 x 16 (an SM's FP64 pipe takes
+//                9 us for a whole tile), and the right-hand side's part, and
+//                marks the fill.
 // k_cc_decide takes the Newton decision of each contact system first;
-// k_cc_subst solves with the factors (blocked forward and backward
-// substitution) and updates q.
+// k_cc_subst runs the backward substitution and updates q.
+// Bound by the chain of tile columns (a panel launch 26 us, most of it the
+// diagonal tile's 32 dependent columns, an update launch 10 us for the seven
+// tiles a side of a 500-node coil).  Measured (GB300): factorisation and solve
+// of that coil 9.0 -> 2.8 ms, of four grippers of 1195 DOFs 21 -> 1.8 ms
+// (before: the full bandwidth, three launches per panel and system, a
+// panel row per thread).
 
 __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -630,184 +667,214 @@ __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {
   a.cbad[c] = 0;
 }
 
-// 1/d from an FP32 seed and two FP64 Newton steps (relative error at the
-// FP64 rounding level) where |d| is well inside the FP32 range, else by
-// division: the panel kernels take many reciprocals, and an FP64 division
-// costs tens of FP64 instructions.
+// 1/d on the integer pipe where d is well inside the normal range, else by
+// division.
 __device__ __forceinline__ double lu_recip(double d) {
-  const double ad = fabs(d);
-  if (!(ad > 1e-30 && ad < 1e30)) return 1.0 / d;
-  double r = (double)__frcp_rn((float)d);
-  double e = fma(-d, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-d, r, 1.0);
-  return fma(r, e, r);
+  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
+  return ex - 64u < 1918u ? rcp_int(d) : 1.0 / d;
 }
 
-__global__ void __launch_bounds__(256) k_lu_diag(ContactArgs a, int c, int k) {
-  if (!a.cgo[c] || a.cbad[c]) return;
-  const int s = a.contact_sys[c];
-  const int n = a.sys_ndof[s];
-  const int nb = min(kNB, n - k);
-  double *A = a.dense + a.sys_dense0[s];
-  __shared__ double D[kNB][kNB + 1];
-  for (int t = threadIdx.x; t < nb * nb; t += blockDim.x) {
-    const int i = t / nb, j = t - i * nb;
-    D[i][j] = A[(size_t)(k + i) * n + k + j];
+// The tiles of row k of a system's pattern beyond k, in order, into list
+// (shared memory); every thread of the block calls it.  Returns their number.
+__device__ __forceinline__ int tile_list(const uint8_t *row, int k, int nt, uint16_t *list, int *count) {
+  if (threadIdx.x < 32) {
+    int m = 0;
+    for (int b = k + 1; b < nt; b += 32) {
+      const int J = b + (int)threadIdx.x;
+      const bool on = J < nt && row[J] != 0;
+      const unsigned mask = __ballot_sync(0xffffffffu, on);
+      if (on) list[m + __popc(mask & ((1u << threadIdx.x) - 1u))] = (uint16_t)J;
+      m += __popc(mask);
+    }
+    if (threadIdx.x == 0) *count = m;
   }
   __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    const double piv = D[j][j];
-    if (!(fabs(piv) > 0.0) || !isfinite(piv)) {
-      if (threadIdx.x == 0) a.cbad[c] = 1;
-      return;  // uniform: every thread read the same pivot
-    }
-    // only the threads that scale the column take the reciprocal
-    if (j + 1 + (int)threadIdx.x < nb) {
-      const double rp = lu_recip(piv);
-      for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) D[i][j] *= rp;
-    }
-    __syncthreads();
-    const int m = nb - 1 - j;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int i = j + 1 + t / m, cc = j + 1 + t % m;
-      D[i][cc] = fma(-D[i][j], D[j][cc], D[i][cc]);
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < nb * nb; t += blockDim.x) {
-    const int i = t / nb, j = t - i * nb;
-    A[(size_t)(k + i) * n + k + j] = D[i][j];
-  }
+  return *count;
 }
 
-// Rows [k+nb, rend): L21 = A21 U11^{-1}; columns [k+nb, cend): U12 = L11^{-1} A12.
-// A thread per row or column, launched in small blocks so that the FP64 work
-// spreads over many SMs; the diagonal block and the reciprocals of its
-// pivots are staged in shared memory, the thread's row or column in
-// registers (loops fully unrolled, zero-padded past nb).
-__global__ void __launch_bounds__(128) k_lu_trsm(ContactArgs a, int c, int k) {
-  if (!a.cgo[c] || a.cbad[c]) return;
+constexpr int kMaxTiles = 1024;  // tile columns of a system (its matrix is at most 8 GB)
+
+__global__ void __launch_bounds__(256) k_lu_panel(ContactArgs a, double *yall, int k) {
+  const int c = blockIdx.y;
+  // (another block of this launch may be setting cbad: the block decides as one)
+  if (__syncthreads_or(!a.cgo[c] || a.cbad[c])) return;
   const int s = a.contact_sys[c];
-  const int n = a.sys_ndof[s];
-  const int nb = min(kNB, n - k);
-  const int bw = max(10, a.sys_bw[s]);
-  const int lo = k + nb, hi = min(n, k + nb + bw);
-  const int cnt = hi - lo;
-  if (cnt <= 0 || blockIdx.x * blockDim.x >= 2 * cnt) return;
-  double *A = a.dense + a.sys_dense0[s];
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB;
+  if (k >= nt) return;
   __shared__ double D[kNB][kNB + 1];
   __shared__ double R[kNB];
-  for (int t = threadIdx.x; t < kNB * kNB; t += blockDim.x) {
-    const int i = t / kNB, j = t - i * kNB;
-    D[i][j] = (i < nb && j < nb) ? A[(size_t)(k + i) * n + k + j] : (i == j ? 1.0 : 0.0);
+  __shared__ uint16_t list[kMaxTiles];
+  __shared__ int count;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double *A = a.dense + a.sys_dense0[s], *y = yall + a.sys_dof0[s];
+  const int k0 = k * kNB, nb = min(kNB, n - k0);
+  // the diagonal tile, four rows per thread (rows warp + 8 t, column lane);
+  // the identity beyond the matrix
+  double e[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int i = warp + 8 * t;
+    e[t] = i < nb && lane < nb ? A[(size_t)(k0 + i) * n + k0 + lane] : i == lane ? 1.0 : 0.0;
+    D[i][lane] = e[t];
+  }
+  const int m = tile_list(a.nz + a.sys_nz0[s] + (size_t)k * nt, k, nt, list, &count);
+  const int nvec = 2 * kNB * m + 1;  // rows of L, columns of U, the right-hand side
+  if (blockIdx.x && (int)blockIdx.x * 8 >= nvec) return;
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) {
+    const double piv = D[j][j];
+    const double r = lu_recip(piv);
+    const double u = D[j][lane] * r;  // row j of U over the pivot
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (8 * t + 7 <= j) continue;
+      const int i = warp + 8 * t;
+      if (i > j) {
+        const double lij = D[i][j];
+        if (lane > j) {
+          e[t] = fma(-lij, u, e[t]);
+          // what the next column reads: its column and its row
+          if (lane == j + 1 || i == j + 1) D[i][lane] = e[t];
+        }
+      }
+    }
+    if (warp == 0 && lane == 0) {
+      R[j] = r;
+      if (!(fabs(piv) > 0.0) || !isfinite(piv)) a.cbad[c] = 1;
+    }
+    __syncthreads();
+  }
+  // D: on and below the diagonal l_ij d_j, above it u_jm; for the solves the
+  // unit factors: L = (l_ij), U' = (u_jm / d_j)
+  if (blockIdx.x == 0) {
+    double *out = a.lud + (size_t)(a.sys_dof0[s] + k0) * kNB;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int i = warp + 8 * t;
+      if (i < nb) out[i * kNB + lane] = i == lane ? R[i] : D[i][lane];
+    }
+  }
+  double lrow[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int i = warp + 8 * t;
+    lrow[t] = lane < i ? D[i][lane] * R[lane] : lane > i ? D[i][lane] * R[i] : 1.0;
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < kNB; j += blockDim.x) R[j] = lu_recip(D[j][j]);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) D[warp + 8 * t][lane] = lrow[t];
   __syncthreads();
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  double x[kNB];
-  if (g < cnt) {  // a row of L21: x U11 = a
-    double *row = A + (size_t)(lo + g) * n + k;
+  const double rl = R[lane];
+  for (int g = (int)blockIdx.x * 8 + warp; g < nvec; g += (int)gridDim.x * 8) {
+    if (g < kNB * m) {  // a row of L: x U = a, w_j = x_j d_j
+      const int row = list[g / kNB] * kNB + g % kNB;
+      if (row >= n) continue;
+      double *p = A + (size_t)row * n + k0 + lane;
+      double w = lane < nb ? *p : 0.0;
 #pragma unroll
-    for (int j = 0; j < kNB; ++j) x[j] = j < nb ? row[j] : 0.0;
+      for (int j = 0; j < kNB - 1; ++j) {
+        const double wj = __shfl_sync(0xffffffffu, w, j);
+        if (lane > j) w = fma(-wj, D[j][lane], w);
+      }
+      if (lane < nb) *p = w * rl;
+    } else {  // a column of U, or the right-hand side: L x = a (unit lower)
+      const int h = g - kNB * m;
+      const bool rhs = h == kNB * m;
+      const int col = rhs ? 0 : list[h / kNB] * kNB + h % kNB;
+      if (col >= n) continue;
+      double *p = rhs ? y + k0 + lane : A + (size_t)(k0 + lane) * n + col;
+      double w = lane < nb ? *p : 0.0;
 #pragma unroll
-    for (int j = 0; j < kNB; ++j) {
-      double v = x[j];
-#pragma unroll
-      for (int m = 0; m < j; ++m) v = fma(-x[m], D[m][j], v);
-      x[j] = v * R[j];
+      for (int j = 0; j < kNB - 1; ++j) {
+        const double wj = __shfl_sync(0xffffffffu, w, j);
+        if (lane > j) w = fma(-wj, D[lane][j], w);
+      }
+      if (lane < nb) *p = w;
     }
-#pragma unroll
-    for (int j = 0; j < kNB; ++j)
-      if (j < nb) row[j] = x[j];
-  } else if (g < 2 * cnt) {  // a column of U12: L11 x = a (unit lower)
-    const int col = lo + (g - cnt);
-#pragma unroll
-    for (int j = 0; j < kNB; ++j) x[j] = j < nb ? A[(size_t)(k + j) * n + col] : 0.0;
-#pragma unroll
-    for (int j = 0; j < kNB; ++j) {
-      double v = x[j];
-#pragma unroll
-      for (int m = 0; m < j; ++m) v = fma(-D[j][m], x[m], v);
-      x[j] = v;
-    }
-#pragma unroll
-    for (int j = 0; j < kNB; ++j)
-      if (j < nb) A[(size_t)(k + j) * n + col] = x[j];
   }
 }
 
-// A22 -= L21 U12 over [k+nb, k+nb+bw)^2 in 64 x 64 tiles, 4 x 4 per thread.
-__global__ void __launch_bounds__(256) k_lu_gemm(ContactArgs a, int c, int k) {
+// Quarter items (16 x 16 of a tile) of the update, then the right-hand side's
+// rows, strided over the system's blocks.
+__global__ void __launch_bounds__(256) k_lu_update(ContactArgs a, double *yall, int k) {
+  const int c = blockIdx.y;
   if (!a.cgo[c] || a.cbad[c]) return;
   const int s = a.contact_sys[c];
-  const int n = a.sys_ndof[s];
-  const int nb = min(kNB, n - k);
-  const int bw = max(10, a.sys_bw[s]);
-  const int lo = k + nb, hi = min(n, k + nb + bw);
-  const int r0 = lo + blockIdx.y * 64, c0 = lo + blockIdx.x * 64;
-  if (r0 >= hi || c0 >= hi) return;
-  if (a.lu_flops && threadIdx.x == 0)
-    atomicAdd(a.lu_flops, 2ull * (unsigned long long)(min(64, hi - r0) * min(64, hi - c0) * nb));
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB;
+  if (k + 1 >= nt) return;
+  __shared__ double Ls[16][kNB + 1];
+  __shared__ double Us[kNB][16 + 1];
+  __shared__ uint16_t list[kMaxTiles];
+  __shared__ int count;
+  uint8_t *nz = a.nz + a.sys_nz0[s];
+  const int m = tile_list(nz + (size_t)k * nt, k, nt, list, &count);
+  double *A = a.dense + a.sys_dense0[s], *y = yall + a.sys_dof0[s];
+  const int k0 = k * kNB, nb = min(kNB, n - k0);
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int items = 4 * m * m;
+  for (int it = blockIdx.x; it < items + m; it += gridDim.x) {
+    if (it >= items) {  // rows of the right-hand side: a quarter of a warp's lanes per term
+      const int I = list[it - items], lane = tid & 31;
+      for (int r = tid >> 5; r < kNB; r += 8) {
+        const int row = I * kNB + r;
+        if (row >= n) break;
+        double v = lane < nb ? A[(size_t)row * n + k0 + lane] * y[k0 + lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) y[row] -= v;
+      }
+      continue;
+    }
+    const int q = it & 3, t = it >> 2, ti = t / m, tj = t - ti * m;
+    const int I = list[ti], J = list[tj];
+    const int r0 = I * kNB + 16 * (q >> 1), c0 = J * kNB + 16 * (q & 1);
+    if (q == 0 && tid == 0) nz[(size_t)I * nt + J] = 1;  // fill
+    if (r0 >= n || c0 >= n) continue;
+    if (a.lu_flops && tid == 0)
+      atomicAdd(a.lu_flops, 2ull * (unsigned long long)(min(16, n - r0) * min(16, n - c0) * nb));
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int i = (tid >> 5) + 8 * e, mm = tid & 31;
+      Ls[i][mm] = r0 + i < n && mm < nb ? A[(size_t)(r0 + i) * n + k0 + mm] : 0.0;
+      const int u = ty + 16 * e;
+      Us[u][tx] = c0 + tx < n && u < nb ? A[(size_t)(k0 + u) * n + c0 + tx] : 0.0;
+    }
+    const bool in = r0 + ty < n && c0 + tx < n;
+    double *p = A + (size_t)(r0 + ty) * n + c0 + tx;
+    const double old = in ? *p : 0.0;
+    __syncthreads();
+    double acc = 0.0;
+#pragma unroll
+    for (int mm = 0; mm < kNB; ++mm) acc = fma(Ls[ty][mm], Us[mm][tx], acc);
+    if (in) *p = old - acc;
+  }
+}
+
+// In-place transpose of the contact systems' matrices (for the adjoint's
+// J^T solve): a block per tile row, the tiles on and right of the diagonal.
+__global__ void __launch_bounds__(256) k_cc_transpose(ContactArgs a) {
+  const int s = a.contact_sys[blockIdx.y];
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.x;
+  if (I >= nt) return;
+  const uint8_t *nz = a.nz + a.sys_nz0[s] + (size_t)I * nt;
   double *A = a.dense + a.sys_dense0[s];
-  __shared__ double Ls[64][kNB + 1];
-  __shared__ double Us[kNB][64 + 1];
-  for (int t = threadIdx.x; t < 64 * kNB; t += blockDim.x) {
-    const int i = t / kNB, m = t - i * kNB;
-    Ls[i][m] = (r0 + i < hi && m < nb) ? A[(size_t)(r0 + i) * n + k + m] : 0.0;
-  }
-  for (int t = threadIdx.x; t < kNB * 64; t += blockDim.x) {
-    const int m = t / 64, j = t - m * 64;
-    Us[m][j] = (c0 + j < hi && m < nb) ? A[(size_t)(k + m) * n + c0 + j] : 0.0;
-  }
-  __syncthreads();
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-  double acc[4][4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int w = 0; w < 4; ++w) acc[u][w] = 0.0;
-  for (int m = 0; m < nb; ++m) {
-    double lv[4], uv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) lv[u] = Ls[ty + 16 * u][m];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) uv[w] = Us[m][tx + 16 * w];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int w = 0; w < 4; ++w) acc[u][w] = fma(lv[u], uv[w], acc[u][w]);
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int i = r0 + ty + 16 * u;
-    if (i >= hi) continue;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const int j = c0 + tx + 16 * w;
-      if (j < hi) A[(size_t)i * n + j] -= acc[u][w];
+  for (int J = I; J < nt; ++J) {
+    if (!nz[J]) continue;
+    for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
+      const int i = I * kNB + e / kNB, j = J * kNB + e % kNB;
+      if (i >= j || i >= n || j >= n) continue;
+      const double x = A[(size_t)i * n + j];
+      A[(size_t)i * n + j] = A[(size_t)j * n + i];
+      A[(size_t)j * n + i] = x;
     }
   }
 }
 
-// In-place transpose of a contact system's matrix within its bandwidth
-// (for the adjoint's J^T solve): one thread per (row, offset) pair.
-__global__ void k_cc_transpose(ContactArgs a, int c) {
-  const int s = a.contact_sys[c];
-  const int n = a.sys_ndof[s];
-  const int bw = max(10, a.sys_bw[s]);
-  double *A = a.dense + a.sys_dense0[s];
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * bw) return;
-  const int i = (int)(t / bw), j = i + 1 + (int)(t - (int64_t)i * bw);
-  if (j >= n) return;
-  const double x = A[(size_t)i * n + j];
-  A[(size_t)i * n + j] = A[(size_t)j * n + i];
-  A[(size_t)j * n + i] = x;
-}
-
-// Blocked substitution with the factors (L unit lower, U upper), q += x.
+// Backward substitution U x = z of each contact system, q += x: a block per
+// system, tile rows from the last one up; the warps take the row's tiles
+// (a warp sums 32 columns of a row by a shuffle tree), warp 0 solves the
+// diagonal tile.
 __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
   const int c = blockIdx.x;
   const int s = a.contact_sys[c];
@@ -821,54 +888,42 @@ __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
     }
     return;
   }
-  const int d0 = v.sys_dof0[s], n = v.sys_ndof[s];
-  const int bw = max(10, a.sys_bw[s]);
+  const int d0 = v.sys_dof0[s], n = v.sys_ndof[s], nt = (n + kNB - 1) / kNB;
   const double *A = a.dense + a.sys_dense0[s];
   double *y = v.dq + d0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) y[i] = -v.f[d0 + i];
-  __syncthreads();
+  __shared__ uint16_t list[kMaxTiles];
+  __shared__ int count;
+  __shared__ double part[32][kNB + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // forward: L y = -f
-  for (int k = 0; k < n; k += kNB) {
-    const int nb = min(kNB, n - k);
-    if (warp == 0) {
-      double yv = lane < nb ? y[k + lane] : 0.0;
-      for (int j = 0; j < nb; ++j) {
-        const double yj = __shfl_sync(0xffffffffu, yv, j);
-        if (lane > j && lane < nb) yv = fma(-A[(size_t)(k + lane) * n + k + j], yj, yv);
-      }
-      if (lane < nb) y[k + lane] = yv;
+  for (int k = nt - 1; k >= 0; --k) {
+    const int k0 = k * kNB, nb = min(kNB, n - k0);
+    const int m = tile_list(a.nz + a.sys_nz0[s] + (size_t)k * nt, k, nt, list, &count);
+    // warp w sums the columns of tiles w, w + 32, ... : lane = row
+    double sum = 0.0;
+    for (int t = warp; t < 4 * m; t += 32) {  // eight columns of a tile
+      const int j0 = list[t >> 2] * kNB + 8 * (t & 3);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (lane < nb && j0 + j < n) sum = fma(A[(size_t)(k0 + lane) * n + j0 + j], y[j0 + j], sum);
     }
+    part[warp][lane] = sum;
     __syncthreads();
-    for (int i = k + nb + threadIdx.x; i < min(n, k + nb + bw); i += blockDim.x) {
-      double v2 = y[i];
-      for (int m = 0; m < nb; ++m) v2 = fma(-A[(size_t)i * n + k + m], y[k + m], v2);
-      y[i] = v2;
-    }
-    __syncthreads();
-  }
-  // backward: U x = y
-  for (int k = ((n - 1) / kNB) * kNB; k >= 0; k -= kNB) {
-    const int nb = min(kNB, n - k);
     if (warp == 0) {
-      double xv = lane < nb ? y[k + lane] : 0.0;
-      // the panel's pivot reciprocals, one per lane, off the sequential chain
-      const double rj = lane < nb ? lu_recip(A[(size_t)(k + lane) * n + k + lane]) : 1.0;
-      for (int j = nb - 1; j >= 0; --j) {
-        double xj = __shfl_sync(0xffffffffu, xv, j) * __shfl_sync(0xffffffffu, rj, j);
-        if (lane == j) xv = xj;
-        if (lane < j) xv = fma(-A[(size_t)(k + lane) * n + k + j], xj, xv);
-      }
+      const double *Dk = a.lud + (size_t)(d0 + k0) * kNB;  // reciprocal pivots, U above
+      double z = lane < nb ? y[k0 + lane] : 0.0;
+      const int nw = min(32, 4 * m);
+      for (int w = 0; w < nw; ++w) z -= part[w][lane];
+      const double r = lane < nb ? Dk[lane * kNB + lane] : 1.0;
+      double urow[kNB];  // the lane's row of U over its pivot
+#pragma unroll
+      for (int j = 0; j < kNB; ++j) urow[j] = lane < nb && j > lane && j < nb ? Dk[lane * kNB + j] * r : 0.0;
+      double x = z * r;
+#pragma unroll
+      for (int j = kNB - 1; j > 0; --j) x = fma(-urow[j], __shfl_sync(0xffffffffu, x, j), x);
       if (lane < nb) {
-        y[k + lane] = xv;
-        atomicAdd(v.q + d0 + k + lane, xv);
+        y[k0 + lane] = x;
+        atomicAdd(v.q + d0 + k0 + lane, x);
       }
-    }
-    __syncthreads();
-    for (int i = max(0, k - bw) + threadIdx.x; i < k; i += blockDim.x) {
-      double v2 = y[i];
-      for (int m = 0; m < nb; ++m) v2 = fma(-A[(size_t)i * n + k + m], y[k + m], v2);
-      y[i] = v2;
     }
     __syncthreads();
   }
@@ -878,6 +933,23 @@ __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
     atomicAdd(&v.ctrl[0], 1);
     if (v.units) atomicAdd(v.units, (unsigned long long)n);
   }
+}
+
+// The whole factorisation and solve: right-hand side in v.dq (k_cc_band).
+cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int max_n, int sms, cudaStream_t st) {
+  const int nt = (max_n + kNB - 1) / kNB, nc = a.n_contact;
+  if (nc == 0) return cudaSuccess;
+  // blocks per system: the chip shared among the systems, no more than a
+  // full column's rows and columns (panel) or tiles (update) can use
+  const int share = std::max(1, (2 * sms + nc - 1) / nc);
+  for (int k = 0; k < nt; ++k) {
+    const int rest = nt - 1 - k;
+    k_lu_panel<<<dim3(std::min(share, std::max(1, 8 * rest + 1)), nc), 256, 0, st>>>(a, v.dq, k);
+    if (rest > 0)
+      k_lu_update<<<dim3(std::min(share, 4 * rest * rest + rest), nc), 256, 0, st>>>(a, v.dq, k);
+  }
+  k_cc_subst<<<nc, 1024, 0, st>>>(a, v);
+  return cudaGetLastError();
 }
 
 }  // namespace dm

@@ -252,7 +252,10 @@ struct ContactArgs {
   const int32_t *sys_dof0, *sys_ndof, *contact_sys, *ls_action;
   const uint8_t *fixed;
   const int64_t *sys_dense0;
-  int32_t *sys_status, *sys_bw;
+  int32_t *sys_status;
+  uint8_t *nz;               // per system: which kNB x kNB tiles of its matrix are in use
+  const int64_t *sys_nz0;
+  double *lud;               // [nd][kNB]: factored diagonal tiles (their pivots inverted)
   unsigned long long *edge_key;
   int32_t *bucket_count, *bucket_start, *bucket_fill, *bucket_edges;
   int32_t *pairs, *npairs;
@@ -262,23 +265,21 @@ struct ContactArgs {
   int nn;  // nodes (ground terms of contact systems)
   unsigned long long *lu_flops;  // profiling: FP64 flops of the LU's trailing updates (or NULL)
 };
-constexpr int kNB = 32;  // panel width of the contact-system LU
+constexpr int kNB = 32;  // tile of the contact systems' matrices and their LU
 __global__ void k_cc_cells(ContactArgs a);
 __global__ void k_cc_scan(ContactArgs a);
 __global__ void k_cc_fill(ContactArgs a);
 __global__ void k_cc_pairs(ContactArgs a);
 __global__ void k_cc_terms(ContactArgs a);
-__global__ void k_cc_band(ContactArgs a);
+__global__ void k_cc_band(ContactArgs a, const double *f, double *y);
 __global__ void k_cc_ground(ContactArgs a, const int32_t *node_dof, const int32_t *node_sys,
                             const double *nt);
 __global__ void k_cc_clear(ContactArgs a);
-__global__ void k_cc_reset_bw(ContactArgs a);
 __global__ void k_cc_decide(ContactArgs a, SolveArgs v);
-__global__ void k_lu_diag(ContactArgs a, int c, int k);
-__global__ void k_lu_trsm(ContactArgs a, int c, int k);
-__global__ void k_lu_gemm(ContactArgs a, int c, int k);
-__global__ void k_cc_subst(ContactArgs a, SolveArgs v);
-__global__ void k_cc_transpose(ContactArgs a, int c);
+__global__ void k_cc_transpose(ContactArgs a);
+// LU and solve of the systems with cgo set: v.dq holds the right-hand side;
+// max_n: DOFs of the largest system.
+cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int max_n, int sms, cudaStream_t st);
 
 // Adjoint of one implicit step (single rods): right-hand side, state and
 // natural-curvature gradients.
