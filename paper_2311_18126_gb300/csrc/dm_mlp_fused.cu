@@ -1,29 +1,32 @@
-// Inference of the warm-start network (64 -> 256 -> 256 -> 256 -> 64, ReLU
-// on the hidden layers; BF16 operands, FP32 accumulation) in one persistent
-// kernel: a CTA per SM takes 128-row tiles of the input in turn and runs the
-// four layers on chip, so the hidden activations never leave shared memory.
+// The warm-start network (64 -> 256 -> 256 -> 256 -> 64, ReLU on the hidden
+// layers; BF16 operands, FP32 accumulation) on chip: one persistent kernel, a
+// CTA per SM taking 128-row tiles of the input in turn, for inference and,
+// with the loss and the whole backward chain behind it, for training; and the
+// weight gradients of all layers in a second kernel.
 //
 //   * operands in shared memory in the tensor core's K-major layout with the
 //     128-byte swizzle (8-row groups of 1024 bytes), written by TMA tiled
 //     loads (cp.async.bulk.tensor, tensor maps with SWIZZLE_128B) for the
 //     input and the weights, and by the epilogue's swizzled stores for the
-//     activations;
-//   * the output layer's weights (64 x 256) stay resident; the 9 weight
-//     blocks of layers 1-3 per tile ([256 x 64] each: layer 1's, then four
-//     K-blocks of each hidden layer) stream through a 3-stage ring from L2,
-//     loaded two blocks ahead of the tensor core;
-//   * warp 0 issues TMA and tcgen05.mma (M = 128, K = 16 per instruction;
-//     lane 0 issues, the whole warp takes the waits, so no lane of it spins
-//     while lane 0 has work); the hidden layers accumulate into 256 fp32
-//     columns of tensor memory, the output layer into 64 others;
-//     tcgen05.commit signals the ring's free slots and the end of a layer;
-//   * eight warps read the accumulator back (tcgen05.ld; warp w the lanes
-//     32 (w % 4).. and half w / 4 of the columns, all loads before one
-//     wait), add the bias, apply ReLU, round to BF16 and store the next
-//     layer's operand with the swizzle, or write the FP32 output;
-//   * the next tile's input is loaded as soon as layer 1 has consumed the
-//     current one, and its layer 1 runs while the output of the current one
-//     is written.
+//     activations (or gradients), which stay in one 64 KB buffer;
+//   * the output layer's weights (64 x 256) stay resident; the other weight
+//     blocks ([256 x 64] each: 9 per tile in inference -- layer 1's, four
+//     K-blocks of each hidden layer -- and the transposed ones of the backward
+//     chain after them in training) stream through a 3-stage ring from L2;
+//   * warp 9 issues the TMA loads, warp 8 the MMAs (M = 128, K = 16 per
+//     instruction) and the TMA stores, warps 0-7 read the accumulators back
+//     (tcgen05.ld; warp w the lanes 32 (w % 4).. and half w / 4 of each 64
+//     columns), add the bias, apply ReLU (or the saved mask), round to BF16
+//     and store the next layer's operand;
+//   * a layer's epilogue hands its operand over in four K-blocks, and two
+//     accumulators (256 fp32 columns of tensor memory each) alternate, so the
+//     next layer's MMAs start when the first 64 columns are ready instead of
+//     after the last: what bounds a tile is the epilogues, the tensor core
+//     works beside them.
+// Training keeps the ReLU masks in registers, forms the loss and its gradient
+// in the output epilogue, and stores the hidden activations and the gradients
+// of every layer row-major by TMA (k_mlp_wgrad reads them as they are, with
+// MN-major descriptors: no transposed copies).
 // Every mbarrier wait is bounded: on timeout the kernel records an error,
 // waits (bounded) for its copies in flight, frees its tensor memory and
 // returns.
@@ -32,29 +35,33 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 
 #include "dm_internal.h"
+#include "dm_mlp.cuh"
 #include "dm_tc.cuh"
 
 namespace dm {
 
 namespace {
 
-constexpr int kTM = 128;  // rows per tile
-constexpr int kThreadsF = 256;  // 8 warps: warp w reads lanes 32 (w % 4).., columns half w / 4
+constexpr int kTM = 128;         // rows per tile
+constexpr int kEpi = 256;        // epilogue threads (8 warps)
+constexpr int kThreadsF = kEpi + 64;  // and the MMA and the TMA warp
 constexpr int kStages = 3;
-constexpr int kBlocksPerTile = 9;  // streamed weight blocks per tile: W1, 4 of W2, 4 of W3
 // shared memory map (bytes from a 1024-aligned base)
 constexpr int kOffW4 = 0;                       // 4 K-blocks of [64][64] bf16: 32 KB
 constexpr int kOffH = kOffW4 + 4 * 64 * 128;    // 4 K-blocks of [128][64]: 64 KB
-constexpr int kOffX = kOffH + 4 * kTM * 128;    // [128][64]: 16 KB
+constexpr int kOffX = kOffH + 4 * kTM * 128;    // [128][64]: 16 KB (input; output gradient)
 constexpr int kOffRing = kOffX + kTM * 128;     // 3 x [256][64]: 96 KB
 constexpr int kStageBytes = 256 * 128;
 constexpr int kOffBias = kOffRing + kStages * kStageBytes;  // fp32 biases: 3 x 256 + 64
 constexpr int kOffBar = kOffBias + (3 * 256 + 64) * 4;
-constexpr int kSmemFused = kOffBar + 128 + 1024;  // barriers, TMEM slot, alignment slack
-constexpr uint32_t kTmemCols = 512;  // hidden accumulator at 0, output accumulator at 256
+constexpr int kNumBars = 2 * kStages + 12;
+constexpr int kSmemFused = kOffBar + 8 * kNumBars + 16 + 1024;  // barriers, TMEM slot, alignment slack
+static_assert(kSmemFused <= 227 * 1024, "shared memory of the fused kernel");
+constexpr uint32_t kTmemCols = 512;  // two accumulators of 256 columns
 
 constexpr unsigned kFullMask = 0xffffffffu;
 
@@ -63,37 +70,90 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// Bounded wait that also gives up when another role of the CTA has failed.
+__device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, volatile int *fail) {
+  const uint32_t a = tc::smem_u32(bar);
+  for (uint32_t it = 0; it < tc::kWaitLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 255u) == 255u && *fail) return false;
+  }
+  *fail = 1;
+  return false;
+}
+__device__ __forceinline__ void arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tma_store_2d(const void *tmap, int x, int y, const void *src) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                   reinterpret_cast<uint64_t>(tmap)),
+               "r"(x), "r"(y), "r"(tc::smem_u32(src))
+               : "memory");
+}
+__device__ __forceinline__ void store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void store_read_wait() {  // the sources have been read
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+struct FusedMaps {
+  CUtensorMap x, w1, w2, w3, w4;  // loads
+  CUtensorMap t4, t3, t2;         // training: transposed weights
+  CUtensorMap a[3], d[3], dy;     // training: stores of activations and gradients
+};
+
+struct TrainArgs {
+  const float *target;  // [M][n_valid]
+  int n_valid;
+  float scale_den;      // M n_valid
+  double loss_den;
+  double *loss;
+  float *gb4;           // [CTAs][4][64] partial sums of the output gradient
+};
+
 }  // namespace
 
+template <bool TRAIN>
 __global__ void __launch_bounds__(kThreadsF, 1)
-    k_mlp_fused(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
-                const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ CUtensorMap tm_w3,
-                const __grid_constant__ CUtensorMap tm_w4, const float *__restrict__ b1,
+    k_mlp_fused(const __grid_constant__ FusedMaps maps, const float *__restrict__ b1,
                 const float *__restrict__ b2, const float *__restrict__ b3,
-                const float *__restrict__ b4, float *__restrict__ Y, int ntiles, int *err) {
+                const float *__restrict__ b4, float *__restrict__ Y, int ntiles, int *err, TrainArgs ta) {
   using namespace tc;
+  constexpr int kBlocks = TRAIN ? 18 : 9;  // streamed weight blocks per tile
   extern __shared__ char smem_raw[];
   char *smem = reinterpret_cast<char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   char *W4s = smem + kOffW4, *Hs = smem + kOffH, *Xs = smem + kOffX, *Ring = smem + kOffRing;
   float *sbias = reinterpret_cast<float *>(smem + kOffBias);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kOffBar);
-  uint64_t *bar_w4 = bar, *bar_x = bar + 1, *bar_mma = bar + 2;
-  uint64_t *bar_full = bar + 3, *bar_free = bar + 3 + kStages;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 3 + 2 * kStages);
+  uint64_t *bar_full = bar, *bar_free = bar + kStages, *bar_acc = bar + 2 * kStages;
+  uint64_t *bar_h = bar_acc + 2, *bar_w4 = bar_h + 4, *bar_x = bar_w4 + 1, *bar_xfree = bar_w4 + 2;
+  uint64_t *bar_dy = bar_w4 + 3, *bar_stored = bar_w4 + 4;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + kNumBars);
   volatile int *fail = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
   const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  const int total_blocks = my_tiles * kBlocksPerTile;
 
-  if (warp == 0) {
+  if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int i = 0; i < 3 + 2 * kStages; ++i) mbar_init(&bar[i], 1);
+    for (int i = 0; i < 2 * kStages + 2; ++i) mbar_init(&bar[i], 1);
+    for (int i = 0; i < 4; ++i) mbar_init(&bar_h[i], kEpi);
+    mbar_init(bar_w4, 1);
+    mbar_init(bar_x, 1);
+    mbar_init(bar_xfree, TRAIN ? 2 : 1);
+    mbar_init(bar_dy, kEpi);
+    mbar_init(bar_stored, 1);
     *fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
@@ -102,206 +162,410 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tmem_slot, tmem_out = tmem + 256;
+  const uint32_t tmem = *tmem_slot;
 
-  // Warp 0 issues the copies and the MMAs: it runs the issue path as a
-  // whole (every lane takes the same waits, lane 0 issues), so that no lane
-  // of it spins on a barrier while lane 0 has work to do.
-  int issued = 0;      // weight blocks whose load was issued (warp 0)
-  int x_loads = 0;     // input tiles whose load was issued (warp 0)
-  bool x_pending = false;
-  // weight block g of this CTA's stream: W1 (g % 9 == 0), else K-block
-  // (g % 9 - 1) % 4 of W2 (g % 9 <= 4) or W3
-  auto load_block = [&](int g) -> bool {  // warp 0
-    const int s = g % kStages, b = g % kBlocksPerTile;
-    bool w = true;
-    if (g >= kStages) w = mbar_wait(&bar_free[s], (uint32_t)((g / kStages - 1) & 1));
-    if (!__all_sync(kFullMask, w)) return false;
-    if (lane == 0) {
-      mbar_expect_tx(&bar_full[s], (uint32_t)kStageBytes);
-      const void *map = b == 0 ? (const void *)&tm_w1 : (b <= 4 ? (const void *)&tm_w2 : (const void *)&tm_w3);
-      tma_load_2d(Ring + s * kStageBytes, map, b == 0 ? 0 : 64 * ((b - 1) % 4), 0, &bar_full[s]);
+  if (warp == 9) {
+    // ---- TMA loads: the resident weights, then per tile its input and the
+    // weight blocks in the order of use, as far ahead as the ring allows
+    if (lane == 0 && my_tiles > 0) {
+      mbar_expect_tx(bar_w4, 4 * 64 * 128);
+      for (int kb = 0; kb < 4; ++kb) tma_load_2d(W4s + kb * 64 * 128, &maps.w4, 64 * kb, 0, bar_w4);
+      int g = 0, loaded = 0;
+      bool ok = true;
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        if (i > 0 && !(ok = wait_on(bar_xfree, (uint32_t)((i - 1) & 1), fail))) break;
+        mbar_expect_tx(bar_x, kTM * 128);
+        tma_load_2d(Xs, &maps.x, 0, ((int)blockIdx.x + i * (int)gridDim.x) * kTM, bar_x);
+        loaded = i + 1;
+        for (int b = 0; b < kBlocks; ++b, ++g) {
+          const int s = g % kStages;
+          if (g >= kStages && !(ok = wait_on(&bar_free[s], (uint32_t)((g / kStages - 1) & 1), fail))) break;
+          mbar_expect_tx(&bar_full[s], (uint32_t)kStageBytes);
+          const CUtensorMap *map = b == 0   ? &maps.w1
+                                   : b <= 4 ? &maps.w2
+                                   : b <= 8 ? &maps.w3
+                                   : b == 9 ? &maps.t4
+                                   : b < 14 ? &maps.t3
+                                            : &maps.t2;
+          const int kb = b == 0 || b == 9 ? 0 : (b < 9 ? (b - 1) & 3 : (b - 10) & 3);
+          tma_load_2d(Ring + s * kStageBytes, map, 64 * kb, 0, &bar_full[s]);
+        }
+      }
+      if (!ok || *fail) {  // what is in flight lands before the CTA leaves (bounded)
+        mbar_wait(bar_w4, 0);
+        for (int k = g > kStages ? g - kStages : 0; k < g; ++k)
+          mbar_wait(&bar_full[k % kStages], (uint32_t)((k / kStages) & 1));
+        if (loaded) mbar_wait(bar_x, (uint32_t)((loaded - 1) & 1));
+      }
     }
-    __syncwarp();
-    issued = g + 1;
-    return true;
-  };
-  // warp 0: the MMAs of weight blocks g0 .. g0 + nb - 1 from the ring into
-  // the hidden accumulator, A = the input tile (layer 1) or the activations
-  // in H; the next loads two blocks ahead; then the layer's commit
-  auto ring_layer = [&](int g0, int nb, bool from_x) -> bool {
-    for (int b = 0; b < nb; ++b) {
-      const int g = g0 + b, s = g % kStages;
-      if (!__all_sync(kFullMask, mbar_wait(&bar_full[s], (uint32_t)((g / kStages) & 1))))
-        return false;
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      if (lane == 0) {
-        const uint32_t a0 = smem_u32(from_x ? Xs : Hs + b * (kTM * 128));
-        const uint32_t w0 = smem_u32(Ring + s * kStageBytes);
+  } else if (warp == 8) {
+    // ---- MMAs and stores, by one lane
+    if (lane == 0 && my_tiles > 0) {
+      int g = 0, ph = 0, hphase = 0;
+      bool ok = true;
+      // K-block b of a layer: A at `a`, B at `w` (N rows), into accumulator ph
+      auto mma_block = [&](const char *a, const char *w, int n, bool first) {
+        const uint32_t a0 = smem_u32(a), w0 = smem_u32(w), d = tmem + 256u * (uint32_t)(ph & 1);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_bf16(tmem, make_desc(a0 + 32 * kk, 16, 1024, kSwizzle128B),
-                   make_desc(w0 + 32 * kk, 16, 1024, kSwizzle128B), make_idesc(kTM, 256),
-                   (b | kk) ? 1u : 0u);
-        mma_commit(&bar_free[s]);
-      }
-      __syncwarp();
-      if (g + 2 < total_blocks && !load_block(g + 2)) return false;
-    }
-    if (lane == 0) mma_commit(bar_mma);
-    __syncwarp();
-    return true;
-  };
-  // warp 0: layer 1 of local tile i (its input and W1 block must land)
-  auto issue_layer1 = [&](int i) -> bool {
-    if (!__all_sync(kFullMask, mbar_wait(bar_x, (uint32_t)(i & 1)))) return false;
-    x_pending = false;
-    return ring_layer(i * kBlocksPerTile, 1, true);
-  };
-
-  if (warp == 0 && my_tiles > 0) {
-    if (lane == 0) {
-      mbar_expect_tx(bar_w4, 4 * 64 * 128);
-      for (int kb = 0; kb < 4; ++kb) tma_load_2d(W4s + kb * 64 * 128, &tm_w4, 64 * kb, 0, bar_w4);
-      mbar_expect_tx(bar_x, kTM * 128);
-      tma_load_2d(Xs, &tm_x, 0, (int)blockIdx.x * kTM, bar_x);
-    }
-    __syncwarp();
-    x_pending = true;
-    x_loads = 1;
-    bool w = true;
-    for (int g = 0; g < 2 && g < total_blocks; ++g) w = w && load_block(g);
-    w = w && __all_sync(kFullMask, mbar_wait(bar_w4, 0));
-    w = w && issue_layer1(0);
-    if (!w && lane == 0) *fail = 1;
-  }
-  __syncthreads();
-  bool ok = !*fail;
-  uint32_t mma_phase = 0;
-  const int quarter = warp & 3, half = warp >> 2;
-  const int row = quarter * 32 + lane;  // this thread's accumulator lane / tile row
-  const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-
-  // all threads: the end of a layer's MMAs (bounded), agreed by the block
-  auto layer_done = [&]() -> bool {
-    bool w = mbar_wait(bar_mma, mma_phase);
-    mma_phase ^= 1u;
-    w = __syncthreads_and(w && !*fail) != 0;
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    return w;
-  };
-  // epilogue of a hidden layer: accumulator + bias, ReLU, BF16 into H; the
-  // thread's row, columns [128 half, 128 half + 128) (eight loads from
-  // tensor memory, one wait)
-  auto hidden_epilogue = [&](const float *bias) {
-    const int cb = 128 * half;
-    uint32_t r[128];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) tmem_ld16_nowait(tmem + lane_off + (uint32_t)(cb + 16 * q), r + 16 * q);
-    tmem_wait();
-#pragma unroll
-    for (int kb = 0; kb < 2; ++kb) {
-      // K-block (cb + 64 kb) / 64 of H, this row's eight 16-byte chunks, swizzled
-      char *rowp = Hs + ((cb >> 6) + kb) * (kTM * 128) + row * 128;
-#pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {
-        const int c = 64 * kb + 8 * ch;
-        const float4 bl = *reinterpret_cast<const float4 *>(bias + cb + c);
-        const float4 bh = *reinterpret_cast<const float4 *>(bias + cb + c + 4);
-        const float *a = reinterpret_cast<const float *>(r + c);
-        const uint32_t p0 = pack_bf16(fmaxf(a[0] + bl.x, 0.0f), fmaxf(a[1] + bl.y, 0.0f));
-        const uint32_t p1 = pack_bf16(fmaxf(a[2] + bl.z, 0.0f), fmaxf(a[3] + bl.w, 0.0f));
-        const uint32_t p2 = pack_bf16(fmaxf(a[4] + bh.x, 0.0f), fmaxf(a[5] + bh.y, 0.0f));
-        const uint32_t p3 = pack_bf16(fmaxf(a[6] + bh.z, 0.0f), fmaxf(a[7] + bh.w, 0.0f));
-        *reinterpret_cast<uint4 *>(rowp + ((ch ^ (row & 7)) << 4)) = make_uint4(p0, p1, p2, p3);
-      }
-    }
-    // the generic-proxy stores become visible to the tensor core's reads
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-  };
-
-  for (int i = 0; i < my_tiles && ok; ++i) {
-    const int tile = (int)blockIdx.x + i * (int)gridDim.x;
-    const int g0 = i * kBlocksPerTile;
-    // layer 1 was issued before (the prologue, or the previous tile)
-    if (!(ok = layer_done())) break;
-    if (warp == 0 && i + 1 < my_tiles) {  // the input buffer is free: next tile's input
-      if (lane == 0) {
-        mbar_expect_tx(bar_x, kTM * 128);
-        tma_load_2d(Xs, &tm_x, 0, (tile + (int)gridDim.x) * kTM, bar_x);
-      }
-      __syncwarp();
-      x_pending = true;
-      ++x_loads;
-    }
-    hidden_epilogue(sbias);
-    // layers 2 and 3: A = H, B = streamed blocks
-    for (int l = 0; l < 2 && ok; ++l) {
-      if (warp == 0 && !*fail && !ring_layer(g0 + 1 + 4 * l, 4, false) && lane == 0) *fail = 1;
-      if (!(ok = layer_done())) break;
-      hidden_epilogue(sbias + 256 * (l + 1));
-    }
-    if (!ok) break;
-    // layer 4 (N = 64, resident weights) into the output accumulator
-    if (warp == 0 && !*fail) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      if (lane == 0) {
-#pragma unroll
-        for (int kb = 0; kb < 4; ++kb) {
-          const uint32_t a0 = smem_u32(Hs + kb * (kTM * 128)), w0 = smem_u32(W4s + kb * 64 * 128);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_bf16(tmem_out, make_desc(a0 + 32 * kk, 16, 1024, kSwizzle128B),
-                     make_desc(w0 + 32 * kk, 16, 1024, kSwizzle128B), make_idesc(kTM, 64),
-                     (kb | kk) ? 1u : 0u);
+          mma_bf16(d, make_desc(a0 + 32 * kk, 16, 1024, kSwizzle128B),
+                   make_desc(w0 + 32 * kk, 16, 1024, kSwizzle128B), make_idesc(kTM, n), (first && kk == 0) ? 0u : 1u);
+      };
+      // a layer whose operand the epilogue leaves in H, K-block by K-block; its
+      // copy to global memory (training) goes out as each block is complete
+      auto h_layer = [&](bool resident, const CUtensorMap *st, int y) {
+        for (int kb = 0; kb < 4 && ok; ++kb) {
+          if (!(ok = wait_on(&bar_h[kb], (uint32_t)(hphase & 1), fail))) return;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          if (TRAIN) tma_store_2d(st, 64 * kb, y, Hs + kb * (kTM * 128));
+          if (resident) {
+            mma_block(Hs + kb * (kTM * 128), W4s + kb * 64 * 128, 64, kb == 0);
+          } else {
+            const int s = g % kStages;
+            if (!(ok = wait_on(&bar_full[s], (uint32_t)((g / kStages) & 1), fail))) return;
+            mma_block(Hs + kb * (kTM * 128), Ring + s * kStageBytes, 256, kb == 0);
+            mma_commit(&bar_free[s]);
+            ++g;
+          }
         }
-        mma_commit(bar_mma);
+        mma_commit(&bar_acc[ph & 1]);
+        ++ph;
+        ++hphase;
+        if (TRAIN) {
+          store_commit();
+          store_read_wait();
+          arrive(bar_stored);
+        }
+      };
+      // a layer whose operand is the input tile (or the output gradient in its place)
+      auto x_layer = [&]() {
+        const int s = g % kStages;
+        if (!(ok = wait_on(&bar_full[s], (uint32_t)((g / kStages) & 1), fail))) return;
+        mma_block(Xs, Ring + s * kStageBytes, 256, true);
+        mma_commit(&bar_free[s]);
+        ++g;
+      };
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        const int y = ((int)blockIdx.x + i * (int)gridDim.x) * kTM;
+        if (!(ok = wait_on(bar_x, (uint32_t)(i & 1), fail))) break;
+        x_layer();
+        if (!ok) break;
+        if (!TRAIN) mma_commit(bar_xfree);
+        mma_commit(&bar_acc[ph & 1]);
+        ++ph;
+        h_layer(false, &maps.a[0], y);
+        if (ok) h_layer(false, &maps.a[1], y);
+        if (ok && i == 0) ok = wait_on(bar_w4, 0, fail);
+        if (ok) h_layer(true, &maps.a[2], y);
+        if (TRAIN && ok) {
+          if (!(ok = wait_on(bar_dy, (uint32_t)(i & 1), fail))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          tma_store_2d(&maps.dy, 0, y, Xs);
+          store_commit();
+          x_layer();
+          if (!ok) break;
+          mma_commit(bar_xfree);
+          mma_commit(&bar_acc[ph & 1]);
+          ++ph;
+          store_read_wait();
+          arrive(bar_xfree);
+          h_layer(false, &maps.d[2], y);
+          if (ok) h_layer(false, &maps.d[1], y);
+          for (int kb = 0; kb < 4 && ok; ++kb) {  // the first layer's gradient is only stored
+            if (!(ok = wait_on(&bar_h[kb], (uint32_t)(hphase & 1), fail))) break;
+            tma_store_2d(&maps.d[0], 64 * kb, y, Hs + kb * (kTM * 128));
+          }
+          if (!ok) break;
+          ++hphase;
+          store_commit();
+          store_read_wait();
+          arrive(bar_stored);
+        }
       }
-      __syncwarp();
+      if (TRAIN) store_wait();
+      if (!ok || *fail) {
+        // every MMA issued so far is done before the tensor memory is freed
+        mma_commit(bar_w4);
+        mbar_wait(bar_w4, 1);
+      }
     }
-    if (!(ok = layer_done())) break;
-    // the next tile's layer 1 (hidden accumulator) runs under this epilogue
-    if (warp == 0 && i + 1 < my_tiles && !issue_layer1(i + 1) && lane == 0) *fail = 1;
-    {
-      // the thread's row, columns [32 half, 32 half + 32) of the output
-      float *yrow = Y + ((size_t)tile * kTM + row) * 64 + 32 * half;
-      const float *bo = sbias + 768 + 32 * half;
-      uint32_t r[32];
-      tmem_ld16_nowait(tmem_out + lane_off + (uint32_t)(32 * half), r);
-      tmem_ld16_nowait(tmem_out + lane_off + (uint32_t)(32 * half + 16), r + 16);
-      tmem_wait();
-      float4 *o = reinterpret_cast<float4 *>(yrow);
+  } else {
+    // ---- epilogues
+    const int quarter = warp & 3, half = warp >> 2;
+    const int row = quarter * 32 + lane;  // this thread's accumulator lane / tile row
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    int ph = 0, stores = 0;
+    bool ok = true;
+    uint32_t mask[TRAIN ? 3 : 1][4];  // training: ReLU masks of the hidden layers
+    float gb = 0.0f;                  // training: output column 32 half + lane's gradient sum
+    auto acc_ready = [&]() -> uint32_t {
+      ok = ok && wait_on(&bar_acc[ph & 1], (uint32_t)((ph >> 1) & 1), fail);
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t t = tmem + 256u * (uint32_t)(ph & 1) + lane_off;
+      ++ph;
+      return t;
+    };
+    // 32 accumulator columns to the thread's row of a K-block in H (or Xs):
+    // its half of the row's eight 16-byte chunks, swizzled
+    auto put = [&](char *blk, const float *v) {
+      char *rowp = blk + row * 128;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float4 bb = *reinterpret_cast<const float4 *>(bo + 4 * j);
-        o[j] = make_float4(__uint_as_float(r[4 * j]) + bb.x, __uint_as_float(r[4 * j + 1]) + bb.y,
-                           __uint_as_float(r[4 * j + 2]) + bb.z, __uint_as_float(r[4 * j + 3]) + bb.w);
+      for (int ch = 0; ch < 4; ++ch) {
+        const float *a = v + 8 * ch;
+        *reinterpret_cast<uint4 *>(rowp + (((4 * half + ch) ^ (row & 7)) << 4)) =
+            make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
+      }
+      // the generic-proxy stores become visible to the tensor core's (and TMA's) reads
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    };
+    // hidden layer l, forward (bias, ReLU) or backward (mask), into H
+    auto hidden = [&](int l, bool back) {
+      const uint32_t t = acc_ready();
+      if (!ok) return;
+      if (TRAIN && stores > 0 && !(ok = wait_on(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
+      ++stores;
+      uint32_t r[2][32];
+      tmem_ld16_nowait(t + (uint32_t)(32 * half), r[0]);
+      tmem_ld16_nowait(t + (uint32_t)(32 * half + 16), r[0] + 16);
+#pragma unroll
+      for (int kb = 0; kb < 4; ++kb) {
+        tmem_wait32(r[kb & 1]);
+        if (kb < 3) {  // the next block's columns come in behind this one's arithmetic
+          tmem_ld16_nowait(t + (uint32_t)(64 * (kb + 1) + 32 * half), r[(kb + 1) & 1]);
+          tmem_ld16_nowait(t + (uint32_t)(64 * (kb + 1) + 32 * half + 16), r[(kb + 1) & 1] + 16);
+        }
+        float v[32];
+        if (!TRAIN || !back) {
+          const float *bias = sbias + 256 * l + 64 * kb + 32 * half;
+          uint32_t mk = 0;
+#pragma unroll
+          for (int j = 0; j < 32; j += 4) {
+            const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
+            v[j] = fmaxf(__uint_as_float(r[kb & 1][j]) + bb.x, 0.0f);
+            v[j + 1] = fmaxf(__uint_as_float(r[kb & 1][j + 1]) + bb.y, 0.0f);
+            v[j + 2] = fmaxf(__uint_as_float(r[kb & 1][j + 2]) + bb.z, 0.0f);
+            v[j + 3] = fmaxf(__uint_as_float(r[kb & 1][j + 3]) + bb.w, 0.0f);
+            if (TRAIN)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) mk |= v[j + k] > 0.0f ? 1u << (j + k) : 0u;
+          }
+          if (TRAIN) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+              if (k == l) mask[TRAIN ? k : 0][kb] = mk;
+          }
+        } else {
+          uint32_t mk = 0;
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            if (k == l) mk = mask[TRAIN ? k : 0][kb];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = (mk >> j) & 1u ? __uint_as_float(r[kb & 1][j]) : 0.0f;
+        }
+        put(Hs + kb * (kTM * 128), v);
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        arrive(&bar_h[kb]);
+      }
+    };
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int tile = (int)blockIdx.x + i * (int)gridDim.x;
+#pragma unroll
+      for (int l = 0; l < 3; ++l)
+        if (ok) hidden(l, false);
+      if (!ok) break;
+      const uint32_t t = acc_ready();
+      if (!ok) break;
+      uint32_t r[32];
+      tmem_ld16_nowait(t + (uint32_t)(32 * half), r);
+      tmem_ld16_nowait(t + (uint32_t)(32 * half + 16), r + 16);
+      tmem_wait32(r);
+      const float *bo = sbias + 768 + 32 * half;
+      if (!TRAIN) {
+        // the thread's row, columns [32 half, 32 half + 32) of the output
+        float4 *o = reinterpret_cast<float4 *>(Y + ((size_t)tile * kTM + row) * 64 + 32 * half);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float4 bb = *reinterpret_cast<const float4 *>(bo + 4 * j);
+          o[j] = make_float4(__uint_as_float(r[4 * j]) + bb.x, __uint_as_float(r[4 * j + 1]) + bb.y,
+                             __uint_as_float(r[4 * j + 2]) + bb.z, __uint_as_float(r[4 * j + 3]) + bb.w);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
+      } else {
+        // loss (summed in FP64) and its gradient on the first n_valid columns
+        const float *yt = ta.target + ((size_t)tile * kTM + row) * ta.n_valid;
+        double ls = 0.0;
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int c = 32 * half + j;
+          v[j] = 0.0f;
+          if (c < ta.n_valid) {  // uniform over the CTA
+            const float d = __uint_as_float(r[j]) + bo[j] - yt[c];
+            ls += (double)d * d;
+            v[j] = 2.0f * d / ta.scale_den;
+            float sum = v[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFullMask, sum, o);
+            if (lane == j) gb += sum;
+          }
+        }
+        put(Xs, v);
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        arrive(bar_dy);
+        if (32 * half < ta.n_valid) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(kFullMask, ls, o);
+          if (lane == 0) atomicAdd(ta.loss, ls / ta.loss_den);
+        }
+#pragma unroll
+        for (int l = 2; l >= 0; --l)
+          if (ok) hidden(l, true);
       }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();  // the output accumulator is read before the next tile's layer 4
-  }
-  if (!ok || *fail) {
-    if (tid == 0) {
-      atomicExch(err, 1);
-      // copies in flight land before the CTA leaves (bounded)
-      for (int g = (int)(issued > 3 ? issued - 3 : 0); g < issued; ++g)
-        mbar_wait(&bar_full[g % kStages], (uint32_t)((g / kStages) & 1));
-      if (x_pending) mbar_wait(bar_x, (uint32_t)((x_loads - 1) & 1));
-      // every MMA issued so far is done before the tensor memory is freed
-      mma_commit(bar_mma);
-      mbar_wait(bar_mma, mma_phase);
-    }
+    if (TRAIN) ta.gb4[((size_t)blockIdx.x * 4 + quarter) * 64 + 32 * half + lane] = gb;
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == 0)
+  if (tid == 0 && *fail) atomicExch(err, 1);
+  if (warp == 8)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 
 namespace {
+
+// ---- weight gradients: dW_l = dZ_l^T A_(l-1) over the batch, all layers in
+// one launch.  A CTA takes 128 rows of one layer's dW (for the output layer,
+// whose 64 rows are too few, of its transpose) and a share of the batch, 64
+// batch rows per stage: both operands are [batch][width] arrays whose width is
+// the MMA's M or N, so the descriptors are MN-major (64-wide boxes with the
+// 128-byte swizzle: 8 batch rows of 128 bytes per swizzle group, the boxes
+// 8 KB apart).  The hidden biases' gradients are the same product with a
+// column of ones (N = 16, one small extra MMA).  Partials per share, summed in
+// a fixed order by k_mlp_update.
+constexpr int kGStages = 4;
+constexpr int kGBox = 64 * 128;                 // bytes of a 64 x 64 box
+constexpr int kGStageBytes = 6 * kGBox;         // 2 boxes of M, up to 4 of N
+constexpr int kGOffOnes = kGStages * kGStageBytes;
+constexpr int kGOffBar = kGOffOnes + 512;
+constexpr int kSmemGrad = kGOffBar + 8 * (2 * kGStages + 1) + 16 + 1024;
+static_assert(kSmemGrad <= 227 * 1024, "shared memory of the weight-gradient kernel");
+
+struct GradMaps {
+  CUtensorMap m[4], n[4];  // per layer: the operand along M, along N
+};
+
+__host__ __device__ constexpr uint32_t make_idesc_mn(int M, int N, bool b_mn) {
+  return tc::make_idesc(M, N) | (1u << 15) | (b_mn ? 1u << 16 : 0u);
+}
+
+__global__ void __launch_bounds__(192, 1)
+    k_mlp_wgrad(const __grid_constant__ GradMaps maps, int nkb, int s_small, int s_big, float *part, int *err) {
+  using namespace tc;
+  extern __shared__ char smem_raw[];
+  char *smem = reinterpret_cast<char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kGOffBar);
+  uint64_t *bar_full = bar, *bar_free = bar + kGStages, *bar_done = bar + 2 * kGStages;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_done + 1);
+  volatile int *fail = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  // block -> layer, row tile, share z of S
+  int u = blockIdx.x, l = 0;
+  int S = s_small;
+  while (u >= 2 * S) {
+    u -= 2 * S;
+    ++l;
+    S = l == 0 || l == 3 ? s_small : s_big;
+  }
+  const int mt = u & 1, z = u >> 1;
+  const int N = l == 0 || l == 3 ? 64 : 256;
+  const int k0 = (int)((int64_t)nkb * z / S), k1 = (int)((int64_t)nkb * (z + 1) / S);
+  const bool bias = l < 3;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2 * kGStages + 1; ++i) mbar_init(&bar[i], 1);
+    *fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (tid < 128) reinterpret_cast<uint32_t *>(smem + kGOffOnes)[tid] = 0x3F803F80u;  // ones, bf16
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tmem_slot;
+  if (warp == 5) {
+    if (lane == 0) {
+      bool ok = true;
+      int g = 0;
+      for (int k = k0; k < k1; ++k, ++g) {
+        const int s = g % kGStages;
+        if (g >= kGStages && !(ok = wait_on(&bar_free[s], (uint32_t)((g / kGStages - 1) & 1), fail))) break;
+        char *st = smem + s * kGStageBytes;
+        mbar_expect_tx(&bar_full[s], (uint32_t)((2 + N / 64) * kGBox));
+        for (int b = 0; b < 2; ++b) tma_load_2d(st + b * kGBox, &maps.m[l], 128 * mt + 64 * b, 64 * k, &bar_full[s]);
+        for (int b = 0; b < N / 64; ++b) tma_load_2d(st + (2 + b) * kGBox, &maps.n[l], 64 * b, 64 * k, &bar_full[s]);
+      }
+      if (!ok || *fail)
+        for (int k = g > kGStages ? g - kGStages : 0; k < g; ++k)
+          mbar_wait(&bar_full[k % kGStages], (uint32_t)((k / kGStages) & 1));
+    }
+  } else if (warp == 4) {
+    if (lane == 0) {
+      int g = 0;
+      for (int k = k0; k < k1; ++k, ++g) {
+        const int s = g % kGStages;
+        if (!wait_on(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t a0 = smem_u32(smem + s * kGStageBytes), b0 = a0 + 2 * kGBox;
+        const uint32_t o0 = smem_u32(smem + kGOffOnes);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {  // 16 batch rows: two swizzle groups of 1024 bytes
+          const uint64_t ad = make_desc(a0 + 2048 * kk, kGBox, 1024, kSwizzle128B);
+          mma_bf16(tmem, ad, make_desc(b0 + 2048 * kk, kGBox, 1024, kSwizzle128B), make_idesc_mn(128, N, true),
+                   (g | kk) ? 1u : 0u);
+          if (bias) mma_bf16(tmem + 256u, ad, make_desc(o0, 128, 256), make_idesc_mn(128, 16, false), (g | kk) ? 1u : 0u);
+        }
+        mma_commit(&bar_free[s]);
+      }
+      mma_commit(bar_done);
+    }
+  }
+  __syncwarp();
+  // the end of every MMA issued (on a failure too, before the tensor memory is freed)
+  const bool done = mbar_wait(bar_done, 0);
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (warp < 4 && done && !*fail) {
+    // partial: [256 or 64 rows][N] of the layer, then its 256 bias sums
+    float *out = part + mlp_part_offset(l, s_small, s_big) + (size_t)z * mlp_part_size(l);
+    const int row = 128 * mt + 32 * warp + lane;
+    const uint32_t t = tmem + ((uint32_t)(32 * warp) << 16);
+    for (int c = 0; c < N; c += 32) {
+      uint32_t r[32];
+      tmem_ld16_nowait(t + (uint32_t)c, r);
+      tmem_ld16_nowait(t + (uint32_t)c + 16, r + 16);
+      tmem_wait32(r);
+      float4 *o = reinterpret_cast<float4 *>(out + (size_t)row * N + c);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        o[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
+                           __uint_as_float(r[4 * j + 3]));
+    }
+    if (bias) {
+      uint32_t r[16];
+      tmem_ld16_nowait(t + 256u, r);
+      tmem_wait();
+      out[(size_t)256 * N + row] = __uint_as_float(r[0]);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (tid == 0 && (*fail || !done)) atomicExch(err, 1);
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -330,6 +594,19 @@ bool encode(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int device_sms() {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+bool encode_forward(FusedMaps &t, int M, const void *X, const void *const W[4]) {
+  return encode(&t.x, X, (uint64_t)M, 64, kTM) && encode(&t.w1, W[0], 256, 64, 256) &&
+         encode(&t.w2, W[1], 256, 256, 256) && encode(&t.w3, W[2], 256, 256, 256) &&
+         encode(&t.w4, W[3], 64, 256, 64);
+}
+
 }  // namespace
 
 // Y [M][64] fp32 = the network on X [M][64] bf16; W[l] the bf16 weights
@@ -338,29 +615,56 @@ bool encode(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint
 // to 1 on a barrier timeout.
 cudaError_t launch_mlp_fused(int M, const void *X, const void *const W[4], const float *const b[4],
                              float *Y, int *err, cudaStream_t st) {
-  static int sms = 0;
-  static bool attr = false;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  CUtensorMap tx, t1, t2, t3, t4;
-  if (!encode(&tx, X, (uint64_t)M, 64, kTM) || !encode(&t1, W[0], 256, 64, 256) ||
-      !encode(&t2, W[1], 256, 256, 256) || !encode(&t3, W[2], 256, 256, 256) ||
-      !encode(&t4, W[3], 64, 256, 64))
-    return cudaErrorInvalidValue;
-  const int ntiles = M / kTM;
-  const int grid = ntiles < sms ? ntiles : sms;
+  FusedMaps t{};
+  if (!encode_forward(t, M, X, W)) return cudaErrorInvalidValue;
+  const int ntiles = M / kTM, grid = std::min(ntiles, device_sms());
   if (grid == 0) return cudaSuccess;
-  k_mlp_fused<<<grid, kThreadsF, kSmemFused, st>>>(tx, t1, t2, t3, t4, b[0], b[1], b[2], b[3], Y,
-                                                     ntiles, err);
+  cudaError_t e =
+      cudaFuncSetAttribute(k_mlp_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
+  if (e != cudaSuccess) return e;
+  k_mlp_fused<false><<<grid, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], Y, ntiles, err, TrainArgs{});
+  return cudaGetLastError();
+}
+
+MlpTrainShape mlp_train_shape(int M) {
+  MlpTrainShape s;
+  const int sms = device_sms(), nkb = M / 64;
+  s.ctas = std::min(M / kTM, sms);
+  // shares of the batch: the hidden layers' products load three times the
+  // bytes of the first and last layer's, all CTAs together one per SM
+  s.s_small = std::max(1, std::min(nkb, sms / 12));
+  s.s_big = std::max(1, std::min(nkb, sms / 6));
+  return s;
+}
+
+// One pass of the training kernels: activations and gradients into `act`
+// [3][M][256], `dz` [3][M][256] and `dy` [M][64] (bf16), the loss added to
+// *loss, partial weight gradients into `part` and the output bias's into
+// `gb4`.
+cudaError_t launch_mlp_train(int M, const void *X, const float *target, int n_valid, const void *const W[4],
+                             const void *const Wt[4], const float *const b[4], void *const act[3],
+                             void *const dz[3], void *dy, double *loss, float *part, float *gb4, int *err,
+                             cudaStream_t st) {
+  FusedMaps t{};
+  GradMaps g{};
+  bool ok = encode_forward(t, M, X, W) && encode(&t.t4, Wt[3], 256, 64, 256) &&
+            encode(&t.t3, Wt[2], 256, 256, 256) && encode(&t.t2, Wt[1], 256, 256, 256) &&
+            encode(&t.dy, dy, (uint64_t)M, 64, kTM);
+  for (int l = 0; l < 3 && ok; ++l)
+    ok = encode(&t.a[l], act[l], (uint64_t)M, 256, kTM) && encode(&t.d[l], dz[l], (uint64_t)M, 256, kTM) &&
+         encode(&g.m[l], dz[l], (uint64_t)M, 256, 64) &&
+         (l == 0 ? encode(&g.n[0], X, (uint64_t)M, 64, 64) : encode(&g.n[l], act[l - 1], (uint64_t)M, 256, 64));
+  ok = ok && encode(&g.m[3], act[2], (uint64_t)M, 256, 64) && encode(&g.n[3], dy, (uint64_t)M, 64, 64);
+  if (!ok) return cudaErrorInvalidValue;
+  const MlpTrainShape s = mlp_train_shape(M);
+  cudaError_t e =
+      cudaFuncSetAttribute(k_mlp_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemGrad);
+  if (e != cudaSuccess) return e;
+  const TrainArgs ta{target, n_valid, (float)(M * n_valid), (double)(M * n_valid), loss, gb4};
+  k_mlp_fused<true><<<s.ctas, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], nullptr, M / kTM, err, ta);
+  k_mlp_wgrad<<<4 * (s.s_small + s.s_big), 192, kSmemGrad, st>>>(g, M / 64, s.s_small, s.s_big, part, err);
   return cudaGetLastError();
 }
 
