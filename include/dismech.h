@@ -260,7 +260,7 @@ dm_status dm_solve_band(int32_t nsys, const int32_t *sys_dof0, const int32_t *sy
  * and separator blocks are eliminated in order, like the full band, and a
  * pivot that is zero, not finite or below 1e-13 times its row's (or its
  * Schur block's) starting diagonal entry returns DM_ERR_DEGENERATE.
- * Allocates device scratch (about 170 bytes per DOF); returns after the
+ * Allocates device scratch (about 200 bytes per DOF); returns after the
  * solve has finished. */
 dm_status dm_solve_band_partitioned(int32_t nsys, const int32_t *sys_dof0,
                                     const int32_t *sys_ndof, int64_t ntot, const double *band,

@@ -2,22 +2,31 @@
 // single-rod Jacobian of Sec. III-C, Eq. 16) that removes the sequential
 // chain over the whole rod: the DOFs of a system are cut into interiors of
 // m - 10 rows separated by 10-row separators, so that interiors do not
-// couple (|i - j| > 10 across a separator).  With B_p the interior blocks,
-// C_p their couplings to the neighbouring separators and B_p = L D L^T:
+// couple (|i - j| > 10 across a separator):
 //
-//   1. per interior, in parallel: L D L^T of B_p; forward solves
-//      Z_p = L^{-1} C_p and z_p = L^{-1} f_p; the Schur contributions
-//      Z_p^T D^{-1} Z_p and Z_p^T D^{-1} z_p (symmetry: only forward solves);
-//   2. per system: the separators' block-tridiagonal Schur system
-//      T x_S = g, T = A_SS - sum_p C_p^T B_p^{-1} C_p, eliminated block by
-//      block (10 x 10 Gauss-Jordan, no pivoting: T is symmetric, and
-//      positive definite whenever the rod Jacobian is);
-//   3. per interior, in parallel: x_p = L^{-T} D^{-1} (z_p - Z_p x_S).
+//   1. k_part_factor, a warp per interior: L D L^T from its first row to its
+//      last, the separator above carried along as ten more rows (and its own
+//      Schur complement in registers), so that what is left in the window at
+//      the end is the separator below with its coupling to the one above;
+//   2. k_part_separators, a block per system: the block-tridiagonal system of
+//      the separators (10 x 10 blocks, Gauss-Jordan without pivoting: a Schur
+//      complement of the symmetric matrix, positive definite whenever the rod
+//      Jacobian is), then x on the separators;
+//   3. k_part_back, a warp per interior: x_i = z_i - L^T x - (the upper
+//      separator's multipliers) x_top.
 //
-// The work per interior is a few times that of the plain band LDL^T, but
-// the sequential depth is m rows plus one 10 x 10 elimination per
-// separator instead of n rows.  One warp per interior or system; an
-// interior keeps its band in shared memory.
+// A column costs 230 (full band) or on average 202 (a rod's envelope: ENV)
+// updates against 65 or 49 without the carried separator, but the sequential
+// depth is m rows plus one block elimination per separator instead of n rows.
+// Bound by the FP64 pipe (64 cycles per warp instruction and SM partition):
+// the updates of a column are dealt evenly over the 32 lanes, its multipliers
+// formed once (one instruction, exchanged through shared memory), 7.75 FP64
+// slots per column of a rod; the reciprocal runs on the integer pipe.
+// Measured (GB300): the solves of one step of 64 rods of 4000-6000 nodes (1.3 M
+// DOFs, interiors of 502 rows) 12.5 -> 2.7 ms against a warp per interior that
+// factored the band, solved for the carried columns and formed the Schur
+// products one after another, with two barriers and a division per column.
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -35,15 +44,12 @@ constexpr int PW = 10;  // half bandwidth = separator width
 // amplify rounding errors without bound.
 constexpr double kTinyPivot = 1e-13;
 
-__device__ __forceinline__ double pb_recip(double d) {
-  const double ad = fabs(d);
-  if (!(ad > 1e-30 && ad < 1e30)) return 1.0 / d;
-  double r = (double)__frcp_rn((float)d);
-  double e = fma(-d, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-d, r, 1.0);
-  return fma(r, e, r);
-}
+constexpr int kRecW = 24;   // a column's record: z, l_1..l_10, 0, the ten carried rows' multipliers, 0, 0
+constexpr int kRowW = 22;   // a window row: 11 diagonals, right-hand side, coupling to the separator above
+constexpr int kPB = 12;     // columns per block (4-periodic like the envelope)
+constexpr int kPWin = 2 * kPB * kRowW;  // doubles of a window buffer
+constexpr int kPCell = 2;               // a fixed cell (the 65th separator sum)
+constexpr int kPSmem = 2 * kPWin + kPB * kRecW + kPCell;
 
 struct PartArgs {
   int64_t ntot;
@@ -53,280 +59,408 @@ struct PartArgs {
   const int32_t *sys_sep0, *sys_nsep;          // per system: first separator, count
   const double *band, *rhs;
   double *x;
-  double *Lf, *Df, *Zt, *zf;   // [ntot][10], 1/D [ntot], [ntot][10], [ntot]
-  double *Zb;                  // [nparts][10][10]: L^{-1} C_bot in the last 10 rows
-  double *ct, *cb, *co;        // [nparts][110]: top/bottom contributions (10x10 + 10), top x bottom (10x10)
+  double *rec;                 // [ntot][kRecW]
+  double *wb, *tt, *xo;        // [nparts][110]: what is left of the separator below (10x10, 10), the
+                               // Schur terms of the one above (10x10, 10), their coupling (10x10)
   double *Xs;                  // [nsep][110]: T'^{-1} [To | g']
   const int32_t *p_sys;        // interior -> system (index into go / bad)
   const int32_t *go;           // per system: solve it (NULL: all)
   int *bad;                    // per system: zero or non-finite pivot
 };
 
-// pair t in [0, 55) -> (u, v), 0 <= v <= u < 10
-__device__ __forceinline__ void pair_uv(int t, int &u, int &v) {
-  u = 0;
-  while ((u + 1) * (u + 2) / 2 <= t) ++u;
-  v = t - u * (u + 1) / 2;
+// Window tasks of a column with R rows below it, in order: row i = 1..R,
+// columns q = 1..i, the right-hand side, the ten carried rows; task t is lane
+// t mod 32's slot t / 32 (the next pivot (1, 1): lane 0's first).  Spare slots
+// repeat the lane's first task, except lane 31's last one (spare for every
+// R), which takes the 65th of the carried rows' own 65 sums (55 and ten of
+// the right-hand side; the other 64 are registers, two per lane).
+__host__ __device__ constexpr int win_tasks(int R) { return R * (R + 1) / 2 + 11 * R; }
+__host__ __device__ constexpr int win_slots(int R) { return (win_tasks(R) + 31) / 32; }
+static_assert(win_slots(10) == 6 && win_slots(9) == 5 && win_slots(8) == 4 && win_slots(7) == 4);
+static_assert(win_tasks(10) <= 191 && win_tasks(9) <= 159 && win_tasks(8) <= 127 && win_tasks(7) <= 127,
+              "lane 31's last slot is spare");
+
+extern __shared__ __align__(16) char g_psm[];
+__device__ __forceinline__ double &psm(int off) { return *reinterpret_cast<double *>(g_psm + off); }
+
+template <bool ENV>
+struct PartLane {
+  static constexpr int T = ENV ? 4 : 1, K = win_slots(10);
+  int to[T][K], uo[T][K], lo[T][K];  // byte offsets: target, column entry, multiplier (in the record)
+  int su[2], sl[2];                  // the lane's two register sums: column entry, multiplier
+  int mo, ro;                        // the lane's multiplier: source, record word
+  int adj;                           // lane 31: -1 (its last task's target does not move)
+  __device__ __forceinline__ void load(int lane, int rec, int cell) {
+    adj = lane == 31 ? -8 * kRowW : 0;
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      const int R = 10 - t, n = win_tasks(R);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        if (k >= win_slots(R)) continue;
+        int e = lane + 32 * k;
+        if (e >= n) e = lane;
+        int i = 1;
+        while (e >= i + 11) e -= i++ + 11;
+        // e < i: column q = e + 1; e == i: right-hand side; beyond: carried row e - i - 1
+        const int c = e < i ? 0 : e == i ? 11 : 12 + e - i - 1;
+        to[t][k] = 8 * (kRowW * i + (e < i ? i - e - 1 : c));
+        uo[t][k] = 8 * (e < i ? (kRowW + 1) * (e + 1) : c);
+        lo[t][k] = rec + 8 * i;
+        if (lane == 31 && k == win_slots(R) - 1) {
+          to[t][k] = cell;
+          uo[t][k] = 8 * 11;
+          lo[t][k] = rec + 8 * 21;
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int e = lane + 32 * h, k = 0;
+      while (e >= k + 2) e -= k++ + 2;
+      su[h] = 8 * (e <= k ? 12 + e : 11);
+      sl[h] = rec + 8 * (12 + k);
+    }
+    // lanes 0-9: l_1..l_10; 10-19: the carried rows; 20: z; the others repeat z
+    mo = lane < 10 ? 8 * (kRowW + 1) * (lane + 1) : lane < 20 ? 8 * (12 + lane - 10) : 8 * 11;
+    ro = rec + 8 * (lane < 10 ? lane + 1 : lane < 20 ? lane + 2 : 0);
+  }
+  // which sum (row k, column e <= k or the right-hand side) register h of the lane is
+  __device__ __forceinline__ int sum_index(int lane, int h) const {
+    int e = lane + 32 * h, k = 0;
+    while (e >= k + 2) e -= k++ + 2;
+    return e <= k ? k * PW + e : 100 + k;
+  }
+};
+
+// Column u of a block at window offset w (bytes): rj its pivot's reciprocal
+// (in), the next column's (out).
+template <bool ENV>
+__device__ __forceinline__ void part_column(const PartLane<ENV> &ln, const int t, const int u, int w, double &rj,
+                                            double (&sum)[2], bool act) {
+  constexpr int K = PartLane<ENV>::K;
+  const int NK = win_slots(10 - t);
+  const int wu = w + 8 * kRowW * u, ru = 8 * kRecW * u;
+  psm(ln.ro + ru) = psm(ln.mo + wu) * rj;
+  double uq[K], dv[K], v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (k < NK) {
+      uq[k] = psm(ln.uo[t][k] + wu);
+      dv[k] = psm(ln.to[t][k] + (k == NK - 1 && ln.adj ? 0 : wu));
+    }
+  const double s0 = psm(ln.su[0] + wu), s1 = psm(ln.su[1] + wu);
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (k < NK) v[k] = fma(-psm(ln.lo[t][k] + ru), uq[k], dv[k]);
+  rj = rcp_any(__shfl_sync(0xffffffffu, v[0], 0));
+  const double p0 = fma(-psm(ln.sl[0] + ru), s0, sum[0]), p1 = fma(-psm(ln.sl[1] + ru), s1, sum[1]);
+  if (act) {
+    sum[0] = p0;
+    sum[1] = p1;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k < NK) psm(ln.to[t][k] + (k == NK - 1 && ln.adj ? 0 : wu)) = v[k];
+  }
+  __syncwarp();
 }
 
+__device__ __forceinline__ void part_cp8(double *dst, const double *src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(on ? 8 : 0) : "memory");
+}
+
+// Interior rows row0 .. row0 + 11 (and beyond its end the separator's) into
+// the window at `buf`, zero past `rows`; the coupling to the separator above
+// (rows 0-9, J[r][k - 10]) where `top`.
+__device__ __forceinline__ void part_stage(const PartArgs &a, int r0, double *buf, int row0, int rows, bool top,
+                                           int lane) {
+#pragma unroll
+  for (int e = lane; e < kPB * kRowW; e += 32) {
+    const int d = e / kPB, s = e - d * kPB, r = row0 + s;
+    bool on = r < rows;
+    const double *src = a.rhs;
+    if (d < 11) {
+      on = on && d <= r;
+      src = a.band + (size_t)d * a.ntot + r0 + r;
+    } else if (d == 11) {
+      src = a.rhs + r0 + r;
+    } else {
+      const int k = d - 12;
+      on = on && top && k >= r;
+      src = a.band + (size_t)(r + PW - k) * a.ntot + r0 + r;
+    }
+    part_cp8(buf + s * kRowW + d, on ? src : a.rhs, on);
+  }
+}
+
+template <bool ENV>
 __global__ void __launch_bounds__(32) k_part_factor(PartArgs a) {
-  extern __shared__ double sm[];
   const int p = blockIdx.x, lane = threadIdx.x;
   const int sys = a.p_sys[p];
   if (a.go && !a.go[sys]) return;
   const int r0 = a.p_a[p], mm = a.p_mm[p];
   const bool top = a.p_top[p] >= 0, bot = a.p_bot[p] >= 0;
-  double *Bs = sm;                     // [mm][11]: band, then multipliers
-  double *Zs = a.Zt + (size_t)r0 * PW;  // [mm][10]: L^{-1} C_top (global, L2-resident)
-  const int64_t N = a.ntot;
-  for (int t = lane; t < mm * 11; t += 32) {
-    const int i = t / 11, d = t - i * 11;
-    Bs[t] = d <= i ? a.band[(size_t)d * N + r0 + i] : 0.0;
-  }
+  const int rows = mm + (bot ? PW : 0);
+  double *W = reinterpret_cast<double *>(g_psm);
+  double *R = W + 2 * kPWin, *cell = R + kPB * kRecW;
+  PartLane<ENV> ln;
+  ln.load(lane, 8 * (2 * kPWin), 8 * (2 * kPWin + kPB * kRecW));
+  // record words that no lane writes stay zero; rows outside the envelope too
+  for (int i = lane; i < kPB * kRecW + kPCell; i += 32) R[i] = 0.0;
+  part_stage(a, r0, W, 0, rows, top, lane);
+  part_stage(a, r0, W + kPB * kRowW, kPB, rows, false, lane);
+  cp_async_commit();
+  cp_async_wait_all();
   __syncwarp();
-  // band L D L^T of the interior
-  for (int j = 0; j < mm; ++j) {
-    const double dj = Bs[j * 11];
-    if (!(fabs(dj) > 0.0) || !isfinite(dj)) {
-      if (lane == 0) atomicExch(a.bad + sys, 1);
-      return;  // uniform: every lane read the same pivot
+  double rj = rcp_any(W[0]), sum[2] = {0.0, 0.0};
+  bool bad = false;
+  const int nblk = (mm + kPB - 1) / kPB;
+  for (int b = 0; b < nblk; ++b) {
+    const int j0 = b * kPB, w = b & 1 ? 8 * kPWin : 0;
+    double *cur = W + (b & 1 ? kPWin : 0), *nxt = W + (b & 1 ? 0 : kPWin);
+    const bool more = b + 1 < nblk;
+    if (more) part_stage(a, r0, nxt + kPB * kRowW, j0 + 2 * kPB, rows, false, lane);
+    cp_async_commit();
+    // the original diagonal entries of the block's rows, for the pivot test
+    const bool mine = lane < kPB && j0 + lane < mm;
+    const double diag = mine ? a.band[r0 + j0 + lane] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kPB; ++u) part_column<ENV>(ln, ENV ? (u & 3) : 0, u, w, rj, sum, j0 + u < mm);
+    if (mine) {
+      const double d = cur[kRowW * lane];
+      if (!(fabs(d) > 0.0) || !isfinite(d) || fabs(diag) * kTinyPivot > fabs(d)) bad = true;
     }
-    const double rj = pb_recip(dj);
-    if (lane == 0) a.Df[r0 + j] = rj;
-    const int i = j + 1 + lane;
-    if (lane < PW && i < mm) Bs[i * 11 + (i - j)] *= rj;  // multiplier l_ij
-    __syncwarp();
-    for (int t = lane; t < 55; t += 32) {
-      int u, v;
-      pair_uv(t, u, v);
-      const int ii = j + 1 + u, kk = j + 1 + v;
-      if (ii < mm)
-        Bs[ii * 11 + (ii - kk)] -= Bs[ii * 11 + (ii - j)] * dj * Bs[kk * 11 + (kk - j)];
+    // the block's records (12 words each of the two halves' 16-byte parts)
+    for (int e = lane; e < kPB * (kRecW / 2); e += 32) {
+      const int u = e / (kRecW / 2), h = e - u * (kRecW / 2);
+      if (j0 + u < mm)
+        *reinterpret_cast<double2 *>(a.rec + (size_t)(r0 + j0 + u) * kRecW + 2 * h) =
+            *reinterpret_cast<const double2 *>(R + u * kRecW + 2 * h);
     }
+    cp_async_wait_all();
+    __syncwarp();  // the staged rows and this block's last columns, by every lane
+    if (more)
+      for (int e = lane; e < kPB * kRowW; e += 32) nxt[e] = cur[kPB * kRowW + e];
     __syncwarp();
   }
-  // a pivot below kTinyPivot times its row's original diagonal entry counts
-  // as zero (the Jacobian need not be positive definite); checked here, in
-  // parallel, off the sequential chain
-  bool tiny = false;
-  for (int j = lane; j < mm; j += 32)
-    if (fabs(a.band[r0 + j]) * kTinyPivot * fabs(a.Df[r0 + j]) > 1.0) tiny = true;
-  if (__any_sync(0xffffffffu, tiny)) {
+  if (__any_sync(0xffffffffu, bad)) {
     if (lane == 0) atomicExch(a.bad + sys, 1);
     return;
   }
-  for (int t = lane; t < mm * PW; t += 32) {
-    const int i = t / PW, d = t - i * PW + 1;
-    a.Lf[(size_t)(r0 + i) * PW + d - 1] = d <= i ? Bs[i * 11 + d] : 0.0;
-  }
-  // forward solves: lanes 0-9 the top coupling columns, lane 10 the
-  // right-hand side, lanes 11-20 the bottom coupling columns (non-zero in
-  // the last 10 rows only)
-  double win[PW];
-#pragma unroll
-  for (int k = 0; k < PW; ++k) win[k] = 0.0;
-  const int c = lane < PW ? lane : lane - 11;
-  const int sa_bot = r0 + mm;  // first row of the bottom separator
-  for (int i = 0; i < mm; ++i) {
-    double z = 0.0;
-    if (lane < PW) {  // C_top[i][c] = A[r0+i][r0-10+c], d = i + 10 - c
-      if (top && c >= i) z = a.band[(size_t)(i + PW - c) * N + r0 + i];
-    } else if (lane == PW) {
-      z = a.rhs[r0 + i];
-    } else if (lane < 2 * PW + 1) {  // C_bot[i][c] = A[sa_bot+c][r0+i], d = mm + c - i
-      if (bot && i >= mm - PW + c) z = a.band[(size_t)(mm + c - i) * N + sa_bot + c];
-    }
-#pragma unroll
-    for (int k = 1; k <= PW; ++k)
-      if (k <= i) z = fma(-Bs[i * 11 + k], win[k - 1], z);
-#pragma unroll
-    for (int k = PW - 1; k > 0; --k) win[k] = win[k - 1];
-    win[0] = z;
-    if (lane < PW) {
-      Zs[i * PW + c] = z;
-    } else if (lane == PW) {
-      a.zf[r0 + i] = z;
-    } else if (lane < 2 * PW + 1 && i >= mm - PW && mm >= PW) {
-      a.Zb[((size_t)p * PW + (i - (mm - PW))) * PW + c] = z;
+  // what is left: the separator below and its coupling to the one above
+  if (bot) {
+    const double *F = W + (nblk & 1 ? 0 : kPWin) + kRowW * (mm - kPB * (nblk - 1));
+    for (int e = lane; e < 210; e += 32) {
+      if (e < 100) {
+        const int i = e / PW, j = e - i * PW, hi = i > j ? i : j, d = i > j ? i - j : j - i;
+        a.wb[(size_t)p * 110 + e] = F[kRowW * hi + d];
+      } else if (e < 110) {
+        a.wb[(size_t)p * 110 + e] = F[kRowW * (e - 100) + 11];
+      } else {
+        const int k = (e - 110) / PW, i = (e - 110) - k * PW;
+        a.xo[(size_t)p * 100 + (e - 110)] = F[kRowW * i + 12 + k];
+      }
     }
   }
-  __syncwarp();
-  // Schur contributions: ct = Zt^T D^{-1} [Zt | zf], cb = Zb^T D^{-1} [Zb | zf]
-  // over the last 10 rows, co = Zt^T D^{-1} Zb
-  const int lo = mm >= PW ? mm - PW : 0;
-  for (int t = lane; t < 110 * 3; t += 32) {
-    const int blk = t / 110, e = t - blk * 110;
-    const int u = e < 100 ? e / PW : e - 100, v = e < 100 ? e % PW : -1;
-    double s = 0.0;
-    if (blk == 0) {  // ct
-      if (!top) continue;
-      for (int i = 0; i < mm; ++i) {
-        const double rd = a.Df[r0 + i];
-        const double zv = v >= 0 ? Zs[i * PW + v] : a.zf[r0 + i];
-        s = fma(Zs[i * PW + u] * rd, zv, s);
-      }
-      a.ct[(size_t)p * 110 + e] = s;
-    } else if (blk == 1) {  // cb
-      if (!bot) continue;
-      for (int i = lo; i < mm; ++i) {
-        const double rd = a.Df[r0 + i];
-        const double zu = a.Zb[((size_t)p * PW + (i - lo)) * PW + u];
-        const double zv = v >= 0 ? a.Zb[((size_t)p * PW + (i - lo)) * PW + v] : a.zf[r0 + i];
-        s = fma(zu * rd, zv, s);
-      }
-      a.cb[(size_t)p * 110 + e] = s;
-    } else {  // co (top row u, bottom column v)
-      if (!top || !bot || v < 0) continue;
-      for (int i = lo; i < mm; ++i) {
-        const double rd = a.Df[r0 + i];
-        s = fma(Zs[i * PW + u] * rd, a.Zb[((size_t)p * PW + (i - lo)) * PW + v], s);
-      }
-      a.co[(size_t)p * 110 + e] = s;
+  if (top) {
+    double *T = a.tt + (size_t)p * 110;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = ln.sum_index(lane, h);
+      T[e] = sum[h];
+      if (e < 100) T[(e % PW) * PW + e / PW] = sum[h];
     }
+    if (lane == 31) T[109] = cell[0];
   }
 }
 
-// Gauss-Jordan on M [10][21] in shared memory, lane j owning column j:
-// M <- [I | M_left^{-1} M_right].  No pivoting: M_left is a Schur complement
-// of the symmetric rod Jacobian (positive definite at small steps, where
-// M/dt^2 dominates).  Returns false on a zero or non-finite pivot, or one
-// below kTinyPivot times the block's starting diagonal entry.
-__device__ bool gj10(double (*M)[22], int lane, int ncol) {
-  double d0[PW];
-#pragma unroll
-  for (int k = 0; k < PW; ++k) d0[k] = M[k][k];
-  __syncwarp();
-  for (int k = 0; k < PW; ++k) {
-    const double pk = M[k][k];
-    if (!(fabs(pk) > 0.0) || !isfinite(pk) || fabs(pk) < kTinyPivot * fabs(d0[k])) return false;
-    const double r = pb_recip(pk);
-    double colk[PW];
-#pragma unroll
-    for (int i = 0; i < PW; ++i) colk[i] = M[i][k];
-    __syncwarp();
-    if (lane < ncol) {
-      const double mk = M[k][lane] * r;
-#pragma unroll
-      for (int i = 0; i < PW; ++i)
-        M[i][lane] = i == k ? mk : fma(-colk[i], mk, M[i][lane]);
-    }
-    __syncwarp();
-  }
-  return true;
-}
-
-__global__ void __launch_bounds__(32) k_part_separators(PartArgs a) {
-  __shared__ double M[PW][22];
-  __shared__ double Tp[PW][PW + 1];  // To of the previous separator
-  const int sys = blockIdx.x, lane = threadIdx.x;
+// Block-tridiagonal elimination over a system's separators, four warps:
+// separator s couples to s + 1 through interior s + 1.  The block [T' | To |
+// g'] (10 x 21) is reduced by Gauss-Jordan, warp w on rows w, w + 4, w + 8,
+// lane j on column j; the next separator's terms are fetched meanwhile.
+constexpr int kSepThreads = 128;
+__global__ void __launch_bounds__(kSepThreads) k_part_separators(PartArgs a) {
+  __shared__ double M[2][PW][22];        // by pivot parity: a column is read while it is rewritten
+  __shared__ double Tp[PW][PW + 1], Xp[PW][PW + 1];  // To and T'^{-1} [To | g'] of the one before
+  __shared__ int fail;
+  const int sys = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int s0 = a.sys_sep0[sys], ns = a.sys_nsep[sys];
   if (ns == 0 || (a.go && !a.go[sys]) || a.bad[sys]) return;
-  const int64_t N = a.ntot;
-  // forward elimination: separator s couples to s+1 through interior s+1
+  if (tid == 0) fail = 0;
+  // this thread's entry of [T | To | g]: T and g from the interior above
+  // (wb) and below (tt), To from the one below
+  auto fetch = [&](int s) -> double {
+    const int pu = s0 + s + sys, pd = pu + 1;
+    double v = 0.0;
+    if (s < ns && tid < 110) {
+      v = a.wb[(size_t)pu * 110 + tid] + a.tt[(size_t)pd * 110 + tid];
+    }
+    return v;
+  };
+  auto fetch_to = [&](int s) -> double {
+    return s + 1 < ns && tid < 100 ? a.xo[(size_t)(s0 + s + sys + 1) * 100 + tid] : 0.0;
+  };
+  double nt = fetch(0), no = fetch_to(0);
   for (int s = 0; s < ns; ++s) {
-    const int gs = s0 + s, sa = a.s_a[gs];
-    const int pu = gs + sys;      // interior above separator s (its bottom side)
-    const int pd = gs + sys + 1;  // interior below (its top side)
-    // T_s = A[S,S] - cb[pu] - ct[pd]; g_s = f_S - cb[pu]_g - ct[pd]_g
-    for (int t = lane; t < PW * PW + PW; t += 32) {
-      if (t < PW * PW) {
-        const int i = t / PW, j = t % PW;
-        const int hi = i > j ? i : j, lo = i > j ? j : i;
-        double v = a.band[(size_t)(hi - lo) * N + sa + hi];
-        v -= a.cb[(size_t)pu * 110 + t] + a.ct[(size_t)pd * 110 + t];
-        M[i][j] = v;
-      } else {
-        const int i = t - PW * PW;
-        M[i][2 * PW] = a.rhs[sa + i] - a.cb[(size_t)pu * 110 + 100 + i] -
-                       a.ct[(size_t)pd * 110 + 100 + i];
-      }
-    }
-    __syncwarp();
-    if (s > 0) {  // T'_s = T_s - To^T X_prev, g'_s = g_s - To^T y_prev
-      const double *Xp = a.Xs + (size_t)(gs - 1) * 110;
-      for (int t = lane; t < PW * PW + PW; t += 32) {
-        const int i = t < PW * PW ? t / PW : t - PW * PW;
-        const int j = t < PW * PW ? t % PW : -1;
-        double v = 0.0;
+    const int i = tid < 100 ? tid / PW : tid - 100, j = tid < 100 ? tid % PW : 2 * PW;
+    if (tid < 110) {
+      double v = nt;
+      if (s > 0) {  // T'_s = T_s - To^T X, g'_s = g_s - To^T y of the separator before
 #pragma unroll
-        for (int k = 0; k < PW; ++k)
-          v = fma(Tp[k][i], j >= 0 ? Xp[k * PW + j] : Xp[100 + k], v);
-        if (j >= 0) M[i][j] -= v;
-        else M[i][2 * PW] -= v;
+        for (int k = 0; k < PW; ++k) v = fma(-Tp[k][i], Xp[k][tid < 100 ? j : PW], v);
       }
-      __syncwarp();
+      M[0][i][j] = v;
     }
-    // To_s = -co[pd] (separator s row, separator s+1 column), if s+1 exists
-    for (int t = lane; t < PW * PW; t += 32) {
-      const int i = t / PW, j = t % PW;
-      const double v = s + 1 < ns ? -a.co[(size_t)pd * 110 + t] : 0.0;
-      M[i][PW + j] = v;
-      Tp[i][j] = v;
+    __syncthreads();
+    if (tid < 100) {
+      M[0][i][PW + j] = no;
+      Tp[i][j] = no;
     }
-    __syncwarp();
-    if (!gj10(M, lane, 2 * PW + 1)) {
-      if (lane == 0) atomicExch(a.bad + sys, 1);
+    nt = fetch(s + 1);
+    no = fetch_to(s + 1);
+    __syncthreads();
+    double d0 = tid < PW ? M[0][tid][tid] : 1.0;  // starting diagonal, for the pivot test
+    double piv = 0.0;
+#pragma unroll
+    for (int k = 0; k < PW; ++k) {
+      const double(*A)[22] = M[k & 1];
+      double(*B)[22] = M[(k + 1) & 1];
+      const double pk = A[k][k], r = rcp_any(pk);
+      if (tid == k) piv = pk;
+      if (lane < 2 * PW + 1) {
+        const double mk = A[k][lane] * r;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const int row = warp + 4 * t;
+          if (row < PW) B[row][lane] = row == k ? mk : fma(-A[row][k], mk, A[row][lane]);
+        }
+      }
+      __syncthreads();
+    }
+    if (tid < PW && (!(fabs(piv) > 0.0) || !isfinite(piv) || fabs(piv) < kTinyPivot * fabs(d0))) fail = 1;
+    if (tid < 110) {  // PW is even: the result is in M[0]
+      const double v = tid < 100 ? M[0][i][PW + j] : M[0][i][2 * PW];
+      Xp[i][tid < 100 ? j : PW] = v;
+      a.Xs[(size_t)(s0 + s) * 110 + tid] = v;
+    }
+    __syncthreads();
+    if (fail) {  // uniform
+      if (tid == 0) atomicExch(a.bad + sys, 1);
       return;
     }
-    double *Xo = a.Xs + (size_t)gs * 110;
-    for (int t = lane; t < 110; t += 32) {
-      const int i = t < 100 ? t / PW : t - 100, j = t < 100 ? PW + t % PW : 2 * PW;
-      Xo[t] = M[i][j];
-    }
-    __syncwarp();
   }
-  // back substitution: x_s = y_s - X_s x_{s+1}
-  double xn = 0.0;  // lane i < 10: x_{s+1}[i]
-  for (int s = ns - 1; s >= 0; --s) {
-    const int gs = s0 + s;
-    const double *X = a.Xs + (size_t)gs * 110;
-    double xv = 0.0;
-    if (lane < PW) {
-      xv = X[100 + lane];
-      if (s + 1 < ns)
-        for (int k = 0; k < PW; ++k)
-          xv = fma(-X[lane * PW + k], __shfl_sync(0x3ffu, xn, k), xv);
-      a.x[a.s_a[gs] + lane] = xv;
+  // back substitution by one warp: x_s = y_s - X_s x_{s+1}, lane i < 10 the row
+  if (warp) return;
+  __syncwarp();
+  double xn = 0.0;
+  double row[PW], yn = 0.0;
+  auto load = [&](int s) {
+    if (lane < PW && s >= 0) {
+      const double *X = a.Xs + (size_t)(s0 + s) * 110;
+#pragma unroll
+      for (int k = 0; k < PW; ++k) row[k] = X[lane * PW + k];
+      yn = X[100 + lane];
     }
-    xn = xv;
-    __syncwarp();
+  };
+  load(ns - 1);
+  for (int s = ns - 1; s >= 0; --s) {
+    double xv = yn, c[PW];
+#pragma unroll
+    for (int k = 0; k < PW; ++k) c[k] = s + 1 < ns ? row[k] : 0.0;
+    load(s - 1);
+    double even = xv, odd = 0.0;
+#pragma unroll
+    for (int k = 0; k < PW; k += 2) {
+      even = fma(-c[k], __shfl_sync(0xffffffffu, xn, k), even);
+      odd = fma(-c[k + 1], __shfl_sync(0xffffffffu, xn, k + 1), odd);
+    }
+    xn = even + odd;
+    if (lane < PW) a.x[a.s_a[s0 + s] + lane] = xn;
   }
 }
 
+// x of an interior, from its last row up: the row of step t is pending in
+// lane t mod 32; a step takes its x by a shuffle and subtracts its part from
+// the next ten rows.  The separator below feeds the first ten steps, the one
+// above enters a row's start value with its record's carried multipliers.
+// Each lane stages the record of its own next row.
 __global__ void __launch_bounds__(32) k_part_back(PartArgs a) {
+  constexpr int kRing = 3;
+  __shared__ __align__(16) double ring[32][kRing * kRecW + 2];
   const int p = blockIdx.x, lane = threadIdx.x;
   if ((a.go && !a.go[a.p_sys[p]]) || a.bad[a.p_sys[p]]) return;
   const int r0 = a.p_a[p], mm = a.p_mm[p];
   const int st = a.p_top[p], sb = a.p_bot[p];
-  const int lo = mm - PW;  // interiors have at least 11 rows
+  const unsigned full = 0xffffffffu;
   double xt = 0.0, xb = 0.0;  // lane c < 10: separator values
   if (lane < PW) {
     if (st >= 0) xt = a.x[a.s_a[st] + lane];
     if (sb >= 0) xb = a.x[a.s_a[sb] + lane];
   }
-  // x_i = (zf_i - (Zt x_top + Zb x_bot)_i) / D_i - sum_{k=1..10} L[i+k][i] x_{i+k},
-  // from the bottom row up; lane k < 10 keeps x_{i+1+k} in `mine`
-  double mine = 0.0;
-  for (int i = mm - 1; i >= 0; --i) {
-    double zc = 0.0, lc = 0.0;
-    if (lane < PW) {
-      if (st >= 0) zc = a.Zt[(size_t)(r0 + i) * PW + lane] * xt;
-      if (sb >= 0 && i >= lo) zc = fma(a.Zb[((size_t)p * PW + (i - lo)) * PW + lane], xb, zc);
-      const int row = i + 1 + lane;
-      if (row < mm) lc = a.Lf[(size_t)(r0 + row) * PW + lane] * mine;
-    }
+  // step t < 10: separator row 9 - t; step t >= 10: interior row mm + 9 - t
+  const int R0 = mm + 9;
+  auto fetch = [&](int g) {
+    const int r = R0 - (32 * g + lane);
+    double *dst = &ring[lane][kRecW * (g % kRing)];
+    if (r >= 0 && r < mm) {
+      const double *src = a.rec + (size_t)(r0 + r) * kRecW;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      zc += __shfl_xor_sync(0xffffffffu, zc, o);
-      lc += __shfl_xor_sync(0xffffffffu, lc, o);
+      for (int e = 0; e < kRecW; e += 2) {
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + e);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src + e) : "memory");
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < kRecW; ++e) dst[e] = 0.0;
     }
-    const double xi = (a.zf[r0 + i] - zc) * a.Df[r0 + i] - lc;
-    mine = __shfl_up_sync(0xffffffffu, mine, 1);
-    if (lane == 0) {
-      mine = xi;
-      a.x[r0 + i] = xi;
+  };
+  auto start = [&](int g) -> double {  // z - (carried multipliers) x_top
+    const double *rc = &ring[lane][kRecW * (g % kRing)];
+    double even = rc[0], odd = 0.0;
+    if (st >= 0) {  // warp-uniform
+#pragma unroll
+      for (int k = 0; k < PW; k += 2) {
+        even = fma(-rc[12 + k], __shfl_sync(full, xt, k), even);
+        odd = fma(-rc[13 + k], __shfl_sync(full, xt, k + 1), odd);
+      }
     }
+    return even + odd;
+  };
+#pragma unroll
+  for (int g = 0; g < kRing; ++g) fetch(g);
+  cp_async_commit();
+  cp_async_wait_all();
+  int idx[32];
+#pragma unroll
+  for (int u = 0; u < 32; ++u) {
+    const int d = (lane - u) & 31;
+    idx[u] = d == 0 || d > 11 ? 11 : d;  // word 11 is zero
   }
+  double v = start(0);
+  const int groups = (R0 + 1 + 31) / 32;
+  for (int g = 0; g < groups; ++g) {
+    const double *ra = &ring[lane][kRecW * (g % kRing)], *rb = &ring[lane][kRecW * ((g + 1) % kRing)];
+    const double zn = start(g + 1);
+    double x_own = 0.0;
+#pragma unroll
+    for (int u = 0; u < 32; ++u) {
+      double x = __shfl_sync(full, v, u);
+      if (g == 0 && u < PW) x = __shfl_sync(full, xb, 9 - u);
+      if (lane == u) {
+        x_own = x;
+        v = zn;
+      }
+      v = fma(-(lane <= u ? rb : ra)[idx[u]], x, v);
+    }
+    const int r = R0 - (32 * g + lane);
+    if (r >= 0 && r < mm) a.x[r0 + r] = x_own;
+    fetch(g + kRing);
+    cp_async_commit();
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+  }
+  cp_async_wait_all();
 }
 
 // Newton rounds of long rods (the partitioned path of dm_step): the
@@ -415,7 +549,6 @@ __global__ void k_long_finish(LongArgs a) {
 // a fixed set of systems.
 struct PartPlan {
   int np = 0, nsep = 0, nsys = 0;
-  size_t smem = 0;
   char *scr = nullptr;
   PartArgs A{};
 };
@@ -461,10 +594,8 @@ static dm_status part_plan_build(int nsys, const int32_t *sys_dof0, const int32_
     bytes += (n * elt + 255) / 256 * 256;
     return o;
   };
-  const size_t oL = take((size_t)ntot * PW, 8), oD = take(ntot, 8), oZ = take((size_t)ntot * PW, 8),
-               oz = take(ntot, 8), oZb = take((size_t)np * PW * PW, 8), oct = take((size_t)np * 110, 8),
-               ocb = take((size_t)np * 110, 8), oco = take((size_t)np * 110, 8),
-               oX = take((size_t)std::max(nsep, 1) * 110, 8),
+  const size_t orec = take((size_t)ntot * kRecW, 8), owb = take((size_t)np * 110, 8), ott = take((size_t)np * 110, 8),
+               oxo = take((size_t)np * 100, 8), oX = take((size_t)std::max(nsep, 1) * 110, 8),
                oI = take(5 * (size_t)np + (size_t)nsep + 3 * (size_t)nsys + 1, 4);
   if (cudaMalloc(&P.scr, bytes) != cudaSuccess) {
     set_error("partitioned band solve: cudaMalloc");
@@ -487,24 +618,13 @@ static dm_status part_plan_build(int nsys, const int32_t *sys_dof0, const int32_
   A.sys_sep0 = ib + 5 * np + nsep;
   A.sys_nsep = ib + 5 * np + nsep + nsys;
   A.bad = ib + 5 * np + nsep + 2 * nsys;
-  A.Lf = reinterpret_cast<double *>(P.scr + oL);
-  A.Df = reinterpret_cast<double *>(P.scr + oD);
-  A.Zt = reinterpret_cast<double *>(P.scr + oZ);
-  A.zf = reinterpret_cast<double *>(P.scr + oz);
-  A.Zb = reinterpret_cast<double *>(P.scr + oZb);
-  A.ct = reinterpret_cast<double *>(P.scr + oct);
-  A.cb = reinterpret_cast<double *>(P.scr + ocb);
-  A.co = reinterpret_cast<double *>(P.scr + oco);
+  A.rec = reinterpret_cast<double *>(P.scr + orec);
+  A.wb = reinterpret_cast<double *>(P.scr + owb);
+  A.tt = reinterpret_cast<double *>(P.scr + ott);
+  A.xo = reinterpret_cast<double *>(P.scr + oxo);
   A.Xs = reinterpret_cast<double *>(P.scr + oX);
   cudaError_t e = cudaMemcpyAsync(ib, ints.data(), ints.size() * sizeof(int32_t),
                                   cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(P.scr + oct, 0, oX - oct, st);
-  int mmax = 0;
-  for (int v : pmm) mmax = std::max(mmax, v);
-  P.smem = (size_t)mmax * 11 * sizeof(double);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_part_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)P.smem);
   if (e != cudaSuccess) {
     part_plan_free(P);
     set_error(std::string("partitioned band solve: ") + cudaGetErrorString(e));
@@ -513,15 +633,20 @@ static dm_status part_plan_build(int nsys, const int32_t *sys_dof0, const int32_
   return DM_OK;
 }
 
+// env: the matrices have the envelope of a rod's Jacobian and every interior
+// starts at a node (part_rows a multiple of four).
 static cudaError_t part_launch(const PartPlan &P, const double *band, const double *rhs,
-                               double *x, const int32_t *go, cudaStream_t st) {
+                               double *x, const int32_t *go, bool env, cudaStream_t st) {
   PartArgs A = P.A;
   A.band = band;
   A.rhs = rhs;
   A.x = x;
   A.go = go;
-  k_part_factor<<<P.np, 32, P.smem, st>>>(A);
-  if (P.nsep > 0) k_part_separators<<<P.nsys, 32, 0, st>>>(A);
+  constexpr size_t smem = kPSmem * sizeof(double);
+  static_assert(smem <= 48 * 1024, "within the default limit");
+  if (env) k_part_factor<true><<<P.np, 32, smem, st>>>(A);
+  else k_part_factor<false><<<P.np, 32, smem, st>>>(A);
+  if (P.nsep > 0) k_part_separators<<<P.nsys, kSepThreads, 0, st>>>(A);
   k_part_back<<<P.np, 32, 0, st>>>(A);
   return cudaGetLastError();
 }
@@ -598,7 +723,7 @@ cudaError_t long_rods_round(LongRods *L, const SolveArgs &v, cudaStream_t st) {
   a.ls_action = v.ls_action;
   a.ls_trial = v.ls_trial;
   k_long_decide<<<a.nlong, 256, 0, st>>>(a);
-  cudaError_t e = part_launch(L->plan, v.band, a.rhs, a.dq, a.go, st);
+  cudaError_t e = part_launch(L->plan, v.band, a.rhs, a.dq, a.go, true, st);
   if (e != cudaSuccess) return e;
   k_long_finish<<<a.nlong, 256, 0, st>>>(a);
   return cudaGetLastError();
@@ -630,7 +755,7 @@ extern "C" dm_status dm_solve_band_partitioned(int32_t nsys, const int32_t *sys_
   PartPlan P;
   dm_status r = part_plan_build(nsys, sys_dof0, sys_ndof, ntot, m, P, st);
   if (r != DM_OK) return r;
-  cudaError_t e = part_launch(P, band, rhs, x, nullptr, st);
+  cudaError_t e = part_launch(P, band, rhs, x, nullptr, false, st);
   std::vector<int> bad(nsys, 0);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(bad.data(), P.A.bad, nsys * sizeof(int), cudaMemcpyDeviceToHost, st);

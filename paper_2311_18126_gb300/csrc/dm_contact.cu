@@ -667,13 +667,6 @@ __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {
   a.cbad[c] = 0;
 }
 
-// 1/d on the integer pipe where d is well inside the normal range, else by
-// division.
-__device__ __forceinline__ double lu_recip(double d) {
-  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
-  return ex - 64u < 1918u ? rcp_int(d) : 1.0 / d;
-}
-
 // The tiles of row k of a system's pattern beyond k, in order, into list
 // (shared memory); every thread of the block calls it.  Returns their number.
 __device__ __forceinline__ int tile_list(const uint8_t *row, int k, int nt, uint16_t *list, int *count) {
@@ -723,7 +716,7 @@ __global__ void __launch_bounds__(256) k_lu_panel(ContactArgs a, double *yall, i
 #pragma unroll
   for (int j = 0; j < kNB; ++j) {
     const double piv = D[j][j];
-    const double r = lu_recip(piv);
+    const double r = rcp_any(piv);
     const double u = D[j][lane] * r;  // row j of U over the pivot
 #pragma unroll
     for (int t = 0; t < 4; ++t) {

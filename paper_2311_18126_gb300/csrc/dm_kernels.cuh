@@ -177,6 +177,13 @@ __device__ __forceinline__ double rcp_int(double d) {
   return __hiloint2double((int)((unsigned)(b >> 32) | (hi & 0x80000000u)), (int)(unsigned)b);
 }
 
+// 1/d on the integer pipe where d is well inside the normal range, else by
+// division.
+__device__ __forceinline__ double rcp_any(double d) {
+  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
+  return ex - 64u < 1918u ? rcp_int(d) : 1.0 / d;
+}
+
 // Asynchronous 8-byte copy global -> shared (both 8-byte aligned), and the
 // group commit / wait for all of this thread's copies.
 __device__ __forceinline__ void cp_async8(double *dst, const double *src) {

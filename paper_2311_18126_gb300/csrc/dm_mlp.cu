@@ -77,22 +77,27 @@ __device__ __forceinline__ float adam(const UpdateArgs &a, float g, float *p, fl
 
 // Gradients (the batch shares' partials in a fixed order), Adam and the BF16
 // weights of every layer in one launch: a thread per weight or hidden bias in
-// the partials' order, then one block for the output bias (a warp per column).
-constexpr int kUpdateThreads = 256;
+// the partials' order, then kBiasBlocks blocks for the output bias (16 columns
+// each, 16 threads per column with several loads in flight).
+constexpr int kUpdateThreads = 256, kBiasBlocks = kOut / 16;
 __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
-  if (blockIdx.x == gridDim.x - 1) {
-    const int lane = threadIdx.x & 31;
-    for (int c = threadIdx.x >> 5; c < kOut; c += kUpdateThreads / 32) {
-      float s = 0.0f;
-      for (int k = lane; k < a.n_gb4; k += 32) s += a.gb4[(size_t)k * kOut + c];
+  const int bias_block = (int)blockIdx.x - ((int)gridDim.x - kBiasBlocks);
+  if (bias_block >= 0) {
+    __shared__ float red[16][17];
+    const int col = threadIdx.x & 15, r0 = threadIdx.x >> 4, c = 16 * bias_block + col;
+    float s = 0.0f;
+#pragma unroll 8
+    for (int k = r0; k < a.n_gb4; k += 16) s += a.gb4[(size_t)k * kOut + c];
+    red[r0][col] = s;
+    __syncthreads();
+    if (r0 != 0) return;
+    s = 0.0f;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane != 0) continue;
-      size_t o = 0;
-      for (int l = 0; l < kLayers; ++l) o += (size_t)(l == 0 || l == 3 ? 64 : 256) * 256 + (l < 3 ? 256 : 0);
-      if (a.grads) a.grads[o + c] = s;
-      if (a.lr > 0.0f) adam(a, s, a.b[3] + c, a.mb[3] + c, a.vb[3] + c, a.maskb[3][c]);
-    }
+    for (int k = 0; k < 16; ++k) s += red[k][col];
+    size_t o = 0;
+    for (int l = 0; l < kLayers; ++l) o += mlp_part_size(l);
+    if (a.grads) a.grads[o + c] = s;
+    if (a.lr > 0.0f) adam(a, s, a.b[3] + c, a.mb[3] + c, a.vb[3] + c, a.maskb[3][c]);
     return;
   }
   int e = blockIdx.x * kUpdateThreads + threadIdx.x, l = 0;
@@ -106,6 +111,7 @@ __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
   const int S = l == 0 || l == 3 ? a.shape.s_small : a.shape.s_big;
   const float *part = a.part + mlp_part_offset(l, a.shape.s_small, a.shape.s_big) + e;
   float g = 0.0f;
+#pragma unroll 8
   for (int z = 0; z < S; ++z) g += part[(size_t)z * mlp_part_size(l)];
   const int in = l == 0 ? kIn : kHid, out = l == 3 ? kOut : kHid;
   if (e >= in * out) {
@@ -430,7 +436,7 @@ dm_status dm_mlp_forward(dm_mlp *m, const void *X, float *Y, int32_t M) {
 // batch's shares, Adam and the BF16 weights in the third.  grads_out (device,
 // optional) receives the fp32 gradients in the dm_mlp_get_params layout;
 // loss_out the loss before the update.
-// Measured (GB300): batch 16384 111 us against 548 us with a launch per layer
+// Measured (GB300): batch 16384 87 us against 548 us with a launch per layer
 // and operation (some 55 launches with transposed copies of every operand).
 dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M, float lr,
                             float *grads_out, double *loss_out) {
@@ -473,7 +479,7 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   a.c2 = 1.0f - std::pow(a.b2, (float)m->step);
   size_t params = 0;
   for (int l = 0; l < kLayers; ++l) params += mlp_part_size(l);
-  k_mlp_update<<<nb((int64_t)params, kUpdateThreads) + 1, kUpdateThreads, 0, st>>>(a);
+  k_mlp_update<<<nb((int64_t)params, kUpdateThreads) + kBiasBlocks, kUpdateThreads, 0, st>>>(a);
   struct {
     double loss;
     int err[2];
