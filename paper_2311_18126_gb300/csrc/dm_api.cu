@@ -113,6 +113,7 @@ struct Extra {
   int32_t *ls_action = nullptr, *ls_trial = nullptr, *ls_nback = nullptr;
   double *ls_alpha = nullptr, *ls_racc = nullptr, *ls_qacc = nullptr, *ls_merit = nullptr;
   int n_rod_sys = 0;
+  int max_rod_nodes = 0;  // of the single rods (the length projection's block)
   struct {
     int table = 0, pair_cap = 0, n_contact = 0;
     double inv_cell = 0.0;
@@ -361,10 +362,11 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
   const int long_min = prm->long_rod_dofs == 0 ? 2048 : prm->long_rod_dofs;
   for (int k = 0; k < S; ++k)
     if (T.sys_kind[k] == SOLVE_ROD_BAND) {
+      s->x.max_rod_nodes = std::max(s->x.max_rod_nodes, (T.sys_ndof[k] + 1) / 4);
       if (long_min > 0 && T.sys_ndof[k] >= long_min) longsys.push_back(k);
       else order.push_back(k);
     }
-  DM_TRY(long_rods_create(s, longsys, 512, &s->x.longr));
+  DM_TRY(long_rods_create(s, longsys, &s->x.longr));
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return T.sys_ndof[a] > T.sys_ndof[b]; });
   s->x.n_rod_sys = (int)order.size();
@@ -1054,8 +1056,8 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       DM_CK(ws_predict(s, st, ws_trial, s->x.d_dof_sys));
     }
     if (s->prm.predictor == 1) {
-      k_project_lengths<<<blocks((int64_t)S * 32, 128), 128, 0, st>>>(
-          S, s->x.d_sys_kind, d.sys_dof0, d.sys_ndof, d.fixed, d.qn, d.q, s->x.midpoint ? 1 : 0);
+      project_lengths(S, s->x.max_rod_nodes, s->x.d_sys_kind, d.sys_dof0, d.sys_ndof, d.fixed, d.qn, d.q,
+                      s->x.midpoint ? 1 : 0, st);
       s->x.launches[K_BEGIN]++;
     }
     if (ls_on) {

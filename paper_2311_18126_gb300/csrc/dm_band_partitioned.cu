@@ -27,6 +27,7 @@
 // factored the band, solved for the carried columns and formed the Schur
 // products one after another, with two barriers and a division per column.
 #include <algorithm>
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -59,6 +60,7 @@ struct PartArgs {
   const int32_t *sys_sep0, *sys_nsep;          // per system: first separator, count
   const double *band, *rhs;
   double *x;
+  double *q;                   // NULL, or q -= x
   double *rec;                 // [ntot][kRecW]
   double *wb, *tt, *xo;        // [nparts][110]: what is left of the separator below (10x10, 10), the
                                // Schur terms of the one above (10x10, 10), their coupling (10x10)
@@ -377,7 +379,11 @@ __global__ void __launch_bounds__(kSepThreads) k_part_separators(PartArgs a) {
       odd = fma(-c[k + 1], __shfl_sync(0xffffffffu, xn, k + 1), odd);
     }
     xn = even + odd;
-    if (lane < PW) a.x[a.s_a[s0 + s] + lane] = xn;
+    if (lane < PW) {
+      const int at = a.s_a[s0 + s] + lane;
+      a.x[at] = xn;
+      if (a.q) a.q[at] -= xn;
+    }
   }
 }
 
@@ -455,7 +461,10 @@ __global__ void __launch_bounds__(32) k_part_back(PartArgs a) {
       v = fma(-(lane <= u ? rb : ra)[idx[u]], x, v);
     }
     const int r = R0 - (32 * g + lane);
-    if (r >= 0 && r < mm) a.x[r0 + r] = x_own;
+    if (r >= 0 && r < mm) {
+      if (a.q) a.q[r0 + r] -= x_own;
+      else a.x[r0 + r] = x_own;
+    }
     fetch(g + kRing);
     cp_async_commit();
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
@@ -464,16 +473,13 @@ __global__ void __launch_bounds__(32) k_part_back(PartArgs a) {
 }
 
 // Newton rounds of long rods (the partitioned path of dm_step): the
-// bookkeeping of the rod solver (converged, failed or solving this round),
-// the right-hand side -f, and after the solve q += dq.
+// bookkeeping of the rod solver (converged, failed or solving this round;
+// the solve itself takes q -= J^-1 f).
 struct LongArgs {
   int nlong;
   const int32_t *sys;                 // long system -> system index
-  const int32_t *sys_dof0, *sys_ndof;  // per system
   double tol;
   int max_iter;
-  const double *f;
-  double *q, *dq, *rhs;
   int32_t *sys_active, *sys_iters, *sys_status;
   const unsigned long long *sys_res;
   int32_t *ctrl;
@@ -484,63 +490,50 @@ struct LongArgs {
 };
 
 __global__ void k_long_decide(LongArgs a) {
-  __shared__ int go_s;
-  const int k = blockIdx.x;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= a.nlong) return;
   const int s = a.sys[k];
-  if (threadIdx.x == 0) {
-    int go = 0;
-    a.bad[k] = 0;
-    if (a.sys_active[s]) {
-      if (a.ls_action && a.ls_action[s] == 1) {  // backtracking: no solve this round
-        atomicAdd(&a.ctrl[0], 1);
+  int go = 0;
+  a.bad[k] = 0;
+  if (a.sys_active[s]) {
+    if (a.ls_action && a.ls_action[s] == 1) {  // backtracking: no solve this round
+      atomicAdd(&a.ctrl[0], 1);
+    } else {
+      const double res = __longlong_as_double((long long)a.sys_res[s]);
+      int st = a.sys_status[s];
+      if (st == 0 && isnan(res)) st = DM_ERR_NONFINITE;
+      if (st == 0 && res <= a.tol) {
+        a.sys_active[s] = 0;
       } else {
-        const double res = __longlong_as_double((long long)a.sys_res[s]);
-        int st = a.sys_status[s];
-        if (st == 0 && isnan(res)) st = DM_ERR_NONFINITE;
-        if (st == 0 && res <= a.tol) {
+        if (st == 0 && a.sys_iters[s] >= a.max_iter) st = DM_ERR_NOT_CONVERGED;
+        if (st != 0) {
+          a.sys_status[s] = st;
           a.sys_active[s] = 0;
+          atomicAdd(&a.ctrl[1], 1);
+          atomicMin(&a.ctrl[2], s);
         } else {
-          if (st == 0 && a.sys_iters[s] >= a.max_iter) st = DM_ERR_NOT_CONVERGED;
-          if (st != 0) {
-            a.sys_status[s] = st;
-            a.sys_active[s] = 0;
-            atomicAdd(&a.ctrl[1], 1);
-            atomicMin(&a.ctrl[2], s);
-          } else {
-            go = 1;
-          }
+          go = 1;
         }
       }
     }
-    a.go[k] = go;
-    go_s = go;
   }
-  __syncthreads();
-  if (!go_s) return;
-  const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a.rhs[d0 + i] = -a.f[d0 + i];
+  a.go[k] = go;
 }
 
 __global__ void k_long_finish(LongArgs a) {
-  const int k = blockIdx.x;
-  if (!a.go[k]) return;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= a.nlong || !a.go[k]) return;
   const int s = a.sys[k];
   if (a.bad[k]) {
-    if (threadIdx.x == 0) {
-      a.sys_status[s] = DM_ERR_DEGENERATE;
-      a.sys_active[s] = 0;
-      atomicAdd(&a.ctrl[1], 1);
-      atomicMin(&a.ctrl[2], s);
-    }
+    a.sys_status[s] = DM_ERR_DEGENERATE;
+    a.sys_active[s] = 0;
+    atomicAdd(&a.ctrl[1], 1);
+    atomicMin(&a.ctrl[2], s);
     return;
   }
-  const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a.q[d0 + i] += a.dq[d0 + i];
-  if (threadIdx.x == 0) {
-    a.sys_iters[s] += 1;
-    if (a.ls_trial) a.ls_trial[s] = 1;
-    atomicAdd(&a.ctrl[0], 1);
-  }
+  a.sys_iters[s] += 1;
+  if (a.ls_trial) a.ls_trial[s] = 1;
+  atomicAdd(&a.ctrl[0], 1);
 }
 
 }  // namespace
@@ -636,11 +629,12 @@ static dm_status part_plan_build(int nsys, const int32_t *sys_dof0, const int32_
 // env: the matrices have the envelope of a rod's Jacobian and every interior
 // starts at a node (part_rows a multiple of four).
 static cudaError_t part_launch(const PartPlan &P, const double *band, const double *rhs,
-                               double *x, const int32_t *go, bool env, cudaStream_t st) {
+                               double *x, double *q, const int32_t *go, bool env, cudaStream_t st) {
   PartArgs A = P.A;
   A.band = band;
   A.rhs = rhs;
   A.x = x;
+  A.q = q;
   A.go = go;
   constexpr size_t smem = kPSmem * sizeof(double);
   static_assert(smem <= 48 * 1024, "within the default limit");
@@ -657,18 +651,37 @@ struct LongRods {
   std::vector<void *> allocs;
 };
 
-dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, int part_rows,
-                           LongRods **out) {
+// Rows per interior (a multiple of four, for the envelope): a column takes
+// about 550 cycles, a separator of the sequential elimination about 14000, so
+// for one rod of n rows the two chains m + 25 n / m are shortest at
+// m = 5 sqrt(n), and half of that costs little more in separators;
+// a large batch takes interiors that still come in several waves, which the
+// block scheduler balances: 64 rods of 20000 rows factor in 0.95 ms with 512
+// rows, in 1.29 ms with 1060 (one uneven wave), while the separators shrink
+// from 0.28 to 0.15 ms.
+static int long_part_rows(int64_t total, int n_max, int sms) {
+  const int64_t m = std::max<int64_t>((int64_t)(2.5 * std::sqrt((double)n_max)), total / (16 * sms));
+  return (int)std::min<int64_t>(2048, std::max<int64_t>(128, m)) / 4 * 4;
+}
+
+dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, LongRods **out) {
   *out = nullptr;
   if (sys.empty()) return DM_OK;
   const HostTopology &T = s->T;
   auto *L = new LongRods();
   const int nl = (int)sys.size();
   std::vector<int32_t> d0(nl), nd(nl);
+  int64_t total = 0;
+  int n_max = 0, dev = 0, sms = 1;
   for (int k = 0; k < nl; ++k) {
     d0[k] = T.sys_dof0[sys[k]];
     nd[k] = T.sys_ndof[sys[k]];
+    total += nd[k];
+    n_max = std::max(n_max, nd[k]);
   }
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int part_rows = long_part_rows(total, n_max, sms);
   dm_status r = part_plan_build(nl, d0.data(), nd.data(), T.n_dofs, part_rows, L->plan, s->stream);
   auto dal = [&](void **p, size_t bytes) {
     if (cudaMalloc(p, bytes) != cudaSuccess) return false;
@@ -676,9 +689,7 @@ dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, int pa
     return true;
   };
   int32_t *dsys = nullptr, *dgo = nullptr;
-  double *drhs = nullptr;
-  if (r == DM_OK && (!dal((void **)&dsys, nl * 4) || !dal((void **)&dgo, nl * 4) ||
-                     !dal((void **)&drhs, (size_t)T.n_dofs * 8))) {
+  if (r == DM_OK && (!dal((void **)&dsys, nl * 4) || !dal((void **)&dgo, nl * 4))) {
     set_error("long rods: cudaMalloc");
     r = DM_ERR_OOM;
   }
@@ -691,7 +702,6 @@ dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, int pa
   L->la.nlong = nl;
   L->la.sys = dsys;
   L->la.go = dgo;
-  L->la.rhs = drhs;
   L->la.bad = L->plan.A.bad;
   *out = L;
   return DM_OK;
@@ -708,13 +718,8 @@ int long_rods_count(const LongRods *L) { return L ? L->la.nlong : 0; }
 
 cudaError_t long_rods_round(LongRods *L, const SolveArgs &v, cudaStream_t st) {
   LongArgs a = L->la;
-  a.sys_dof0 = v.sys_dof0;
-  a.sys_ndof = v.sys_ndof;
   a.tol = v.tol;
   a.max_iter = v.max_iter;
-  a.f = v.f;
-  a.q = v.q;
-  a.dq = v.dq;
   a.sys_active = v.sys_active;
   a.sys_iters = v.sys_iters;
   a.sys_status = v.sys_status;
@@ -722,10 +727,11 @@ cudaError_t long_rods_round(LongRods *L, const SolveArgs &v, cudaStream_t st) {
   a.ctrl = v.ctrl;
   a.ls_action = v.ls_action;
   a.ls_trial = v.ls_trial;
-  k_long_decide<<<a.nlong, 256, 0, st>>>(a);
-  cudaError_t e = part_launch(L->plan, v.band, a.rhs, a.dq, a.go, true, st);
+  const int nb = (a.nlong + 127) / 128;
+  k_long_decide<<<nb, 128, 0, st>>>(a);
+  cudaError_t e = part_launch(L->plan, v.band, v.f, v.dq, v.q, a.go, true, st);
   if (e != cudaSuccess) return e;
-  k_long_finish<<<a.nlong, 256, 0, st>>>(a);
+  k_long_finish<<<nb, 128, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -755,7 +761,7 @@ extern "C" dm_status dm_solve_band_partitioned(int32_t nsys, const int32_t *sys_
   PartPlan P;
   dm_status r = part_plan_build(nsys, sys_dof0, sys_ndof, ntot, m, P, st);
   if (r != DM_OK) return r;
-  cudaError_t e = part_launch(P, band, rhs, x, nullptr, false, st);
+  cudaError_t e = part_launch(P, band, rhs, x, nullptr, nullptr, false, st);
   std::vector<int> bad(nsys, 0);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(bad.data(), P.A.bad, nsys * sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -201,11 +201,9 @@ int32_t *ws_trial_flags(dm_system *s);
 cudaError_t ws_keep_velocity(dm_system *s, cudaStream_t st);
 
 // Long rods (dm_band_partitioned.cu): the systems `sys` are solved in the
-// Newton rounds by the partitioned band solve (interiors of part_rows - 10
-// rows).  long_rods_round is declared with the kernel arguments.
+// Newton rounds by the partitioned band solve.  long_rods_round is declared with the kernel arguments.
 struct LongRods;
-dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, int part_rows,
-                           LongRods **out);
+dm_status long_rods_create(dm_system *s, const std::vector<int32_t> &sys, LongRods **out);
 void long_rods_free(LongRods *L);
 int long_rods_count(const LongRods *L);
 

@@ -184,6 +184,22 @@ __device__ __forceinline__ double rcp_any(double d) {
   return ex - 64u < 1918u ? rcp_int(d) : 1.0 / d;
 }
 
+// sqrt(x), x >= 0: where x is well inside the FP32 range, the FP32 reciprocal
+// root r of its leading 23 bits, moved between the formats by integer
+// operations as in rcp64_seed, and with h = x r, e = 1 - h r the series
+// h (1 + e/2 + 3 e^2/8) of h / sqrt(1 - e): five FP64 instructions, relative
+// error below 2 * 2^-53.
+__device__ __forceinline__ double sqrt_any(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (hi - ((1023u - 100u) << 20) >= (200u << 20)) return sqrt(x);
+  float sf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(sf) : "f"(__uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29))));
+  const unsigned sb = __float_as_uint(sf);
+  const double r = __hiloint2double((int)((sb >> 3) + 0x38000000u), (int)(sb << 29));
+  const double h = x * r, e = fma(-h, r, 1.0);
+  return fma(h, e * fma(0.375, e, 0.5), h);
+}
+
 // Asynchronous 8-byte copy global -> shared (both 8-byte aligned), and the
 // group commit / wait for all of this thread's copies.
 __device__ __forceinline__ void cp_async8(double *dst, const double *src) {
@@ -368,9 +384,9 @@ __global__ void k_frame_chain_nodes(FrameChainArgs a);
 __global__ void k_frames_out(int ne, const double *soa, double *aos);
 __global__ void k_frames_in(int ne, const double *aos, double *soa);
 __global__ void k_begin_step(StepArgs a);
-__global__ void k_project_lengths(int nsys, const int32_t *sys_kind, const int32_t *sys_dof0,
-                                  const int32_t *sys_ndof, const uint8_t *fixed,
-                                  const double *qn, double *q, int midpoint);
+void project_lengths(int nsys, int max_nodes, const int32_t *sys_kind, const int32_t *sys_dof0,
+                     const int32_t *sys_ndof, const uint8_t *fixed, const double *qn, double *q, int midpoint,
+                     cudaStream_t st);
 __global__ void k_commit(StepArgs a);
 __global__ void k_restore(StepArgs a);
 __global__ void k_round_continue(int32_t *ctrl, int max_rounds, cudaGraphConditionalHandle h);
