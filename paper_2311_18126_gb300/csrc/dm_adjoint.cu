@@ -64,26 +64,18 @@ __global__ void k_adj_midpoint_out(int nd, const uint8_t *fixed, const double *g
   if (!fixed[i]) gv0[i] -= 0.5 * gv2[i];
 }
 
-// dst = transposed condensation-path storage: per limb the band
-// B'[p][k + 10] = B[p + k][10 - k], C' = R^T, R' = C^T (one thread per entry)
+// dst = transposed condensation-path storage: per limb C' = R^T, R' = C^T
+// (the limb's band is formed transposed by its factor kernel); a block per limb
 __global__ void k_gen_transpose(SolveGenArgs a, const double *src, double *dst) {
-  const int L = blockIdx.y;
+  const int L = blockIdx.x;
   if (L >= a.nlimb || !a.gs_fast[a.lb_gsys[L]]) return;
-  const int n = a.lb_n[L], m = a.lb_m[L], nbc = a.lb_nbc[L];
-  const double *B = src + a.lb_band[L];
-  double *Bt = dst + a.lb_band[L];
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * 21; e += gridDim.x * blockDim.x) {
-    const int p = e / 21, k = e - p * 21 - 10;
-    Bt[e] = (p + k >= 0 && p + k < n) ? B[(size_t)(p + k) * 21 + (10 - k)] : 0.0;
-  }
-  if (blockIdx.x == 0) {
-    const double *C = src + a.lb_C[L], *R = src + a.lb_R[L];
-    double *Ct = dst + a.lb_C[L], *Rt = dst + a.lb_R[L];
-    for (int e = threadIdx.x; e < m * nbc; e += blockDim.x) {
-      const int r = e / nbc, b = e - r * nbc;
-      Ct[e] = R[(size_t)b * m + r];
-      Rt[(size_t)b * m + r] = C[e];
-    }
+  const int m = a.lb_m[L], nbc = a.lb_nbc[L];
+  const double *C = src + a.lb_C[L], *R = src + a.lb_R[L];
+  double *Ct = dst + a.lb_C[L], *Rt = dst + a.lb_R[L];
+  for (int e = threadIdx.x; e < m * nbc; e += blockDim.x) {
+    const int r = e / nbc, b = e - r * nbc;
+    Ct[e] = R[(size_t)b * m + r];
+    Rt[(size_t)b * m + r] = C[e];
   }
 }
 

@@ -490,6 +490,14 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     DM_TRY(upload(s, &d.lb_nbc, T.lb_nbc));
     DM_TRY(upload(s, &d.lb_bc0, T.lb_bc0));
     DM_TRY(upload(s, &d.lb_bcols, T.lb_bcols));
+    DM_TRY(upload(s, &d.lb_rod, T.lb_rod));
+    DM_TRY(upload(s, &d.lb_first, T.lb_first));
+    DM_TRY(upload(s, &d.npr, T.npr));
+    {
+      std::vector<int32_t> slot0(T.n_rods + 1, 0);
+      for (int r = 0; r < T.n_rods; ++r) slot0[r + 1] = slot0[r] + T.npr[r] - 2;
+      DM_TRY(upload(s, &d.rod_slot0, slot0));
+    }
     DM_TRY(dalloc(s, &d.gen_go, T.gen_sys.size()));
     DM_TRY(dalloc(s, &d.gen_bad, T.gen_sys.size()));
     DM_CK(cudaMemset(d.gen_bad, 0, T.gen_sys.size() * sizeof(int32_t)));
@@ -502,25 +510,36 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
         s->x.n_slow++;
       }
     }
-    if (s->x.border_smem > 48 * 1024)
-      DM_CK(cudaFuncSetAttribute(k_gen_border, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)s->x.border_smem));
+    // the limit of a block, not this system's need: the attribute is the
+    // kernel's, and a later, smaller system must not lower it for this one
+    int dev = 0, smem_max = 0;
+    DM_CK(cudaGetDevice(&dev));
+    DM_CK(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    auto raise_limit = [&](const void *kernel) {
+      cudaFuncAttributes fa;
+      cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 smem_max - (int)fa.sharedSizeBytes);
+      return e;
+    };
+    DM_CK(raise_limit((const void *)k_gen_border));
     for (size_t L = 0; L < T.lb_n.size(); ++L)
       if (T.gs_fast[T.lb_gsys[L]]) s->x.limb_nmax = std::max(s->x.limb_nmax, T.lb_n[L]);
     {
       // warps per block: up to 4, within 200 KB of shared memory per block
       const size_t pf = gen_factor_smem(s->x.limb_nmax) * sizeof(double);
-      const size_t pb = gen_back_smem(s->x.limb_nmax) * sizeof(double);
+      const size_t pb = gen_back_smem() * sizeof(double);
       s->x.wpb_factor = (int)std::max<size_t>(1, std::min<size_t>(4, (200 << 10) / pf));
       s->x.wpb_back = (int)std::max<size_t>(1, std::min<size_t>(4, (200 << 10) / pb));
       s->x.wpb_factor_max = s->x.wpb_factor;
       s->x.wpb_back_max = s->x.wpb_back;
       s->x.smem_factor = pf * s->x.wpb_factor;
       s->x.smem_back = pb * s->x.wpb_back;
-      DM_CK(cudaFuncSetAttribute(k_gen_limb_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)s->x.smem_factor));
-      DM_CK(cudaFuncSetAttribute(k_gen_limb_back, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)s->x.smem_back));
+      // one limb per block: the few limbs of a late round spread over the SMs
+      s->x.wpb_factor = s->x.wpb_back = 1;
+      DM_CK(raise_limit((const void *)k_gen_limb_factor));
+      DM_CK(raise_limit((const void *)k_gen_limb_back));
     }
     DM_TRY(upload(s, &d.asm_target, T.asm_target));
     DM_TRY(upload(s, &d.asm_sys, T.asm_sys));
@@ -585,6 +604,18 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
   }
   DM_CK(cudaDeviceSynchronize());
   return DM_OK;
+}
+
+// What the limb kernels need to form their rows (trans: of the transpose).
+static void limb_terms(const dm_system_ext *s, SolveGenArgs &ga, int trans) {
+  const HostTopology &T = s->T;
+  const DevArrays &d = s->d;
+  ga.lb_rod = d.lb_rod; ga.lb_first = d.lb_first; ga.npr = d.npr; ga.rod_slot0 = d.rod_slot0;
+  ga.rod_edge0 = s->x.d_rod_edge0; ga.slot2st = s->x.d_slot2st; ga.dof_node = d.dof_node;
+  ga.fixed = d.fixed; ga.sh = d.sh; ga.es = d.es; ga.nt = T.ground ? d.nt : nullptr;
+  ga.dconst = d.dconst;
+  ga.ns = (int)T.n_stencils; ga.ne = (int)T.n_edges; ga.nn = (int)T.n_nodes;
+  ga.trans = trans;
 }
 
 // Event bracket around one kernel launch when profiling is on.
@@ -799,6 +830,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
   ga.gs_fast = d.gs_fast; ga.lb_gsys = d.lb_gsys; ga.lb_dir = d.lb_dir; ga.lb_m = d.lb_m;
   ga.lb_nbc = d.lb_nbc; ga.lb_bc0 = d.lb_bc0; ga.lb_bcols = d.lb_bcols;
   ga.gen_go = d.gen_go; ga.gen_bad = d.gen_bad;
+  limb_terms(s, ga, 0);
   LineSearchArgs la{S, nd, d.sys_active, s->x.d_dof_sys, d.sys_dof0, d.sys_ndof, d.f, d.rscale,
                     s->x.ls_action, s->x.ls_trial, s->x.ls_nback, s->x.ls_alpha, s->x.ls_racc,
                     s->x.ls_merit, d.q, s->x.ls_qacc, nullptr};
@@ -1825,15 +1857,15 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     ga.gs_fast = d.gs_fast; ga.lb_gsys = d.lb_gsys; ga.lb_dir = d.lb_dir; ga.lb_m = d.lb_m;
     ga.lb_nbc = d.lb_nbc; ga.lb_bc0 = d.lb_bc0; ga.lb_bcols = d.lb_bcols;
     ga.gen_go = go; ga.gen_bad = bad;
-    if (ga.nlimb > 0)
-      k_gen_transpose<<<dim3(4, ga.nlimb), 256, 0, st>>>(ga, d.gen, A.gen2);
+    limb_terms(s, ga, 1);
+    if (ga.nlimb > 0) k_gen_transpose<<<ga.nlimb, 128, 0, st>>>(ga, d.gen, A.gen2);
     k_gen_transpose_border<<<ngen, 256, 0, st>>>(ga, d.gen, A.gen2);
     const int wf = s->x.wpb_factor, wb = s->x.wpb_back;
     if (ga.nlimb)
-      k_gen_limb_factor<<<(ga.nlimb + wf - 1) / wf, 32 * wf, s->x.smem_factor, st>>>(ga);
+      k_gen_limb_factor<<<(ga.nlimb + wf - 1) / wf, 32 * wf, s->x.smem_factor / s->x.wpb_factor_max * wf, st>>>(ga);
     k_gen_border<<<ngen, kGenBorderThreads, s->x.border_smem, st>>>(ga);
     if (ga.nlimb)
-      k_gen_limb_back<<<(ga.nlimb + wb - 1) / wb, 32 * wb, s->x.smem_back, st>>>(ga);
+      k_gen_limb_back<<<(ga.nlimb + wb - 1) / wb, 32 * wb, s->x.smem_back / s->x.wpb_back_max * wb, st>>>(ga);
     DM_CK(cudaGetLastError());
     int32_t h[4] = {0, 0, 0, 0};
     DM_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));

@@ -85,23 +85,33 @@ __global__ void k_nodes(NodeArgs a) {
   for (int k = 0; k < 9; ++k) a.nt[(3 + k) * NN + v] = J[k];
 }
 
-__global__ void __launch_bounds__(256) k_rows_gen(RowGenArgs a) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.nd) return;
-  const int s = a.dof_sys[i];
-  if (a.sys_kind[s] != SOLVE_GENERAL || !a.sys_active[s]) return;
+// Row i's force balance; the scaled residual's bits.
+__device__ __forceinline__ unsigned long long rows_gen_one(const RowGenArgs &a, int i) {
   count_active(a.units);
+  // eight terms at a time, loaded side by side (a joint node has dozens) and
+  // summed in order
   double F = 0.0;
-  for (int k = a.gat_ptr[i]; k < a.gat_ptr[i + 1]; ++k) {
-    const int code = a.gat_ent[k];
-    const int idx = code >> 5;
-    if (code & 16) {
-      const int slot = code & 15;
-      const double v = a.es[(slot % 3) * a.ne + idx];
-      F += slot < 3 ? v : -v;
-    } else {
-      F -= a.sg[(code & 15) * a.ns + idx];
+  const int k1 = a.gat_ptr[i + 1];
+  for (int k = a.gat_ptr[i]; k < k1; k += 8) {
+    int code[8];
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) code[u] = k + u < k1 ? a.gat_ent[k + u] : -1;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int slot = code[u] & 15, idx = code[u] >> 5;
+      x[u] = 0.0;
+      if (code[u] < 0) continue;
+      if (code[u] & 16) {
+        const double v = a.es[(slot % 3) * a.ne + idx];
+        x[u] = slot < 3 ? v : -v;
+      } else {
+        x[u] = -a.sg[slot * a.ns + idx];
+      }
     }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k + u < k1) F += x[u];
   }
   const int c = a.dof_comp[i];
   const double m = a.mass[i], idt = a.idt;
@@ -113,8 +123,17 @@ __global__ void __launch_bounds__(256) k_rows_gen(RowGenArgs a) {
   double f = m * idt * idt * (a.q[i] - a.qn[i]) - m * idt * a.vn[i] - F;
   if (a.fixed[i]) f = 0.0;
   a.f[i] = f;
-  const double rr = fabs(f) * a.rscale[i];
-  atomicMax(&a.sys_res[s], (unsigned long long)__double_as_longlong(rr));
+  return (unsigned long long)__double_as_longlong(fabs(f) * a.rscale[i]);
+}
+
+__global__ void __launch_bounds__(256) k_rows_gen(RowGenArgs a) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int s = i < a.nd ? a.dof_sys[i] : -1;
+  if (s >= 0 && (a.sys_kind[s] != SOLVE_GENERAL || !a.sys_active[s])) s = -1;
+  unsigned long long r = 0;
+  if (s >= 0) r = rows_gen_one(a, i);
+  __syncwarp();
+  max_residual(a.sys_res, s, r);  // (takes every lane)
 }
 
 // Grid (system, chunk of kAsmPerBlock targets): blocks of systems that do
@@ -131,16 +150,24 @@ __global__ void k_assemble_gen(AsmArgs a) {
   for (int u = 0; u < kAsmPerBlock / 256; ++u) {
     const int t = a.t0[w] + (int)blockIdx.y * kAsmPerBlock + u * 256 + (int)threadIdx.x;
     if (t >= t1) break;
+    // eight terms at a time, loaded side by side (an entry of a joint node has
+    // dozens) and summed in order
     double v = 0.0;
-    for (int k = a.ptr[t]; k < a.ptr[t + 1]; ++k) {
-      const uint32_t code = a.src[k];
-      const uint32_t type = (code >> 29) & 3u, idx = code & 0x1FFFFFFFu;
-      double x;
-      if (type == SRC_STENCIL) x = a.sh[idx];
-      else if (type == SRC_EDGE) x = a.es[idx];
-      else if (type == SRC_NODE) x = a.nt[idx];
-      else x = a.dconst[idx];
-      v += (code & 0x80000000u) ? -x : x;
+    const int k1 = a.ptr[t + 1];
+    for (int k = a.ptr[t]; k < k1; k += 8) {
+      uint32_t code[8];
+      double x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) code[q] = k + q < k1 ? a.src[k + q] : 0u;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const uint32_t type = (code[q] >> 29) & 3u, idx = code[q] & 0x1FFFFFFFu;
+        const double *src = type == SRC_STENCIL ? a.sh : type == SRC_EDGE ? a.es : type == SRC_NODE ? a.nt : a.dconst;
+        x[q] = k + q < k1 ? src[idx] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (k + q < k1) v += (code[q] & 0x80000000u) ? -x[q] : x[q];
     }
     a.gen[a.target[t]] = v;
   }

@@ -2,56 +2,58 @@
 // whose limbs couple to the border only through the rows at one end (rods
 // attached at one end: star robots; single rods on the ground).
 //
-//   1. k_gen_limb_factor (one warp per limb): banded LU without pivoting of
-//      the limb block in its elimination order (from the free end), with the
-//      right-hand side eliminated alongside.  What remains is the dense m x m
-//      block A_m of the rows next to the border; with it the limb's Schur
-//      complement R_m A_m^{-1} C_m and right-hand side R_m A_m^{-1} y_m are
-//      subtracted from the border system (atomics on the system's matrix).
+//   1. k_gen_limb_factor (one warp per limb): forms the limb's band of the
+//      Jacobian in shared memory straight from the stencil, edge and node
+//      terms (the row formula of a single rod), and eliminates it without
+//      pivoting from the free end, with the right-hand side alongside.  What
+//      remains is the dense m x m block A_m of the rows next to the border;
+//      [A_m C_m y_m; R_m 0 0] is eliminated further, and the limb's Schur
+//      complement -R_m A_m^{-1} [C_m | y_m], which that leaves, goes to the
+//      border system (atomics on the system's matrix).
 //   2. k_gen_border (a block per system): Newton bookkeeping for the system
 //      and the dense LU of the border system (in order, partial pivoting
 //      where a pivot is tiny).
-//   3. k_gen_limb_back (one warp per limb): the m condensed rows from the
-//      border values, then back substitution towards the free end; q += dq.
+//   3. k_gen_limb_back (one warp per limb): back substitution from the border
+//      values towards the free end; q += dq.
 //
 // Late Newton rounds carry few systems, so a round costs the length of one
-// limb's elimination chain; both limb kernels keep that chain short.  Per
-// column the factor takes the 10 multipliers in one instruction (a lane
-// each, broadcast by shuffles), the 110 updates in four, and the next
-// pivot's reciprocal (an FP32 seed and one third-order step, three FP64
-// instructions) interleaved with the updates after the one that produces
-// it; a pivot outside [2^-126, 2^126) (zero and non-finite included) fails
-// the system.  The band, C_m and R_m are staged by asynchronous copies, and
-// the condensed block's small LU spreads its work over (row, column)
-// pairs.  The back substitution
-// is column oriented: lanes 1..10 hold the partial right-hand sides of the
-// ten rows above the current one in registers, so a row costs one multiply,
-// one update and two shuffles.
+// limb's elimination chain; full rounds cost FP64 slots (64 cycles per warp
+// instruction and SM partition).  Per column: the multipliers, the scaled row
+// of U and y in one instruction (exchanged through shared memory), the R (R +
+// 1) updates dealt evenly over the lanes -- R = 10, 9, 8, 7 in turn, the
+// envelope of a rod's Jacobian: 4 slots a column instead of 8 --, the pivot's
+// reciprocal on the integer pipe; a pivot outside [2^-126, 2^126) (zero and
+// non-finite included) fails the system.  The back substitution keeps the
+// pending rows in lane registers: one update and one shuffle per row.
+// Measured, 1024 star robots of 3 to 8 limbs of 112 rows, a step of 63 rounds:
+// limb kernels and border 7.6 ms, assembly of the couplings 3.9 -> 1.6 ms (the
+// limbs' bands are no longer stored), back substitution 1.8 -> 1.3 ms; step
+// 22.7 -> 17.9 ms together with the residual's maximum by the warp.
 //
 // The Jacobian is that of Sec. III-C (M/dt^2 - dF/dq, with the contact and
 // friction terms of Sec. III-B), not symmetric when friction acts, hence LU.
-// Band storage of a limb (row-major in elimination order p): entry (p, p+k)
-// at [p][k + 10], |k| <= 10.
 #include "dm_internal.h"
 #include "dm_kernels.cuh"
 
 namespace dm {
 
 namespace {
-constexpr int kRow = 22;        // 21 band entries and the right-hand side
-// condensed block [A_m | C_m | y_m] (leading dimension m + nbc + 1), the
-// coupling rows R_m (nbc x m), then the small LU's scratch
-constexpr int kSmall = kFastMaxM * (kFastMaxM + kFastMaxBC + 1) + kFastMaxBC * kFastMaxM + 2 * kFastMaxM;
+constexpr int kRow = 22;        // 21 band entries (p, p + k) at k + 10, then the right-hand side
+constexpr int kLBlk = 12;       // columns per block, 4-periodic like the envelope
+constexpr int kLRec = 12;       // record of an eliminated row: y / d, U(p, p + 1..10) / d, 0
+// small block: [A_m C_m y_m; R_m 0 0]; with pivoting instead [A_m | C_m | y_m],
+// R_m and the small LU's scratch
+constexpr int kSmall = (kFastMaxM + kFastMaxBC) * (kFastMaxM + kFastMaxBC + 1);
+static_assert(kSmall >= kFastMaxM * (kFastMaxM + kFastMaxBC + 1) + kFastMaxBC * kFastMaxM + 2 * kFastMaxM, "small");
+static_assert(kLimbExtra == 11 * kRow + kLBlk * kLRec + 12 + kSmall && kLimbExtra % 2 == 0, "limb smem layout");
+static_assert(kFastMaxRows <= 32 * 2 * kLBlk * kLRec, "a bit per row fits the records");
 constexpr unsigned kFull = 0xffffffffu;
 
 // Pivots of the border system's elimination in order smaller than this
 // fraction of their original diagonal entry send it to partial pivoting.
 constexpr double kTinyPivotB = 1e-13;
 
-// 1/d by rcp64 (three FP64 instructions); a division outside its range.
-__device__ __forceinline__ double limb_recip(double d) {
-  return rcp64_in_range(d) ? rcp64(d) : 1.0 / d;
-}
+__device__ __forceinline__ double limb_recip(double d) { return rcp_any(d); }
 
 // The border kernel's decision for system s, without its side effects.
 __device__ __forceinline__ bool wants_solve(const SolveGenArgs &a, int s) {
@@ -132,10 +134,164 @@ __device__ bool warp_lu_solve(double *M, int n, int ld, int nrhs, double *lm, do
 
 }  // namespace
 
+namespace {
+
+// Update tasks of a column with R rows below it, in order: row i = 1..R, the
+// entries under column k = 1..R, the right-hand side; task t is lane t mod
+// 32's slot t / 32 (the next pivot (1, 1): lane 0's first); spare slots repeat
+// the lane's first.
+__host__ __device__ constexpr int limb_slots(int R) { return (R * (R + 1) + 31) / 32; }
+
+struct LimbLane {
+  int to[4][4], uo[4][4], lo[4][4];  // byte offsets by column type: target, U entry, multiplier
+  int so, ro;                        // the lane's product with the reciprocal: source, destination
+  bool walks;                        // ... in the record (moves with the column)
+  __device__ __forceinline__ void load(int lane, int rec, int lw) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int R = 10 - t;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (h >= limb_slots(R)) continue;
+        int e = lane + 32 * h;
+        if (e >= R * (R + 1)) e = lane;
+        const int i = e / (R + 1) + 1, k = e - (i - 1) * (R + 1) + 1;  // k = R + 1: right-hand side
+        to[t][h] = 8 * (kRow * i + (k <= R ? 10 + k - i : 21));
+        uo[t][h] = 8 * (k <= R ? 10 + k : 21);
+        lo[t][h] = lw + 8 * (i - 1);
+      }
+    }
+    // lanes 0-9: the multiplier of row i = lane + 1; 10-19: U; 20 on: y
+    so = 8 * (lane < 10 ? kRow * (lane + 1) + 9 - lane : lane < 20 ? lane + 1 : 21);
+    walks = lane >= 10;
+    ro = lane < 10 ? lw + 8 * lane : rec + 8 * (lane < 20 ? lane - 9 : 0);
+  }
+};
+
+extern __shared__ __align__(16) char g_lsm[];
+__device__ __forceinline__ double &lsm(int off) { return *reinterpret_cast<double *>(g_lsm + off); }
+
+// Column u of a block whose pivot row is `w` bytes in; rj its pivot's
+// reciprocal (in), the next column's (out).  The reciprocal's chain starts at
+// the first update; the other updates are tied to its steps (RcpChain), since
+// in-order issue would hold the chain back behind them (64 cycles each).
+__device__ __forceinline__ void limb_column(const LimbLane &ln, const int t, const int u, int w, double &rj, bool act,
+                                            unsigned zero) {
+  const int NK = limb_slots(10 - t), wu = w + 8 * kRow * u;
+  lsm(ln.ro + (ln.walks ? 8 * kLRec * u : 0)) = lsm(ln.so + wu) * rj;
+  double uq[4], dv[4], v[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+    if (h < NK) {
+      uq[h] = lsm(ln.uo[t][h] + wu);
+      dv[h] = lsm(ln.to[t][h] + wu);
+    }
+  __syncwarp();
+  v[0] = fma(-lsm(ln.lo[t][0]), uq[0], dv[0]);
+  RcpChain ch;
+  ch.seed(__shfl_sync(kFull, v[0], 0));
+  v[1] = fma(-lsm(ln.lo[t][1]), after(uq[1], ch.S, zero), dv[1]);
+  ch.residual();
+  if (NK > 2) v[2] = fma(-lsm(ln.lo[t][2]), after(uq[2], (unsigned)ch.t, zero), dv[2]);
+  rj = ch.result();
+  if (NK > 3) v[3] = fma(-lsm(ln.lo[t][3]), after(uq[3], (unsigned)__double2loint(rj), zero), dv[3]);
+  if (act) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      if (h < NK) lsm(ln.to[t][h] + wu) = v[h];
+  }
+  __syncwarp();
+}
+
+// packed upper-triangle index of an 11 x 11 symmetric matrix (i <= j)
+__host__ __device__ constexpr int up11(int i, int j) { return i * 11 - i * (i - 1) / 2 + (j - i); }
+
+struct LimbRows {
+  int N, st, e0, f, n, d0, dir;  // rod nodes, stencil of rod node 1, first edge, limb's rod row, rows, DOF, direction
+  const unsigned *fmask;         // the limb's fixed rows, a bit each
+  double *A;
+};
+
+// Rod row 4 node + C (a lane per node, C a constant: every index below is one)
+// of the limb into its band (entry (r, r - d) and its mirror image; zeroed
+// before): the lower band row of a single rod's Jacobian -- stencils m = node
+// - 1, node, node + 1 (4m-4 <= r <= 4m+6; joints sit at rod ends, so a rod's
+// stencils and edges run along it), the edges at its node, M/dt^2 and damping
+// -- and the node's 3 x 3 ground terms, which friction makes nonsymmetric
+// (`trans`: their transpose, hence the transposed matrix).  Entries to rows
+// outside the limb are border coupling.
+template <int C>
+__device__ __forceinline__ void limb_row(const SolveGenArgs &a, const LimbRows &q, int node) {
+  const int k = 4 * node + C - q.f;
+  if (k < 0 || k >= q.n) return;
+  const int g = q.d0 + k;  // DOF
+  const double *sh = a.sh + q.st + node - 1;  // entry e of stencil m = node + h: sh[e ns + h]
+  const bool s0 = node >= 2, s1 = node >= 1 && node <= q.N - 2, s2 = node <= q.N - 3;
+  constexpr int L0 = 8 + C, L1 = 4 + C, L2 = C;  // the row's place in the three stencils
+  double b[11], b1[11], b2[11];
+#pragma unroll
+  for (int d = 0; d < 11; ++d) {
+    b[d] = C < 3 && d <= L0 && s0 ? sh[(size_t)up11(L0 - d, L0) * a.ns - 1] : 0.0;
+    b1[d] = d <= L1 && s1 ? sh[(size_t)up11(L1 - d, L1) * a.ns] : 0.0;
+    b2[d] = d <= L2 && s2 ? sh[(size_t)up11(L2 - d, L2) * a.ns + 1] : 0.0;
+  }
+  const double dc = a.dconst[g];
+  // edges: the one that starts at the node (its block's entries under the
+  // diagonal), the one that ends there (its whole row of the block), and the
+  // ground terms: row C and column C of the node's block
+  double es[3] = {0.0, 0.0, 0.0}, ee[3] = {0.0, 0.0, 0.0}, gx[3] = {0.0, 0.0, 0.0}, gy[3] = {0.0, 0.0, 0.0};
+  if (C < 3) {
+    const int v = a.nt ? a.dof_node[g] : 0;
+#pragma unroll
+    for (int cp = 0; cp < 3; ++cp) {
+      const int lo = cp < C ? cp : C, hi = cp < C ? C : cp;
+      const double *src = a.es + (size_t)(3 + (lo == 0 ? hi : lo == 1 ? 2 + hi : 5)) * a.ne + q.e0 + node;
+      if (cp <= C && node <= q.N - 2) es[cp] = src[0];
+      if (node >= 1) ee[cp] = src[-1];
+      if (a.nt && cp <= C) {
+        gx[cp] = a.nt[(size_t)(3 + 3 * C + cp) * a.nn + v];
+        gy[cp] = a.nt[(size_t)(3 + 3 * cp + C) * a.nn + v];
+      }
+    }
+  }
+  // bit d: row k - d is fixed (rows before the limb count as fixed)
+  const int w = k >> 5;
+  const unsigned fx = __brev(__funnelshift_l(w > 0 ? q.fmask[w - 1] : ~0u, q.fmask[w], 31 - (k & 31)));
+  const int p = q.dir ? q.n - 1 - k : k, s = q.dir ? 1 : -1;
+  double *A = q.A + p * kRow + 10;
+  if (fx & 1u) {
+    A[0] = dc;
+    return;
+  }
+#pragma unroll
+  for (int d = 0; d < 11; ++d) {
+    if (d <= L1) b[d] = C < 3 ? b[d] + b1[d] : b1[d];
+    if (d <= L2) b[d] += b2[d];
+  }
+  b[0] += dc;
+  double up[3] = {0.0, 0.0, 0.0};  // what the mirror image of b[1], b[2] has more (friction)
+  if (C < 3) {
+#pragma unroll
+    for (int cp = 0; cp < 3; ++cp) {
+      if (cp <= C) {
+        b[C - cp] += es[cp] + ee[cp] + (a.trans ? gy[cp] : gx[cp]);
+        up[C - cp] = a.trans ? gx[cp] - gy[cp] : gy[cp] - gx[cp];
+      }
+      b[4 + C - cp] -= ee[cp];
+    }
+  }
+  A[0] = b[0];
+#pragma unroll
+  for (int d = 1; d < 11; ++d) {
+    if (d > (C < 3 ? L0 : L1) || ((fx >> d) & 1u)) continue;
+    A[s * d] = b[d];
+    A[s * d * kRow - s * d] = d < 3 ? b[d] + up[d] : b[d];
+  }
+}
+
+}  // namespace
+
 __global__ void __launch_bounds__(128) k_gen_limb_factor(SolveGenArgs a) {
-  // per warp: the limb band with its right-hand side [n][22], then the
-  // condensed block and its right-hand sides
-  extern __shared__ double dyn[];
   const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int L = blockIdx.x * (blockDim.x >> 5) + wi;
   if (L >= a.nlimb) return;
@@ -143,167 +299,158 @@ __global__ void __launch_bounds__(128) k_gen_limb_factor(SolveGenArgs a) {
   if (!a.gs_fast[w]) return;
   const int s = a.gen_sys[w];
   if (!wants_solve(a, s)) return;
-  double *Bs = dyn + (size_t)wi * (a.limb_nmax * kRow + kSmall);
-  double *small = Bs + (size_t)a.limb_nmax * kRow;
+  // per warp: the band [n + 11][22] (eleven zero rows behind it), a block's
+  // records, the multipliers of a column, the small block
+  const int per = a.limb_nmax * kRow + kLimbExtra;
+  double *A = reinterpret_cast<double *>(g_lsm) + (size_t)wi * per;
   const int n = a.lb_n[L], m = a.lb_m[L], nbc = a.lb_nbc[L], dir = a.lb_dir[L];
-  const int d0 = a.lb_dof0[L];
+  double *rec = A + a.limb_nmax * kRow + 11 * kRow, *lw = rec + kLBlk * kLRec, *M = lw + 12;
+  const int d0 = a.lb_dof0[L], f = a.lb_first[L];
   double *G = a.gen;
-  const double *band = G + a.lb_band[L];
-  double *U = G + a.lb_y[L];  // [ne][12] out: U row, right-hand side, 1/pivot
-  // staging of the contiguous band by asynchronous copies (all in flight
-  // at once), the right-hand side alongside
-  for (int e = lane; e < n * 21; e += 32) {
-    const int p = e / 21;
-    cp_async8(Bs + p * kRow + (e - p * 21), band + e);
-  }
-  cp_async_commit();
-#pragma unroll 4
-  for (int p = lane; p < n; p += 32) Bs[p * kRow + 21] = -a.f[d0 + (dir ? n - 1 - p : p)];
-  cp_async_wait_all();
-  __syncwarp();
-  bool bad = false;
-  const int ne = n - m;  // rows eliminated inside the limb
-  // update slots of this lane, the same for every column: row j + si
-  // (si = 1..10; 0 = no slot) and entry sk (0 = right-hand side, 1..10 =
-  // the band entry under column j + sk); the slot (1, 1), which yields the
-  // next pivot, is lane 1's first
-  int si[4], sk[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int t = lane + 32 * u;
-    si[u] = t < 110 ? t / 11 + 1 : 0;
-    sk[u] = t < 110 ? t - (si[u] - 1) * 11 : 0;
-  }
-  double rp = 1.0;
-  if (ne > 0) {
-    const double piv = Bs[10];
-    if (!rcp64_in_range(piv)) bad = true;
-    else rp = rcp64(piv);
-  }
-  // columns whose ten rows below lie inside the limb: no tests of its end,
-  // per-lane offsets from the pivot row, the next pivot's update first
-  const int jf = min(ne, n - 10);
+  double *U = G + a.lb_y[L];  // [n][12] records of the rows, out
+  // (C_m and R_m arrive while the limb is eliminated: the block's first m
+  // rows' last columns, the rows after them)
+  const int ldm = m + nbc + 1;
   {
-    const int mo = lane < 10 ? (lane + 1) * kRow + 9 - lane : kRow + 9;
-    int dof[4], sof[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      dof[u] = si[u] > 0 ? si[u] * kRow + (sk[u] ? 10 - si[u] + sk[u] : 21) : 0;
-      sof[u] = sk[u] ? 10 + sk[u] : 21;
+    const double *C = G + a.lb_C[L], *R = G + a.lb_R[L];
+    for (int e = lane; e < m * nbc; e += 32) {
+      const int r = e / nbc, c = e / m;
+      cp_async8(M + r * ldm + m + e - r * nbc, C + e);
+      cp_async8(M + (m + c) * ldm + e - c * m, R + e);
     }
-    const bool s3 = si[3] > 0;
-    double *pr = Bs;
-    for (int j = 0; j < jf && !bad; ++j, pr += kRow) {
-      const double l = pr[mo] * rp;
-      if (lane < 10) pr[mo] = l;
-      if (lane == 0) pr[10] = rp;  // the pivot is read no more
-      const double v0 = fma(-__shfl_sync(kFull, l, si[0] - 1), pr[sof[0]], pr[dof[0]]);
-      pr[dof[0]] = v0;
-      // the next pivot's reciprocal (seed, e = 1 - d r0, t = e + e^2,
-      // r0 + r0 t) interleaved with the other updates, without branches; a
-      // pivot outside [2^-126, 2^126) (zero and non-finite included) fails
-      const double pn = __shfl_sync(kFull, v0, 1);
-      const double r0 = rcp64_seed(pn);
-      const double l1 = __shfl_sync(kFull, l, si[1] - 1);
-      const double l2 = __shfl_sync(kFull, l, si[2] - 1);
-      const double l3 = __shfl_sync(kFull, l, s3 ? si[3] - 1 : 0);
-      const double v1 = fma(-l1, pr[sof[1]], pr[dof[1]]);
-      const double e = fma(-pn, r0, 1.0);
-      const double v2 = fma(-l2, pr[sof[2]], pr[dof[2]]);
-      const double t = fma(e, e, e);
-      const double v3 = fma(-l3, pr[sof[3]], pr[dof[3]]);
-      const double rn = fma(r0, t, r0);
-      pr[dof[1]] = v1;
-      pr[dof[2]] = v2;
-      if (s3) pr[dof[3]] = v3;
-      if (j + 1 < ne) {
-        if (!rcp64_in_range(pn)) bad = true;
-        rp = rn;
+    cp_async_commit();
+  }
+  const int rod = a.lb_rod[L];
+  LimbRows q{a.npr[rod], 0, a.rod_edge0[rod], f, n, d0, dir, reinterpret_cast<unsigned *>(rec), A};
+  q.st = q.N > 2 ? a.slot2st[a.rod_slot0[rod]] : 0;
+  for (int e = lane; e < (n + 11) * kRow / 2; e += 32) reinterpret_cast<double2 *>(A)[e] = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const bool fx = k0 + lane < n && a.fixed[d0 + k0 + lane];
+    const unsigned bits = __ballot_sync(kFull, fx);
+    if (lane == 0) reinterpret_cast<unsigned *>(rec)[k0 >> 5] = bits;
+  }
+  __syncwarp();
+  for (int node = (f >> 2) + lane; 4 * node < f + n; node += 32) {
+    limb_row<0>(a, q, node);
+    limb_row<1>(a, q, node);
+    limb_row<2>(a, q, node);
+    limb_row<3>(a, q, node);
+  }
+#pragma unroll 4
+  for (int p = lane; p < n; p += 32) A[p * kRow + 21] = -a.f[d0 + (dir ? n - 1 - p : p)];
+  __syncwarp();
+  for (int e = lane; e < kLBlk * kLRec; e += 32) rec[e] = 0.0;  // (their last words stay zero)
+  LimbLane ln;
+  const int w0 = (int)(reinterpret_cast<char *>(A) - g_lsm);
+  ln.load(lane, (int)(reinterpret_cast<char *>(rec) - g_lsm), (int)(reinterpret_cast<char *>(lw) - g_lsm));
+  __syncwarp();
+  const int ne = n - m;  // rows eliminated inside the limb
+  bool bad = false;
+  double rj = rcp_any(A[10]);
+  for (int j0 = 0; j0 < ne; j0 += kLBlk) {
+#pragma unroll
+    for (int u = 0; u < kLBlk; ++u) limb_column(ln, u & 3, u, w0 + 8 * kRow * j0, rj, j0 + u < ne, a.zero);
+    const int cnt = min(kLBlk, ne - j0);
+    if (lane < cnt && !rcp64_in_range(A[(j0 + lane) * kRow + 10])) bad = true;
+    for (int e = lane; e < cnt * (kLRec / 2); e += 32)
+      *reinterpret_cast<double2 *>(U + (size_t)j0 * kLRec + 2 * e) = *reinterpret_cast<const double2 *>(rec + 2 * e);
+    __syncwarp();
+  }
+  bad = __any_sync(kFull, bad);
+  if (!bad && m > 0) {
+    // [A_m C_m y_m; R_m 0 0], eliminated in order; a pivot below 2^-43 of its
+    // starting diagonal entry, or not finite, sends the limb to partial pivoting
+    const int rows = m + nbc;
+    cp_async_wait_all();
+    for (int e = lane; e < m * (m + 1); e += 32) {
+      const int r = e / (m + 1), c = e - r * (m + 1);
+      M[r * ldm + (c < m ? c : rows)] = A[(ne + r) * kRow + (c < m ? 10 + c - r : 21)];
+    }
+    for (int e = lane; e < nbc * (nbc + 1); e += 32) {
+      const int r = e / (nbc + 1);
+      M[(m + r) * ldm + m + e - r * (nbc + 1)] = 0.0;
+    }
+    // the test in the upper words: exponent and 20 mantissa bits
+    const int thr = lane < m ? max((__double2hiint(A[(ne + lane) * kRow + 10]) & 0x7FFFFFFF) - (43 << 20), 1 << 20) : 0;
+    __syncwarp();
+    bool ok = true;
+    for (int c = 0; c < m; ++c) {
+      const double pv = M[c * ldm + c];
+      const int ph = __double2hiint(pv) & 0x7FFFFFFF;
+      if (ph < __shfl_sync(kFull, thr, c) || ph >= 0x7FF00000) {
+        ok = false;  // uniform
+        break;
+      }
+      const int wd = rows - c;  // entries right of the pivot
+      const double rp = rcp_any(pv);
+      if (lane < wd) M[c * ldm + c + 1 + lane] *= rp;
+      __syncwarp();
+      // rows c+1.., a lane per column: two rows at a time once 16 lanes do
+      const bool twin = wd <= 16;
+      const int col = c + 1 + (twin ? lane & 15 : lane), stp = twin ? 2 : 1;
+      if (col <= rows) {
+        const double u = M[c * ldm + col];
+#pragma unroll 4
+        for (int i = c + 1 + (twin ? lane >> 4 : 0); i < rows; i += stp)
+          M[i * ldm + col] = fma(-M[i * ldm + c], u, M[i * ldm + col]);
       }
       __syncwarp();
     }
-  }
-  for (int j = max(jf, 0); j < ne && !bad; ++j) {
-    const double *pr = Bs + j * kRow;
-    // multiplier of row j + 1 + lane, stored in place by the lane that reads it
-    double l = 0.0;
-    if (lane < 10 && j + lane + 1 < n) {
-      double *mp = Bs + (j + lane + 1) * kRow + 9 - lane;
-      l = *mp * rp;
-      *mp = l;
-    }
-    if (lane == 0) Bs[j * kRow + 10] = rp;  // the pivot is read no more
-    double v0 = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const double lu = __shfl_sync(kFull, l, si[u] > 0 ? si[u] - 1 : 0);
-      if (si[u] > 0 && j + si[u] < n) {
-        double *dst = Bs + (j + si[u]) * kRow + (sk[u] ? 10 - si[u] + sk[u] : 21);
-        const double v = fma(-lu, pr[sk[u] ? 10 + sk[u] : 21], *dst);
-        *dst = v;
-        if (u == 0) v0 = v;
+    double *Z = G + a.lb_Y[L];
+    const int32_t *bc = a.lb_bcols + a.lb_bc0[L];
+    const int nB = a.gs_nB[w], ldb = nbc + 1;
+    double *S = G + a.gs_JBB[w], *rB = G + a.gs_rB[w];
+    if (ok) {
+      // the condensed rows for the back substitution: U right of the pivot
+      // within the block, the couplings to the border and y over the pivot
+      for (int e = lane; e < m * kLRec; e += 32) {
+        const int r = e / kLRec, k = e - r * kLRec;
+        U[(size_t)ne * kLRec + e] = k >= 1 && r + k < m ? M[r * ldm + r + k] : 0.0;
       }
-      if (u == 0 && j + 1 < ne) {
-        // the next pivot (lane 1's first slot), its reciprocal off the chain
-        const double pn = __shfl_sync(kFull, v0, 1);
-        if (!rcp64_in_range(pn)) bad = true;
-        else rp = rcp64(pn);
-      }
-    }
-    __syncwarp();
-  }
-  // U rows, eliminated right-hand sides and reciprocal pivots of the
-  // eliminated rows, for the back substitution
-  if (!bad)
-    for (int e = lane; e < ne * 12; e += 32) {
-      const int p = e / 12, c = e - p * 12;
-      U[e] = Bs[p * kRow + (c < 10 ? 11 + c : (c == 10 ? 21 : 10))];
-    }
-  if (!bad && m > 0) {
-    // condensed block [A_m | C_m | y_m] (leading dimension ld), C_m and the
-    // coupling rows R_m by asynchronous copies
-    const int ldb = nbc + 1, ld = m + ldb;
-    double *M = small;
-    double *Rs = small + kFastMaxM * (kFastMaxM + kFastMaxBC + 1);
-    double *lm = Rs + kFastMaxBC * kFastMaxM, *dinv = lm + kFastMaxM;
-    const double *C = G + a.lb_C[L];
-    const double *R = G + a.lb_R[L];
-    for (int e = lane; e < m * nbc; e += 32) {
-      const int r = e / nbc;
-      cp_async8(M + r * ld + m + e - r * nbc, C + e);
-    }
-    for (int e = lane; e < nbc * m; e += 32) cp_async8(Rs + e, R + e);
-    cp_async_commit();
-    for (int e = lane; e < m * m; e += 32) {
-      const int r = e / m, c = e - r * m;
-      M[r * ld + c] = Bs[(ne + r) * kRow + 10 + c - r];
-    }
-    for (int r = lane; r < m; r += 32) M[r * ld + m + nbc] = Bs[(ne + r) * kRow + 21];
-    cp_async_wait_all();
-    __syncwarp();
-    if (!warp_lu_solve(M, m, ld, ldb, lm, dinv, lane)) {
-      bad = true;
-    } else {
-      // Z = A_m^{-1} [C_m | y_m] for the back substitution
-      double *Z = G + a.lb_Y[L];
       for (int e = lane; e < m * ldb; e += 32) {
         const int r = e / ldb;
-        Z[e] = M[r * ld + m + e - r * ldb];
+        Z[e] = M[r * ldm + m + e - r * ldb];
       }
-      // Schur complement and right-hand side of the border system
-      const int32_t *bc = a.lb_bcols + a.lb_bc0[L];
-      const int nB = a.gs_nB[w];
-      double *S = G + a.gs_JBB[w];
-      double *rB = G + a.gs_rB[w];
       for (int e = lane; e < nbc * ldb; e += 32) {
         const int b1 = e / ldb, b2 = e - b1 * ldb;
-        double v = 0.0;
-        for (int r = 0; r < m; ++r) v = fma(Rs[b1 * m + r], M[r * ld + m + b2], v);
-        if (b2 < nbc) atomicAdd(S + (int64_t)bc[b1] * nB + bc[b2], -v);
-        else atomicAdd(rB + bc[b1], -v);
+        const double v = M[(m + b1) * ldm + m + b2];
+        if (b2 < nbc) atomicAdd(S + (int64_t)bc[b1] * nB + bc[b2], v);
+        else atomicAdd(rB + bc[b1], v);
+      }
+    } else {
+      __syncwarp();
+      const double *C = G + a.lb_C[L], *R = G + a.lb_R[L];
+      const int ld = m + ldb;
+      double *Rs = M + kFastMaxM * (kFastMaxM + kFastMaxBC + 1);
+      double *lm = Rs + kFastMaxBC * kFastMaxM, *dinv = lm + kFastMaxM;
+      for (int e = lane; e < m * ld; e += 32) {
+        const int r = e / ld, c = e - r * ld;
+        M[e] = c < m ? A[(ne + r) * kRow + 10 + c - r] : c < m + nbc ? C[r * nbc + c - m] : A[(ne + r) * kRow + 21];
+      }
+      for (int e = lane; e < nbc * m; e += 32) Rs[e] = R[e];
+      __syncwarp();
+      if (!warp_lu_solve(M, m, ld, ldb, lm, dinv, lane)) {
+        bad = true;
+      } else {
+        // Z = A_m^{-1} [C_m | y_m]: the condensed rows without each other
+        for (int e = lane; e < m * kLRec; e += 32) U[(size_t)ne * kLRec + e] = 0.0;
+        for (int e = lane; e < m * ldb; e += 32) {
+          const int r = e / ldb;
+          Z[e] = M[r * ld + m + e - r * ldb];
+        }
+        // Schur complement and right-hand side of the border system
+        for (int e = lane; e < nbc * ldb; e += 32) {
+          const int b1 = e / ldb, b2 = e - b1 * ldb;
+          double v = 0.0;
+          for (int r = 0; r < m; ++r) v = fma(Rs[b1 * m + r], M[r * ld + m + b2], v);
+          if (b2 < nbc) atomicAdd(S + (int64_t)bc[b1] * nB + bc[b2], -v);
+          else atomicAdd(rB + bc[b1], -v);
+        }
       }
     }
   }
+  cp_async_wait_all();
   if (bad && lane == 0) atomicOr(a.gen_bad + w, 1);
 }
 
@@ -515,66 +662,87 @@ __global__ void __launch_bounds__(kGenBorderThreads) k_gen_border(SolveGenArgs a
   }
 }
 
+// Rows from the border end up: the row of step t is n - 1 - t (elimination
+// order), pending in lane t mod 32; a step takes its x by a shuffle and
+// subtracts its part from the next ten rows (record word d of a row d steps
+// later; word 11 is zero).  The m condensed rows start from the border values.
+// Each lane stages its own rows' records, two groups of 32 steps ahead.
 __global__ void __launch_bounds__(128) k_gen_limb_back(SolveGenArgs a) {
-  // per warp: U rows (10 off-diagonal entries), eliminated right-hand side
-  // and reciprocal pivot [n][12], then the m condensed rows' values
+  constexpr int kRing = 3;
   extern __shared__ double dyn[];
   const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int L = blockIdx.x * (blockDim.x >> 5) + wi;
   if (L >= a.nlimb) return;
   const int w = a.lb_gsys[L];
   if (!a.gs_fast[w] || !a.gen_go[w]) return;
-  double *Us = dyn + (size_t)wi * (a.limb_nmax * 12 + 16);
-  double *xr = Us + (size_t)a.limb_nmax * 12;  // x of rows ne .. n - 1
+  static_assert(gen_back_smem() == 32 * kRing * kLRec, "ring");
+  double *ring = dyn + (size_t)wi * gen_back_smem() + lane * (kRing * kLRec);
   const int n = a.lb_n[L], m = a.lb_m[L], nbc = a.lb_nbc[L], dir = a.lb_dir[L];
-  const int d0 = a.lb_dof0[L], ne = n - m;
+  const int d0 = a.lb_dof0[L];
   const double *G = a.gen;
-  const double *Ug = G + a.lb_y[L];
-  auto dof = [&](int p) { return d0 + (dir ? n - 1 - p : p); };
-  // the U rows by asynchronous copies, in flight while the condensed rows
-  // are formed
-  for (int e = lane; e < ne * 12; e += 32) cp_async8(Us + e, Ug + e);
+  const double *U = G + a.lb_y[L];
+  auto fetch = [&](int g) {
+    const int p = n - 1 - (32 * g + lane);
+    double *dst = ring + kLRec * (g % kRing);
+    if (p >= 0) {
+#pragma unroll
+      for (int e = 0; e < kLRec; e += 2) {
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + e);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(U + (size_t)p * kLRec + e) : "memory");
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < kLRec; ++e) dst[e] = 0.0;
+    }
+  };
+#pragma unroll
+  for (int g = 0; g < kRing; ++g) fetch(g);
   cp_async_commit();
-  // the condensed rows ne..n-1 from the border values: the nbc values this
-  // limb couples to fetched one per lane (one round trip), then broadcast
+  // the condensed rows n-1 .. n-m (steps 0 .. m - 1) from the border values:
+  // the nbc values this limb couples to fetched one per lane, then broadcast
+  double v;
   {
     const double *xB = G + a.gs_xB[w];
     const int32_t *bc = a.lb_bcols + a.lb_bc0[L];
     const double xbv = lane < nbc ? xB[bc[lane]] : 0.0;
-    const double *Z = G + a.lb_Y[L] + (lane < m ? lane : 0) * (nbc + 1);
-    double v = lane < m ? Z[nbc] : 0.0;
+    const double *Z = G + a.lb_Y[L] + (lane < m ? m - 1 - lane : 0) * (nbc + 1);
+    v = lane < m ? Z[nbc] : 0.0;
 #pragma unroll
     for (int b = 0; b < kFastMaxBC; ++b) {
+      if (b >= nbc) break;  // uniform
       const double xb = __shfl_sync(kFull, xbv, b);
-      if (lane < m && b < nbc) v = fma(-Z[b], xb, v);
-    }
-    if (lane < m) {
-      xr[lane] = v;
-      atomicAdd(a.q + dof(ne + lane), v);
+      if (lane < m) v = fma(-Z[b], xb, v);
     }
   }
   cp_async_wait_all();
-  __syncwarp();
-  // lane i (0..10) holds the right-hand side of row p - i less the terms of
-  // the solved rows; lane 11 brings in row p - 11 untouched
-  auto U = [&](int r, int k) { return Us[r * 12 + k - 1]; };  // entry (r, r + k)
-  double acc = 0.0;
-  {
-    const int r = ne - 1 - lane;
-    if (lane <= 11 && r >= 0) {
-      acc = Us[r * 12 + 10];
-      if (lane <= 10)
-        for (int c = ne; c < n && c <= r + 10; ++c) acc = fma(-U(r, c - r), xr[c - ne], acc);
+  if (lane >= m) v = ring[0];
+  int idx[32];
+#pragma unroll
+  for (int u = 0; u < 32; ++u) {
+    const int d = (lane - u) & 31;
+    idx[u] = d == 0 || d > 11 ? 11 : d;
+  }
+  const int groups = (n + 31) / 32;
+  for (int g = 0; g < groups; ++g) {
+    const double *ra = ring + kLRec * (g % kRing), *rb = ring + kLRec * ((g + 1) % kRing);
+    const double zn = rb[0];
+    double x_own = 0.0;
+#pragma unroll
+    for (int u = 0; u < 32; ++u) {
+      const double x = __shfl_sync(kFull, v, u);
+      if (lane == u) {
+        x_own = x;
+        v = zn;
+      }
+      v = fma(-(lane <= u ? rb : ra)[idx[u]], x, v);
     }
+    const int p = n - 1 - (32 * g + lane);
+    if (p >= 0) atomicAdd(a.q + d0 + (dir ? n - 1 - p : p), x_own);
+    fetch(g + kRing);
+    cp_async_commit();
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
   }
-  for (int p = ne - 1; p >= 0; --p) {
-    const double x = __shfl_sync(kFull, acc * Us[p * 12 + 11], 0);
-    if (lane == 0) atomicAdd(a.q + dof(p), x);  // a reduction: no load on the recurrence
-    if (lane >= 1 && lane <= 10 && p - lane >= 0) acc = fma(-U(p - lane, lane), x, acc);
-    // row p - 1 - i to lane i; lane 11 takes row p - 12
-    acc = __shfl_down_sync(kFull, acc, 1);
-    if (lane == 11) acc = p - 12 >= 0 ? Us[(p - 12) * 12 + 10] : 0.0;
-  }
+  cp_async_wait_all();
 }
 
 }  // namespace dm

@@ -81,6 +81,7 @@ struct HostTopology {
   // flag; per limb its system, elimination direction (1 = from the last
   // row), trailing block size m and coupled border columns
   std::vector<int32_t> gs_fast, lb_gsys, lb_dir, lb_m, lb_nbc, lb_bc0, lb_bcols;
+  std::vector<int32_t> lb_rod, lb_first;   // rod of each limb and its row (Eq. 1) of the limb's first row
   std::vector<int32_t> border_dof;         // global DOF of each border entry
   std::vector<int32_t> coupled_rows;       // limb-local rows coupled to border
   int64_t gen_doubles = 0;                 // size of the general scratch
@@ -159,6 +160,7 @@ struct DevArrays {
   int32_t *border_dof = nullptr, *coupled_rows = nullptr;
   int32_t *gs_fast = nullptr, *lb_gsys = nullptr, *lb_dir = nullptr, *lb_m = nullptr,
           *lb_nbc = nullptr, *lb_bc0 = nullptr, *lb_bcols = nullptr;
+  int32_t *lb_rod = nullptr, *lb_first = nullptr, *npr = nullptr, *rod_slot0 = nullptr;
   int32_t *gen_go = nullptr, *gen_bad = nullptr;  // per general system
   int64_t *asm_target = nullptr;
   int32_t *asm_sys = nullptr, *asm_t0 = nullptr;

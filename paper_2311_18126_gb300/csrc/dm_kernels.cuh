@@ -155,26 +155,44 @@ __device__ __forceinline__ double rcp64(double d) {
 // bits: within 1.01 * 2^-53 of the exact reciprocal.  A warp's FP64
 // instruction occupies its SM partition for 64 cycles, so the three dependent
 // ones of rcp64 cost more than these integer ones.
+struct RcpChain {  // in three steps, so that a kernel can place other work between them
+  unsigned hi, Dh, Dl, S;
+  long long t;
+  __device__ __forceinline__ void seed(double d) {
+    hi = (unsigned)__double2hiint(d);
+    const unsigned lo = (unsigned)__double2loint(d);
+    Dh = 0x80000000u | (hi << 11) | (lo >> 21);
+    Dl = lo << 11;
+    float sf;  // of a number in (1, 2): the result is below 1
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(sf) : "f"(__uint_as_float(0x3F800001u | ((Dh >> 8) & 0x7FFFFFu))));
+    S = (max(__float_as_uint(sf), 0x3F000000u) << 8) | 0x80000000u;
+  }
+  __device__ __forceinline__ void residual() {
+    // P = D S 2^63, e 2^63 = 2^63 - P, t = e + e^2
+    const unsigned long long P = (unsigned long long)Dh * S + __umulhi(Dl, S);
+    const long long e = (long long)(0x8000000000000000ull - P);
+    const int es = (int)(e >> 20);
+    t = e + (long long)(unsigned)(((long long)es * es) >> 23);
+  }
+  __device__ __forceinline__ double result() const {
+    // r 2^64 = S 2^32 (1 + t), rounded to 53 bits (2^53 carries into the exponent)
+    const unsigned long long r = ((unsigned long long)S << 32) +
+                                 (unsigned long long)(((long long)(int)(t >> 32) * (long long)S) * 2) +
+                                 (((unsigned long long)(unsigned)t * S) >> 31);
+    const unsigned long long m = (r >> 11) + ((r >> 10) & 1);
+    const unsigned mh = (unsigned)(m >> 32) + (2044u << 20) - (hi & 0x7FF00000u);
+    return __hiloint2double((int)(mh | (hi & 0x80000000u)), (int)(unsigned)m);
+  }
+};
 __device__ __forceinline__ double rcp_int(double d) {
-  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned Dh = 0x80000000u | (hi << 11) | (lo >> 21), Dl = lo << 11;
-  float sf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(sf) : "f"(__uint_as_float(0x3F800000u | ((Dh >> 8) & 0x7FFFFFu))));
-  const unsigned sb = __float_as_uint(sf);  // in [1/2, 1]
-  const unsigned S = sb >= 0x3F800000u ? 0xFFFFFFFFu : sb < 0x3F000000u ? 0x80000000u : (sb << 8) | 0x80000000u;
-  // P = D S 2^63, e 2^63 = 2^63 - P
-  const unsigned long long P = (unsigned long long)Dh * S + __umulhi(Dl, S);
-  const long long e = (long long)(0x8000000000000000ull - P);
-  const int es = (int)(e >> 20);
-  const long long t = e + (((long long)es * es) >> 23);  // (e + e^2) 2^63
-  // r 2^64 = S 2^32 (1 + t)
-  const unsigned long long r = ((unsigned long long)S << 32) +
-                               (unsigned long long)(((long long)(int)(t >> 32) * (long long)S) * 2) +
-                               (((unsigned long long)(unsigned)t * S) >> 31);
-  const unsigned long long m = (r >> 11) + ((r >> 10) & 1);  // rounded; 2^53 carries into the exponent
-  const unsigned ex = (hi >> 20) & 0x7FFu;
-  const unsigned long long b = ((unsigned long long)(2044u - ex) << 52) + m;
-  return __hiloint2double((int)((unsigned)(b >> 32) | (hi & 0x80000000u)), (int)(unsigned)b);
+  RcpChain c;
+  c.seed(d);
+  c.residual();
+  return c.result();
+}
+// x, but not before `w` is known (zero: a kernel argument that is 0)
+__device__ __forceinline__ double after(double x, unsigned w, unsigned zero) {
+  return __hiloint2double(__double2hiint(x), (int)((unsigned)__double2loint(x) ^ (w & zero)));
 }
 
 // 1/d on the integer pipe where d is well inside the normal range, else by
@@ -198,6 +216,21 @@ __device__ __forceinline__ double sqrt_any(double x) {
   const double r = __hiloint2double((int)((sb >> 3) + 0x38000000u), (int)(sb << 29));
   const double h = x * r, e = fma(-h, r, 1.0);
   return fma(h, e * fma(0.375, e, 0.5), h);
+}
+
+// Maximum of the scaled residuals (their bits) per system (-1: none), order
+// independent: one atomic per warp and system; every lane of the warp calls
+// it.  A thread's own atomics serialised on the few addresses of a batch of
+// long rods (64 systems of 20000 rows: 687 us a launch, 59 us with the warp's
+// maximum first).
+__device__ __forceinline__ void max_residual(unsigned long long *sys_res, int sys, unsigned long long r) {
+  const unsigned full = 0xffffffffu;
+  if (__all_sync(full, sys < 0)) return;
+  const unsigned grp = __match_any_sync(full, sys);
+  const unsigned hi = (unsigned)(r >> 32), mh = __reduce_max_sync(grp, hi);
+  const unsigned ml = __reduce_max_sync(grp, hi == mh ? (unsigned)r : 0u);
+  if (sys >= 0 && (threadIdx.x & 31) == (unsigned)(__ffs(grp) - 1))
+    atomicMax(&sys_res[sys], ((unsigned long long)mh << 32) | ml);
 }
 
 // Asynchronous 8-byte copy global -> shared (both 8-byte aligned), and the
@@ -247,16 +280,22 @@ struct SolveGenArgs {
   int nlimb, limb_nmax;  // limbs; most rows of a condensation-path limb
   const int32_t *gs_fast, *lb_gsys, *lb_dir, *lb_m, *lb_nbc, *lb_bc0, *lb_bcols;
   int32_t *gen_go, *gen_bad;
+  // the limbs' rows, formed by the factor kernel: rod and its row of a limb's
+  // first row; element terms; `trans`: the transposed matrix
+  const int32_t *lb_rod, *lb_first, *npr, *rod_slot0, *rod_edge0, *slot2st, *dof_node;
+  const uint8_t *fixed;
+  const double *sh, *es, *nt, *dconst;
+  int ns, ne, nn, trans;
+  unsigned zero;  // 0 (see after())
 };
 
 // shared memory (doubles) per warp of the condensation-path limb kernels:
-// the factor's limb band, its condensed block [A_m | C_m | y_m], the
-// coupling rows R_m and the small LU's scratch
-__host__ __device__ constexpr size_t gen_factor_smem(int nmax) {
-  return (size_t)nmax * 22 + kFastMaxM * (kFastMaxM + kFastMaxBC + 1) + kFastMaxBC * kFastMaxM +
-         2 * kFastMaxM;
-}
-__host__ __device__ constexpr size_t gen_back_smem(int nmax) { return (size_t)nmax * 12 + 16; }
+// the factor's limb band with its zero rows, a block's records, a column's
+// multipliers and the small block; the back substitution's records
+constexpr int kLimbExtra = 11 * 22 + 12 * 12 + 12 +
+                           (kFastMaxM + kFastMaxBC) * (kFastMaxM + kFastMaxBC + 1);
+__host__ __device__ constexpr size_t gen_factor_smem(int nmax) { return (size_t)nmax * 22 + kLimbExtra; }
+__host__ __device__ constexpr size_t gen_back_smem() { return 32 * 3 * 12; }
 
 struct LineSearchArgs {
   int nsys, nd;

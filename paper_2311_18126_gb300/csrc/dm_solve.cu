@@ -147,33 +147,19 @@ __device__ __forceinline__ unsigned long long k_rows_rod_one(const RowArgs &a, c
   return 0;
 }
 
-// Maximum of the scaled residuals per system (order independent): one atomic
-// per warp and system.  A thread's own atomics serialised on the few
-// addresses of a batch of long rods (64 systems of 20000 rows: 687 us a
-// launch, 59 us with the warp's maximum first).
-__device__ __forceinline__ void max_residual(const RowArgs &a, int sys, unsigned long long r) {
-  const unsigned full = 0xffffffffu;
-  if (__all_sync(full, sys < 0)) return;
-  const unsigned grp = __match_any_sync(full, sys);
-  const unsigned hi = (unsigned)(r >> 32), mh = __reduce_max_sync(grp, hi);
-  const unsigned ml = __reduce_max_sync(grp, hi == mh ? (unsigned)r : 0u);
-  if (sys >= 0 && (threadIdx.x & 31) == (unsigned)(__ffs(grp) - 1))
-    atomicMax(&a.sys_res[sys], ((unsigned long long)mh << 32) | ml);
-}
-
 // block-uniform grid-stride loops (count_units synchronises the block)
 __global__ void __launch_bounds__(256) k_rows_rod(RowArgs a) {
   for (int b0 = blockIdx.x * blockDim.x; b0 < a.nd; b0 += gridDim.x * blockDim.x) {
     int sys;
     const unsigned long long r = k_rows_rod_one<0>(a, b0 + threadIdx.x, sys);
-    max_residual(a, sys, r);
+    max_residual(a.sys_res, sys, r);
   }
 }
 __global__ void __launch_bounds__(256) k_rows_rod_res(RowArgs a) {
   for (int b0 = blockIdx.x * blockDim.x; b0 < a.nd; b0 += gridDim.x * blockDim.x) {
     int sys;
     const unsigned long long r = k_rows_rod_one<1>(a, b0 + threadIdx.x, sys);
-    max_residual(a, sys, r);
+    max_residual(a.sys_res, sys, r);
   }
 }
 __global__ void __launch_bounds__(256) k_rows_rod_band(RowArgs a) {

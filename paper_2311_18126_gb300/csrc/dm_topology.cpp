@@ -340,7 +340,7 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
   T.sys_ndof.assign(S, 0);
   T.sys_kind.assign(S, SOLVE_ROD_BAND);
   std::vector<char> bnode(nn, 0), bedge(ne, 0);
-  std::vector<int32_t> limb_sys, limb_rod, limb_d0, limb_n;
+  std::vector<int32_t> limb_sys, limb_rod, limb_first, limb_d0, limb_n;
   std::vector<std::vector<int32_t>> sys_border(S);
   int32_t ndof = 0;
   for (int s = 0; s < S; ++s) {
@@ -399,6 +399,7 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
       if (count > 0) {
         limb_sys.push_back(s);
         limb_rod.push_back(r);
+        limb_first.push_back(first);
         limb_d0.push_back(ndof);
         limb_n.push_back(count);
       }
@@ -621,6 +622,8 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
       const int L = (int)T.lb_dof0.size();
       T.lb_dof0.push_back(limb_d0[li]);
       T.lb_n.push_back(limb_n[li]);
+      T.lb_rod.push_back(limb_rod[li]);
+      T.lb_first.push_back(limb_first[li]);
       for (int k = 0; k < limb_n[li]; ++k) {
         dof_limb[limb_d0[li] + k] = L;
         dof_row[limb_d0[li] + k] = k;
@@ -735,14 +738,15 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
           bcmap[l][bcl[l][k]] = (int32_t)k;
         }
       if (fast) {
-        T.lb_band.push_back(off); off += 21 * n;   // row-major [n][21]
-        T.lb_piv.push_back(off); off += n;         // reciprocal pivots
+        off += off & 1;                            // the records move by 16 bytes
+        // [n][12]: y / d and the row of U over its pivot, per row in
+        // elimination order (the limb's band is formed in shared memory)
+        T.lb_y.push_back(off); off += 12 * n;
+        T.lb_band.push_back(off);
+        T.lb_piv.push_back(off);
         T.lb_C.push_back(off); off += m * nbc;
         T.lb_R.push_back(off); off += nbc * m;
         T.lb_Y.push_back(off); off += m * (nbc + 1);
-        // [n][12]: U row (10 entries), eliminated right-hand side and
-        // reciprocal pivot of each eliminated row (the band stays assembled)
-        T.lb_y.push_back(off); off += 12 * n;
       } else {
         T.lb_band.push_back(off); off += 31 * n;   // kl = 10, ku + fill = 20
         T.lb_piv.push_back(off); off += n;
@@ -756,7 +760,7 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
     T.gs_rB.push_back(off); off += nB;
     T.gs_S.push_back(off); off += (int64_t)nB * nB;
     T.gs_xB.push_back(off); off += nB;
-    T.gs_mat0.push_back(T.lb_band.empty() || nl == 0 ? T.gs_JBB.back() : T.lb_band[mylimbs[0]]);
+    T.gs_mat0.push_back(nl == 0 ? T.gs_JBB.back() : fast ? T.lb_y[mylimbs[0]] : T.lb_band[mylimbs[0]]);
     T.gs_mat1.push_back(off);
     for (auto &t : ent) {
       const int32_t g1 = std::get<0>(t), g2 = std::get<1>(t);
@@ -771,12 +775,8 @@ bool build_topology(const dm_system_desc *D, const dm_params *P, HostTopology &T
           set_error("internal: element couples DOFs outside a limb band");
           return false;
         }
-        if (fast) {
-          const int p1 = mapped(L1, r1), p2 = mapped(L1, r2);
-          tgt = T.lb_band[L1] + (int64_t)p1 * 21 + (p2 - p1 + 10);
-        } else {
-          tgt = T.lb_band[L1] + (int64_t)(r2 - r1 + 10) * T.lb_n[L1] + r1;
-        }
+        if (fast) continue;  // formed by the limb's factor kernel
+        tgt = T.lb_band[L1] + (int64_t)(r2 - r1 + 10) * T.lb_n[L1] + r1;
       } else if (L1 >= 0) {
         if (fast) {
           const int a = mapped(L1, dof_row[g1]) - (T.lb_n[L1] - T.lb_m[L1]);
