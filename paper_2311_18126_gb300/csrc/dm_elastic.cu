@@ -3,20 +3,27 @@
 //  k_edge     -- one thread per edge: tangent, time-parallel reference frame
 //                (Sec. III), material frame, stretching force and Hessian
 //                (Sec. III-A, Eq. 2-3).
-//  k_stencil  -- one thread per bend-twist stencil: curvature binormal
-//                (Eq. 4), material curvatures (Eq. 5), reference twist and
-//                twist (Eq. 7), and the gradient and Hessian of
-//                1/2 EI/V |kappa - kappabar|^2 + 1/2 GJ/V (tau - taubar)^2
-//                (Eq. 6, 8) in closed form: first in the at-point gauge
-//                (reference frames carried by parallel transport from the
-//                current iterate), then corrected by the holonomy of the
-//                time-parallel transport so that they are the exact
-//                derivatives of the energy whose frames are carried from the
-//                committed step.
+//  k_stencil  -- one thread per bend-twist stencil: material curvatures
+//                (Eq. 4, 5), reference twist and twist (Eq. 7), and the
+//                gradient and Hessian of 1/2 EI/V |kappa - kappabar|^2 +
+//                1/2 GJ/V (tau - taubar)^2 (Eq. 6, 8) in closed form.
 //
-// The GB300 FP64 pipe is narrow (about 1 TFLOP/s) and charges a full warp
-// slot for every FP64 instruction whatever its active mask, so each thread
-// owns one whole edge or stencil and all 32 lanes do useful FP64 work.
+// With C the 3 x 3 rotation from one edge's material frame to the other's and
+// chi = 1 + C33, the strains are kappa1 = (C13 - C31)/chi, kappa2 = (C23 -
+// C32)/chi, and twist = the angle of (C11 + C22, C21 - C12); a rotation of a
+// frame maps entries of C to entries of C, so gradient and Hessian over the six
+// variables (two tangent-plane directions and the angle, per edge) are short
+// polynomials in C's nine entries.  They are formed in these variables (21
+// entries instead of 36 in space), the holonomy of the time-parallel transport
+// shifts the angles there too, and only the result goes to space.
+//
+// What bounds these kernels is the FP64 pipe: it charges a full warp slot (64
+// cycles of an SM partition) for every FP64 instruction whatever its active
+// mask, so each thread owns one whole edge or stencil and all 32 lanes do
+// useful work; reciprocals run on the integer pipe.  FP64 instructions per
+// stencil, from the kernels' times: gradient 295 -> 195, Hessian 1060 -> 570,
+// both in one pass 1000 -> 525.  4096 rods (450046 stencils): fused pass 846 ->
+// 444 us, a step's Hessians 1.24 -> 0.67 ms and gradients 0.60 -> 0.39 ms.
 #include "dm_internal.h"
 #include "dm_kernels.cuh"
 
@@ -110,23 +117,10 @@ __device__ __forceinline__ v3 axpy(double s, v3 x, v3 y) {  // s x + y
 }
 // component access by compile-time index
 __device__ __forceinline__ double cmp(const v3 &a, int i) { return i == 0 ? a.x : (i == 1 ? a.y : a.z); }
-// P_perp(t) v = v - (t.v) t
-__device__ __forceinline__ v3 perp(v3 t, v3 v) { return axpy(-dot(t, v), t, v); }
-
 // packed upper-triangle index of an n x n symmetric matrix (i <= j)
 template <int n>
 __host__ __device__ constexpr int up(int i, int j) {
   return i * n - i * (i - 1) / 2 + (j - i);
-}
-
-// H8[blk] += s * (x y^T + y x^T) on a 3x3 diagonal block starting at o
-__device__ __forceinline__ void add_sym(double *h, int o, double s, v3 x, v3 y) {
-  const v3 sx = s * x;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i; j < 3; ++j)
-      h[up<8>(o + i, o + j)] = fma(cmp(sx, i), cmp(y, j), fma(cmp(y, i), cmp(sx, j), h[up<8>(o + i, o + j)]));
 }
 
 // s x for s = +-1 given as a sign word (0 or 0x80000000): the sign bit
@@ -140,14 +134,85 @@ __device__ __forceinline__ v3 sgn3(int s, v3 v) {
   return mk(sgnmul(sw, v.x), sgnmul(sw, v.y), sgnmul(sw, v.z));
 }
 
-__device__ __forceinline__ void load_edge(const double *ef, int NE, int e, int sgn,
-                                          v3 &t, double &il, v3 &d1, v3 &m1, v3 &m2) {
+// An edge's material frame (m1, m2, t), right-handed and orthonormal, in the
+// stencil's orientation (a reversed edge: t and m2 flipped), and its 1/l.
+struct Frame {
+  v3 m1, m2, t;
+  double il;
+  __device__ __forceinline__ void load(const double *ef, int NE, int e, int sgn) {
+    const unsigned sw = sign_word(sgn);
+    t = mk(sgnmul(sw, ef[e]), sgnmul(sw, ef[NE + e]), sgnmul(sw, ef[2 * NE + e]));
+    il = ef[3 * NE + e];
+    m1 = mk(ef[7 * NE + e], ef[8 * NE + e], ef[9 * NE + e]);
+    m2 = mk(sgnmul(sw, ef[10 * NE + e]), sgnmul(sw, ef[11 * NE + e]), sgnmul(sw, ef[12 * NE + e]));
+  }
+};
+
+// Holonomy of the time-parallel transport: moving the edge's tangent t also
+// rotates the director carried from the committed tangent t_n about t, by the
+// holonomy chi of the geodesic triangle (t_n, t, t').  In the material frame,
+// over tangent-plane displacements: grad chi = (r, -p), hess chi =
+// -[r p, (r^2 - p^2)/2; ., -r p], with (p, r) = (t_n.m1, t_n.m2)/(1 + t_n.t).
+__device__ __forceinline__ void holonomy(const double *tn, int NE, int e, int sgn, const Frame &f, double &p,
+                                         double &r) {
   const unsigned sw = sign_word(sgn);
-  t = mk(sgnmul(sw, ef[e]), sgnmul(sw, ef[NE + e]), sgnmul(sw, ef[2 * NE + e]));
-  il = ef[3 * NE + e];
-  d1 = mk(ef[4 * NE + e], ef[5 * NE + e], ef[6 * NE + e]);
-  m1 = mk(ef[7 * NE + e], ef[8 * NE + e], ef[9 * NE + e]);
-  m2 = mk(sgnmul(sw, ef[10 * NE + e]), sgnmul(sw, ef[11 * NE + e]), sgnmul(sw, ef[12 * NE + e]));
+  const v3 n = mk(sgnmul(sw, tn[e]), sgnmul(sw, tn[NE + e]), sgnmul(sw, tn[2 * NE + e]));
+  const double ic = rcp_int(1.0 + dot(n, f.t));  // k_edge: 1 + t_n.t > 1e-12
+  const v3 d = n - f.t;                          // m.t = 0: the short difference loses nothing
+  p = ic * dot(f.m1, d);
+  r = ic * dot(f.m2, d);
+}
+
+// The holonomy's part in the Hessian block H (rows and columns: tangent plane
+// 0, 1, angle 2): with E the energy's derivative in the angle, the angle
+// shifts by -grad chi . phi - phi . hess chi phi / 2.
+__device__ __forceinline__ void shift_block(double &h00, double &h01, double &h11, double &h02, double &h12,
+                                            double h22, double E, double p, double r) {
+  const double hh = 0.5 * h22;
+  const double v0 = fma(-0.5 * E, p, fma(-hh, r, h02)), v1 = fma(-0.5 * E, r, fma(hh, p, h12));
+  h00 = fma(-2.0 * r, v0, h00);
+  h01 = fma(-r, v1, fma(p, v0, h01));
+  h11 = fma(2.0 * p, v1, h11);
+  h02 = fma(-r, h22, h02);
+  h12 = fma(p, h22, h12);
+}
+
+// x m1 + y m2
+__device__ __forceinline__ v3 span(double x, v3 m1, double y, v3 m2) {
+  return mk(fma(x, m1.x, y * m2.x), fma(x, m1.y, y * m2.y), fma(x, m1.z, y * m2.z));
+}
+
+// 3 x 3 block of an edge in space: [h00 h01; h01 h11] in the (scaled) basis
+// (m1, m2), and the terms -(g t^T + t g^T) of the angle's second order in the
+// edge vector, into h at offset o
+__device__ __forceinline__ void expand_block(double *h, int o, double h00, double h01, double h11, double g0,
+                                             double g1, v3 m1, v3 m2, v3 t) {
+  const v3 u = axpy(-g0, t, span(0.5 * h00, m1, h01, m2)), w = span(0.5 * h11, m2, -g1, t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i; j < 3; ++j) {
+      const double x = fma(cmp(m1, i), cmp(u, j), cmp(m2, i) * cmp(w, j));
+      h[up<8>(o + i, o + j)] = i == j ? x + x : fma(cmp(u, i), cmp(m1, j), fma(cmp(w, i), cmp(m2, j), x));
+    }
+}
+
+// atan2(v, u): for |v| <= u/8 by the Taylor series of atan (nine terms: the
+// tenth is below 2^-56 of the sum), which costs a fifth of the general
+// function's FP64 instructions.
+__device__ __forceinline__ double twist_angle(double v, double u) {
+  if (!(fabs(v) <= 0.125 * u && rcp64_in_range(u))) return atan2(v, u);
+  const double x = v * rcp_int(u), y = x * x;
+  double s = -1.0 / 19.0;
+  s = fma(s, y, 1.0 / 17.0);
+  s = fma(s, y, -1.0 / 15.0);
+  s = fma(s, y, 1.0 / 13.0);
+  s = fma(s, y, -1.0 / 11.0);
+  s = fma(s, y, 1.0 / 9.0);
+  s = fma(s, y, -1.0 / 7.0);
+  s = fma(s, y, 1.0 / 5.0);
+  s = fma(s, y, -1.0 / 3.0);
+  return fma(x * y, s, x);
 }
 
 // Slot p of the 11 DOFs [x0 (0-2), th_a (3), x1 (4-6), th_b (7), x2 (8-10)]
@@ -208,31 +273,29 @@ __device__ __forceinline__ void k_stencil_one(StencilArgs a, const int k) {
   const int NS = a.ns, NE = a.ne;
   const int sg = a.st_sg[k];
   const int sa = (sg & 1) ? -1 : 1, sb = (sg & 2) ? -1 : 1;
-  v3 ta, d1a, m1a, m2a, tb, d1b, m1b, m2b;
-  double ila, ilb;
-  load_edge(a.ef, NE, a.st_ed[k], sa, ta, ila, d1a, m1a, m2a);
-  load_edge(a.ef, NE, a.st_ed[NS + k], sb, tb, ilb, d1b, m1b, m2b);
+  const int ea = a.st_ed[k], eb = a.st_ed[NS + k];
+  Frame A, B;
+  A.load(a.ef, NE, ea, sa);
+  B.load(a.ef, NE, eb, sb);
 
-  // Eq. 4: curvature binormal
-  const double chi = 1.0 + dot(ta, tb);
+  // frame b seen from frame a: C = [m1a m2a ta]^T [m1b m2b tb]; its last
+  // column and row from tb - ta
+  const double z = dot(A.t, B.t), chi = 1.0 + z;
   if (!(chi > 1e-12)) {
     if (MODE != 2) atomicMax(&a.sys_status[sys], (int)DM_ERR_DEGENERATE);
     return;
   }
-  const double ichi = rcp64(chi);  // chi in (1e-12, 2]
-  const v3 kb = (2.0 * ichi) * cross(ta, tb);
-  const v3 M1 = m1a + m1b, M2 = m2a + m2b;
-  // Eq. 5: material curvatures
-  const double k1 = 0.5 * dot(kb, M2);
-  const double k2 = -0.5 * dot(kb, M1);
-  // Eq. 7: reference twist, continued from the committed value
-  const v3 s_ab = ta + tb;
+  const double ic = rcp_int(chi);  // chi in (1e-12, 2]
+  const v3 d = B.t - A.t;
+  const double C11 = dot(A.m1, B.m1), C12 = dot(A.m1, B.m2), C21 = dot(A.m2, B.m1), C22 = dot(A.m2, B.m2);
+  // Eq. 7: reference twist, continued from the committed value: the angle of
+  // C's twist about the tangent less the difference of the material angles
+  const double th = sgnmul(sign_word(sb), a.q[a.st_th[NS + k]]) - sgnmul(sign_word(sa), a.q[a.st_th[k]]);
   double beta;
   if (MODE == 2) {
     beta = a.beta_it[k];
   } else {
-    const v3 u = axpy(-dot(d1a, tb) * ichi, s_ab, d1a);
-    const double ang = atan2(dot(tb, cross(u, d1b)), dot(u, d1b));
+    const double ang = twist_angle(C21 - C12, C11 + C22) - th;
     const double bn = a.beta_n[k];
     double dd = ang - bn;
     dd -= 6.283185307179586 * rint(dd * 0.15915494309189535);
@@ -240,282 +303,150 @@ __device__ __forceinline__ void k_stencil_one(StencilArgs a, const int k) {
     a.beta_it[k] = beta;
     if (a.frames_only) return;
   }
-  const double tha = a.q[a.st_th[k]], thb = a.q[a.st_th[NS + k]];
-  const double tau = sgnmul(sign_word(sb), thb) - sgnmul(sign_word(sa), tha) + beta;
+  // everything over chi from here on: C's last column (a, b, z), row (c, d, z)
+  const double av = ic * dot(A.m1, d), bv = ic * dot(A.m2, d);
+  const double cv = -ic * dot(B.m1, d), dv = -ic * dot(B.m2, d);
+  const double zi = ic * z, C11i = ic * C11, C12i = ic * C12, C21i = ic * C21, C22i = ic * C22;
+  // Eq. 4, 5: material curvatures
+  const double k1 = av - cv, k2 = bv - dv;
   const double kbs = a.st_kb[k], kts = a.st_kt[k];
   const double c1 = kbs * (k1 - a.kbar[k]);
   const double c2 = kbs * (k2 - a.kbar[NS + k]);
-  const double c3 = kts * (tau - a.taubar[k]);
+  const double c3 = kts * (th + beta - a.taubar[k]);
 
-  // gradients of kappa1, kappa2, tau in (e_a, e_b, theta_a, theta_b)
-  const v3 tt = ichi * s_ab, mt1 = ichi * M1, mt2 = ichi * M2;
-  double g1[8], g2[8], g3[8];
-  {
-    v3 x;
-    x = ila * (cross(tb, mt2) - k1 * tt);
-    g1[0] = x.x; g1[1] = x.y; g1[2] = x.z;
-    x = ilb * ((-k1) * tt - cross(ta, mt2));
-    g1[3] = x.x; g1[4] = x.y; g1[5] = x.z;
-    g1[6] = -0.5 * dot(kb, m1a);
-    g1[7] = -0.5 * dot(kb, m1b);
-    x = ila * ((-k2) * tt - cross(tb, mt1));
-    g2[0] = x.x; g2[1] = x.y; g2[2] = x.z;
-    x = ilb * (cross(ta, mt1) - k2 * tt);
-    g2[3] = x.x; g2[4] = x.y; g2[5] = x.z;
-    g2[6] = -0.5 * dot(kb, m2a);
-    g2[7] = -0.5 * dot(kb, m2b);
-    g3[0] = 0.5 * ila * kb.x; g3[1] = 0.5 * ila * kb.y; g3[2] = 0.5 * ila * kb.z;
-    g3[3] = 0.5 * ilb * kb.x; g3[4] = 0.5 * ilb * kb.y; g3[5] = 0.5 * ilb * kb.z;
-    g3[6] = -1.0;
-    g3[7] = 1.0;
-  }
-  // energy gradient (8-space) and its outer-product Hessian part
+  // gradients of kappa1, kappa2 and tau over (tangent plane of a, angle a,
+  // tangent plane of b, angle b)
+  const double zc1 = zi + C11i, zc2 = zi + C22i;
+  const double x1[6] = {-fma(k1, av, zc1), -fma(k1, bv, C21i), bv, fma(-k1, cv, zc1), fma(-k1, dv, C12i), -dv};
+  const double x2[6] = {-fma(k2, av, C12i), -fma(k2, bv, zc2), -av, fma(-k2, cv, C21i), fma(-k2, dv, zc2), cv};
+  const double x3[6] = {-bv, av, -1.0, dv, -cv, 1.0};
+  // the curvature energy's gradient, then the energy's
+  double ck[6], g[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) ck[i] = fma(c1, x1[i], c2 * x2[i]);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) g[i] = fma(c3, x3[i], ck[i]);
+  double pa, ra, pb, rb;  // holonomies of the two edges
+  holonomy(a.tn, NE, ea, sa, A, pa, ra);
+  holonomy(a.tn, NE, eb, sb, B, pb, rb);
+  const double EA = g[2], EB = g[5], g0 = g[0], g1 = g[1];
+  g[0] = fma(-ra, EA, g[0]);
+  g[1] = fma(pa, EA, g[1]);
+  g[3] = fma(-rb, EB, g[3]);
+  g[4] = fma(pb, EB, g[4]);
+  // the edges' bases over their lengths: tangent plane -> edge vector
+  const v3 A1 = A.il * A.m1, A2 = A.il * A.m2, B1 = B.il * B.m1, B2 = B.il * B.m2;
   double g8[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) g8[i] = fma(c1, g1[i], fma(c2, g2[i], c3 * g3[i]));
+  {
+    const v3 x = span(g[0], A1, g[1], A2), y = span(g[3], B1, g[4], B2);
+    g8[0] = x.x; g8[1] = x.y; g8[2] = x.z;
+    g8[3] = y.x; g8[4] = y.y; g8[5] = y.z;
+    g8[6] = EA;
+    g8[7] = EB;
+  }
   if (MODE == 1) {
-    // the holonomy correction of the gradient (see the Hessian block below)
-    const v3 tna = sgn3(sa, mk(a.tn[a.st_ed[k]], a.tn[NE + a.st_ed[k]], a.tn[2 * NE + a.st_ed[k]]));
-    const v3 tnb = sgn3(sb, mk(a.tn[a.st_ed[NS + k]], a.tn[NE + a.st_ed[NS + k]],
-                                   a.tn[2 * NE + a.st_ed[NS + k]]));
-    const v3 ga = ila * (rcp64(1.0 + dot(tna, ta)) * cross(tna, ta));
-    const v3 gb = ilb * (rcp64(1.0 + dot(tnb, tb)) * cross(tnb, tb));
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      g8[i] -= g8[6] * cmp(ga, i);
-      g8[3 + i] -= g8[7] * cmp(gb, i);
-    }
     write_gradient(a, k, g8, sa, sb);
     return;
   }
-  double h[36];
-  {
-    // gradients pre-scaled by the stiffnesses: three FP64 instructions an entry
-    double a1[8], a2[8], a3[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      a1[i] = kbs * g1[i];
-      a2[i] = kbs * g2[i];
-      a3[i] = kts * g3[i];
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = i; j < 8; ++j) h[up<8>(i, j)] = fma(a1[i], g1[j], fma(a2[i], g2[j], a3[i] * g3[j]));
-  }
 
-  // second-derivative part, first in tangent space then projected
-  const v3 w = c1 * M2 - c2 * M1;
-  const double kw = dot(kb, w);
-  const double ichi2 = ichi * ichi;
-  const v3 pb = perp(ta, tb);   // P_a t_b
-  const v3 pa = perp(tb, ta);   // P_b t_a
-  // t-space gradient of E (the extension of the energy off the sphere)
-  const v3 tbxw = cross(tb, w), wxta = cross(w, ta);
-  const v3 gta = axpy(ichi, tbxw, axpy(-0.5 * kw * ichi, tb, (0.5 * c3) * kb));
-  const v3 gtb = axpy(ichi, wxta, axpy(-0.5 * kw * ichi, ta, (0.5 * c3) * kb));
-  const double tga = 0.5 * kw * ichi;  // t_a . g_ta == t_b . g_tb
-  const v3 hga = perp(ta, gta), hgb = perp(tb, gtb);
-  const v3 Pa = c1 * m2a - c2 * m1a, Pb = c1 * m2b - c2 * m1b;
-  const v3 Ra = c1 * m1a + c2 * m2a, Rb = c1 * m1b + c2 * m2b;
-  // aa block
+  // Hessian over the six variables, upper triangle.  With k = c1 kappa1 + c2
+  // kappa2 and N = chi k: Hess k = (Hess N - grad k grad chi^T - grad chi grad
+  // k^T - k Hess chi)/chi, where N and chi are entries of C, whose second
+  // derivatives under F -> F exp(phi) exp(theta t) are entries of C again.
+  double H[21];
   {
-    const double s2 = ila * ila;
-    const v3 Xa = axpy(-ichi2, perp(ta, tbxw), axpy(0.5 * kw * ichi2, pb, (-0.25 * c3 * ichi) * kb));
-    add_sym(h, 0, s2, Xa, pb);
-    add_sym(h, 0, 0.25 * s2, perp(ta, Pa), kb);
-    add_sym(h, 0, -s2, ta, hga);
-    {
-      // - s2 tga (I - t_a t_a^T)
-      const double c = s2 * tga;
-      const v3 ct = c * ta;
+    const double P = fma(c1, av, c2 * bv), Q = fma(c1, cv, c2 * dv), kk = P - Q;
+    const double Sa = fma(kk, zi, Q), Sb = fma(kk, zi, -P);
+    const double h1 = fma(0.5, fma(-c3, bv, c1), ck[0]), h2 = fma(0.5, fma(c3, av, c2), ck[1]);
+    const double f1 = fma(0.5, fma(c3, dv, -c1), ck[3]), f2 = fma(-0.5, fma(c3, cv, c2), ck[4]);
+    const double c1z = c1 * zi, c2z = c2 * zi;
+    H[up<6>(0, 0)] = fma(-2.0 * av, h1, Sa);
+    H[up<6>(0, 1)] = -fma(bv, h1, av * h2);
+    H[up<6>(1, 1)] = fma(-2.0 * bv, h2, Sa);
+    H[up<6>(0, 2)] = fma(-ck[2], av, c2z);
+    H[up<6>(1, 2)] = fma(-ck[2], bv, -c1z);
+    H[up<6>(2, 2)] = -P;
+    H[up<6>(3, 3)] = fma(-2.0 * cv, f1, Sb);
+    H[up<6>(3, 4)] = -fma(dv, f1, cv * f2);
+    H[up<6>(4, 4)] = fma(-2.0 * dv, f2, Sb);
+    H[up<6>(3, 5)] = fma(-ck[5], cv, -c2z);
+    H[up<6>(4, 5)] = fma(-ck[5], dv, c1z);
+    H[up<6>(5, 5)] = Q;
+    H[up<6>(0, 3)] = fma(-c3, C21i, fma(-kk, C11i, fma(-ck[3], av, fma(-g0, cv, c1 * k1))));
+    H[up<6>(0, 4)] = fma(-c3, C22i, fma(-kk, C12i, fma(-ck[4], av, fma(-g0, dv, fma(c2, av, -c1 * dv)))));
+    H[up<6>(1, 3)] = fma(c3, C11i, fma(-kk, C21i, fma(-ck[3], bv, fma(-g1, cv, fma(c1, bv, -c2 * cv)))));
+    H[up<6>(1, 4)] = fma(c3, C12i, fma(-kk, C22i, fma(-ck[4], bv, fma(-g1, dv, c2 * k2))));
+    H[up<6>(0, 5)] = fma(-ck[5], av, fma(c2, C11i, -c1 * C12i));
+    H[up<6>(1, 5)] = fma(-ck[5], bv, fma(c2, C21i, -c1 * C22i));
+    H[up<6>(2, 3)] = fma(-ck[2], cv, fma(c1, C21i, -c2 * C11i));
+    H[up<6>(2, 4)] = fma(-ck[2], dv, fma(c1, C22i, -c2 * C12i));
+    H[up<6>(2, 5)] = 0.0;
+    // outer products of the gradients
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 6; ++i) {
+      const double y1 = kbs * x1[i], y2 = kbs * x2[i], y3 = i == 2 ? -kts : i == 5 ? kts : kts * x3[i];
 #pragma unroll
-        for (int j = i; j < 3; ++j)
-          h[up<8>(i, j)] = fma(cmp(ct, i), cmp(ta, j), i == j ? h[up<8>(i, j)] - c : h[up<8>(i, j)]);
+      for (int j = i; j < 6; ++j) {
+        const double t = j == 2 ? -y3 : j == 5 ? y3 : 0.0;  // y3 x3[j] for x3[j] = -+1
+        const double v = i == 2 && j == 5 ? 0.0 : H[up<6>(i, j)];
+        H[up<6>(i, j)] = fma(y1, x1[j], fma(y2, x2[j], j == 2 || j == 5 ? v + t : fma(y3, x3[j], v)));
+      }
     }
   }
-  // bb block
-  {
-    const double s2 = ilb * ilb;
-    const v3 Xb = axpy(-ichi2, perp(tb, wxta), axpy(0.5 * kw * ichi2, pa, (-0.25 * c3 * ichi) * kb));
-    add_sym(h, 3, s2, Xb, pa);
-    add_sym(h, 3, 0.25 * s2, perp(tb, Pb), kb);
-    add_sym(h, 3, -s2, tb, hgb);
-    {
-      const double c = s2 * tga;
-      const v3 ct = c * tb;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j)
-          h[up<8>(3 + i, 3 + j)] =
-              fma(cmp(ct, i), cmp(tb, j), i == j ? h[up<8>(3 + i, 3 + j)] - c : h[up<8>(3 + i, 3 + j)]);
-    }
-  }
-  // ab block: M = -ichi [w]x - ichi^2 (alpha_a t_a^T + t_b alpha_b^T)
-  //               + (kw ichi^2) t_b t_a^T - kw ichi/2 I
-  //               + c3 ichi [t_a]x - c3 ichi/2 kb t_a^T,  then P_a M P_b
-  {
-    double Mab[3][3];
-    const double ca = -0.5 * kw * ichi;
-    // the rank-one parts as Ev t_a^T + Bv wxta^T
-    const v3 Ev = axpy(-ichi2, tbxw, axpy(kw * ichi2, tb, (-0.5 * c3 * ichi) * kb));
-    const v3 Bv = (-ichi2) * tb;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const double v = fma(cmp(Ev, i), cmp(ta, j), cmp(Bv, i) * cmp(wxta, j));
-        Mab[i][j] = i == j ? v + ca : v;
-      }
-    // skew parts: -ichi [w]x + c3 ichi [t_a]x = [z]x with z = ichi (c3 t_a - w)
-    const v3 z = ichi * axpy(c3, ta, (-1.0) * w);
-    Mab[0][1] -= z.z; Mab[0][2] += z.y;
-    Mab[1][0] += z.z; Mab[1][2] -= z.x;
-    Mab[2][0] -= z.y; Mab[2][1] += z.x;
-    // P_a M P_b
-    double r[3], cc[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) r[j] = ta.x * Mab[0][j] + ta.y * Mab[1][j] + ta.z * Mab[2][j];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) cc[i] = Mab[i][0] * tb.x + Mab[i][1] * tb.y + Mab[i][2] * tb.z;
-    const double sc = r[0] * tb.x + r[1] * tb.y + r[2] * tb.z;
-    const double s2 = ila * ilb;
-    // M - t_a r^T - cc t_b^T + sc t_a t_b^T = M - t_a (r - sc t_b)^T - cc t_b^T
-#pragma unroll
-    for (int j = 0; j < 3; ++j) r[j] = fma(-sc, cmp(tb, j), r[j]);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const double v = fma(-cmp(ta, i), r[j], fma(-cc[i], cmp(tb, j), Mab[i][j]));
-        h[up<8>(i, 3 + j)] = fma(s2, v, h[up<8>(i, 3 + j)]);
-      }
-  }
-  // theta cross blocks: -1/2 P ga(R), ga(v) = 2 ichi (t_b x v) - (kb.v) ichi t_b,
-  //                                     gb(v) = 2 ichi (v x t_a) - (kb.v) ichi t_a
-  {
-    const double kRa = dot(kb, Ra), kRb = dot(kb, Rb);
-    v3 x;
-    x = (-0.5 * ila) * axpy(2.0 * ichi, perp(ta, cross(tb, Ra)), (-kRa * ichi) * pb);
-    h[up<8>(0, 6)] += x.x; h[up<8>(1, 6)] += x.y; h[up<8>(2, 6)] += x.z;
-    x = (-0.5 * ilb) * axpy(2.0 * ichi, perp(tb, cross(Ra, ta)), (-kRa * ichi) * pa);
-    h[up<8>(3, 6)] += x.x; h[up<8>(4, 6)] += x.y; h[up<8>(5, 6)] += x.z;
-    x = (-0.5 * ila) * axpy(2.0 * ichi, perp(ta, cross(tb, Rb)), (-kRb * ichi) * pb);
-    h[up<8>(0, 7)] += x.x; h[up<8>(1, 7)] += x.y; h[up<8>(2, 7)] += x.z;
-    x = (-0.5 * ilb) * axpy(2.0 * ichi, perp(tb, cross(Rb, ta)), (-kRb * ichi) * pa);
-    h[up<8>(3, 7)] += x.x; h[up<8>(4, 7)] += x.y; h[up<8>(5, 7)] += x.z;
-    h[up<8>(6, 6)] += -0.5 * dot(kb, Pa);
-    h[up<8>(7, 7)] += -0.5 * dot(kb, Pb);
-  }
-
   // Exact derivatives of the energy with the reference frames carried from
-  // the committed step by time-parallel transport (Eq. 9): moving the edge
-  // tangent t also rotates its time-transported director about t by the
-  // holonomy chi of the geodesic triangle (t_n, t, t'), which acts like a
-  // twist-angle shift.  With Phi the at-point energy above:
-  //   grad E = grad Phi - sum_x E_x grad chi_x
-  //   hess E = H - sum_x sym(H[:, x], grad chi_x) + sum_xy H[x, y] grad chi_x grad chi_y^T
-  //            - sum_x E_x hess chi_x,      x in {A, B} (effective angles)
-  // grad_e chi = w / l with w = (t_n x t)/(1 + t_n.t), and
-  // hess_e chi = -[ (n s^T + s n^T) / (2 c^2) + w t^T + t w^T ] / l^2,
-  // n = t_n x t, c = 1 + t_n.t, s = t_n - (t_n.t) t.
+  // the committed step by time-parallel transport (Eq. 9): the angles shift by
+  // the holonomies, first a's, then b's.
+  shift_block(H[up<6>(0, 0)], H[up<6>(0, 1)], H[up<6>(1, 1)], H[up<6>(0, 2)], H[up<6>(1, 2)], H[up<6>(2, 2)], EA, pa, ra);
+#pragma unroll
+  for (int j = 3; j < 6; ++j) {
+    H[up<6>(0, j)] = fma(-ra, H[up<6>(2, j)], H[up<6>(0, j)]);
+    H[up<6>(1, j)] = fma(pa, H[up<6>(2, j)], H[up<6>(1, j)]);
+  }
+  shift_block(H[up<6>(3, 3)], H[up<6>(3, 4)], H[up<6>(4, 4)], H[up<6>(3, 5)], H[up<6>(4, 5)], H[up<6>(5, 5)], EB, pb, rb);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    H[up<6>(i, 3)] = fma(-rb, H[up<6>(i, 5)], H[up<6>(i, 3)]);
+    H[up<6>(i, 4)] = fma(pb, H[up<6>(i, 5)], H[up<6>(i, 4)]);
+  }
+  // to edge vectors and angles
+  double h[36];
+  expand_block(h, 0, H[up<6>(0, 0)], H[up<6>(0, 1)], H[up<6>(1, 1)], g[0], g[1], A1, A2, A.il * A.t);
+  expand_block(h, 3, H[up<6>(3, 3)], H[up<6>(3, 4)], H[up<6>(4, 4)], g[3], g[4], B1, B2, B.il * B.t);
   {
-    const v3 tna = sgn3(sa, mk(a.tn[a.st_ed[k]], a.tn[NE + a.st_ed[k]], a.tn[2 * NE + a.st_ed[k]]));
-    const v3 tnb = sgn3(sb, mk(a.tn[a.st_ed[NS + k]], a.tn[NE + a.st_ed[NS + k]],
-                                   a.tn[2 * NE + a.st_ed[NS + k]]));
-    v3 ga, gb;
-    double Ha[6], Hb[6];
-    {
-      const double c = 1.0 + dot(tna, ta), ic = rcp64(c);
-      const v3 n = cross(tna, ta), w = ic * n;
-      const v3 sp = axpy(-dot(tna, ta), ta, tna);
-      ga = ila * w;
-      const double f1 = -0.5 * ic * ic * ila * ila, f2 = -ila * ila;
-      const v3 fn = f1 * n, fw = f2 * w;
-      int e = 0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j, ++e)
-          Ha[e] = fma(cmp(fn, i), cmp(sp, j),
-                      fma(cmp(sp, i), cmp(fn, j), fma(cmp(fw, i), cmp(ta, j), cmp(ta, i) * cmp(fw, j))));
-    }
-    {
-      const double c = 1.0 + dot(tnb, tb), ic = rcp64(c);
-      const v3 n = cross(tnb, tb), w = ic * n;
-      const v3 sp = axpy(-dot(tnb, tb), tb, tnb);
-      gb = ilb * w;
-      const double f1 = -0.5 * ic * ic * ilb * ilb, f2 = -ilb * ilb;
-      const v3 fn = f1 * n, fw = f2 * w;
-      int e = 0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = i; j < 3; ++j, ++e)
-          Hb[e] = fma(cmp(fn, i), cmp(sp, j),
-                      fma(cmp(sp, i), cmp(fn, j), fma(cmp(fw, i), cmp(tb, j), cmp(tb, i) * cmp(fw, j))));
-    }
-    double colA[8], colB[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      colA[i] = i <= 6 ? h[up<8>(i, 6)] : h[up<8>(6, i)];
-      colB[i] = h[up<8>(i < 7 ? i : 7, 7)];
-    }
-    const double EA = g8[6], EB = g8[7];
-    const double HAA = h[up<8>(6, 6)], HBB = h[up<8>(7, 7)], HAB = h[up<8>(6, 7)];
+    const v3 x = span(H[up<6>(0, 3)], B1, H[up<6>(0, 4)], B2), y = span(H[up<6>(1, 3)], B1, H[up<6>(1, 4)], B2);
+    const v3 aA = span(H[up<6>(0, 2)], A1, H[up<6>(1, 2)], A2), aB = span(H[up<6>(0, 5)], A1, H[up<6>(1, 5)], A2);
+    const v3 bA = span(H[up<6>(2, 3)], B1, H[up<6>(2, 4)], B2), bB = span(H[up<6>(3, 5)], B1, H[up<6>(4, 5)], B2);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      g8[i] -= EA * cmp(ga, i);
-      g8[3 + i] -= EB * cmp(gb, i);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) h[up<8>(i, 3 + j)] = fma(cmp(A1, i), cmp(x, j), cmp(A2, i) * cmp(y, j));
+      h[up<8>(i, 6)] = cmp(aA, i);
+      h[up<8>(i, 7)] = cmp(aB, i);
+      h[up<8>(3 + i, 6)] = cmp(bA, i);
+      h[up<8>(3 + i, 7)] = cmp(bB, i);
     }
-    // grad chi_A lives on entries 0-2, grad chi_B on 3-5: only the terms
-    // whose factors are not structurally zero are formed (a product with a
-    // literal zero is not dropped by an IEEE-conforming compiler)
-    v3 hga_a = HAA * ga, hab_a = HAB * ga, hgb_b = HBB * gb;
+    h[up<8>(6, 6)] = H[up<6>(2, 2)];
+    h[up<8>(6, 7)] = H[up<6>(2, 5)];
+    h[up<8>(7, 7)] = H[up<6>(5, 5)];
+  }
+  if (a.dk) {
+    // gradients of kappa1 and kappa2 as functions of the 11 DOFs (the same
+    // shift of the angles), for the adjoint: d(grad E)/d(kappabar_c) =
+    // -EI/V grad kappa_c
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int c = 0; c < 2; ++c) {
+      const double *x = c == 0 ? x1 : x2;
+      const v3 xa = span(fma(-ra, x[2], x[0]), A1, fma(pa, x[2], x[1]), A2);
+      const v3 xb = span(fma(-rb, x[5], x[3]), B1, fma(pb, x[5], x[4]), B2);
+      double *o = a.dk + (size_t)(11 * c) * NS + k;
 #pragma unroll
-      for (int j = i; j < 8; ++j) {
-        const bool ai = i < 3, aj = j < 3, bi = i >= 3 && i < 6, bj = j >= 3 && j < 6;
-        if (!ai && !bi) continue;  // i, j >= 6: no correction
-        double v = h[up<8>(i, j)];
-        if (aj) v = fma(-colA[i], cmp(ga, j), v);
-        if (ai) v = fma(-cmp(ga, i), colA[j], v);
-        if (bj) v = fma(-colB[i], cmp(gb, j - 3), v);
-        if (bi) v = fma(-cmp(gb, i - 3), colB[j], v);
-        if (ai && aj) v = fma(cmp(hga_a, i), cmp(ga, j), fma(-EA, Ha[up<3>(i, j)], v));
-        if (ai && bj) v = fma(cmp(hab_a, i), cmp(gb, j - 3), v);
-        if (bi && bj) v = fma(cmp(hgb_b, i - 3), cmp(gb, j - 3), fma(-EB, Hb[up<3>(i - 3, j - 3)], v));
-        h[up<8>(i, j)] = v;
+      for (int i = 0; i < 3; ++i) {
+        o[(size_t)i * NS] = -cmp(xa, i);
+        o[(size_t)(4 + i) * NS] = cmp(xa, i) - cmp(xb, i);
+        o[(size_t)(8 + i) * NS] = cmp(xb, i);
       }
-    if (a.dk) {
-      // gradients of kappa1 and kappa2 as functions of the 11 DOFs (the
-      // same holonomy correction as the energy gradient), for the adjoint:
-      // d(grad E)/d(kappabar_c) = -EI/V grad kappa_c
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const double *gc = c == 0 ? g1 : g2;
-        double e8[8];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          e8[i] = gc[i] - gc[6] * cmp(ga, i);
-          e8[3 + i] = gc[3 + i] - gc[7] * cmp(gb, i);
-        }
-        e8[6] = gc[6];
-        e8[7] = gc[7];
-        double *o = a.dk + (size_t)(11 * c) * NS + k;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          o[(size_t)i * NS] = -e8[i];
-          o[(size_t)(4 + i) * NS] = e8[i] - e8[3 + i];
-          o[(size_t)(8 + i) * NS] = e8[3 + i];
-        }
-        o[(size_t)3 * NS] = sgnmul(sign_word(sa), e8[6]);
-        o[(size_t)7 * NS] = sgnmul(sign_word(sb), e8[7]);
-      }
+      o[(size_t)3 * NS] = sgnmul(sign_word(sa), x[2]);
+      o[(size_t)7 * NS] = sgnmul(sign_word(sb), x[5]);
     }
   }
 
