@@ -60,6 +60,20 @@ dm_status upload(dm_system *s, T **p, const std::vector<T> &h) {
 
 inline int blocks(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
+// A kernel's dynamic shared memory up to the limit of a block, not a system's
+// need: the attribute is the kernel's, and a later, smaller system must not
+// lower it for an earlier one.
+cudaError_t raise_limit(const void *kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+  return e;
+}
+
 __global__ void k_gather_layout(int n, const int32_t *map, const double *src, double *dst) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = src[map[i]];
@@ -125,6 +139,8 @@ struct Extra {
     int64_t *sys_dense0 = nullptr, *sys_nz0 = nullptr;
     uint8_t *nz = nullptr;
     double *lud = nullptr;
+    int32_t *lu_level = nullptr, *lu_bar = nullptr;
+    uint16_t *lu_adj = nullptr;
     int max_n = 0;  // DOFs of the largest contact system
     unsigned long long *edge_key = nullptr;
   } cc;  // edge-edge contact
@@ -419,6 +435,10 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     DM_TRY(upload(s, &c.sys_nz0, nz0));
     DM_TRY(dalloc(s, &c.nz, tiles));
     DM_TRY(dalloc(s, &c.lud, kNB * nd));
+    DM_TRY(dalloc(s, &c.lu_adj, tiles));
+    DM_TRY(dalloc(s, &c.lu_bar, S));
+    DM_TRY(dalloc(s, &c.lu_level, (int64_t)S * blocks(c.max_n, kNB) * kLevelInts));
+    DM_CK(raise_limit((const void *)k_lu_order));
     DM_TRY(dalloc(s, &c.cgo, S));
     DM_TRY(dalloc(s, &c.cbad, S));
     DM_CK(cudaMemset(c.dense, 0, tot * sizeof(double)));
@@ -510,19 +530,6 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
         s->x.n_slow++;
       }
     }
-    // the limit of a block, not this system's need: the attribute is the
-    // kernel's, and a later, smaller system must not lower it for this one
-    int dev = 0, smem_max = 0;
-    DM_CK(cudaGetDevice(&dev));
-    DM_CK(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    auto raise_limit = [&](const void *kernel) {
-      cudaFuncAttributes fa;
-      cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem_max - (int)fa.sharedSizeBytes);
-      return e;
-    };
     DM_CK(raise_limit((const void *)k_gen_border));
     for (size_t L = 0; L < T.lb_n.size(); ++L)
       if (T.gs_fast[T.lb_gsys[L]]) s->x.limb_nmax = std::max(s->x.limb_nmax, T.lb_n[L]);
@@ -762,8 +769,9 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     ca.sys_dof0 = d.sys_dof0; ca.sys_ndof = d.sys_ndof; ca.contact_sys = c.contact_sys;
     ca.ls_action = s->prm.line_search ? s->x.ls_action : nullptr;
     ca.fixed = d.fixed; ca.sys_dense0 = c.sys_dense0; ca.sys_status = d.sys_status;
-    ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud; ca.edge_key = c.edge_key; ca.bucket_count = c.bucket_count;
-    ca.bucket_start = c.bucket_start; ca.bucket_fill = c.bucket_fill;
+    ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud;
+    ca.max_tiles = blocks(c.max_n, kNB); ca.lu_level = c.lu_level; ca.lu_adj = c.lu_adj; ca.lu_bar = c.lu_bar;
+    ca.edge_key = c.edge_key; ca.bucket_count = c.bucket_count; ca.bucket_start = c.bucket_start; ca.bucket_fill = c.bucket_fill;
     ca.bucket_edges = c.bucket_edges; ca.pairs = c.pairs; ca.npairs = c.npairs;
     ca.fc = c.fc; ca.dense = c.dense;
     ca.n_contact = c.n_contact; ca.cgo = c.cgo; ca.cbad = c.cbad;
@@ -965,7 +973,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       Timed t(s, K_SOLVE_CONTACT, rs);
       k_cc_band<<<blocks(nd, 256), 256, 0, rs>>>(ca, d.f, d.dq);
       k_cc_decide<<<blocks(s->x.cc.n_contact, 128), 128, 0, rs>>>(ca, va);
-      DM_CK(lu_solve(ca, va, s->x.cc.max_n, s->x.sms, rs));
+      DM_CK(lu_solve(ca, va, s->x.sms, rs));
     }
     if (gen_on) {
       {
@@ -1773,7 +1781,9 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     ca.sys_kind = s->x.d_sys_kind; ca.sys_active = d.sys_active; ca.dof_sys = s->x.d_dof_sys;
     ca.sys_dof0 = d.sys_dof0; ca.sys_ndof = d.sys_ndof; ca.contact_sys = c.contact_sys;
     ca.ls_action = nullptr; ca.fixed = d.fixed; ca.sys_dense0 = c.sys_dense0;
-    ca.sys_status = d.sys_status; ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud; ca.edge_key = c.edge_key;
+    ca.sys_status = d.sys_status; ca.nz = c.nz; ca.sys_nz0 = c.sys_nz0; ca.lud = c.lud;
+    ca.max_tiles = blocks(c.max_n, kNB); ca.lu_level = c.lu_level; ca.lu_adj = c.lu_adj; ca.lu_bar = c.lu_bar;
+    ca.edge_key = c.edge_key;
     ca.bucket_count = c.bucket_count; ca.bucket_start = c.bucket_start;
     ca.bucket_fill = c.bucket_fill; ca.bucket_edges = c.bucket_edges; ca.pairs = c.pairs;
     ca.npairs = c.npairs; ca.fc = c.fc; ca.dense = c.dense;
@@ -1898,7 +1908,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     vs.nd = nd; vs.sys_dof0 = d.sys_dof0; vs.sys_ndof = d.sys_ndof; vs.f = nrhs;
     vs.q = lam; vs.dq = d.dq; vs.sys_active = d.sys_active; vs.sys_iters = its;
     vs.sys_status = sts; vs.ctrl = ctl;
-    DM_CK(lu_solve(ca, vs, s->x.cc.max_n, s->x.sms, st));
+    DM_CK(lu_solve(ca, vs, s->x.sms, st));
     int32_t h[4] = {0, 0, 0, 0};
     DM_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
     DM_CK(cudaStreamSynchronize(st));

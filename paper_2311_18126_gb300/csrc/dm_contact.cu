@@ -20,12 +20,14 @@
 //                             the Hessian into the system's dense matrix.
 //  k_cc_band               -- adds the rod's own band (11 lower diagonals of
 //                             the symmetric Jacobian) to the dense matrix.
-//  k_lu_* / k_cc_subst     -- blocked LU without pivoting over the nonzero
+//  k_lu* / k_cc_subst      -- blocked LU without pivoting over the nonzero
 //                             32 x 32 tiles of the matrix (the rod band, the
 //                             contacts and their fill), all systems at once,
 //                             then the solve, q += dq.
 #include <algorithm>
 #include <cmath>
+
+#include <cooperative_groups.h>
 
 #include "dm_internal.h"
 #include "dm_kernels.cuh"
@@ -617,26 +619,35 @@ __global__ void __launch_bounds__(256) k_cc_clear(ContactArgs a) {
 //
 // The rods' Jacobian with the contact blocks is sparse in 32 x 32 tiles: the
 // band along each rod, the tiles that touching edges couple, and the fill
-// between them (its pattern is symmetric).  `nz` marks the tiles in use; for
-// each tile column k in turn, all systems at once:
-//   k_lu_panel   factors the diagonal tile (in every block, which saves a
-//                launch; block 0 keeps it in `lud`) and solves the tiles below
-//                (L = A U^-1) and right of it (U = L^-1 A) and the right-hand
-//                side, a warp per row or column: 32 steps of a shuffle and one
-//                FMA, the pivots' reciprocals moved out of the chain into
-//                the rows of U;
-//   k_lu_update  subtracts L(I,k) U(k,J) from the tiles (I, J) of the column's
-//                nonzero rows, in quarters of 16 x 16 (an SM's FP64 pipe takes
-//                9 us for a whole tile), and the right-hand side's part, and
-//                marks the fill.
+// between them (its pattern is symmetric).  `nz` marks the tiles in use.
+//   k_lu_order   orders the elimination by levels from the pattern alone, a
+//                block per system: a level takes up to eight tile columns
+//                (fronts) of the fewest neighbours (one more allowed), no two
+//                of them coupled, the outermost first; it lists each front's
+//                remaining neighbours and marks the fill.  Rods eliminate from
+//                both ends, separate rods side by side.
+//   k_lu         all levels in one launch, the chip's blocks shared among the
+//                systems, which each meet at their own counter twice a level:
+//                panel -- the fronts' diagonal tiles are factored (in every
+//                block, which saves a meeting; a front's first block keeps its
+//                tile in `lud`) and the tiles below (L = A U^-1) and right of
+//                it (U = L^-1 A) and the right-hand side solved, a warp per row
+//                or column: 32 steps of a shuffle and one FMA, the pivots'
+//                reciprocals moved out of the chain into the rows of U;
+//                update -- L(I,k) U(k,J) subtracted from the tiles (I, J) of a
+//                front's neighbours, in quarters of 16 x 16 (an SM's FP64 pipe
+//                takes 9 us for a whole tile), and the right-hand side's part.
 // k_cc_decide takes the Newton decision of each contact system first;
-// k_cc_subst runs the backward substitution and updates q.
-// Bound by the chain of tile columns (a panel launch 26 us, most of it the
-// diagonal tile's 32 dependent columns, an update launch 10 us for the seven
-// tiles a side of a 500-node coil).  Measured (GB300): factorisation and solve
-// of that coil 9.0 -> 2.8 ms, of four grippers of 1195 DOFs 21 -> 1.8 ms
-// (before: the full bandwidth, three launches per panel and system, a
-// panel row per thread).
+// k_cc_subst runs the backward substitution, level by level, and updates q.
+// Bound by the chain of levels: a 500-node coil (63 tile columns, up to 12
+// neighbours) has 24, a gripper of five 60-node fingers (38) has 8.  The
+// diagonal tile's 32 dependent columns run on four warps (one per SM
+// partition).
+// Measured (GB300): a level 45 k cycles and up -- the diagonal tile 23 k, its
+// solves 7 k, the two meetings 4 k each, the update from 6 k (few tiles) to 85 k
+// (2400 quarters: the FP64 pipes' rate); factorisation and solve of the coil 2.8
+// -> 1.1 ms, of four grippers 1.8 -> 0.4 ms (before: tile columns in their
+// order, two launches for each; before that, the full bandwidth: 9 and 21 ms).
 
 __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -667,180 +678,353 @@ __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {
   a.cbad[c] = 0;
 }
 
-// The tiles of row k of a system's pattern beyond k, in order, into list
-// (shared memory); every thread of the block calls it.  Returns their number.
-__device__ __forceinline__ int tile_list(const uint8_t *row, int k, int nt, uint16_t *list, int *count) {
-  if (threadIdx.x < 32) {
-    int m = 0;
-    for (int b = k + 1; b < nt; b += 32) {
-      const int J = b + (int)threadIdx.x;
-      const bool on = J < nt && row[J] != 0;
-      const unsigned mask = __ballot_sync(0xffffffffu, on);
-      if (on) list[m + __popc(mask & ((1u << threadIdx.x) - 1u))] = (uint16_t)J;
-      m += __popc(mask);
-    }
-    if (threadIdx.x == 0) *count = m;
+constexpr int kMaxTiles = 1024;  // tile columns of a system (its matrix is at most 8 GB)
+constexpr int kFronts = 8;       // tile columns eliminated at once
+constexpr unsigned kDegreeSlack = 1;
+static_assert(kLevelInts > 1 + 2 * kFronts + 1, "a level's record");
+// a level's record: number of fronts, their tile columns, their neighbours'
+// counts (zero fronts: past the last level); the first one ends with the
+// number of levels
+
+struct Level {
+  int nf, k[kFronts], m[kFronts];
+};
+
+// Bit rows of the pattern in shared memory, word w of tile i at row[w nt + i];
+// a thread per tile.
+__global__ void __launch_bounds__(1024) k_lu_order(ContactArgs a) {
+  const int c = blockIdx.x;
+  if (!a.cgo[c]) return;
+  const int s = a.contact_sys[c], n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, W = (nt + 31) / 32;
+  extern __shared__ unsigned row[];
+  __shared__ unsigned rem[kMaxTiles / 32], best[2][kFronts];
+  int32_t *lev = a.lu_level + (size_t)c * a.max_tiles * kLevelInts;
+  uint8_t *nz = a.nz + a.sys_nz0[s];
+  uint16_t *adj = a.lu_adj + a.sys_nz0[s];
+  const int i = threadIdx.x, lane = i & 31;
+#pragma unroll 4
+  for (int e = i >> 5; e < nt * W; e += blockDim.x >> 5) {
+    const int r = e / W, J = (e - r * W) * 32 + lane;
+    const unsigned bits = __ballot_sync(0xffffffffu, J < nt && J != r && nz[(size_t)r * nt + J] != 0);
+    if (lane == 0) row[(e - r * W) * nt + r] = bits;
   }
+  if (i < W) rem[i] = i == W - 1 && (nt & 31) ? (1u << (nt & 31)) - 1u : 0xffffffffu;
+  if (i == 0) a.lu_bar[c] = 0;
+  if (i < 2 * kFronts) best[i / kFronts][i % kFronts] = 0xffffffffu;
   __syncthreads();
-  return *count;
+  const auto bit = [&](int p) { return i < nt && ((row[(p >> 5) * nt + i] >> (p & 31)) & 1u); };  // i ~ p
+  int l = 0;
+  for (;; ++l) {
+    // fewest remaining neighbours, then farthest from the middle, then first
+    unsigned key = 0xffffffffu;
+    const bool alive = i < nt && ((rem[i >> 5] >> lane) & 1u);
+    if (alive) {
+      unsigned deg = 0;
+      for (int w = 0; w < W; ++w) deg += __popc(row[w * nt + i] & rem[w]);
+      key = (deg << 21) | ((unsigned)(1024 - abs(2 * i - (nt - 1))) << 10) | (unsigned)i;
+    }
+    int nf = 0, pick[kFronts];
+    unsigned lim = 0;
+#pragma unroll
+    for (int f = 0; f < kFronts; ++f) {
+      if (nf < f) break;
+      const unsigned v = __reduce_min_sync(0xffffffffu, key);
+      if (lane == 0) atomicMin(&best[l & 1][f], v);
+      __syncthreads();
+      const unsigned b = best[l & 1][f];
+      if (f == 0) lim = (b >> 21) + kDegreeSlack;
+      if (b == 0xffffffffu || (b >> 21) > lim) break;
+      pick[f] = (int)(b & 1023u);
+      nf = f + 1;
+      if (i == pick[f] || bit(pick[f])) key = 0xffffffffu;
+    }
+    if (nf == 0) break;
+    __syncthreads();  // (best of this level read, rem read)
+#pragma unroll
+    for (int f = 0; f < kFronts; ++f)
+      if (f < nf && i == pick[f]) atomicAnd(&rem[i >> 5], ~(1u << lane));
+    if (i < kFronts) best[l & 1][i] = 0xffffffffu;  // (next used two levels on)
+    __syncthreads();
+#pragma unroll
+    for (int f = 0; f < kFronts; ++f) {
+      if (f >= nf) break;
+      const int p = pick[f];
+      if (i == 32 * f % (int)blockDim.x) {  // (a thread of another warp for each)
+        int m = 0;
+        for (int w = 0; w < W; ++w) m += __popc(row[w * nt + p] & rem[w]);
+        lev[l * kLevelInts + 1 + f] = p;
+        lev[l * kLevelInts + 1 + kFronts + f] = m;
+      }
+      if (alive && bit(p) && ((rem[i >> 5] >> lane) & 1u)) {
+        int rank = 0;
+        for (int w = 0; w < W; ++w) {
+          const unsigned x = row[w * nt + p] & rem[w];
+          if (w < i >> 5) rank += __popc(x);
+          if (w == i >> 5) rank += __popc(x & ((1u << lane) - 1u));
+          row[w * nt + i] |= w == i >> 5 ? x & ~(1u << lane) : x;  // fill (own row only)
+        }
+        adj[(size_t)p * nt + rank] = (uint16_t)i;
+      }
+    }
+    if (i == 0) lev[l * kLevelInts] = nf;
+    __syncthreads();
+  }
+  if (i == 0) lev[kLevelInts - 1] = l;
+  for (int x = l + i; x < a.max_tiles; x += blockDim.x) lev[x * kLevelInts] = 0;
+  for (int e = i >> 5; e < nt * W; e += blockDim.x >> 5) {
+    const int r = e / W, J = (e - r * W) * 32 + lane;
+    if ((row[(e - r * W) * nt + r] >> lane) & 1u) nz[(size_t)r * nt + J] = 1;
+  }
 }
 
-constexpr int kMaxTiles = 1024;  // tile columns of a system (its matrix is at most 8 GB)
+// LU of the 32 x 32 tile D (shared memory; four zero rows behind it) by warps
+// 0-3; every thread of the block calls it.  Leaves the unit factors (L below
+// the diagonal, U over its pivots above it) in D and the pivots' reciprocals in
+// R.  Column j: rows j + 1 + warp, + 4, ..., a lane per column; no branches (the
+// zero rows take what is too much, and reciprocals are those of the integer
+// pipe): 705 cycles a column, 496 of them the chain of product, first row,
+// exchange, reciprocal and barrier.  False if a pivot was outside the
+// reciprocal's range; `exact`: any pivot, by division (thrice the time).
+template <bool exact>
+__device__ __forceinline__ bool factor_tile(double (*D)[kNB + 1], double *R) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < 4) {
+    double r = exact ? 1.0 / D[0][0] : rcp_int(D[0][0]);
+    if (warp == 0 && lane == 0) R[0] = r;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      const int NT = 8 - p;  // rows of a warp in columns 4 p .. 4 p + 3
+#pragma unroll 1
+      for (int j = 4 * p; j < (p < 7 ? 4 * p + 4 : kNB - 1); ++j) {
+        const int i0 = j + 1 + warp;
+        double m[8], d[8];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          m[t] = D[i0 + 4 * t][j];
+          d[t] = D[i0 + 4 * t][lane];
+        }
+        const double x = D[j][lane] * r, u = lane > j ? x : 0.0;
+        d[0] = fma(-m[0], u, d[0]);
+        const double piv = __shfl_sync(0xffffffffu, d[0], j + 1);  // (warp 0's)
+        const double rn = exact ? 1.0 / piv : rcp_int(piv);
+#pragma unroll
+        for (int t = 1; t < NT; ++t) d[t] = fma(-m[t], u, d[t]);
+#pragma unroll
+        for (int t = 0; t < NT; ++t) D[i0 + 4 * t][lane] = d[t];
+        if (warp == 0 && lane == 0) R[j + 1] = rn;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        r = R[j + 1];
+      }
+    }
+  }
+  __syncthreads();
+  return exact || !__syncthreads_or(warp == 0 && !rcp64_in_range(D[lane][lane]));
+}
 
-__global__ void __launch_bounds__(256) k_lu_panel(ContactArgs a, double *yall, int k) {
+// The blocks of a system meet (all of them are resident: a cooperative launch
+// when there are several).  False: a wait ran out, or (`check`) a zero pivot.
+constexpr int kSpinLimit = 1 << 22;  // a few seconds
+__device__ __forceinline__ bool lu_barrier(int32_t *bar, int32_t *bad, int blocks, int &target, bool check) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int fine = 1;
+    if (blocks > 1) {
+      target += blocks;
+      __threadfence();
+      atomicAdd(bar, 1);
+      int seen = 0, spins = 0;
+      do {
+        asm volatile("ld.acquire.gpu.s32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      } while (seen < target && ++spins < kSpinLimit);
+      if (seen < target) {
+        atomicExch(bad, 1);
+        fine = 0;
+      }
+      __threadfence();
+    }
+    // (a zero pivot is written before the barrier that follows its panel, and
+    // none while any block is between that barrier and the next)
+    if (check && *reinterpret_cast<volatile int32_t *>(bad)) fine = 0;
+    ok = fine;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Factorisation of all levels: gridDim.x blocks per system.
+constexpr int kLuThreads = 512;
+__global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yall) {
   const int c = blockIdx.y;
-  // (another block of this launch may be setting cbad: the block decides as one)
-  if (__syncthreads_or(!a.cgo[c] || a.cbad[c])) return;
+  if (!a.cgo[c]) return;
   const int s = a.contact_sys[c];
   const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB;
-  if (k >= nt) return;
-  __shared__ double D[kNB][kNB + 1];
-  __shared__ double R[kNB];
-  __shared__ uint16_t list[kMaxTiles];
-  __shared__ int count;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ Level lv;
+  __shared__ double D[kNB + 4][kNB + 1], R[kNB];
+  __shared__ double Lh[2][16][kNB + 1];
+  __shared__ double Uh[2][kNB][16 + 1];
+  __shared__ uint16_t list[kFronts][kMaxTiles];
+  __shared__ unsigned reach[kMaxTiles / 4];  // per tile, a byte: the fronts it neighbours
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int half = tid >> 8, ty = (tid & 255) >> 4, tx = tid & 15;  // of the update
+  double (*Ls)[kNB + 1] = Lh[half], (*Us)[16 + 1] = Uh[half];
   double *A = a.dense + a.sys_dense0[s], *y = yall + a.sys_dof0[s];
-  const int k0 = k * kNB, nb = min(kNB, n - k0);
-  // the diagonal tile, four rows per thread (rows warp + 8 t, column lane);
-  // the identity beyond the matrix
-  double e[4];
+  const uint16_t *adj = a.lu_adj + a.sys_nz0[s];
+  const int32_t *lev = a.lu_level + (size_t)c * a.max_tiles * kLevelInts;
+  const int levels = lev[kLevelInts - 1];
+  const auto fronts = [&](int I) { return (reach[I >> 2] >> (8 * (I & 3))) & 0xffu; };
+  const int blocks = gridDim.x;
+  int target = 0;
+  for (int l = 0; l < levels; ++l) {
+    if (tid < 1 + 2 * kFronts) reinterpret_cast<int *>(&lv)[tid] = lev[l * kLevelInts + tid];
+    for (int e = tid; e < (nt + 3) / 4; e += kLuThreads) reach[e] = 0;
+    __syncthreads();
+    const int nf = lv.nf;
+    int items = 0, vecs = 0;
+    for (int f = 0; f < nf; ++f) {
+      const uint16_t *src = adj + (size_t)lv.k[f] * nt;
+      for (int e = tid; e < lv.m[f]; e += kLuThreads) {
+        const int I = src[e];
+        list[f][e] = (uint16_t)I;
+        atomicOr(&reach[I >> 2], 1u << (8 * (I & 3) + f));
+      }
+      items += 4 * lv.m[f] * lv.m[f];
+      vecs += lv.m[f];
+    }
+    __syncthreads();
+
+    // panel: the blocks are dealt to the fronts by their vectors (rows of L,
+    // columns of U, the right-hand side: a warp each), so that a block factors
+    // one diagonal tile; fronts in turn when there are fewer blocks
+    for (int f = 0, start = 0; f < nf; ++f) {
+      const int k = lv.k[f], m = lv.m[f], k0 = k * kNB, nb = min(kNB, n - k0), vec = 2 * kNB * m + 1;
+      int part = 0, parts = 1;
+      if (blocks >= nf) {
+        parts += (blocks - nf) * vec / (2 * kNB * vecs + nf);
+        part = (int)blockIdx.x - start;
+        start += parts;
+        if (part < 0 || part >= parts) continue;
+      } else if (f % blocks != (int)blockIdx.x) {
+        continue;
+      }
+      const int each = min((vec + parts - 1) / parts, kLuThreads / 32);  // vectors of a block at a time
+      if (part * each >= vec) continue;
+      const auto load = [&] {  // the identity beyond the matrix
+        __syncthreads();
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int i = warp + 8 * t;
-    e[t] = i < nb && lane < nb ? A[(size_t)(k0 + i) * n + k0 + lane] : i == lane ? 1.0 : 0.0;
-    D[i][lane] = e[t];
-  }
-  const int m = tile_list(a.nz + a.sys_nz0[s] + (size_t)k * nt, k, nt, list, &count);
-  const int nvec = 2 * kNB * m + 1;  // rows of L, columns of U, the right-hand side
-  if (blockIdx.x && (int)blockIdx.x * 8 >= nvec) return;
+        for (int t = 0; t < kNB * 32 / kLuThreads; ++t) {
+          const int i = warp + kLuThreads / 32 * t;
+          D[i][lane] = i < nb && lane < nb ? A[(size_t)(k0 + i) * n + k0 + lane] : i == lane ? 1.0 : 0.0;
+        }
+        if (warp < 4) D[kNB + warp][lane] = 0.0;
+        __syncthreads();
+      };
+      load();
+      if (!factor_tile<false>(D, R)) {
+        load();
+        factor_tile<true>(D, R);
+        if (warp == 0 && zero_or_nonfinite(D[lane][lane])) a.cbad[c] = 1;
+        __syncthreads();
+      }
+      const double rl = R[lane];
 #pragma unroll
-  for (int j = 0; j < kNB; ++j) {
-    const double piv = D[j][j];
-    const double r = rcp_any(piv);
-    const double u = D[j][lane] * r;  // row j of U over the pivot
+      for (int t = 0; t < kNB * 32 / kLuThreads; ++t) {
+        const int i = warp + kLuThreads / 32 * t;
+        D[i][lane] = lane == i ? 1.0 : D[i][lane] * (lane < i ? rl : R[i]);
+      }
+      __syncthreads();
+      if (part == 0) {
+        double *out = a.lud + (size_t)(a.sys_dof0[s] + k0) * kNB;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      if (8 * t + 7 <= j) continue;
-      const int i = warp + 8 * t;
-      if (i > j) {
-        const double lij = D[i][j];
-        if (lane > j) {
-          e[t] = fma(-lij, u, e[t]);
-          // what the next column reads: its column and its row
-          if (lane == j + 1 || i == j + 1) D[i][lane] = e[t];
+        for (int t = 0; t < kNB * 32 / kLuThreads; ++t) {
+          const int i = warp + kLuThreads / 32 * t;
+          if (i < nb) out[i * kNB + lane] = i == lane ? R[i] : D[i][lane];
+        }
+      }
+      for (int g = part * each + warp; g < vec && warp < each; g += parts * each) {
+        if (g < kNB * m) {  // a row of L: x U = a, w_j = x_j d_j
+          const int row = list[f][g / kNB] * kNB + g % kNB;
+          if (row >= n) continue;
+          double *p = A + (size_t)row * n + k0 + lane;
+          double w = lane < nb ? *p : 0.0;
+#pragma unroll
+          for (int j = 0; j < kNB - 1; ++j) {
+            const double wj = __shfl_sync(0xffffffffu, w, j);
+            if (lane > j) w = fma(-wj, D[j][lane], w);
+          }
+          if (lane < nb) *p = w * R[lane];
+        } else {  // a column of U, or the right-hand side: L x = a (unit lower)
+          const int h = g - kNB * m;
+          const bool rhs = h == kNB * m;
+          const int col = rhs ? 0 : list[f][h / kNB] * kNB + h % kNB;
+          if (col >= n) continue;
+          double *p = rhs ? y + k0 + lane : A + (size_t)(k0 + lane) * n + col;
+          double w = lane < nb ? *p : 0.0;
+#pragma unroll
+          for (int j = 0; j < kNB - 1; ++j) {
+            const double wj = __shfl_sync(0xffffffffu, w, j);
+            if (lane > j) w = fma(-wj, D[lane][j], w);
+          }
+          if (lane < nb) *p = w;
         }
       }
     }
-    if (warp == 0 && lane == 0) {
-      R[j] = r;
-      if (!(fabs(piv) > 0.0) || !isfinite(piv)) a.cbad[c] = 1;
-    }
-    __syncthreads();
-  }
-  // D: on and below the diagonal l_ij d_j, above it u_jm; for the solves the
-  // unit factors: L = (l_ij), U' = (u_jm / d_j)
-  if (blockIdx.x == 0) {
-    double *out = a.lud + (size_t)(a.sys_dof0[s] + k0) * kNB;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int i = warp + 8 * t;
-      if (i < nb) out[i * kNB + lane] = i == lane ? R[i] : D[i][lane];
-    }
-  }
-  double lrow[4];
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int i = warp + 8 * t;
-    lrow[t] = lane < i ? D[i][lane] * R[lane] : lane > i ? D[i][lane] * R[i] : 1.0;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < 4; ++t) D[warp + 8 * t][lane] = lrow[t];
-  __syncthreads();
-  const double rl = R[lane];
-  for (int g = (int)blockIdx.x * 8 + warp; g < nvec; g += (int)gridDim.x * 8) {
-    if (g < kNB * m) {  // a row of L: x U = a, w_j = x_j d_j
-      const int row = list[g / kNB] * kNB + g % kNB;
-      if (row >= n) continue;
-      double *p = A + (size_t)row * n + k0 + lane;
-      double w = lane < nb ? *p : 0.0;
-#pragma unroll
-      for (int j = 0; j < kNB - 1; ++j) {
-        const double wj = __shfl_sync(0xffffffffu, w, j);
-        if (lane > j) w = fma(-wj, D[j][lane], w);
-      }
-      if (lane < nb) *p = w * rl;
-    } else {  // a column of U, or the right-hand side: L x = a (unit lower)
-      const int h = g - kNB * m;
-      const bool rhs = h == kNB * m;
-      const int col = rhs ? 0 : list[h / kNB] * kNB + h % kNB;
-      if (col >= n) continue;
-      double *p = rhs ? y + k0 + lane : A + (size_t)(k0 + lane) * n + col;
-      double w = lane < nb ? *p : 0.0;
-#pragma unroll
-      for (int j = 0; j < kNB - 1; ++j) {
-        const double wj = __shfl_sync(0xffffffffu, w, j);
-        if (lane > j) w = fma(-wj, D[lane][j], w);
-      }
-      if (lane < nb) *p = w;
-    }
-  }
-}
+    if (l + 1 == levels) return;  // (the last level has no neighbours left)
+    if (!lu_barrier(a.lu_bar + c, a.cbad + c, blocks, target, true)) return;
 
-// Quarter items (16 x 16 of a tile) of the update, then the right-hand side's
-// rows, strided over the system's blocks.
-__global__ void __launch_bounds__(256) k_lu_update(ContactArgs a, double *yall, int k) {
-  const int c = blockIdx.y;
-  if (!a.cgo[c] || a.cbad[c]) return;
-  const int s = a.contact_sys[c];
-  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB;
-  if (k + 1 >= nt) return;
-  __shared__ double Ls[16][kNB + 1];
-  __shared__ double Us[kNB][16 + 1];
-  __shared__ uint16_t list[kMaxTiles];
-  __shared__ int count;
-  uint8_t *nz = a.nz + a.sys_nz0[s];
-  const int m = tile_list(nz + (size_t)k * nt, k, nt, list, &count);
-  double *A = a.dense + a.sys_dense0[s], *y = yall + a.sys_dof0[s];
-  const int k0 = k * kNB, nb = min(kNB, n - k0);
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int items = 4 * m * m;
-  for (int it = blockIdx.x; it < items + m; it += gridDim.x) {
-    if (it >= items) {  // rows of the right-hand side: a quarter of a warp's lanes per term
-      const int I = list[it - items], lane = tid & 31;
-      for (int r = tid >> 5; r < kNB; r += 8) {
-        const int row = I * kNB + r;
-        if (row >= n) break;
-        double v = lane < nb ? A[(size_t)row * n + k0 + lane] * y[k0 + lane] : 0.0;
+    // update, by half a block: quarter items (16 x 16 of a tile), front by front,
+    // then the right-hand side's rows; a tile or row of several fronts belongs to the
+    // first, which takes the others' parts along
+    for (int f = 0, base = 0, it = blockIdx.x + half * blocks; it < items + vecs; it += 2 * blocks) {
+      if (it >= items) {  // right-hand side: a lane per term
+        int g = it - items, fv = 0;
+        while (g >= lv.m[fv]) g -= lv.m[fv++];
+        const int I = list[fv][g];
+        const unsigned on = fronts(I);
+        if (__ffs(on) - 1 != fv) continue;
+        for (int r = warp & 7; r < kNB; r += 8) {
+          const int row = I * kNB + r;
+          if (row >= n) break;
+          double v = 0.0;
+          for (unsigned q = on; q; q &= q - 1) {
+            const int k0 = lv.k[__ffs(q) - 1] * kNB;
+            if (lane < n - k0) v = fma(A[(size_t)row * n + k0 + lane], y[k0 + lane], v);
+          }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) y[row] -= v;
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) y[row] -= v;
+        }
+        continue;
       }
-      continue;
-    }
-    const int q = it & 3, t = it >> 2, ti = t / m, tj = t - ti * m;
-    const int I = list[ti], J = list[tj];
-    const int r0 = I * kNB + 16 * (q >> 1), c0 = J * kNB + 16 * (q & 1);
-    if (q == 0 && tid == 0) nz[(size_t)I * nt + J] = 1;  // fill
-    if (r0 >= n || c0 >= n) continue;
-    if (a.lu_flops && tid == 0)
-      atomicAdd(a.lu_flops, 2ull * (unsigned long long)(min(16, n - r0) * min(16, n - c0) * nb));
-    __syncthreads();
+      while (it >= base + 4 * lv.m[f] * lv.m[f]) base += 4 * lv.m[f] * lv.m[f], ++f;
+      const int q = (it - base) & 3, t = (it - base) >> 2, ti = t / lv.m[f], tj = t - ti * lv.m[f];
+      const int I = list[f][ti], J = list[f][tj];
+      const int r0 = I * kNB + 16 * (q >> 1), c0 = J * kNB + 16 * (q & 1);
+      const unsigned on = fronts(I) & fronts(J);
+      if (__ffs(on) - 1 != f || r0 >= n || c0 >= n) continue;
+      if (a.lu_flops && (tid & 255) == 0)
+        atomicAdd(a.lu_flops, 2ull * (unsigned long long)(min(16, n - r0) * min(16, n - c0) * kNB * __popc(on)));
+      const bool in = r0 + ty < n && c0 + tx < n;
+      double *p = A + (size_t)(r0 + ty) * n + c0 + tx;
+      const double old = in ? *p : 0.0;
+      double acc = 0.0;
+      for (unsigned qf = on; qf; qf &= qf - 1) {
+        const int k0 = lv.k[__ffs(qf) - 1] * kNB, nb = min(kNB, n - k0);
+        asm volatile("bar.sync %0, 256;" ::"r"(2 + half) : "memory");
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int i = (tid >> 5) + 8 * e, mm = tid & 31;
-      Ls[i][mm] = r0 + i < n && mm < nb ? A[(size_t)(r0 + i) * n + k0 + mm] : 0.0;
-      const int u = ty + 16 * e;
-      Us[u][tx] = c0 + tx < n && u < nb ? A[(size_t)(k0 + u) * n + c0 + tx] : 0.0;
-    }
-    const bool in = r0 + ty < n && c0 + tx < n;
-    double *p = A + (size_t)(r0 + ty) * n + c0 + tx;
-    const double old = in ? *p : 0.0;
-    __syncthreads();
-    double acc = 0.0;
+        for (int e = 0; e < 2; ++e) {
+          const int i = (warp & 7) + 8 * e, mm = lane;
+          Ls[i][mm] = r0 + i < n && mm < nb ? A[(size_t)(r0 + i) * n + k0 + mm] : 0.0;
+          const int u = ty + 16 * e;
+          Us[u][tx] = c0 + tx < n && u < nb ? A[(size_t)(k0 + u) * n + c0 + tx] : 0.0;
+        }
+        asm volatile("bar.sync %0, 256;" ::"r"(2 + half) : "memory");
 #pragma unroll
-    for (int mm = 0; mm < kNB; ++mm) acc = fma(Ls[ty][mm], Us[mm][tx], acc);
-    if (in) *p = old - acc;
+        for (int mm = 0; mm < kNB; ++mm) acc = fma(Ls[ty][mm], Us[mm][tx], acc);
+      }
+      if (in) *p = old - acc;
+    }
+    if (!lu_barrier(a.lu_bar + c, a.cbad + c, blocks, target, false)) return;
   }
 }
 
@@ -864,16 +1048,20 @@ __global__ void __launch_bounds__(256) k_cc_transpose(ContactArgs a) {
   }
 }
 
-// Backward substitution U x = z of each contact system, q += x: a block per
-// system, tile rows from the last one up; the warps take the row's tiles
-// (a warp sums 32 columns of a row by a shuffle tree), warp 0 solves the
+// Backward substitution U x = z of each contact system, q += x: a cluster of
+// blocks per system, levels from the last one up; the level's fronts are dealt
+// to a block's warps, a front's tiles to the blocks (eight columns at a time,
+// lane = row); a front's own block adds the blocks' sums and solves the
 // diagonal tile.
-__global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
-  const int c = blockIdx.x;
+constexpr int kSubstWarps = 16;
+__global__ void __launch_bounds__(32 * kSubstWarps) k_cc_subst(ContactArgs a, SolveArgs v) {
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int c = blockIdx.x / blocks;
   const int s = a.contact_sys[c];
   if (!a.cgo[c]) return;
   if (a.cbad[c]) {
-    if (threadIdx.x == 0) {
+    if (rank == 0 && threadIdx.x == 0) {
       v.sys_status[s] = DM_ERR_DEGENERATE;
       v.sys_active[s] = 0;
       atomicAdd(&v.ctrl[1], 1);
@@ -883,33 +1071,50 @@ __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
   }
   const int d0 = v.sys_dof0[s], n = v.sys_ndof[s], nt = (n + kNB - 1) / kNB;
   const double *A = a.dense + a.sys_dense0[s];
+  const uint16_t *adj = a.lu_adj + a.sys_nz0[s];
+  const int32_t *lev = a.lu_level + (size_t)c * a.max_tiles * kLevelInts;
   double *y = v.dq + d0;
-  __shared__ uint16_t list[kMaxTiles];
-  __shared__ int count;
-  __shared__ double part[32][kNB + 1];
+  __shared__ double part[kSubstWarps][kNB + 1], tot[kFronts][kNB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int k = nt - 1; k >= 0; --k) {
+  for (int l = lev[kLevelInts - 1] - 1; l >= 0; --l) {
+    const int32_t *rec = lev + l * kLevelInts;
+    const int nf = rec[0], sh = nf <= 1 ? 0 : 32 - __clz(nf - 1);  // fronts, rounded up to 2^sh
+    const int per = kSubstWarps >> sh, f = warp / per, slot = warp - f * per;
+    const bool on = f < nf, first = on && slot == 0, own = first && f % blocks == rank;
+    const int k = on ? rec[1 + f] : 0, m = on ? rec[1 + kFronts + f] : 0;
     const int k0 = k * kNB, nb = min(kNB, n - k0);
-    const int m = tile_list(a.nz + a.sys_nz0[s] + (size_t)k * nt, k, nt, list, &count);
-    // warp w sums the columns of tiles w, w + 32, ... : lane = row
     double sum = 0.0;
-    for (int t = warp; t < 4 * m; t += 32) {  // eight columns of a tile
-      const int j0 = list[t >> 2] * kNB + 8 * (t & 3);
+    for (int t = rank + blocks * slot; t < 4 * m; t += blocks * per) {
+      const int j0 = adj[(size_t)k * nt + (t >> 2)] * kNB + 8 * (t & 3);
+      double x[8], z[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (lane < nb && j0 + j < n) sum = fma(A[(size_t)(k0 + lane) * n + j0 + j], y[j0 + j], sum);
+      for (int j = 0; j < 8; ++j) {
+        const bool in = lane < nb && j0 + j < n;
+        x[j] = in ? A[(size_t)(k0 + lane) * n + j0 + j] : 0.0;
+        z[j] = in ? y[j0 + j] : 0.0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum = fma(x[j], z[j], sum);
     }
     part[warp][lane] = sum;
-    __syncthreads();
-    if (warp == 0) {
-      const double *Dk = a.lud + (size_t)(d0 + k0) * kNB;  // reciprocal pivots, U above
-      double z = lane < nb ? y[k0 + lane] : 0.0;
-      const int nw = min(32, 4 * m);
-      for (int w = 0; w < nw; ++w) z -= part[w][lane];
-      const double r = lane < nb ? Dk[lane * kNB + lane] : 1.0;
-      double urow[kNB];  // the lane's row of U over its pivot
+    // the lane's row of U over its pivot
+    const double *Dk = a.lud + (size_t)(d0 + k0) * kNB;
+    double urow[kNB], r = 0.0, z = 0.0;
+    if (own) {
 #pragma unroll
-      for (int j = 0; j < kNB; ++j) urow[j] = lane < nb && j > lane && j < nb ? Dk[lane * kNB + j] * r : 0.0;
+      for (int j = 0; j < kNB; ++j) urow[j] = lane < nb && j > lane && j < nb ? Dk[lane * kNB + j] : 0.0;
+      r = lane < nb ? Dk[lane * kNB + lane] : 1.0;
+      z = lane < nb ? y[k0 + lane] : 0.0;
+    }
+    __syncthreads();
+    if (first) {
+      const int got = min(per, (4 * m - rank + blocks - 1) / blocks);  // slots with tiles
+      for (int w = 1; w < got; ++w) sum += part[warp + w][lane];
+      tot[f][lane] = sum;
+    }
+    cluster.sync();
+    if (own) {
+      for (int b = 0; b < min(blocks, 4 * m); ++b) z -= cluster.map_shared_rank(&tot[f][0], b)[lane];
       double x = z * r;
 #pragma unroll
       for (int j = kNB - 1; j > 0; --j) x = fma(-urow[j], __shfl_sync(0xffffffffu, x, j), x);
@@ -918,9 +1123,9 @@ __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
         atomicAdd(v.q + d0 + k0 + lane, x);
       }
     }
-    __syncthreads();
+    cluster.sync();
   }
-  if (threadIdx.x == 0) {
+  if (rank == 0 && threadIdx.x == 0) {
     v.sys_iters[s] += 1;
     if (v.ls_trial) v.ls_trial[s] = 1;
     atomicAdd(&v.ctrl[0], 1);
@@ -929,20 +1134,35 @@ __global__ void __launch_bounds__(1024) k_cc_subst(ContactArgs a, SolveArgs v) {
 }
 
 // The whole factorisation and solve: right-hand side in v.dq (k_cc_band).
-cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int max_n, int sms, cudaStream_t st) {
-  const int nt = (max_n + kNB - 1) / kNB, nc = a.n_contact;
+cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStream_t st) {
+  const int nt = a.max_tiles, nc = a.n_contact;
   if (nc == 0) return cudaSuccess;
-  // blocks per system: the chip shared among the systems, no more than a
-  // full column's rows and columns (panel) or tiles (update) can use
-  const int share = std::max(1, (2 * sms + nc - 1) / nc);
-  for (int k = 0; k < nt; ++k) {
-    const int rest = nt - 1 - k;
-    k_lu_panel<<<dim3(std::min(share, std::max(1, 8 * rest + 1)), nc), 256, 0, st>>>(a, v.dq, k);
-    if (rest > 0)
-      k_lu_update<<<dim3(std::min(share, 4 * rest * rest + rest), nc), 256, 0, st>>>(a, v.dq, k);
-  }
-  k_cc_subst<<<nc, 1024, 0, st>>>(a, v);
-  return cudaGetLastError();
+  const int words = nt * ((nt + 31) / 32), threads = std::max(256, (nt + 31) / 32 * 32);
+  k_lu_order<<<nc, threads, 4 * words, st>>>(a);
+  // the chip shared among the systems; several blocks of a system wait for one
+  // another, so all of them must be resident (two per SM fit)
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg{};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cfg.stream = st;
+  const int share = std::max(1, std::min(sms / nc, 4 * nt * nt));
+  cfg.gridDim = dim3(share, nc);
+  cfg.blockDim = dim3(kLuThreads);
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = share > 1 ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_lu, a, v.dq);
+  if (e != cudaSuccess) return e;
+  // a cluster of up to eight blocks while the systems leave SMs idle
+  int cs = 8;
+  while (cs > 1 && cs * nc > sms) cs >>= 1;
+  cfg.gridDim = dim3(nc * cs);
+  cfg.blockDim = dim3(32 * kSubstWarps);
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  e = cudaLaunchKernelEx(&cfg, k_cc_subst, a, v);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace dm

@@ -317,6 +317,10 @@ struct ContactArgs {
   int32_t *sys_status;
   uint8_t *nz;               // per system: which kNB x kNB tiles of its matrix are in use
   const int64_t *sys_nz0;
+  int max_tiles;             // tile columns of the largest system
+  int32_t *lu_level;         // [n_contact][max_tiles][kLevelInts]: the elimination's levels
+  int32_t *lu_bar;           // per contact system: its blocks' meetings
+  uint16_t *lu_adj;          // like nz: the neighbours left of each tile column at its elimination
   double *lud;               // [nd][kNB]: factored diagonal tiles (their pivots inverted)
   unsigned long long *edge_key;
   int32_t *bucket_count, *bucket_start, *bucket_fill, *bucket_edges;
@@ -340,8 +344,10 @@ __global__ void k_cc_clear(ContactArgs a);
 __global__ void k_cc_decide(ContactArgs a, SolveArgs v);
 __global__ void k_cc_transpose(ContactArgs a);
 // LU and solve of the systems with cgo set: v.dq holds the right-hand side;
-// max_n: DOFs of the largest system.
-cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int max_n, int sms, cudaStream_t st);
+// its ordering takes (max_tiles^2 / 8) bytes of shared memory.
+constexpr int kLevelInts = 20;
+__global__ void k_lu_order(ContactArgs a);
+cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStream_t st);
 
 // Adjoint of one implicit step (single rods): right-hand side, state and
 // natural-curvature gradients.
