@@ -12,11 +12,9 @@
 //                             below C + delta (C = sum of the radii).
 //  k_cc_terms              -- a warp per active pair: D and its first and
 //                             second derivatives with respect to the 12
-//                             node coordinates (second-order forward-mode
-//                             dual numbers through the closest-point
-//                             computation, their 78 second derivatives spread
-//                             over the lanes), k_c E(D) of Eq. 10 by the chain
-//                             rule; -grad into the contact force vector,
+//                             node coordinates (in closed form at the closest
+//                             points, the 78 second ones spread over the
+//                             lanes), k_c E(D) of Eq. 10 by the chain rule; -grad into the contact force vector,
 //                             the Hessian into the system's dense matrix.
 //  k_cc_band               -- adds the rod's own band (11 lower diagonals of
 //                             the symmetric Jacobian) to the dense matrix.
@@ -39,18 +37,6 @@ namespace {
 constexpr int kNH = 78;  // packed upper 12x12
 constexpr int kHP = 3;   // entries of it per lane
 
-// Second-order dual number in the 12 coordinates x[0..11] of a pair (p0, p1,
-// q0, q1), spread over a warp: every lane has the value; lane l has the
-// second derivatives of the packed upper entries l, l + 32 and l + 64 (below
-// 78) and the first derivatives at their rows and columns, and lanes 0-11 the
-// first derivative of their own coordinate.  An operation touches 14 first
-// derivatives, 3 second ones and the value per lane instead of 12 + 78 + 1 by
-// one thread, whose numbers did not fit its registers (11 KB of local memory).
-struct HD {
-  double v, own;
-  double gi[kHP], gj[kHP], h[kHP];
-};
-
 // The lane's entries: coordinates (i, j) of each, and its own coordinate.
 struct HLane {
   int i[kHP], j[kHP], own;
@@ -69,80 +55,12 @@ struct HLane {
   }
 };
 
-__device__ __forceinline__ HD hd_const(double v) {
-  HD o;
-  o.v = v;
-  o.own = 0.0;
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) o.gi[k] = o.gj[k] = o.h[k] = 0.0;
-  return o;
-}
-
-__device__ __forceinline__ HD hd_mul(const HD &a, const HD &b) {
-  HD o;
-  o.v = a.v * b.v;
-  o.own = a.v * b.own + b.v * a.own;
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    o.gi[k] = a.v * b.gi[k] + b.v * a.gi[k];
-    o.gj[k] = a.v * b.gj[k] + b.v * a.gj[k];
-    o.h[k] = a.v * b.h[k] + b.v * a.h[k] + a.gi[k] * b.gj[k] + a.gj[k] * b.gi[k];
-  }
-  return o;
-}
-
-__device__ __forceinline__ HD hd_add(const HD &a, const HD &b) {
-  HD o;
-  o.v = a.v + b.v;
-  o.own = a.own + b.own;
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    o.gi[k] = a.gi[k] + b.gi[k];
-    o.gj[k] = a.gj[k] + b.gj[k];
-    o.h[k] = a.h[k] + b.h[k];
-  }
-  return o;
-}
-
-__device__ __forceinline__ HD hd_sub(const HD &a, const HD &b) {
-  HD o;
-  o.v = a.v - b.v;
-  o.own = a.own - b.own;
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    o.gi[k] = a.gi[k] - b.gi[k];
-    o.gj[k] = a.gj[k] - b.gj[k];
-    o.h[k] = a.h[k] - b.h[k];
-  }
-  return o;
-}
-
-// f(a) for a scalar function with f(a.v) = f0, f' = f1, f'' = f2
-__device__ __forceinline__ HD hd_apply(const HD &a, double f0, double f1, double f2) {
-  HD o;
-  o.v = f0;
-  o.own = f1 * a.own;
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    o.h[k] = f1 * a.h[k] + f2 * (a.gi[k] * a.gj[k]);
-    o.gi[k] = f1 * a.gi[k];
-    o.gj[k] = f1 * a.gj[k];
-  }
-  return o;
-}
-
-__device__ __forceinline__ HD hd_div(const HD &a, const HD &b) {
-  const double r = 1.0 / b.v;
-  return hd_mul(a, hd_apply(b, r, -r * r, 2.0 * r * r * r));
-}
-
 // First-order dual number in the 12 coordinates of a pair (value in every
 // lane, the derivative in coordinate l in lane l < 12), for the friction force
 // whose Jacobian is not a Hessian.
 struct D1 {
   double v, g;
 };
-__device__ __forceinline__ D1 d1_of(const HD &a) { return {a.v, a.own}; }
 __device__ __forceinline__ D1 d1_const(double v) { return {v, 0.0}; }
 __device__ __forceinline__ D1 operator+(const D1 &a, const D1 &b) { return {a.v + b.v, a.g + b.g}; }
 __device__ __forceinline__ D1 operator-(const D1 &a, const D1 &b) { return {a.v - b.v, a.g - b.g}; }
@@ -153,106 +71,86 @@ __device__ __forceinline__ D1 operator*(double c, const D1 &a) { return {c * a.v
 // f(a) with f(a.v) = f0, f'(a.v) = f1
 __device__ __forceinline__ D1 d1_apply(const D1 &a, double f0, double f1) { return {f0, f1 * a.g}; }
 
-// Coordinates of a pair: x[0..2] = p0, x[3..5] = p1, x[6..8] = q0,
-// x[9..11] = q1.  The vectors a = p1 - p0, b = q1 - q0, r = p0 - q0 are
-// linear in x: component c is +1 at variable P + c and -1 at N + c.
-struct Lin {
-  double v[3];
-  int P, N;
-  // derivative of component c in coordinate x
-  __device__ __forceinline__ double at(int x, int c) const {
-    return x == P + c ? 1.0 : x == N + c ? -1.0 : 0.0;
-  }
+// A pair's distance D and its derivatives, spread over a warp.  With f = D^2/2
+// as a function of the 12 coordinates x and of (s, t), d = sum_n w_n x_n, w =
+// (1 - s, s, t - 1, -t): at the closest points f's derivative in a free s or t
+// is zero, so D's gradient is f_x / D and its Hessian comes from f_xx + f_xz z_x
+// + (f_xz z_x)^T + z_x^T f_zz z_x, where z_x = (s_x, t_x) are the closest
+// points' own derivatives (zero for a clamped one).  Every lane has the values;
+// lanes 0-11 the derivatives of their own coordinate, which the lanes' second
+// derivatives fetch.  (Second-order dual numbers through the whole computation
+// took 1400 FP64 instructions a pair, 94 us a launch for 897 pairs.)
+struct Distance {
+  double D, s, t, d[3];
+  double sx, tx, Dx;  // of the lane's own coordinate
+  double dx[3];       // d's, likewise
+  double h[kHP], gi[kHP], gj[kHP];
 };
 
-__device__ __forceinline__ double lin_dot_grad(const Lin &u, const Lin &w, int x) {
-  double g = 0.0;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) g += u.at(x, c) * w.v[c] + w.at(x, c) * u.v[c];
-  return g;
-}
-
-// u . w for linear vectors
-__device__ __forceinline__ HD hd_lindot(const Lin &u, const Lin &w, const HLane &ln) {
-  HD o;
-  o.v = u.v[0] * w.v[0] + u.v[1] * w.v[1] + u.v[2] * w.v[2];
-  o.own = lin_dot_grad(u, w, ln.own);
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    const int x = ln.i[k], y = ln.j[k];
-    o.gi[k] = lin_dot_grad(u, w, x);
-    o.gj[k] = lin_dot_grad(u, w, y);
-    double h = 0.0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) h += u.at(x, c) * w.at(y, c) + u.at(y, c) * w.at(x, c);
-    o.h[k] = h;
-  }
-  return o;
-}
-
-// o += sign * s * L_c (scalar dual times component c of a linear vector)
-__device__ __forceinline__ void hd_add_scaled_lin(const HD &s, const Lin &L, int c, double sign, const HLane &ln,
-                                                  HD &o) {
-  const double lv = sign * L.v[c], sv = sign * s.v;
-  o.v += s.v * lv;
-  o.own += lv * s.own + sv * L.at(ln.own, c);
-#pragma unroll
-  for (int k = 0; k < kHP; ++k) {
-    const double li = L.at(ln.i[k], c), lj = L.at(ln.j[k], c);
-    o.gi[k] += lv * s.gi[k] + sv * li;
-    o.gj[k] += lv * s.gj[k] + sv * lj;
-    o.h[k] += lv * s.h[k] + sign * (lj * s.gi[k] + li * s.gj[k]);
-  }
-}
-
-// clamp to [0, 1]: outside the interval the result is a constant
-__device__ __forceinline__ HD hd_clamp01(const HD &a) {
-  if (a.v < 0.0) return hd_const(0.0);
-  if (a.v > 1.0) return hd_const(1.0);
-  return a;
-}
-
-// Segment distance with its derivatives, by the same closest-point rule
-// as the definition it follows: s from the unconstrained minimiser clamped
-// to [0, 1] (s = 0 for near-parallel segments), t for that s clamped, then s
-// again for the clamped t, clamped.
-__device__ __forceinline__ HD segment_distance_hd(const double *x, const HLane &ln, HD &s, HD &t, HD (&d)[3]) {
-  Lin a, b, r;
+// By the same closest-point rule as the plain distance below: s from the
+// unconstrained minimiser clamped to [0, 1] (s = 0 for near-parallel
+// segments), t for that s clamped, then s again for the clamped t, clamped.
+__device__ __forceinline__ Distance pair_distance(const double *x, const HLane &ln) {
+  constexpr unsigned full = 0xffffffffu;
+  Distance q;
+  double a[3], b[3], r[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    a.v[c] = x[3 + c] - x[c];
-    b.v[c] = x[9 + c] - x[6 + c];
-    r.v[c] = x[c] - x[6 + c];
+    a[c] = x[3 + c] - x[c];
+    b[c] = x[9 + c] - x[6 + c];
+    r[c] = x[c] - x[6 + c];
   }
-  a.P = 3; a.N = 0;
-  b.P = 9; b.N = 6;
-  r.P = 0; r.N = 6;
-  const HD A = hd_lindot(a, a, ln), B = hd_lindot(a, b, ln), Cc = hd_lindot(b, b, ln);
-  const HD Dd = hd_lindot(a, r, ln), Ee = hd_lindot(b, r, ln);
-  const HD den = hd_sub(hd_mul(A, Cc), hd_mul(B, B));
-  if (den.v < 1e-12 * A.v * Cc.v) {
-    s = hd_const(0.0);
-  } else {
-    s = hd_clamp01(hd_div(hd_sub(hd_mul(B, Ee), hd_mul(Cc, Dd)), den));
-  }
-  t = hd_clamp01(hd_div(hd_add(hd_mul(B, s), Ee), Cc));
-  s = hd_clamp01(hd_div(hd_sub(hd_mul(B, t), Dd), A));
-  // d = r + s a - t b; D = |d|
+  const auto dot3 = [](const double *u, const double *v) { return fma(u[0], v[0], fma(u[1], v[1], u[2] * v[2])); };
+  const double A = dot3(a, a), B = dot3(a, b), C = dot3(b, b), Dd = dot3(a, r), Ee = dot3(b, r);
+  const double den = A * C - B * B, iA = rcp_any(A), iC = rcp_any(C), iden = rcp_any(den);
+  const bool parallel = den < 1e-12 * A * C;
+  const double s0 = parallel ? 0.0 : (B * Ee - C * Dd) * iden;
+  const double s1 = fmin(fmax(s0, 0.0), 1.0);
+  const double t0 = fma(B, s1, Ee) * iC;
+  q.t = fmin(fmax(t0, 0.0), 1.0);
+  const double s2 = fma(B, q.t, -Dd) * iA;
+  q.s = fmin(fmax(s2, 0.0), 1.0);
+  const bool joint = !parallel && s0 == s1, tfree = t0 == q.t, sfree = s2 == q.s;
+  double d1[3];  // d at (s1, t)
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    d[c] = hd_const(r.v[c]);
-    d[c].own = r.at(ln.own, c);
-#pragma unroll
-    for (int k = 0; k < kHP; ++k) {
-      d[c].gi[k] = r.at(ln.i[k], c);
-      d[c].gj[k] = r.at(ln.j[k], c);
-    }
-    hd_add_scaled_lin(s, a, c, 1.0, ln, d[c]);
-    hd_add_scaled_lin(t, b, c, -1.0, ln, d[c]);
+    const double rt = fma(-q.t, b[c], r[c]);
+    q.d[c] = fma(q.s, a[c], rt);
+    d1[c] = fma(s1, a[c], rt);
   }
-  const HD u = hd_add(hd_add(hd_mul(d[0], d[0]), hd_mul(d[1], d[1])), hd_mul(d[2], d[2]));
-  const double sq = sqrt(u.v);
-  return hd_apply(u, sq, 0.5 / sq, -0.25 / (sq * u.v));
+  const double u = dot3(q.d, q.d);
+  q.D = sqrt_any(u);
+  const double iD = rcp_any(q.D);
+  // the lane's own coordinate: node m, component c
+  const int m = ln.own / 3, c = ln.own - 3 * m;
+  const auto pick = [&](const double *v) { return c == 0 ? v[0] : c == 1 ? v[1] : v[2]; };
+  const double ac = pick(a), bc = pick(b), dc = pick(q.d);
+  const double w = m == 0 ? 1.0 - q.s : m == 1 ? q.s : m == 2 ? q.t - 1.0 : -q.t;
+  const double w1 = m == 0 ? 1.0 - s1 : m == 1 ? s1 : w;
+  const double ms = m == 0 ? -1.0 : m == 1 ? 1.0 : 0.0, mt = m == 2 ? 1.0 : m == 3 ? -1.0 : 0.0;
+  const double fs = fma(w, ac, ms * dc), ft = fma(-w, bc, mt * dc);
+  q.tx = !tfree ? 0.0 : joint ? -fma(B, fs, A * ft) * iden : fma(w1, bc, -mt * pick(d1)) * iC;
+  q.sx = !sfree ? 0.0 : fma(B, q.tx, -fs) * iA;
+  // (the last term vanishes but for near-parallel segments, where t is the
+  // closest point of s = 0)
+  q.Dx = iD * fma(-dot3(q.d, b), q.tx, w * dc);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) q.dx[e] = fma(a[e], q.sx, fma(-b[e], q.tx, e == c ? w : 0.0));
+  const double ps = fma(0.5, fma(A, q.sx, -B * q.tx), fs), pt = fma(0.5, fma(C, q.tx, -B * q.sx), ft);
+#pragma unroll
+  for (int k = 0; k < kHP; ++k) {
+    const int i = ln.i[k], j = ln.j[k];
+    const double wi = __shfl_sync(full, w, i), wj = __shfl_sync(full, w, j);
+    double h = i % 3 == j % 3 ? wi * wj : 0.0;
+    h = fma(__shfl_sync(full, ps, i), __shfl_sync(full, q.sx, j), h);
+    h = fma(__shfl_sync(full, pt, i), __shfl_sync(full, q.tx, j), h);
+    h = fma(__shfl_sync(full, q.sx, i), __shfl_sync(full, ps, j), h);
+    h = fma(__shfl_sync(full, q.tx, i), __shfl_sync(full, pt, j), h);
+    q.gi[k] = __shfl_sync(full, q.Dx, i);
+    q.gj[k] = __shfl_sync(full, q.Dx, j);
+    q.h[k] = iD * fma(-q.gi[k], q.gj[k], h);
+  }
+  return q;
 }
 
 // Plain segment distance (same rule), for the candidate filter.
@@ -469,21 +367,20 @@ __global__ void __launch_bounds__(64) k_cc_terms(ContactArgs a) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) x[3 * n + k] = a.q[nodes[n] + k];
     auto dof = [&](int i) { return (i < 6 ? (i < 3 ? nodes[0] : nodes[1]) : (i < 9 ? nodes[2] : nodes[3])) + i % 3; };
-    HD st, tt, d[3];
-    const HD D = segment_distance_hd(x, ln, st, tt, d);
+    const Distance q = pair_distance(x, ln);
     const double C = a.edge_h[e] + a.edge_h[f];
     double e0, e1, e2;
-    imc(D.v, C, a.delta, e0, e1, e2);
+    imc(q.D, C, a.delta, e0, e1, e2);
     const double kc = a.kc;
     const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
     double *M = a.dense + a.sys_dense0[s];
     const bool mine = lane < 12 && !a.fixed[dof(ln.own)];
-    if (mine) atomicAdd(a.fc + dof(ln.own), -kc * e1 * D.own);  // F = -dE/dq (Eq. 11)
+    if (mine) atomicAdd(a.fc + dof(ln.own), -kc * e1 * q.Dx);  // F = -dE/dq (Eq. 11)
 #pragma unroll
     for (int k = 0; k < kHP; ++k) {
       const int di = dof(ln.i[k]), dj = dof(ln.j[k]);
       if (!ln.on[k] || a.fixed[di] || a.fixed[dj]) continue;
-      const double hv = kc * (e1 * D.h[k] + e2 * D.gi[k] * D.gj[k]);
+      const double hv = kc * (e1 * q.h[k] + e2 * q.gi[k] * q.gj[k]);
       const int r = di - d0, c = dj - d0;
       atomicAdd(M + (size_t)r * n + c, hv);
       if (r != c) atomicAdd(M + (size_t)c * n + r, hv);
@@ -496,13 +393,13 @@ __global__ void __launch_bounds__(64) k_cc_terms(ContactArgs a) {
     // edge b, spread by the closest-point weights; |F_con| = k_c |dE/dD|.
     // Derivatives by first-order dual numbers; at |u| = 0 the limit
     // gamma/|u| -> K2/2 of the smooth law.
-    const D1 sD = d1_of(st), tD = d1_of(tt), Dd = d1_of(D), one = d1_const(1.0);
+    const D1 sD = {q.s, q.sx}, tD = {q.t, q.tx}, Dd = {q.D, q.Dx}, one = d1_const(1.0);
     const D1 iD = d1_apply(Dd, 1.0 / Dd.v, -1.0 / (Dd.v * Dd.v));
     const double idt = 1.0 / a.dt;
     D1 nrm[3], ur[3], u[3], Fa[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      nrm[c] = d1_of(d[c]) * iD;
+      nrm[c] = D1{q.d[c], q.dx[c]} * iD;
       D1 v[4];
 #pragma unroll
       for (int m = 0; m < 4; ++m)
@@ -697,7 +594,8 @@ __global__ void __launch_bounds__(1024) k_lu_order(ContactArgs a) {
   if (!a.cgo[c]) return;
   const int s = a.contact_sys[c], n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, W = (nt + 31) / 32;
   extern __shared__ unsigned row[];
-  __shared__ unsigned rem[kMaxTiles / 32], best[2][kFronts];
+  __shared__ unsigned rem[kMaxTiles / 32], best[2][kFronts][32];
+  __shared__ int levels;
   int32_t *lev = a.lu_level + (size_t)c * a.max_tiles * kLevelInts;
   uint8_t *nz = a.nz + a.sys_nz0[s];
   uint16_t *adj = a.lu_adj + a.sys_nz0[s];
@@ -710,65 +608,70 @@ __global__ void __launch_bounds__(1024) k_lu_order(ContactArgs a) {
   }
   if (i < W) rem[i] = i == W - 1 && (nt & 31) ? (1u << (nt & 31)) - 1u : 0xffffffffu;
   if (i == 0) a.lu_bar[c] = 0;
-  if (i < 2 * kFronts) best[i / kFronts][i % kFronts] = 0xffffffffu;
   __syncthreads();
-  const auto bit = [&](int p) { return i < nt && ((row[(p >> 5) * nt + i] >> (p & 31)) & 1u); };  // i ~ p
   int l = 0;
-  for (;; ++l) {
-    // fewest remaining neighbours, then farthest from the middle, then first
-    unsigned key = 0xffffffffu;
-    const bool alive = i < nt && ((rem[i >> 5] >> lane) & 1u);
-    if (alive) {
-      unsigned deg = 0;
-      for (int w = 0; w < W; ++w) deg += __popc(row[w * nt + i] & rem[w]);
-      key = (deg << 21) | ((unsigned)(1024 - abs(2 * i - (nt - 1))) << 10) | (unsigned)i;
-    }
-    int nf = 0, pick[kFronts];
-    unsigned lim = 0;
-#pragma unroll
-    for (int f = 0; f < kFronts; ++f) {
-      if (nf < f) break;
-      const unsigned v = __reduce_min_sync(0xffffffffu, key);
-      if (lane == 0) atomicMin(&best[l & 1][f], v);
-      __syncthreads();
-      const unsigned b = best[l & 1][f];
-      if (f == 0) lim = (b >> 21) + kDegreeSlack;
-      if (b == 0xffffffffu || (b >> 21) > lim) break;
-      pick[f] = (int)(b & 1023u);
-      nf = f + 1;
-      if (i == pick[f] || bit(pick[f])) key = 0xffffffffu;
-    }
-    if (nf == 0) break;
-    __syncthreads();  // (best of this level read, rem read)
-#pragma unroll
-    for (int f = 0; f < kFronts; ++f)
-      if (f < nf && i == pick[f]) atomicAnd(&rem[i >> 5], ~(1u << lane));
-    if (i < kFronts) best[l & 1][i] = 0xffffffffu;  // (next used two levels on)
-    __syncthreads();
-#pragma unroll
-    for (int f = 0; f < kFronts; ++f) {
-      if (f >= nf) break;
-      const int p = pick[f];
-      if (i == 32 * f % (int)blockDim.x) {  // (a thread of another warp for each)
-        int m = 0;
-        for (int w = 0; w < W; ++w) m += __popc(row[w * nt + p] & rem[w]);
-        lev[l * kLevelInts + 1 + f] = p;
-        lev[l * kLevelInts + 1 + kFronts + f] = m;
+  if (i < 32 * W) {  // (the other warps wait at the end)
+    const auto meet = [&] { asm volatile("bar.sync 1, %0;" ::"r"(32 * W) : "memory"); };
+    const auto bit = [&](int p) { return i < nt && ((row[(p >> 5) * nt + i] >> (p & 31)) & 1u); };  // i ~ p
+    for (;; ++l) {
+      // fewest remaining neighbours, then farthest from the middle, then first
+      unsigned key = 0xffffffffu;
+      const bool alive = i < nt && ((rem[i >> 5] >> lane) & 1u);
+      if (alive) {
+        unsigned deg = 0;
+        for (int w = 0; w < W; ++w) deg += __popc(row[w * nt + i] & rem[w]);
+        key = (deg << 21) | ((unsigned)(1024 - abs(2 * i - (nt - 1))) << 10) | (unsigned)i;
       }
-      if (alive && bit(p) && ((rem[i >> 5] >> lane) & 1u)) {
-        int rank = 0;
-        for (int w = 0; w < W; ++w) {
-          const unsigned x = row[w * nt + p] & rem[w];
-          if (w < i >> 5) rank += __popc(x);
-          if (w == i >> 5) rank += __popc(x & ((1u << lane) - 1u));
-          row[w * nt + i] |= w == i >> 5 ? x & ~(1u << lane) : x;  // fill (own row only)
+      int nf = 0, pick[kFronts];
+      unsigned lim = 0;
+#pragma unroll
+      for (int f = 0; f < kFronts; ++f) {
+        if (nf < f) break;
+        unsigned b = __reduce_min_sync(0xffffffffu, key);
+        if (lane == 0) best[l & 1][f][i >> 5] = b;
+        meet();
+        for (int w = 0; w < W; ++w) b = min(b, best[l & 1][f][w]);
+        if (f == 0) lim = (b >> 21) + kDegreeSlack;
+        if (b == 0xffffffffu || (b >> 21) > lim) break;
+        pick[f] = (int)(b & 1023u);
+        nf = f + 1;
+        if (i == pick[f] || bit(pick[f])) key = 0xffffffffu;
+      }
+      if (nf == 0) break;
+      meet();  // (rem read)
+#pragma unroll
+      for (int f = 0; f < kFronts; ++f)
+        if (f < nf && i == pick[f]) atomicAnd(&rem[i >> 5], ~(1u << lane));
+      meet();
+      const bool left = alive && ((rem[i >> 5] >> lane) & 1u);
+#pragma unroll
+      for (int f = 0; f < kFronts; ++f) {
+        if (f >= nf) break;
+        const int p = pick[f];
+        if (i == p) {
+          int m = 0;
+          for (int w = 0; w < W; ++w) m += __popc(row[w * nt + p] & rem[w]);
+          lev[l * kLevelInts + 1 + f] = p;
+          lev[l * kLevelInts + 1 + kFronts + f] = m;
         }
-        adj[(size_t)p * nt + rank] = (uint16_t)i;
+        if (left && bit(p)) {
+          int rank = 0;
+          for (int w = 0; w < W; ++w) {
+            const unsigned x = row[w * nt + p] & rem[w];
+            if (w < i >> 5) rank += __popc(x);
+            if (w == i >> 5) rank += __popc(x & ((1u << lane) - 1u));
+            row[w * nt + i] |= w == i >> 5 ? x & ~(1u << lane) : x;  // fill (own row only)
+          }
+          adj[(size_t)p * nt + rank] = (uint16_t)i;
+        }
       }
+      if (i == 0) lev[l * kLevelInts] = nf;
+      meet();
     }
-    if (i == 0) lev[l * kLevelInts] = nf;
-    __syncthreads();
   }
+  if (i == 0) levels = l;
+  __syncthreads();
+  l = levels;
   if (i == 0) lev[kLevelInts - 1] = l;
   for (int x = l + i; x < a.max_tiles; x += blockDim.x) lev[x * kLevelInts] = 0;
   for (int e = i >> 5; e < nt * W; e += blockDim.x >> 5) {
@@ -1137,7 +1040,7 @@ __global__ void __launch_bounds__(32 * kSubstWarps) k_cc_subst(ContactArgs a, So
 cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStream_t st) {
   const int nt = a.max_tiles, nc = a.n_contact;
   if (nc == 0) return cudaSuccess;
-  const int words = nt * ((nt + 31) / 32), threads = std::max(256, (nt + 31) / 32 * 32);
+  const int words = nt * ((nt + 31) / 32), threads = std::max(512, (nt + 31) / 32 * 32);
   k_lu_order<<<nc, threads, 4 * words, st>>>(a);
   // the chip shared among the systems; several blocks of a system wait for one
   // another, so all of them must be resident (two per SM fit)
