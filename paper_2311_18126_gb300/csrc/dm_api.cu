@@ -752,6 +752,9 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
   EdgeArgs ea{ne, d.q, d.edge_a, d.edge_b, d.edge_th, d.edge_sys, d.edge_EA, d.edge_ilbar,
               d.tn, d.d1n, d.sys_active, d.sys_status, d.ef, d.es,
               s->x.prof ? s->x.d_units + K_EDGE : nullptr};
+  ea.sys_res = d.sys_res;
+  ea.ctrl = d.ctrl;
+  ea.nsys = S;
   StencilArgs ka{ns, ne, d.q, d.ef, d.tn, d.st_ed, d.st_th, d.st_sg, d.st_sys, d.st_kb, d.st_kt,
                  d.kbar, d.taubar, d.beta_n, d.sys_active, d.sys_status, d.beta_it, d.sg, d.sh,
                  s->x.prof ? s->x.d_units + K_STENCIL : nullptr};
@@ -858,11 +861,11 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     stats->max_iterations = 0;
   }
   std::vector<int32_t> iters;
-  // residual and Jacobian passes apart, except with rod networks; the first
-  // round of a step, whose guess essentially never meets the tolerance, runs
-  // the fused passes (without a learned guess, whose trial round may be
-  // rejected)
-  const bool split = !gen_on;
+  // residual and Jacobian passes apart, except with rod networks without line
+  // search (below); the first round of a step, whose guess essentially never
+  // meets the tolerance, runs the fused passes (without a learned guess, whose
+  // trial round may be rejected)
+  const bool split = !gen_on || ls_on;
   const bool fuse_first = split && !ws_on && s->x.fused_first;
   // the node terms run beside the edge and stencil kernels (not while
   // profiling, whose events time each kernel alone)
@@ -875,10 +878,6 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
   // One Newton round: every phase's launches, in stream order on rs.
   auto round = [&](cudaStream_t rs, int it, bool first) -> dm_status {
     const bool sp = split && !first;
-    k_reset_res<<<blocks(S, 256), 256, 0, rs>>>(0, S, d.sys_active, d.sys_res);
-    s->x.launches[K_BEGIN]++;
-    DM_CK(cudaMemsetAsync(d.ctrl, 0, sizeof(int32_t), rs));
-    DM_CK(cudaMemsetAsync(d.ctrl + 3, 0, sizeof(int32_t), rs));
     if (fork_nodes) {
       DM_CK(cudaEventRecord(s->x.ev_fork, rs));
       DM_CK(cudaStreamWaitEvent(s->x.side_stream, s->x.ev_fork, 0));
@@ -897,9 +896,11 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     }
     // residual pass: reference twist and gradients, then the residual rows;
     // the Jacobian pass (stencil Hessians, band rows) below runs only for
-    // systems whose residual is still above the tolerance.  Batches with rod
-    // networks keep one fused pass: most of their many rounds carry systems
-    // that iterate on, for which the split would only add work.
+    // systems whose residual is still above the tolerance and that the line
+    // search does not pull back.  Rod networks without line search keep one
+    // fused pass: most of their rounds carry systems that iterate on, for which
+    // the split would only add work.  With line search most rounds only pull
+    // back (64 robots: a round's stencil pass 24.5 us fused, 12.7 us split).
     const int st_tb = s->x.tune.stencil_threads;
     const int st_grid = blocks(ns, (int64_t)st_tb * s->x.tune.stencil_per_thread);
     if (ns > 0 && sp) {
@@ -1132,6 +1133,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       k_midpoint_finish<<<blocks(std::max(nd, S), 256), 256, 0, st>>>(sa, d.dq);
       EdgeArgs ef_args = ea;
       ef_args.units = nullptr;
+      ef_args.sys_res = nullptr;
       k_edge<<<blocks(ne, 256), 256, 0, st>>>(ef_args);
       if (ns > 0) {
         StencilArgs kf = ka;

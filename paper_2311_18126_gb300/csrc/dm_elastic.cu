@@ -93,6 +93,12 @@ __device__ __forceinline__ void k_edge_one(EdgeArgs a, const int e) {
 }
 
 __global__ void k_edge(EdgeArgs a) {
+  if (a.sys_res) {  // (a system that has stopped keeps its residual)
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int s = t; s < a.nsys; s += gridDim.x * blockDim.x)
+      if (a.sys_active[s]) a.sys_res[s] = 0ull;
+    if (t == 0) a.ctrl[0] = a.ctrl[3] = 0;
+  }
   // block-uniform grid-stride loop (count_units synchronises the block)
   for (int b0 = blockIdx.x * blockDim.x; b0 < a.ne; b0 += gridDim.x * blockDim.x)
     k_edge_one(a, b0 + threadIdx.x);

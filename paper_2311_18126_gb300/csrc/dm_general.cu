@@ -88,17 +88,17 @@ __global__ void k_nodes(NodeArgs a) {
 // Row i's force balance; the scaled residual's bits.
 __device__ __forceinline__ unsigned long long rows_gen_one(const RowGenArgs &a, int i) {
   count_active(a.units);
-  // eight terms at a time, loaded side by side (a joint node has dozens) and
+  // sixteen terms at a time, loaded side by side (a joint node has dozens) and
   // summed in order
   double F = 0.0;
   const int k1 = a.gat_ptr[i + 1];
-  for (int k = a.gat_ptr[i]; k < k1; k += 8) {
-    int code[8];
-    double x[8];
+  for (int k = a.gat_ptr[i]; k < k1; k += 16) {
+    int code[16];
+    double x[16];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) code[u] = k + u < k1 ? a.gat_ent[k + u] : -1;
+    for (int u = 0; u < 16; ++u) code[u] = k + u < k1 ? a.gat_ent[k + u] : -1;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 16; ++u) {
       const int slot = code[u] & 15, idx = code[u] >> 5;
       x[u] = 0.0;
       if (code[u] < 0) continue;
@@ -110,7 +110,7 @@ __device__ __forceinline__ unsigned long long rows_gen_one(const RowGenArgs &a, 
       }
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 16; ++u)
       if (k + u < k1) F += x[u];
   }
   const int c = a.dof_comp[i];

@@ -13,6 +13,11 @@ struct EdgeArgs {
   int32_t *sys_status;
   double *ef, *es;
   unsigned long long *units;
+  // first kernel of a Newton round (else NULL): clears the residuals of the
+  // systems still iterating and the round's counters
+  unsigned long long *sys_res;
+  int32_t *ctrl;
+  int nsys;
 };
 
 struct StencilArgs {
@@ -436,8 +441,6 @@ __global__ void k_commit(StepArgs a);
 __global__ void k_restore(StepArgs a);
 __global__ void k_round_continue(int32_t *ctrl, int max_rounds, cudaGraphConditionalHandle h);
 __global__ void k_round_count(int32_t *ctrl);
-__global__ void k_reset_res(int lo, int hi, const int32_t *sys_active,
-                            unsigned long long *sys_res);
 
 __global__ void k_midpoint_finish(StepArgs a, double *vnew);
 // Newton round of the long rods: bookkeeping, partitioned solve, q += dq.

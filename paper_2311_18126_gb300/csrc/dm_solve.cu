@@ -184,7 +184,20 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (s >= a.nsys || !a.sys_active[s]) return;  // block-uniform
   const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
+  // the decision's inputs and the move's first DOFs on the way while the merit
+  // is summed
+  constexpr int U = 8;
+  const int trial = a.trial[s], nback = a.nback[s], wstry = a.wstry ? a.wstry[s] : 0;
+  const double alpha0 = a.alpha[s], racc = a.racc[s];
+  double qv[U], qa[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = tid + u * kLineSearchThreads;
+    qv[u] = i < n ? a.q[d0 + i] : 0.0;
+    qa[u] = i < n ? a.qacc[d0 + i] : 0.0;
+  }
   double acc = 0.0;
+#pragma unroll 4
   for (int i = tid; i < n; i += kLineSearchThreads) {
     const double v = a.f[d0 + i] * a.rscale[d0 + i];
     acc = fma(v, v, acc);
@@ -202,11 +215,11 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
     int action = 0;
     double alpha = 1.0;
     bool done = false;
-    if (a.wstry && a.wstry[s]) {
+    if (wstry) {
       // the learned guess is kept only if it lowers the merit below that of
       // the extrapolation; otherwise the iterate returns to the extrapolation
       a.wstry[s] = 0;
-      if (!(m <= (1.0 - 1e-4) * a.racc[s])) {
+      if (!(m <= (1.0 - 1e-4) * racc)) {
         action = 1;
         alpha = 0.0;
         a.trial[s] = 0;
@@ -215,10 +228,10 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
       }
     }
     if (!done) {
-      if (a.trial[s] && a.nback[s] < 12 && !(m <= (1.0 - 1e-4 * a.alpha[s]) * a.racc[s])) {
+      if (trial && nback < 12 && !(m <= (1.0 - 1e-4 * alpha0) * racc)) {
         action = 1;
-        alpha = 0.5 * a.alpha[s];
-        a.nback[s] += 1;
+        alpha = 0.5 * alpha0;
+        a.nback[s] = nback + 1;
       } else {
         a.trial[s] = 0;
         a.nback[s] = 0;
@@ -233,7 +246,14 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   __syncthreads();
   const int action = s_action;
   const double alpha = s_alpha;
-  for (int i = d0 + tid; i < d0 + n; i += kLineSearchThreads) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = tid + u * kLineSearchThreads;
+    if (i >= n) break;
+    if (action == 1) a.q[d0 + i] = alpha == 0.0 ? qa[u] : 0.5 * (qv[u] + qa[u]);
+    else a.qacc[d0 + i] = qv[u];
+  }
+  for (int i = d0 + tid + U * kLineSearchThreads; i < d0 + n; i += kLineSearchThreads) {
     if (action == 1) a.q[i] = alpha == 0.0 ? a.qacc[i] : 0.5 * (a.q[i] + a.qacc[i]);
     else a.qacc[i] = a.q[i];
   }

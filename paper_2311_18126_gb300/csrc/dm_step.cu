@@ -211,15 +211,6 @@ __global__ void k_round_count(int32_t *ctrl) {
   if (threadIdx.x == 0 && blockIdx.x == 0) ++ctrl[4];
 }
 
-// Clears the residual slots of the systems [lo, hi) still iterating before a
-// round's row kernels max-reduce into them; a system that has stopped keeps
-// the residual of its last evaluated iterate (the value dm_step reports).
-__global__ void k_reset_res(int lo, int hi, const int32_t *sys_active,
-                            unsigned long long *sys_res) {
-  const int s = lo + blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < hi && sys_active[s]) sys_res[s] = 0ull;
-}
-
 // Committed tangents recomputed from q (after a state is set).
 __global__ void k_tangents(int ne, const int32_t *edge_a, const int32_t *edge_b,
                            const double *q, double *tn, int32_t *bad) {
