@@ -125,6 +125,8 @@ struct Extra {
   int32_t *d_bad = nullptr;
   int32_t *d_sys_kind = nullptr;
   int32_t *ls_action = nullptr, *ls_trial = nullptr, *ls_nback = nullptr;
+  // edges, nodes and stencils by system (line search of general systems)
+  int32_t *by_sys[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   double *ls_alpha = nullptr, *ls_racc = nullptr, *ls_qacc = nullptr, *ls_merit = nullptr;
   int n_rod_sys = 0;
   int max_rod_nodes = 0;  // of the single rods (the length projection's block)
@@ -453,6 +455,18 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     DM_TRY(dalloc(s, &s->x.ls_racc, S));
     DM_TRY(dalloc(s, &s->x.ls_merit, S));
     DM_TRY(dalloc(s, &s->x.ls_qacc, nd));
+    if (T.any_general) {
+      const std::vector<int32_t> *of[3] = {&T.edge_sys, &T.node_sys, &T.st_sys};
+      for (int k = 0; k < 3; ++k) {
+        std::vector<int32_t> ptr(S + 1, 0), list(of[k]->size());
+        for (int32_t x : *of[k]) ++ptr[x + 1];
+        for (int x = 0; x < S; ++x) ptr[x + 1] += ptr[x];
+        std::vector<int32_t> at(ptr.begin(), ptr.end() - 1);
+        for (size_t e = 0; e < list.size(); ++e) list[at[(*of[k])[e]]++] = (int32_t)e;
+        DM_TRY(upload(s, &s->x.by_sys[2 * k], ptr));
+        DM_TRY(upload(s, &s->x.by_sys[2 * k + 1], list));
+      }
+    }
   }
   // general path
   DM_TRY(upload(s, &d.dof_node, T.dof_node));
@@ -875,6 +889,12 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     DM_CK(cudaEventCreateWithFlags(&s->x.ev_fork, cudaEventDisableTiming));
     DM_CK(cudaEventCreateWithFlags(&s->x.ev_join, cudaEventDisableTiming));
   }
+  LineLoopArgs lb{};
+  lb.edges = ea; lb.stencils = ka; lb.nodes = na; lb.rows = rg;
+  lb.edges.units = lb.stencils.units = lb.nodes.units = lb.rows.units = nullptr;
+  lb.edge_ptr = s->x.by_sys[0]; lb.edge_list = s->x.by_sys[1];
+  lb.node_ptr = s->x.by_sys[2]; lb.node_list = s->x.by_sys[3];
+  lb.st_ptr = s->x.by_sys[4]; lb.st_list = s->x.by_sys[5];
   // One Newton round: every phase's launches, in stream order on rs.
   auto round = [&](cudaStream_t rs, int it, bool first) -> dm_status {
     const bool sp = split && !first;
@@ -944,7 +964,8 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       k_rows_gen<<<blocks(nd, 256), 256, 0, rs>>>(rg);
     }
     if (ls_on) {
-      k_line_search<<<S, kLineSearchThreads, 0, rs>>>(la);
+      if (gen_on) k_line_search_loop<<<S * kLoopBlocks, kLineSearchThreads, 0, rs>>>(la, lb);
+      else k_line_search<<<S, kLineSearchThreads, 0, rs>>>(la);
       if (ws_trial && it == 0) DM_CK(ws_inject(s, rs, s->x.ls_action, s->x.ls_trial));
     }
     if (sp && ns > 0) {

@@ -24,8 +24,11 @@
 // stencil, from the kernels' times: gradient 295 -> 195, Hessian 1060 -> 570,
 // both in one pass 1000 -> 525.  4096 rods (450046 stencils): fused pass 846 ->
 // 444 us, a step's Hessians 1.24 -> 0.67 ms and gradients 0.60 -> 0.39 ms.
+#include <cooperative_groups.h>
+
 #include "dm_internal.h"
 #include "dm_kernels.cuh"
+#include "dm_terms.cuh"
 
 namespace dm {
 
@@ -503,6 +506,93 @@ __global__ void __launch_bounds__(128) k_stencil_grad(StencilArgs a) {
 __global__ void __launch_bounds__(128) k_stencil_hess(StencilArgs a) {
   for (int b0 = blockIdx.x * blockDim.x; b0 < a.ns; b0 += gridDim.x * blockDim.x)
     k_stencil_one<2>(a, b0 + threadIdx.x);
+}
+
+// Line search of batches with general systems: a cluster of four blocks per
+// system.  The first decision is on the residual that the round's kernels left
+// (the same sums as k_line_search); a small system that is pulled back is then
+// evaluated here, again and again until it accepts -- edges and nodes, stencil
+// gradients, rows, merit -- instead of a round for every trial point (most
+// rounds of a batch of robots did nothing else: 75 us each for the chain of ten
+// launches, 64 robots).  Each block decides for itself on the same numbers.
+// Bound by the chain of a trial point's FP64 instructions (about 500 of 64
+// cycles).  Larger systems (over kLoopDofs) keep a round per trial point: the
+// whole chip's threads pay off there.
+constexpr int kLoopDofs = 4096;
+__global__ void __cluster_dims__(kLoopBlocks, 1, 1) __launch_bounds__(kLineSearchThreads)
+    k_line_search_loop(LineSearchArgs a, LineLoopArgs b) {
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  __shared__ double part[kLineSearchThreads / 32];
+  __shared__ unsigned long long most[kLineSearchThreads / 32];
+  const int rank = (int)cluster.block_rank(), s = blockIdx.x / kLoopBlocks;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int t0 = rank * kLineSearchThreads + tid;
+  constexpr int kT = kLoopBlocks * kLineSearchThreads;
+  if (!a.sys_active[s]) return;  // the whole cluster
+  const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
+  const bool small = b.rows.sys_kind[s] == SOLVE_GENERAL && n <= kLoopDofs;
+  LineState ls{a.trial[s], a.nback[s], a.wstry ? a.wstry[s] : 0, a.alpha[s], a.racc[s]};
+  const int e0 = b.edge_ptr[s], ne = b.edge_ptr[s + 1] - e0, v0 = b.node_ptr[s];
+  const int nv = b.rows.nt ? b.node_ptr[s + 1] - v0 : 0, k0 = b.st_ptr[s], nk = b.st_ptr[s + 1] - k0;
+  const int ne32 = (ne + 31) & ~31;
+  double m = 0.0;
+  unsigned long long res = 0;
+  int action = 0;
+  bool again = false;
+  for (;;) {
+    double acc = 0.0;
+    res = 0;
+#pragma unroll 4
+    for (int i = tid; i < n; i += kLineSearchThreads) {
+      const double v = a.f[d0 + i] * a.rscale[d0 + i];
+      acc = fma(v, v, acc);
+      res = max(res, (unsigned long long)__double_as_longlong(fabs(v)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      res = max(res, __shfl_xor_sync(0xffffffffu, res, o));
+    }
+    if (lane == 0) {
+      part[warp] = acc;
+      most[warp] = res;
+    }
+    __syncthreads();
+    double tot = 0.0;
+#pragma unroll
+    for (int w = 0; w < kLineSearchThreads / 32; ++w) {
+      tot += part[w];
+      res = max(res, most[w]);
+    }
+    m = sqrt(tot);
+    action = line_search_decide(m, ls);
+    for (int i = d0 + t0; i < d0 + n; i += kT) {
+      if (action == 1) a.q[i] = ls.alpha == 0.0 ? a.qacc[i] : 0.5 * (a.q[i] + a.qacc[i]);
+      else a.qacc[i] = a.q[i];
+    }
+    if (!action || !small) break;
+    again = true;
+    cluster.sync();
+    for (int i = t0; i < ne32 + nv; i += kT) {
+      if (i < ne) k_edge_one(b.edges, b.edge_list[e0 + i]);
+      else if (i >= ne32) node_one(b.nodes, b.node_list[v0 + i - ne32]);
+    }
+    cluster.sync();
+    for (int i = t0; i < nk; i += kT) k_stencil_one<1>(b.stencils, b.st_list[k0 + i]);
+    cluster.sync();
+    for (int i = t0; i < n; i += kT) rows_gen_one(b.rows, d0 + i);
+    cluster.sync();
+  }
+  if (rank == 0 && tid == 0) {
+    a.merit[s] = m;
+    if (a.wstry) a.wstry[s] = 0;
+    a.trial[s] = ls.trial;
+    a.nback[s] = ls.nback;
+    a.racc[s] = ls.racc;
+    a.action[s] = action;
+    a.alpha[s] = ls.alpha;
+    if (again) b.rows.sys_res[s] = res;
+  }
 }
 
 }  // namespace dm

@@ -310,6 +310,17 @@ struct LineSearchArgs {
   double *alpha, *racc, *merit, *q, *qacc;
   int32_t *wstry;  // NULL, or 1 while the trial is the learned initial guess
 };
+// The evaluation of a trial point inside the line search: the terms' arguments
+// and each system's edges, nodes and stencils.
+constexpr int kLoopBlocks = 4;  // blocks (a cluster) per system
+struct LineLoopArgs {
+  EdgeArgs edges;
+  StencilArgs stencils;
+  NodeArgs nodes;
+  RowGenArgs rows;
+  const int32_t *edge_ptr, *edge_list, *node_ptr, *node_list, *st_ptr, *st_list;
+};
+
 struct ContactArgs {
   int ne, nd, nsys, table_mask, pair_cap;
   double inv_cell, delta, kc;
@@ -387,6 +398,7 @@ __global__ void k_adj_midpoint_out(int nd, const uint8_t *fixed, const double *g
 
 constexpr int kLineSearchThreads = 128;
 __global__ void k_line_search(LineSearchArgs a);  // one block per system
+__global__ void k_line_search_loop(LineSearchArgs a, LineLoopArgs b);  // a cluster per system
 
 __global__ void k_nodes(NodeArgs a);
 __global__ void k_rows_gen(RowGenArgs a);

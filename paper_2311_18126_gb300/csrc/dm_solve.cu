@@ -11,6 +11,7 @@
 //  k_line_search -- one block per system: Armijo test and backtracking.
 #include "dm_internal.h"
 #include "dm_kernels.cuh"
+#include "dm_terms.cuh"
 
 namespace dm {
 
@@ -187,8 +188,7 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   // the decision's inputs and the move's first DOFs on the way while the merit
   // is summed
   constexpr int U = 8;
-  const int trial = a.trial[s], nback = a.nback[s], wstry = a.wstry ? a.wstry[s] : 0;
-  const double alpha0 = a.alpha[s], racc = a.racc[s];
+  LineState ls{a.trial[s], a.nback[s], a.wstry ? a.wstry[s] : 0, a.alpha[s], a.racc[s]};
   double qv[U], qa[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -212,36 +212,15 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
     for (int w = 0; w < kLineSearchThreads / 32; ++w) tot += part[w];
     const double m = sqrt(tot);
     a.merit[s] = m;
-    int action = 0;
-    double alpha = 1.0;
-    bool done = false;
-    if (wstry) {
-      // the learned guess is kept only if it lowers the merit below that of
-      // the extrapolation; otherwise the iterate returns to the extrapolation
-      a.wstry[s] = 0;
-      if (!(m <= (1.0 - 1e-4) * racc)) {
-        action = 1;
-        alpha = 0.0;
-        a.trial[s] = 0;
-        a.nback[s] = 0;
-        done = true;
-      }
-    }
-    if (!done) {
-      if (trial && nback < 12 && !(m <= (1.0 - 1e-4 * alpha0) * racc)) {
-        action = 1;
-        alpha = 0.5 * alpha0;
-        a.nback[s] = nback + 1;
-      } else {
-        a.trial[s] = 0;
-        a.nback[s] = 0;
-        a.racc[s] = m;
-      }
-    }
+    const int action = line_search_decide(m, ls);
+    if (a.wstry) a.wstry[s] = 0;
+    a.trial[s] = ls.trial;
+    a.nback[s] = ls.nback;
+    a.racc[s] = ls.racc;
     a.action[s] = action;
-    a.alpha[s] = alpha;
+    a.alpha[s] = ls.alpha;
     s_action = action;
-    s_alpha = alpha;
+    s_alpha = ls.alpha;
   }
   __syncthreads();
   const int action = s_action;

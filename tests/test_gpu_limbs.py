@@ -68,3 +68,52 @@ def _networks(lengths, ground):
 def test_limb_lengths_against_oracle(lengths, ground):
     desc, params = _networks(lengths, ground)
     _run(desc, params, 3, 1e-10)  # the Newton tolerance both sides step to
+
+
+def test_line_search_inside_and_across_rounds():
+    """Trial points of small general systems are evaluated inside the line
+    search, those of larger systems (over 4096 DOFs) and of single rods in
+    rounds of their own; both follow the oracle's backtracking."""
+    from oracle import OracleSystems
+    from paper_2311_18126_gb300 import System
+    desc, params, _ = workloads.star_robots(n_robots=2, seed=9, nodes_per_limb=7)
+    rng = np.random.default_rng(2)
+    big, N = 1100, 9  # 4399 DOFs
+    x = [np.asarray(desc["x0"])]
+    for n, y in ((big, 3.0), (N, 4.0)):
+        x.append(np.c_[0.004 * np.arange(n), np.full(n, y), np.full(n, desc["radius"][0])])
+    x0 = np.concatenate(x)
+    npr = list(desc["nodes_per_rod"]) + [big, N]
+    R = len(npr)
+    ext = lambda k: np.concatenate([np.asarray(desc[k], float), [desc[k][0]] * 2])
+    v0 = np.zeros_like(x0)
+    v0[-(big + N):, 2] = np.repeat(0.3 * rng.normal(size=(big + N + 4) // 4), 4)[:big + N]  # rough: trial points fail
+    d = dict(nodes_per_rod=npr, x0=x0, v0=v0, joints=desc["joints"],
+             fixed=np.zeros(int(sum(4 * n - 1 for n in npr)), np.uint8),
+             **{k: ext(k) for k in ("E", "nu", "rho", "radius", "ground_mu", "ground_kc")})
+    p = dict(params, line_search=True)
+    s = System(d, p)
+    s.step(1)
+    together = np.array(s.get_state()[0])
+    s.close()
+    # the large rod alone, its trial points in rounds, against the whole batch,
+    # where the same kernels ran beside the robots' loop
+    off = np.concatenate([[0], np.cumsum([4 * n - 1 for n in npr])])
+    small = [r for r in range(R) if npr[r] != big]
+    keep = np.concatenate([np.arange(off[r], off[r + 1]) for r in small])
+    nodes = np.concatenate([[0], np.cumsum(npr)])
+    kn = np.concatenate([np.arange(nodes[r], nodes[r + 1]) for r in small])
+    ds = dict(d, nodes_per_rod=[npr[r] for r in small], x0=x0[kn], v0=v0[kn], fixed=d["fixed"][keep],
+              **{k: d[k][small] for k in ("E", "nu", "rho", "radius", "ground_mu", "ground_kc")})
+    ora = OracleSystems(ds, p)
+    st = ora.step(1)
+    assert all(t[0] == 0 for t in st), st
+    qo = np.asarray(ora.get_state()[0])
+    assert np.abs(together[keep] - qo).max() < 1e-10 * 4.0  # the Newton tolerance, at 4 m
+    dl = dict(d, nodes_per_rod=[big], x0=x0[nodes[-3]:nodes[-2]], v0=v0[nodes[-3]:nodes[-2]], joints=[],
+              fixed=d["fixed"][off[-3]:off[-2]],
+              **{k: d[k][-2:-1] for k in ("E", "nu", "rho", "radius", "ground_mu", "ground_kc")})
+    s = System(dl, p)
+    s.step(1)
+    assert np.array_equal(np.array(s.get_state()[0]), together[off[-3]:off[-2]])
+    s.close()
