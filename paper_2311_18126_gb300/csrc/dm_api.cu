@@ -823,6 +823,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
   NodeArgs na{nn, s->p.dt, s->prm.ground_z, s->prm.delta, s->prm.slip_nu, d.q, d.qn,
               d.node_dof_arr, d.node_sys, d.node_h, d.node_mu, d.node_kc, d.sys_active, d.nt,
               s->x.prof ? s->x.d_units + K_NODES : nullptr};
+  na.constants();
   RowGenArgs rg{};
   rg.units = s->x.prof ? s->x.d_units + K_ROWS_GEN : nullptr;
   rg.nd = nd; rg.ns = ns; rg.ne = ne; rg.nn = nn; rg.dt = s->p.dt; rg.idt = 1.0 / s->p.dt;
@@ -1790,6 +1791,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
   if (T.ground) {
     NodeArgs na{nn, s->p.dt, s->prm.ground_z, s->prm.delta, s->prm.slip_nu, d.q, d.qn,
                 d.node_dof_arr, d.node_sys, d.node_h, d.node_mu, d.node_kc, d.sys_active, d.nt};
+    na.constants();
     k_nodes<<<blocks(nn, 256), 256, 0, st>>>(na);
   }
   if (ns > 0) k_stencil<<<blocks(ns, 128), 128, 0, st>>>(ka);

@@ -511,8 +511,8 @@ __global__ void __launch_bounds__(128) k_stencil_hess(StencilArgs a) {
 // Line search of batches with general systems: a cluster of four blocks per
 // system.  The first decision is on the residual that the round's kernels left
 // (the same sums as k_line_search); a small system that is pulled back is then
-// evaluated here, again and again until it accepts -- edges and nodes, stencil
-// gradients, rows, merit -- instead of a round for every trial point (most
+// evaluated here, again and again until it accepts -- edges, stencil gradients
+// and nodes, rows, merit -- instead of a round for every trial point (most
 // rounds of a batch of robots did nothing else: 75 us each for the chain of ten
 // launches, 64 robots).  Each block decides for itself on the same numbers.
 // Bound by the chain of a trial point's FP64 instructions (about 500 of 64
@@ -534,7 +534,7 @@ __global__ void __cluster_dims__(kLoopBlocks, 1, 1) __launch_bounds__(kLineSearc
   LineState ls{a.trial[s], a.nback[s], a.wstry ? a.wstry[s] : 0, a.alpha[s], a.racc[s]};
   const int e0 = b.edge_ptr[s], ne = b.edge_ptr[s + 1] - e0, v0 = b.node_ptr[s];
   const int nv = b.rows.nt ? b.node_ptr[s + 1] - v0 : 0, k0 = b.st_ptr[s], nk = b.st_ptr[s + 1] - k0;
-  const int ne32 = (ne + 31) & ~31;
+  const int nk32 = (nk + 31) & ~31;
   double m = 0.0;
   unsigned long long res = 0;
   int action = 0;
@@ -573,12 +573,12 @@ __global__ void __cluster_dims__(kLoopBlocks, 1, 1) __launch_bounds__(kLineSearc
     if (!action || !small) break;
     again = true;
     cluster.sync();
-    for (int i = t0; i < ne32 + nv; i += kT) {
-      if (i < ne) k_edge_one(b.edges, b.edge_list[e0 + i]);
-      else if (i >= ne32) node_one(b.nodes, b.node_list[v0 + i - ne32]);
-    }
+    for (int i = t0; i < ne; i += kT) k_edge_one(b.edges, b.edge_list[e0 + i]);
     cluster.sync();
-    for (int i = t0; i < nk; i += kT) k_stencil_one<1>(b.stencils, b.st_list[k0 + i]);
+    for (int i = t0; i < nk32 + nv; i += kT) {  // other warps than the stencils' take the nodes
+      if (i < nk) k_stencil_one<1>(b.stencils, b.st_list[k0 + i]);
+      else if (i >= nk32) node_one(b.nodes, b.node_list[v0 + i - nk32]);
+    }
     cluster.sync();
     for (int i = t0; i < n; i += kT) rows_gen_one(b.rows, d0 + i);
     cluster.sync();

@@ -96,6 +96,13 @@ struct NodeArgs {
   const int32_t *sys_active;
   double *nt;
   unsigned long long *units;  // profiling: nodes evaluated (or NULL)
+  double K1, iK1, K2, idt;    // 15/delta, delta/15, 15/slip_nu, 1/dt (constants())
+  void constants() {
+    K1 = 15.0 / delta;
+    iK1 = delta / 15.0;
+    K2 = 15.0 / slip_nu;
+    idt = 1.0 / dt;
+  }
 };
 
 struct RowGenArgs {

@@ -7,37 +7,37 @@
 
 namespace dm {
 
-__device__ __forceinline__ double softplus(double x) {
-  return fmax(x, 0.0) + log1p(exp(-fabs(x)));
-}
-
-// Node v's contact and friction terms.
+// Node v's contact and friction terms.  Bound by their chain of FP64
+// instructions: one exponential for the softplus and its derivatives,
+// constants from the host, reciprocals of the integer pipe (20 k cycles a node
+// before).
 __device__ __forceinline__ void node_one(const NodeArgs &a, int v) {
   count_active(a.units);
   const int NN = a.nn;
   const int d = a.node_dof[v];
   const double z = a.q[d + 2] - a.ground_z;
-  const double C = a.node_h[v], dl = a.delta, K1 = 15.0 / dl, kc = a.node_kc[v];
+  const double C = a.node_h[v], dl = a.delta, kc = a.node_kc[v];
   // Eq. 10 and its first two derivatives in D
   double dE = 0.0, d2E = 0.0;
   if (z <= C - dl) {
     dE = -2.0 * (C - z);
     d2E = 2.0;
   } else if (z < C + dl) {
-    const double s = K1 * (C - z);
-    const double sp = softplus(s);
-    const double sg = 1.0 / (1.0 + exp(-s));
-    dE = -2.0 * sp * sg / K1;
-    d2E = 2.0 * (sg * sg + sp * sg * (1.0 - sg));
+    // softplus(s) = max(s, 0) + log(1 + e), its derivative the logistic sg
+    const double s = a.K1 * (C - z), e = exp(-fabs(s)), r = rcp_any(1.0 + e), er = e * r;
+    const double sp = fmax(s, 0.0) + log1p(e);
+    const double sg = s >= 0.0 ? r : er, gs = s >= 0.0 ? er : r;  // gs = 1 - sg
+    dE = -2.0 * sp * sg * a.iK1;
+    d2E = 2.0 * sg * fma(sp, gs, sg);
   }
   const double Fn = -kc * dE;
   double F[3] = {0.0, 0.0, Fn};
   double J[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, kc * d2E};
   const double mu = a.node_mu[v];
   if (mu > 0.0 && Fn != 0.0) {
-    const double K2 = 15.0 / a.slip_nu, idt = 1.0 / a.dt;
+    const double K2 = a.K2, idt = a.idt;
     const double ux = (a.q[d] - a.qn[d]) * idt, uy = (a.q[d + 1] - a.qn[d + 1]) * idt;
-    const double s = sqrt(ux * ux + uy * uy);
+    const double s = sqrt_any(ux * ux + uy * uy);
     const double fn = fabs(Fn);
     if (s == 0.0) {
       // limit of -mu |F_n| gamma(|u|) u/|u| at u = 0 (reading C14)
@@ -47,11 +47,11 @@ __device__ __forceinline__ void node_one(const NodeArgs &a, int v) {
     } else {
       const double th = tanh(0.5 * K2 * s);   // gamma of Eq. 12
       const double dth = 0.5 * K2 * (1.0 - th * th);
-      const double hx = ux / s, hy = uy / s;
+      const double is = rcp_any(s), hx = ux * is, hy = uy * is;
       F[0] = -mu * th * hx * fn;
       F[1] = -mu * th * hy * fn;
       // -dF/dx in the plane: mu |F_n| [g/s (I - u u^T) + g' u u^T] / dt
-      const double a1 = mu * fn * th / s * idt, a2 = mu * fn * dth * idt;
+      const double a1 = mu * fn * th * is * idt, a2 = mu * fn * dth * idt;
       J[0] = a1 * (1.0 - hx * hx) + a2 * hx * hx;
       J[1] = (a2 - a1) * hx * hy;
       J[3] = J[1];
