@@ -13,11 +13,12 @@
 //     blocks ([256 x 64] each: 9 per tile in inference -- layer 1's, four
 //     K-blocks of each hidden layer -- and the transposed ones of the backward
 //     chain after them in training) stream through a 3-stage ring from L2;
-//   * warp 9 issues the TMA loads, warp 8 the MMAs (M = 128, K = 16 per
-//     instruction) and the TMA stores, warps 0-7 read the accumulators back
-//     (tcgen05.ld; warp w the lanes 32 (w % 4).. and half w / 4 of each 64
+//   * warp 17 issues the TMA loads, warp 16 the MMAs (M = 128, K = 16 per
+//     instruction) and the TMA stores, warps 0-15 read the accumulators back
+//     (tcgen05.ld; warp w the lanes 32 (w % 4).. and half (w / 4) % 2 of 64
 //     columns), add the bias, apply ReLU (or the saved mask), round to BF16
-//     and store the next layer's operand;
+//     and store the next layer's operand: two groups of eight warps, a group
+//     the even, the other the odd 64-column blocks;
 //   * a layer's epilogue hands its operand over in four K-blocks, and two
 //     accumulators (256 fp32 columns of tensor memory each) alternate, so the
 //     next layer's MMAs start when the first 64 columns are ready instead of
@@ -47,7 +48,8 @@ namespace dm {
 namespace {
 
 constexpr int kTM = 128;         // rows per tile
-constexpr int kEpi = 256;        // epilogue threads (8 warps)
+constexpr int kGroup = 256;      // threads of an epilogue group (8 warps)
+constexpr int kEpi = 2 * kGroup;
 constexpr int kThreadsF = kEpi + 64;  // and the MMA and the TMA warp
 constexpr int kStages = 3;
 // shared memory map (bytes from a 1024-aligned base)
@@ -68,6 +70,21 @@ constexpr unsigned kFullMask = 0xffffffffu;
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// bf16 pair of (x + b, y + c), and the larger of it and 0 (NaN: 0)
+__device__ __forceinline__ uint32_t bias_pair(uint32_t x, uint32_t y, float b, float c) {
+  uint64_t v, w;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(x), "r"(y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "f"(b), "f"(c));
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(v), "l"(w));
+  float lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+  return pack_bf16(lo, hi);
+}
+__device__ __forceinline__ uint32_t relu_bf16(uint32_t x) {
+  const __nv_bfloat162 z = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&x), __nv_bfloat162(0.0f, 0.0f));
+  return *reinterpret_cast<const uint32_t *>(&z);
 }
 
 // Bounded wait that also gives up when another role of the CTA has failed.
@@ -140,7 +157,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
 
   const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-  if (warp == 8) {
+  if (warp == 16) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(kTmemCols));
@@ -148,7 +165,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   }
   if (tid == 0) {
     for (int i = 0; i < 2 * kStages + 2; ++i) mbar_init(&bar[i], 1);
-    for (int i = 0; i < 4; ++i) mbar_init(&bar_h[i], kEpi);
+    for (int i = 0; i < 4; ++i) mbar_init(&bar_h[i], kGroup);
     mbar_init(bar_w4, 1);
     mbar_init(bar_x, 1);
     mbar_init(bar_xfree, TRAIN ? 2 : 1);
@@ -164,7 +181,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 9) {
+  if (warp == 17) {
     // ---- TMA loads: the resident weights, then per tile its input and the
     // weight blocks in the order of use, as far ahead as the ring allows
     if (lane == 0 && my_tiles > 0) {
@@ -198,7 +215,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         if (loaded) mbar_wait(bar_x, (uint32_t)((loaded - 1) & 1));
       }
     }
-  } else if (warp == 8) {
+  } else if (warp == 16) {
     // ---- MMAs and stores, by one lane
     if (lane == 0 && my_tiles > 0) {
       int g = 0, ph = 0, hphase = 0;
@@ -291,13 +308,13 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     }
   } else {
     // ---- epilogues
-    const int quarter = warp & 3, half = warp >> 2;
+    const int quarter = warp & 3, part = warp >> 2, half = part & 1, group = warp >> 3;
     const int row = quarter * 32 + lane;  // this thread's accumulator lane / tile row
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     int ph = 0, stores = 0;
     bool ok = true;
-    uint32_t mask[TRAIN ? 3 : 1][4];  // training: ReLU masks of the hidden layers
-    float gb = 0.0f;                  // training: output column 32 half + lane's gradient sum
+    uint32_t mask[TRAIN ? 3 : 1][2];  // training: ReLU masks of the hidden layers
+    float gb = 0.0f;                  // training: output column 16 part + lane's gradient sum
     auto acc_ready = [&]() -> uint32_t {
       ok = ok && wait_on(&bar_acc[ph & 1], (uint32_t)((ph >> 1) & 1), fail);
       asm volatile("tcgen05.fence::after_thread_sync;");
@@ -305,64 +322,76 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       ++ph;
       return t;
     };
-    // 32 accumulator columns to the thread's row of a K-block in H (or Xs):
-    // its half of the row's eight 16-byte chunks, swizzled
-    auto put = [&](char *blk, const float *v) {
-      char *rowp = blk + row * 128;
-#pragma unroll
-      for (int ch = 0; ch < 4; ++ch) {
-        const float *a = v + 8 * ch;
-        *reinterpret_cast<uint4 *>(rowp + (((4 * half + ch) ^ (row & 7)) << 4)) =
-            make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
-      }
-      // the generic-proxy stores become visible to the tensor core's (and TMA's) reads
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // eight columns (chunk ch of the row's eight, swizzled) of the thread's row
+    // of a K-block in H (or Xs)
+    auto put = [&](char *blk, int ch, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+      *reinterpret_cast<uint4 *>(blk + row * 128 + ((ch ^ (row & 7)) << 4)) = make_uint4(a, b, c, d);
     };
+    // the generic-proxy stores become visible to the tensor core's (and TMA's) reads
+    auto publish = [] { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); };
     // hidden layer l, forward (bias, ReLU) or backward (mask), into H
     auto hidden = [&](int l, bool back) {
       const uint32_t t = acc_ready();
       if (!ok) return;
       if (TRAIN && stores > 0 && !(ok = wait_on(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
       ++stores;
-      uint32_t r[2][32];
-      tmem_ld16_nowait(t + (uint32_t)(32 * half), r[0]);
-      tmem_ld16_nowait(t + (uint32_t)(32 * half + 16), r[0] + 16);
+      uint32_t r[2][32];  // the group's K-blocks: group, group + 2
+      const uint32_t tc0 = t + (uint32_t)(64 * group + 32 * half);
+      tmem_ld16_nowait(tc0, r[0]);
+      tmem_ld16_nowait(tc0 + 16u, r[0] + 16);
 #pragma unroll
-      for (int kb = 0; kb < 4; ++kb) {
-        tmem_wait32(r[kb & 1]);
-        if (kb < 3) {  // the next block's columns come in behind this one's arithmetic
-          tmem_ld16_nowait(t + (uint32_t)(64 * (kb + 1) + 32 * half), r[(kb + 1) & 1]);
-          tmem_ld16_nowait(t + (uint32_t)(64 * (kb + 1) + 32 * half + 16), r[(kb + 1) & 1] + 16);
+      for (int u = 0; u < 2; ++u) {
+        const int kb = group + 2 * u;
+        tmem_wait32(r[u]);
+        if (u == 0) {  // the next block's columns come in behind this one's arithmetic
+          tmem_ld16_nowait(tc0 + 128u, r[1]);
+          tmem_ld16_nowait(tc0 + 144u, r[1] + 16);
         }
-        float v[32];
-        if (!TRAIN || !back) {
-          const float *bias = sbias + 256 * l + 64 * kb + 32 * half;
-          uint32_t mk = 0;
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
-            v[j] = fmaxf(__uint_as_float(r[kb & 1][j]) + bb.x, 0.0f);
-            v[j + 1] = fmaxf(__uint_as_float(r[kb & 1][j + 1]) + bb.y, 0.0f);
-            v[j + 2] = fmaxf(__uint_as_float(r[kb & 1][j + 2]) + bb.z, 0.0f);
-            v[j + 3] = fmaxf(__uint_as_float(r[kb & 1][j + 3]) + bb.w, 0.0f);
-            if (TRAIN)
-#pragma unroll
-              for (int k = 0; k < 4; ++k) mk |= v[j + k] > 0.0f ? 1u << (j + k) : 0u;
-          }
-          if (TRAIN) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-              if (k == l) mask[TRAIN ? k : 0][kb] = mk;
-          }
-        } else {
-          uint32_t mk = 0;
+        char *blk = Hs + kb * (kTM * 128);
+        const float *bias = sbias + 256 * l + 64 * kb + 32 * half;
+        uint32_t mk = 0;
+        if (TRAIN && back) {
 #pragma unroll
           for (int k = 0; k < 3; ++k)
-            if (k == l) mk = mask[TRAIN ? k : 0][kb];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = (mk >> j) & 1u ? __uint_as_float(r[kb & 1][j]) : 0.0f;
+            if (k == l) mk = mask[TRAIN ? k : 0][u];
         }
-        put(Hs + kb * (kTM * 128), v);
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 8; e += 4) {
+            const int j = 8 * ch + e;
+            if (!TRAIN) {
+              // packed: bias, rounding, ReLU of the rounded pair (the same result)
+              const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
+              w[e / 2] = relu_bf16(bias_pair(r[u][j], r[u][j + 1], bb.x, bb.y));
+              w[e / 2 + 1] = relu_bf16(bias_pair(r[u][j + 2], r[u][j + 3], bb.z, bb.w));
+            } else {
+              float v[4];
+              if (!back) {
+                const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
+                const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  v[k] = fmaxf(__uint_as_float(r[u][j + k]) + b4[k], 0.0f);
+                  mk |= v[k] > 0.0f ? 1u << (j + k) : 0u;
+                }
+              } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = (mk >> (j + k)) & 1u ? __uint_as_float(r[u][j + k]) : 0.0f;
+              }
+              w[e / 2] = pack_bf16(v[0], v[1]);
+              w[e / 2 + 1] = pack_bf16(v[2], v[3]);
+            }
+          }
+          put(blk, 4 * half + ch, w[0], w[1], w[2], w[3]);
+        }
+        if (TRAIN && !back) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            if (k == l) mask[TRAIN ? k : 0][u] = mk;
+        }
+        publish();
         asm volatile("tcgen05.fence::before_thread_sync;");
         arrive(&bar_h[kb]);
       }
@@ -375,16 +404,14 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       if (!ok) break;
       const uint32_t t = acc_ready();
       if (!ok) break;
-      uint32_t r[32];
-      tmem_ld16_nowait(t + (uint32_t)(32 * half), r);
-      tmem_ld16_nowait(t + (uint32_t)(32 * half + 16), r + 16);
-      tmem_wait32(r);
-      const float *bo = sbias + 768 + 32 * half;
+      // the output layer: 16 columns a warp
+      uint32_t r[16];
+      tmem_ld16(t + (uint32_t)(16 * part), r);
+      const float *bo = sbias + 768 + 16 * part;
       if (!TRAIN) {
-        // the thread's row, columns [32 half, 32 half + 32) of the output
-        float4 *o = reinterpret_cast<float4 *>(Y + ((size_t)tile * kTM + row) * 64 + 32 * half);
+        float4 *o = reinterpret_cast<float4 *>(Y + ((size_t)tile * kTM + row) * 64 + 16 * part);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
           const float4 bb = *reinterpret_cast<const float4 *>(bo + 4 * j);
           o[j] = make_float4(__uint_as_float(r[4 * j]) + bb.x, __uint_as_float(r[4 * j + 1]) + bb.y,
                              __uint_as_float(r[4 * j + 2]) + bb.z, __uint_as_float(r[4 * j + 3]) + bb.w);
@@ -394,12 +421,12 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         // loss (summed in FP64) and its gradient on the first n_valid columns
         const float *yt = ta.target + ((size_t)tile * kTM + row) * ta.n_valid;
         double ls = 0.0;
-        float v[32];
+        float v[16];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int c = 32 * half + j;
+        for (int j = 0; j < 16; ++j) {
+          const int c = 16 * part + j;
           v[j] = 0.0f;
-          if (c < ta.n_valid) {  // uniform over the CTA
+          if (c < ta.n_valid) {  // uniform over the warp
             const float d = __uint_as_float(r[j]) + bo[j] - yt[c];
             ls += (double)d * d;
             v[j] = 2.0f * d / ta.scale_den;
@@ -409,10 +436,16 @@ __global__ void __launch_bounds__(kThreadsF, 1)
             if (lane == j) gb += sum;
           }
         }
-        put(Xs, v);
+#pragma unroll
+        for (int ch = 0; ch < 2; ++ch) {
+          const float *a = v + 8 * ch;
+          put(Xs, 2 * part + ch, pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
+              pack_bf16(a[6], a[7]));
+        }
+        publish();
         asm volatile("tcgen05.fence::before_thread_sync;");
         arrive(bar_dy);
-        if (32 * half < ta.n_valid) {
+        if (16 * part < ta.n_valid) {
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(kFullMask, ls, o);
           if (lane == 0) atomicAdd(ta.loss, ls / ta.loss_den);
@@ -422,12 +455,12 @@ __global__ void __launch_bounds__(kThreadsF, 1)
           if (ok) hidden(l, true);
       }
     }
-    if (TRAIN) ta.gb4[((size_t)blockIdx.x * 4 + quarter) * 64 + 32 * half + lane] = gb;
+    if (TRAIN && lane < 16) ta.gb4[((size_t)blockIdx.x * 4 + quarter) * 64 + 16 * part + lane] = gb;
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (tid == 0 && *fail) atomicExch(err, 1);
-  if (warp == 8)
+  if (warp == 16)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 
