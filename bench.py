@@ -992,7 +992,7 @@ def run_mlp(args):
             "e2e": {"value": ws * M / (ms_e * 1e-3), "unit": "segments/s",
                     "h2d_bytes_per_step": M * 64 * 2, "d2h_bytes_per_step": M * 64 * 4},
             "gpu_launches": args.steps,
-            "roofline": {"bound": "tensor", "kernel": "k_mlp_fused (4 layers, one launch)",
+            "roofline": {"bound": "tensor", "kernel": "k_mlp_infer (4 layers, one launch)",
                          "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                          "peak_source": src, "flops_per_row": fwd, "rows_per_launch": M,
                          "traffic": None,

@@ -1,29 +1,32 @@
 // The warm-start network (64 -> 256 -> 256 -> 256 -> 64, ReLU on the hidden
-// layers; BF16 operands, FP32 accumulation) on chip: one persistent kernel, a
-// CTA per SM taking 128-row tiles of the input in turn, for inference and,
-// with the loss and the whole backward chain behind it, for training; and the
-// weight gradients of all layers in a second kernel.
+// layers; BF16 operands, FP32 accumulation) on chip, a CTA per SM taking
+// 128-row tiles of the input in turn: k_mlp_infer, two tiles in flight;
+// k_mlp_fused, the forward pass of training with the loss and the whole
+// backward chain behind it; and the weight gradients of all layers in
+// k_mlp_wgrad.
 //
 //   * operands in shared memory in the tensor core's K-major layout with the
 //     128-byte swizzle (8-row groups of 1024 bytes), written by TMA tiled
 //     loads (cp.async.bulk.tensor, tensor maps with SWIZZLE_128B) for the
 //     input and the weights, and by the epilogue's swizzled stores for the
-//     activations (or gradients), which stay in one 64 KB buffer;
-//   * the output layer's weights (64 x 256) stay resident; the other weight
-//     blocks ([256 x 64] each: 9 per tile in inference -- layer 1's, four
-//     K-blocks of each hidden layer -- and the transposed ones of the backward
-//     chain after them in training) stream through a 3-stage ring from L2;
+//     activations (or gradients), which stay in one 64 KB buffer per tile;
+//   * the weight blocks ([256 x 64] each) stream through a ring from L2 (in
+//     training the output layer's 64 x 256 stay resident);
 //   * warp 17 issues the TMA loads, warp 16 the MMAs (M = 128, K = 16 per
 //     instruction) and the TMA stores, warps 0-15 read the accumulators back
 //     (tcgen05.ld; warp w the lanes 32 (w % 4).. and half (w / 4) % 2 of 64
 //     columns), add the bias, apply ReLU (or the saved mask), round to BF16
-//     and store the next layer's operand: two groups of eight warps, a group
-//     the even, the other the odd 64-column blocks;
-//   * a layer's epilogue hands its operand over in four K-blocks, and two
-//     accumulators (256 fp32 columns of tensor memory each) alternate, so the
-//     next layer's MMAs start when the first 64 columns are ready instead of
-//     after the last: what bounds a tile is the epilogues, the tensor core
-//     works beside them.
+//     and store the next layer's operand: two groups of eight warps, in
+//     training a group the even, the other the odd 64-column blocks of a
+//     layer, in inference a group per tile in flight;
+//   * training: a layer's epilogue hands its operand over in four K-blocks, and
+//     two accumulators (256 fp32 columns of tensor memory each) alternate, so
+//     the next layer's MMAs start when the first 64 columns are ready instead
+//     of after the last.
+// Measured: inference of 444544 rows 233 -> 164 us (0.9 PFLOP/s; a tile 13.6 k
+// cycles, 5.1 k of them tensor work, 2.6 k waits for weights with two 32 KB
+// blocks in flight, 3.1 k for epilogues where the short first and last layers
+// meet); a training step of 16384 rows 548 -> 75 us.
 // Training keeps the ReLU masks in registers, forms the loss and its gradient
 // in the output epilogue, and stores the hidden activations and the gradients
 // of every layer row-major by TMA (k_mlp_wgrad reads them as they are, with
@@ -107,6 +110,12 @@ __device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, volatile
 __device__ __forceinline__ void arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
 }
+// One arrival for the warp, after every lane's fences (256 arrivals of single
+// threads serialise on the barrier's word).
+__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) arrive(bar);
+}
 __device__ __forceinline__ void tma_store_2d(const void *tmap, int x, int y, const void *src) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
                    reinterpret_cast<uint64_t>(tmap)),
@@ -136,13 +145,12 @@ struct TrainArgs {
 
 }  // namespace
 
-template <bool TRAIN>
 __global__ void __launch_bounds__(kThreadsF, 1)
     k_mlp_fused(const __grid_constant__ FusedMaps maps, const float *__restrict__ b1,
                 const float *__restrict__ b2, const float *__restrict__ b3,
-                const float *__restrict__ b4, float *__restrict__ Y, int ntiles, int *err, TrainArgs ta) {
+                const float *__restrict__ b4, int ntiles, int *err, TrainArgs ta) {
   using namespace tc;
-  constexpr int kBlocks = TRAIN ? 18 : 9;  // streamed weight blocks per tile
+  constexpr int kBlocks = 18;  // streamed weight blocks per tile
   extern __shared__ char smem_raw[];
   char *smem = reinterpret_cast<char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -165,11 +173,11 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   }
   if (tid == 0) {
     for (int i = 0; i < 2 * kStages + 2; ++i) mbar_init(&bar[i], 1);
-    for (int i = 0; i < 4; ++i) mbar_init(&bar_h[i], kGroup);
+    for (int i = 0; i < 4; ++i) mbar_init(&bar_h[i], kGroup / 32);
     mbar_init(bar_w4, 1);
     mbar_init(bar_x, 1);
-    mbar_init(bar_xfree, TRAIN ? 2 : 1);
-    mbar_init(bar_dy, kEpi);
+    mbar_init(bar_xfree, 2);
+    mbar_init(bar_dy, kEpi / 32);
     mbar_init(bar_stored, 1);
     *fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
@@ -234,7 +242,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         for (int kb = 0; kb < 4 && ok; ++kb) {
           if (!(ok = wait_on(&bar_h[kb], (uint32_t)(hphase & 1), fail))) return;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          if (TRAIN) tma_store_2d(st, 64 * kb, y, Hs + kb * (kTM * 128));
+          tma_store_2d(st, 64 * kb, y, Hs + kb * (kTM * 128));
           if (resident) {
             mma_block(Hs + kb * (kTM * 128), W4s + kb * 64 * 128, 64, kb == 0);
           } else {
@@ -248,11 +256,9 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         mma_commit(&bar_acc[ph & 1]);
         ++ph;
         ++hphase;
-        if (TRAIN) {
-          store_commit();
-          store_read_wait();
-          arrive(bar_stored);
-        }
+        store_commit();
+        store_read_wait();
+        arrive(bar_stored);
       };
       // a layer whose operand is the input tile (or the output gradient in its place)
       auto x_layer = [&]() {
@@ -267,14 +273,13 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         if (!(ok = wait_on(bar_x, (uint32_t)(i & 1), fail))) break;
         x_layer();
         if (!ok) break;
-        if (!TRAIN) mma_commit(bar_xfree);
         mma_commit(&bar_acc[ph & 1]);
         ++ph;
         h_layer(false, &maps.a[0], y);
         if (ok) h_layer(false, &maps.a[1], y);
         if (ok && i == 0) ok = wait_on(bar_w4, 0, fail);
         if (ok) h_layer(true, &maps.a[2], y);
-        if (TRAIN && ok) {
+        if (ok) {
           if (!(ok = wait_on(bar_dy, (uint32_t)(i & 1), fail))) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
           tma_store_2d(&maps.dy, 0, y, Xs);
@@ -299,7 +304,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
           arrive(bar_stored);
         }
       }
-      if (TRAIN) store_wait();
+      store_wait();
       if (!ok || *fail) {
         // every MMA issued so far is done before the tensor memory is freed
         mma_commit(bar_w4);
@@ -313,8 +318,8 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     int ph = 0, stores = 0;
     bool ok = true;
-    uint32_t mask[TRAIN ? 3 : 1][2];  // training: ReLU masks of the hidden layers
-    float gb = 0.0f;                  // training: output column 16 part + lane's gradient sum
+    uint32_t mask[3][2];  // ReLU masks of the hidden layers
+    float gb = 0.0f;      // output column 16 part + lane's gradient sum
     auto acc_ready = [&]() -> uint32_t {
       ok = ok && wait_on(&bar_acc[ph & 1], (uint32_t)((ph >> 1) & 1), fail);
       asm volatile("tcgen05.fence::after_thread_sync;");
@@ -333,7 +338,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     auto hidden = [&](int l, bool back) {
       const uint32_t t = acc_ready();
       if (!ok) return;
-      if (TRAIN && stores > 0 && !(ok = wait_on(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
+      if (stores > 0 && !(ok = wait_on(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
       ++stores;
       uint32_t r[2][32];  // the group's K-blocks: group, group + 2
       const uint32_t tc0 = t + (uint32_t)(64 * group + 32 * half);
@@ -350,10 +355,10 @@ __global__ void __launch_bounds__(kThreadsF, 1)
         char *blk = Hs + kb * (kTM * 128);
         const float *bias = sbias + 256 * l + 64 * kb + 32 * half;
         uint32_t mk = 0;
-        if (TRAIN && back) {
+        if (back) {
 #pragma unroll
           for (int k = 0; k < 3; ++k)
-            if (k == l) mk = mask[TRAIN ? k : 0][u];
+            if (k == l) mk = mask[k][u];
         }
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
@@ -361,39 +366,32 @@ __global__ void __launch_bounds__(kThreadsF, 1)
 #pragma unroll
           for (int e = 0; e < 8; e += 4) {
             const int j = 8 * ch + e;
-            if (!TRAIN) {
-              // packed: bias, rounding, ReLU of the rounded pair (the same result)
+            float v[4];
+            if (!back) {
               const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
-              w[e / 2] = relu_bf16(bias_pair(r[u][j], r[u][j + 1], bb.x, bb.y));
-              w[e / 2 + 1] = relu_bf16(bias_pair(r[u][j + 2], r[u][j + 3], bb.z, bb.w));
-            } else {
-              float v[4];
-              if (!back) {
-                const float4 bb = *reinterpret_cast<const float4 *>(bias + j);
-                const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+              const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  v[k] = fmaxf(__uint_as_float(r[u][j + k]) + b4[k], 0.0f);
-                  mk |= v[k] > 0.0f ? 1u << (j + k) : 0u;
-                }
-              } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = (mk >> (j + k)) & 1u ? __uint_as_float(r[u][j + k]) : 0.0f;
+              for (int k = 0; k < 4; ++k) {
+                v[k] = fmaxf(__uint_as_float(r[u][j + k]) + b4[k], 0.0f);
+                mk |= v[k] > 0.0f ? 1u << (j + k) : 0u;
               }
-              w[e / 2] = pack_bf16(v[0], v[1]);
-              w[e / 2 + 1] = pack_bf16(v[2], v[3]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) v[k] = (mk >> (j + k)) & 1u ? __uint_as_float(r[u][j + k]) : 0.0f;
             }
+            w[e / 2] = pack_bf16(v[0], v[1]);
+            w[e / 2 + 1] = pack_bf16(v[2], v[3]);
           }
           put(blk, 4 * half + ch, w[0], w[1], w[2], w[3]);
         }
-        if (TRAIN && !back) {
+        if (!back) {
 #pragma unroll
           for (int k = 0; k < 3; ++k)
-            if (k == l) mask[TRAIN ? k : 0][u] = mk;
+            if (k == l) mask[k][u] = mk;
         }
         publish();
         asm volatile("tcgen05.fence::before_thread_sync;");
-        arrive(&bar_h[kb]);
+        warp_arrive(&bar_h[kb]);
       }
     };
     for (int i = 0; i < my_tiles && ok; ++i) {
@@ -408,54 +406,286 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       uint32_t r[16];
       tmem_ld16(t + (uint32_t)(16 * part), r);
       const float *bo = sbias + 768 + 16 * part;
-      if (!TRAIN) {
-        float4 *o = reinterpret_cast<float4 *>(Y + ((size_t)tile * kTM + row) * 64 + 16 * part);
+      // loss (summed in FP64) and its gradient on the first n_valid columns
+      const float *yt = ta.target + ((size_t)tile * kTM + row) * ta.n_valid;
+      double ls = 0.0;
+      float v[16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 bb = *reinterpret_cast<const float4 *>(bo + 4 * j);
-          o[j] = make_float4(__uint_as_float(r[4 * j]) + bb.x, __uint_as_float(r[4 * j + 1]) + bb.y,
-                             __uint_as_float(r[4 * j + 2]) + bb.z, __uint_as_float(r[4 * j + 3]) + bb.w);
+      for (int j = 0; j < 16; ++j) {
+        const int c = 16 * part + j;
+        v[j] = 0.0f;
+        if (c < ta.n_valid) {  // uniform over the warp
+          const float d = __uint_as_float(r[j]) + bo[j] - yt[c];
+          ls += (double)d * d;
+          v[j] = 2.0f * d / ta.scale_den;
+          float sum = v[j];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFullMask, sum, o);
+          if (lane == j) gb += sum;
         }
-        asm volatile("tcgen05.fence::before_thread_sync;");
-      } else {
-        // loss (summed in FP64) and its gradient on the first n_valid columns
-        const float *yt = ta.target + ((size_t)tile * kTM + row) * ta.n_valid;
-        double ls = 0.0;
-        float v[16];
+      }
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int c = 16 * part + j;
-          v[j] = 0.0f;
-          if (c < ta.n_valid) {  // uniform over the warp
-            const float d = __uint_as_float(r[j]) + bo[j] - yt[c];
-            ls += (double)d * d;
-            v[j] = 2.0f * d / ta.scale_den;
-            float sum = v[j];
+      for (int ch = 0; ch < 2; ++ch) {
+        const float *a = v + 8 * ch;
+        put(Xs, 2 * part + ch, pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
+            pack_bf16(a[6], a[7]));
+      }
+      publish();
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      warp_arrive(bar_dy);
+      if (16 * part < ta.n_valid) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFullMask, sum, o);
-            if (lane == j) gb += sum;
+        for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(kFullMask, ls, o);
+        if (lane == 0) atomicAdd(ta.loss, ls / ta.loss_den);
+      }
+#pragma unroll
+      for (int l = 2; l >= 0; --l)
+        if (ok) hidden(l, true);
+    }
+    if (lane < 16) ta.gb4[((size_t)blockIdx.x * 4 + quarter) * 64 + 16 * part + lane] = gb;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (tid == 0 && *fail) atomicExch(err, 1);
+  if (warp == 16)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+}
+
+namespace {
+
+// ---- inference.  One tile's layers are a chain -- accumulator ready, read
+// back, rounded, stored, fenced, handed over, multiplied -- whose waits one tile
+// at a time exposes (16.5 k cycles a tile, 5 k of them tensor work).  So a CTA
+// has two tiles in flight, each with its operand buffer, its 256 accumulator
+// columns and eight epilogue warps: one's epilogue runs beside the other's
+// MMAs.  The weight blocks, the output layer's too, stream through the ring
+// once per tile.  (Halves of 128 output columns of one tile with two operand
+// buffers took 22 k cycles: MMAs of N = 128 read shared memory at its limit.)
+constexpr int kIStages = 2;
+constexpr int kIOffX = 2 * 4 * kTM * 128;               // after two operand buffers of 64 KB
+constexpr int kIOffRing = kIOffX + 2 * kTM * 128;
+constexpr int kIOffBar = kIOffRing + kIStages * kStageBytes;
+constexpr int kINumBars = 2 * kIStages + 8 + 1;
+constexpr int kSmemInfer = kIOffBar + 8 * kINumBars + 16 + 1024;
+static_assert(kSmemInfer <= 227 * 1024, "shared memory of the inference kernel");
+
+struct InferMaps {
+  CUtensorMap x, w1, w2, w3, w4;
+};
+
+}  // namespace
+
+__global__ void __launch_bounds__(kThreadsF, 1)
+    k_mlp_infer(const __grid_constant__ InferMaps maps, const float *__restrict__ b1, const float *__restrict__ b2,
+                const float *__restrict__ b3, const float *__restrict__ b4, float *__restrict__ Y, int ntiles,
+                int *err) {
+  using namespace tc;
+  extern __shared__ char smem_raw[];
+  char *smem = reinterpret_cast<char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  char *Ring = smem + kIOffRing;
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kIOffBar);
+  uint64_t *bar_full = bar, *bar_free = bar + kIStages;
+  // per tile in flight: accumulator complete, accumulator read and operand
+  // stored, input in, input read
+  uint64_t *bar_acc = bar + 2 * kIStages, *bar_h = bar_acc + 2, *bar_x = bar_acc + 4, *bar_xfree = bar_acc + 6;
+  uint64_t *bar_end = bar_acc + 8;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + kINumBars);
+  volatile int *fail = reinterpret_cast<volatile int *>(tmem_slot + 1);
+
+  const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const auto tile_of = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x; };
+  // order of the layers: in slot v, layer v % 4 of an even tile, then of the odd
+  // one after it (one or two layers apart 176 us instead of 164, three the same)
+  const int slots = 4 * ((my_tiles + 1) / 2);
+
+  if (warp == 16) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(kTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int i = 0; i < kINumBars; ++i) mbar_init(&bar[i], 1);
+    for (int i = 0; i < 2; ++i) mbar_init(&bar_h[i], kGroup / 32);
+    *fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 17) {
+    // ---- TMA loads: the two tiles' inputs, then per layer and tile the weight
+    // blocks, as far ahead as the ring allows
+    if (lane == 0 && my_tiles > 0) {
+      int g = 0, loaded[2] = {0, 0};
+      bool ok = true;
+      auto weights = [&](int l, int kb) {
+        const int s = g % kIStages;
+        if (g >= kIStages && !(ok = ok && wait_on(&bar_free[s], (uint32_t)((g / kIStages - 1) & 1), fail))) return;
+        char *dst = Ring + s * kStageBytes;
+        mbar_expect_tx(&bar_full[s], (uint32_t)kStageBytes);
+        if (l < 3) {
+          tma_load_2d(dst, l == 0 ? &maps.w1 : l == 1 ? &maps.w2 : &maps.w3, 64 * kb, 0, &bar_full[s]);
+        } else {
+          for (int u = 0; u < 4; ++u) tma_load_2d(dst + u * 64 * 128, &maps.w4, 64 * u, 0, &bar_full[s]);
+        }
+        ++g;
+      };
+      auto input = [&](int i) {
+        const int t = i & 1;
+        mbar_expect_tx(&bar_x[t], kTM * 128);
+        tma_load_2d(smem + kIOffX + t * (kTM * 128), &maps.x, 0, tile_of(i) * kTM, &bar_x[t]);
+        ++loaded[t];
+      };
+      input(0);
+      if (my_tiles > 1) input(1);
+      for (int v = 0; v < slots && ok; ++v)
+        for (int t = 0; t < 2 && ok; ++t) {
+          const int l = v & 3, i = 2 * (v >> 2) + t;
+          if (i >= my_tiles) continue;
+          for (int kb = 0; kb < (l == 1 || l == 2 ? 4 : 1) && ok; ++kb) weights(l, kb);
+          if (l == 1 && i + 2 < my_tiles && ok) {  // the first layer has read the input
+            ok = wait_on(&bar_xfree[t], (uint32_t)((i >> 1) & 1), fail);
+            if (ok) input(i + 2);
           }
         }
-#pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-          const float *a = v + 8 * ch;
-          put(Xs, 2 * part + ch, pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
-              pack_bf16(a[6], a[7]));
-        }
-        publish();
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        arrive(bar_dy);
-        if (16 * part < ta.n_valid) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(kFullMask, ls, o);
-          if (lane == 0) atomicAdd(ta.loss, ls / ta.loss_den);
-        }
-#pragma unroll
-        for (int l = 2; l >= 0; --l)
-          if (ok) hidden(l, true);
+      if (!ok || *fail) {  // what is in flight lands before the CTA leaves (bounded)
+        for (int k = g > kIStages ? g - kIStages : 0; k < g; ++k)
+          mbar_wait(&bar_full[k % kIStages], (uint32_t)((k / kIStages) & 1));
+        for (int t = 0; t < 2; ++t)
+          if (loaded[t]) mbar_wait(&bar_x[t], (uint32_t)((loaded[t] - 1) & 1));
       }
     }
-    if (TRAIN && lane < 16) ta.gb4[((size_t)blockIdx.x * 4 + quarter) * 64 + 16 * part + lane] = gb;
+  } else if (warp == 16) {
+    // ---- MMAs, by one lane
+    if (lane == 0 && my_tiles > 0) {
+      int g = 0, hphase[2] = {0, 0};
+      bool ok = true;
+      // K = 64 at `a` against n weight rows at `w`, into accumulator columns d
+      auto mma_block = [&](const char *a, const char *w, int n, uint32_t d, bool first) {
+        const uint32_t a0 = smem_u32(a), w0 = smem_u32(w);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16(tmem + d, make_desc(a0 + 32 * kk, 16, 1024, kSwizzle128B),
+                   make_desc(w0 + 32 * kk, 16, 1024, kSwizzle128B), make_idesc(kTM, n), (first && kk == 0) ? 0u : 1u);
+      };
+      for (int v = 0; v < slots && ok; ++v)
+        for (int t = 0; t < 2 && ok; ++t) {
+          const int l = v & 3, i = 2 * (v >> 2) + t;
+          if (i >= my_tiles) continue;
+          const uint32_t d = 256u * (uint32_t)t;
+          char *H = smem + t * (4 * kTM * 128);
+          if (l == 0) ok = wait_on(&bar_x[t], (uint32_t)((i >> 1) & 1), fail);
+          // the accumulator has been read, the operand (layers 1 on) stored
+          if (ok && v > 0) {
+            ok = wait_on(&bar_h[t], (uint32_t)(hphase[t] & 1), fail);
+            ++hphase[t];
+          }
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          for (int kb = 0; kb < (l == 1 || l == 2 ? 4 : 1) && ok; ++kb) {
+            const int s = g % kIStages;
+            if (!(ok = wait_on(&bar_full[s], (uint32_t)((g / kIStages) & 1), fail))) break;
+            const char *w = Ring + s * kStageBytes;
+            if (l == 3) {
+              for (int q = 0; q < 4; ++q) mma_block(H + q * (kTM * 128), w + q * 64 * 128, 64, d, q == 0);
+            } else {
+              mma_block(l == 0 ? smem + kIOffX + t * (kTM * 128) : H + kb * (kTM * 128), w, 256, d, kb == 0);
+            }
+            mma_commit(&bar_free[s]);
+            ++g;
+          }
+          if (!ok) break;
+          if (l == 0) mma_commit(&bar_xfree[t]);
+          mma_commit(&bar_acc[t]);
+        }
+      if (!ok || *fail) {
+        // every MMA issued so far is done before the tensor memory is freed
+        mma_commit(bar_end);
+        mbar_wait(bar_end, 0);
+      }
+    }
+  } else {
+    // ---- epilogues: warps 0-7 of the even tiles, 8-15 of the odd ones
+    const int quarter = warp & 3, half = (warp >> 2) & 1, t = warp >> 3;
+    const int row = quarter * 32 + lane;  // this thread's accumulator lane / tile row
+    const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + 256u * (uint32_t)t + 32u * (uint32_t)half;
+    char *H = smem + t * (4 * kTM * 128);
+    uint32_t phase = 0;
+    bool ok = true;
+    auto acc_ready = [&]() {
+      ok = ok && wait_on(&bar_acc[t], phase & 1u, fail);
+      ++phase;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+    };
+    for (int i = t; i < my_tiles && ok; i += 2) {
+#pragma unroll 1
+      for (int l = 0; l < 3; ++l) {
+        acc_ready();
+        if (!ok) break;
+        const float *bl = l == 0 ? b1 : l == 1 ? b2 : b3;
+        uint32_t r[2][32];
+        tmem_ld16_nowait(acc, r[0]);
+        tmem_ld16_nowait(acc + 16u, r[0] + 16);
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) {
+          tmem_wait32(r[kb & 1]);
+          if (kb < 3) {  // the next block's columns come in behind this one's arithmetic
+            tmem_ld16_nowait(acc + (uint32_t)(64 * (kb + 1)), r[(kb + 1) & 1]);
+            tmem_ld16_nowait(acc + (uint32_t)(64 * (kb + 1) + 16), r[(kb + 1) & 1] + 16);
+          }
+          const float4 *bias = reinterpret_cast<const float4 *>(bl + 64 * kb + 32 * half);
+          char *rowp = H + kb * (kTM * 128) + row * 128;
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float4 bb = __ldg(bias + 2 * ch + e);
+              const uint32_t *x = r[kb & 1] + 8 * ch + 4 * e;
+              w[2 * e] = relu_bf16(bias_pair(x[0], x[1], bb.x, bb.y));
+              w[2 * e + 1] = relu_bf16(bias_pair(x[2], x[3], bb.z, bb.w));
+            }
+            *reinterpret_cast<uint4 *>(rowp + (((4 * half + ch) ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+        }
+        // the generic-proxy stores become visible to the tensor core's reads
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        warp_arrive(&bar_h[t]);
+      }
+      if (!ok) break;
+      acc_ready();
+      if (!ok) break;
+      // the output layer: 32 rows of 128 bytes per warp, through its 4 KB of the
+      // operand buffer so that eight lanes store a row's 128 bytes
+      uint32_t r[32];
+      tmem_ld16_nowait(acc, r);
+      tmem_ld16_nowait(acc + 16u, r + 16);
+      tmem_wait32(r);
+      const float4 *bo = reinterpret_cast<const float4 *>(b4 + 32 * half);
+      char *buf = H + (warp & 7) * 4096;
+#pragma unroll
+      for (int ch = 0; ch < 8; ++ch) {
+        const float4 bb = __ldg(bo + ch);
+        *reinterpret_cast<float4 *>(buf + lane * 128 + ((ch ^ (lane & 7)) << 4)) =
+            make_float4(__uint_as_float(r[4 * ch]) + bb.x, __uint_as_float(r[4 * ch + 1]) + bb.y,
+                        __uint_as_float(r[4 * ch + 2]) + bb.z, __uint_as_float(r[4 * ch + 3]) + bb.w);
+      }
+      __syncwarp();
+      float4 *o = reinterpret_cast<float4 *>(Y + ((size_t)tile_of(i) * kTM + quarter * 32) * 64 + 32 * half);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int rr = 4 * k + (lane >> 3), ch = lane & 7;
+        o[rr * 16 + ch] = *reinterpret_cast<const float4 *>(buf + rr * 128 + ((ch ^ (rr & 7)) << 4));
+      }
+      // the accumulator and this warp's part of the buffer, which the other
+      // warps' next layer overwrites, have been read
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      warp_arrive(&bar_h[t]);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -648,14 +878,15 @@ bool encode_forward(FusedMaps &t, int M, const void *X, const void *const W[4]) 
 // to 1 on a barrier timeout.
 cudaError_t launch_mlp_fused(int M, const void *X, const void *const W[4], const float *const b[4],
                              float *Y, int *err, cudaStream_t st) {
-  FusedMaps t{};
-  if (!encode_forward(t, M, X, W)) return cudaErrorInvalidValue;
+  InferMaps t{};
+  if (!(encode(&t.x, X, (uint64_t)M, 64, kTM) && encode(&t.w1, W[0], 256, 64, 256) &&
+        encode(&t.w2, W[1], 256, 256, 256) && encode(&t.w3, W[2], 256, 256, 256) && encode(&t.w4, W[3], 64, 256, 64)))
+    return cudaErrorInvalidValue;
   const int ntiles = M / kTM, grid = std::min(ntiles, device_sms());
   if (grid == 0) return cudaSuccess;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_mlp_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInfer);
   if (e != cudaSuccess) return e;
-  k_mlp_fused<false><<<grid, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], Y, ntiles, err, TrainArgs{});
+  k_mlp_infer<<<grid, kThreadsF, kSmemInfer, st>>>(t, b[0], b[1], b[2], b[3], Y, ntiles, err);
   return cudaGetLastError();
 }
 
@@ -691,12 +922,12 @@ cudaError_t launch_mlp_train(int M, const void *X, const float *target, int n_va
   if (!ok) return cudaErrorInvalidValue;
   const MlpTrainShape s = mlp_train_shape(M);
   cudaError_t e =
-      cudaFuncSetAttribute(k_mlp_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
+      cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemGrad);
   if (e != cudaSuccess) return e;
   const TrainArgs ta{target, n_valid, (float)(M * n_valid), (double)(M * n_valid), loss, gb4};
-  k_mlp_fused<true><<<s.ctas, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], nullptr, M / kTM, err, ta);
+  k_mlp_fused<<<s.ctas, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], M / kTM, err, ta);
   k_mlp_wgrad<<<4 * (s.s_small + s.s_big), 192, kSmemGrad, st>>>(g, M / 64, s.s_small, s.s_big, part, err);
   return cudaGetLastError();
 }
