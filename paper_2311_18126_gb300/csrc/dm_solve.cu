@@ -1,7 +1,7 @@
 // Residual, Jacobian assembly and line search of the backward-Euler Newton
 // iteration (DisMech, arXiv 2311.18126, Sec. III-C, Eq. 15-16), FP64.
 //
-//  k_rows_rod   -- one thread per DOF row of a single-rod system: gathers the
+//  k_rows_rod   -- the DOF rows of single-rod systems: gathers the
 //                  forces of the stencils/edges that touch the DOF (Eq. 9 plus
 //                  gravity and damping), forms the residual
 //                  f = M/dt^2 (q - q_n) - M/dt qdot_n - F, its scaled size
@@ -20,154 +20,181 @@ __device__ __forceinline__ constexpr int upk(int i, int j) {
   return i * n - i * (i - 1) / 2 + (j - i);
 }
 
-__device__ __forceinline__ int ksym(int c, int cp) {  // packed 3x3 (xx,xy,xz,yy,yz,zz)
-  int i = c < cp ? c : cp, j = c < cp ? cp : c;
+__host__ __device__ constexpr int ksym(int c, int cp) {  // packed 3x3 (xx,xy,xz,yy,yz,zz)
+  const int i = c < cp ? c : cp, j = c < cp ? cp : c;
   return 3 + (i == 0 ? j : (i == 1 ? 2 + j : 5));
 }
 
-// The band pass runs for a system only if the solver will factor its
-// Jacobian this round (the test of the Hessian pass of the stencils).
-__device__ __forceinline__ bool band_due(const RowArgs &a, int s) {
-  if (a.sys_status[s] != 0) return false;
-  if (a.ls_action && a.ls_action[s] == 1) return false;
-  return !(__longlong_as_double((long long)a.sys_res[s]) <= a.tol);
-}
-
-// One DOF row (the work of one thread); returns early when inactive.
+// Rows of a rod, a block of T threads per T DOFs, in two steps.  First a thread
+// sums the element terms of DOF b0 + 4 (t mod T/4) + t / (T/4): a quarter of the
+// block has one component c of consecutive nodes (rods have 4 N - 1 DOFs, so c
+// changes only where a rod ends), so that every index of the sums is a constant
+// and the loads of a term are consecutive.  Then, through shared memory, a
+// thread per DOF in order adds the diagonal, the masks and the residual and
+// stores.  (One thread per DOF from the start: the four components of a node in
+// one warp ran one after the other, 70 FP64 instructions a row, 240 us for the
+// fused pass of 1828856 rows whose bytes take 59; now 154, the band pass 80 ->
+// 63, the residual pass 56 -> 46.  Bound by the chain of loads, so four blocks
+// per SM: two took 103 and 260.)
 // MODE 0: residual and band row; 1: residual only (the residual pass of a
 // round); 2: band row of the systems the solver will factor (the Jacobian
-// pass).  Returns the row's scaled residual |f| / (D l) (as its bits; 0 where
-// there is none) for the system in `sys` (-1: none).
-template <int MODE>
-__device__ __forceinline__ unsigned long long k_rows_rod_one(const RowArgs &a, const int i, int &sys) {
-  sys = -1;
-  bool act = i < a.nd && a.sys_active[a.dof_sys[i]] &&
-             a.sys_kind[a.dof_sys[i]] != SOLVE_GENERAL;
-  if (MODE == 2 && act) act = band_due(a, a.dof_sys[i]);
-  count_units(a.units, act);
-  if (!act) return 0;
-  const int s = a.dof_sys[i];
-  const int rod = a.dof_rod[i];
-  const int base = a.rod_dof0[rod];
-  const int r = i - base;
-  const int n = a.rod_ndof[rod];
-  const int N = (n + 1) >> 2;
-  const int node = r >> 2, c = r & 3;
-  const int st0 = a.rod_st0[rod], e0 = a.rod_edge0[rod];
-  const int NS = a.ns, NE = a.ne;
-  // G = minus the sum of the forces on DOF i (the residual adds it), so
-  // that the sums start from their first term, not from an add to zero
-  double G = 0.0;
-  double brow[11];
-  // stencils m (interior nodes 1..N-2) with 4m-4 <= r <= 4m+6
-  int mlo = (r - 6 + 3) >= 0 ? (r - 6 + 3) / 4 : 0;
-  if (mlo < 1) mlo = 1;
-  int mhi = (r + 4) / 4;
-  if (mhi > N - 2) mhi = N - 2;
-  {
-    const bool any = mlo <= mhi;
-    const int lr = r - 4 * (mlo - 1);
-    const int st = st0 + mlo - 1;
-    if (MODE != 2 && any) G = a.sg[lr * NS + st];
-#pragma unroll
-    for (int d = 0; d < 11; ++d) {
-      const int lc = lr - d;
-      brow[d] = (MODE != 1 && any && lc >= 0) ? a.sh[upk<11>(lc, lr) * NS + st] : 0.0;
+// pass).
+constexpr int kRowThreads = 256;  // at most
+__device__ __forceinline__ int row_pitch(int T) { return T / 4 + 4; }  // (conflict-free both ways)
+
+// Loaded without a branch in between, so that system and rod arrive together
+// (the kernel is a chain of dependent loads).
+struct RowPlace {
+  int sys, N, r, st0, e0;
+  bool due;
+  template <int MODE>
+  __device__ __forceinline__ void load(const RowArgs &a, int i0) {
+    const int i = min(i0, a.nd - 1), rod = a.dof_rod[i];
+    sys = a.dof_sys[i];
+    const int base = a.rod_dof0[rod], n = a.rod_ndof[rod], act = a.sys_active[sys], kind = a.sys_kind[sys];
+    st0 = a.rod_st0[rod];
+    e0 = a.rod_edge0[rod];
+    due = act && kind != SOLVE_GENERAL && i0 < a.nd;
+    if (MODE == 2) {  // only if the solver will factor its Jacobian this round (as the stencils' Hessian pass)
+      const int st = a.sys_status[sys], act2 = a.ls_action ? a.ls_action[sys] : 0;
+      const double res = __longlong_as_double((long long)a.sys_res[sys]);
+      due = due && st == 0 && act2 != 1 && !(res <= a.tol);
     }
+    r = i - base;
+    N = (n + 1) >> 2;
   }
-  for (int m = mlo + 1; m <= mhi; ++m) {
-    const int lr = r - 4 * (m - 1);
-    const int st = st0 + m - 1;
-    if (MODE != 2) G += a.sg[lr * NS + st];
-    if (MODE != 1) {
-#pragma unroll
-      for (int d = 0; d < 11; ++d) {
-        const int lc = lr - d;
-        if (lc >= 0) brow[d] += a.sh[upk<11>(lc, lr) * NS + st];
-      }
+};
+
+// Row C of `node` of a rod of N nodes: its band entries without the diagonal's
+// mass and damping, and minus the sum of the elastic forces on it (the
+// residual adds it), to out[0..10] and out[11], `plane` doubles apart.
+template <int MODE, int C>
+__device__ __forceinline__ void rod_row(const RowArgs &a, int N, int node, int st0, int e0, double *out, int plane) {
+  constexpr int L0 = 8 + C, L1 = 4 + C, L2 = C;  // the row's place in the stencils of node - 1, node, node + 1
+  const bool h0 = C < 3 && node >= 2, h1 = node >= 1 && node <= N - 2, h2 = node <= N - 3;
+  const int st = st0 + node - 1, NS = a.ns, NE = a.ne;
+  const bool es = C < 3 && node <= N - 2, ee = C < 3 && node >= 1;  // edges that start and end here
+  if (MODE != 2) {
+    double G = h0 ? a.sg[(size_t)(C < 3 ? L0 : 0) * NS + st - 1] : 0.0;
+    const double g1 = h1 ? a.sg[(size_t)L1 * NS + st] : 0.0, g2 = h2 ? a.sg[(size_t)L2 * NS + st + 1] : 0.0;
+    if (C < 3) {
+      const double x = es ? a.es[(size_t)C * NE + e0 + node] : 0.0, y = ee ? a.es[(size_t)C * NE + e0 + node - 1] : 0.0;
+      G = (((G + g1) + g2) - x) + y;
+    } else {
+      G = g1 + g2;
     }
-  }
-  const double m_i = a.mass[i];
-  const double idt = a.idt;
-  if (c < 3) {
-    // one copy per component, so that every index of brow is a constant
-    // (brow stays in registers)
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      if (cc != c) continue;
-      if (node <= N - 2) {  // edge `node` starts here
-        const int e = e0 + node;
-        if (MODE != 2) G -= a.es[cc * NE + e];
-        if (MODE != 1) {
-#pragma unroll
-          for (int cp = 0; cp <= cc; ++cp) brow[cc - cp] += a.es[ksym(cc, cp) * NE + e];
-        }
-      }
-      if (node >= 1) {  // edge `node-1` ends here
-        const int e = e0 + node - 1;
-        if (MODE != 2) G += a.es[cc * NE + e];
-        if (MODE != 1) {
-#pragma unroll
-          for (int cp = 0; cp <= 2; ++cp) {
-            const double kv = a.es[ksym(cc, cp) * NE + e];
-            if (cp <= cc) brow[cc - cp] += kv;
-            brow[4 + cc - cp] -= kv;
-          }
-        }
-      }
-    }
-    const double cd = a.damp[i];
-    if (MODE != 2) {
-      G = fma(-m_i, a.g[c], G);
-      G = fma(cd, a.q[i] - a.qn[i], G);
-    }
-    brow[0] += cd;
+    out[11 * plane] = G;
   }
   if (MODE != 1) {
-    brow[0] += m_i * idt * idt;
-    if (a.fixed[i]) {
-      brow[0] = 1.0;
+    double v[11], v1[11], v2[11], x[3], y[3];
 #pragma unroll
-      for (int d = 1; d < 11; ++d) brow[d] = 0.0;
-    } else {
-#pragma unroll
-      for (int d = 1; d < 11; ++d)
-        if (r - d < 0 || a.fixed[i - d]) brow[d] = 0.0;
+    for (int d = 0; d < 11; ++d) {
+      v[d] = C < 3 && d <= L0 && h0 ? a.sh[(size_t)upk<11>(C < 3 ? L0 - d : 0, C < 3 ? L0 : 0) * NS + st - 1] : 0.0;
+      v1[d] = d <= L1 && h1 ? a.sh[(size_t)upk<11>(d <= L1 ? L1 - d : 0, L1) * NS + st] : 0.0;
+      v2[d] = d <= L2 && h2 ? a.sh[(size_t)upk<11>(d <= L2 ? L2 - d : 0, L2) * NS + st + 1] : 0.0;
     }
 #pragma unroll
-    for (int d = 0; d < 11; ++d) a.band[(size_t)d * a.nd + i] = brow[d];
+    for (int cp = 0; cp < 3; ++cp) {
+      x[cp] = cp <= C && es ? a.es[(size_t)ksym(C < 3 ? C : 0, cp) * NE + e0 + node] : 0.0;
+      y[cp] = ee ? a.es[(size_t)ksym(C < 3 ? C : 0, cp) * NE + e0 + node - 1] : 0.0;
+    }
+#pragma unroll
+    for (int d = 0; d < 11; ++d) {
+      double w = C < 3 ? v[d] : v1[d];
+      if (C < 3 && d <= L1) w += v1[d];
+      if (d <= L2) w += v2[d];
+      if (C < 3) {
+        if (d <= C) w += x[C - d < 0 ? 0 : C - d];
+        if (d <= C) w += y[C - d < 0 ? 0 : C - d];
+        if (d >= 2 + C && d <= 4 + C) w -= y[4 + C - d < 0 ? 0 : 4 + C - d > 2 ? 2 : 4 + C - d];
+      }
+      out[d * plane] = w;
+    }
   }
-  if (MODE != 2) {
-    if (a.fc) G -= a.fc[i];
-    double f = m_i * idt * idt * (a.q[i] - a.qn[i]) - m_i * idt * a.vn[i] + G;
-    if (a.fixed[i]) f = 0.0;
-    a.f[i] = f;
-    sys = s;
-    return (unsigned long long)__double_as_longlong(fabs(f) * a.rscale[i]);
-  }
-  return 0;
 }
 
-// block-uniform grid-stride loops (count_units synchronises the block)
-__global__ void __launch_bounds__(256) k_rows_rod(RowArgs a) {
-  for (int b0 = blockIdx.x * blockDim.x; b0 < a.nd; b0 += gridDim.x * blockDim.x) {
-    int sys;
-    const unsigned long long r = k_rows_rod_one<0>(a, b0 + threadIdx.x, sys);
-    max_residual(a.sys_res, sys, r);
+template <int MODE>
+__device__ __forceinline__ void rows_rod(const RowArgs &a, double *sm) {
+  const int T = blockDim.x, t = threadIdx.x, pitch = row_pitch(T), plane = 4 * pitch, q = t / (T / 4);
+  for (int b0 = blockIdx.x * T; b0 < a.nd; b0 += gridDim.x * T) {
+    RowPlace pa, pb;
+    pa.load<MODE>(a, b0 + 4 * (t - q * (T / 4)) + q);
+    pb.load<MODE>(a, b0 + t);
+    // the second step's inputs, on the way during the first
+    const int i = min(b0 + t, a.nd - 1), c = pb.r & 3;
+    const double m = a.mass[i], damp = a.damp[i];
+    double dq = 0.0, vn = 0.0, rscale = 0.0, fc = 0.0;
+    if (MODE != 2) {
+      dq = a.q[i] - a.qn[i];
+      vn = a.vn[i];
+      rscale = a.rscale[i];
+      if (a.fc) fc = a.fc[i];
+    }
+    unsigned fixed = a.fixed[i] != 0;  // bit d: row i - d is fixed
+    if (MODE != 1) {
+#pragma unroll
+      for (int d = 1; d < 11; ++d) fixed |= a.fixed[max(i - d, 0)] ? 1u << d : 0u;
+    }
+    if (pa.due) {
+      double *out = sm + q * pitch + t - q * (T / 4);
+      const int node = pa.r >> 2;
+      switch (pa.r & 3) {
+        case 0: rod_row<MODE, 0>(a, pa.N, node, pa.st0, pa.e0, out, plane); break;
+        case 1: rod_row<MODE, 1>(a, pa.N, node, pa.st0, pa.e0, out, plane); break;
+        case 2: rod_row<MODE, 2>(a, pa.N, node, pa.st0, pa.e0, out, plane); break;
+        default: rod_row<MODE, 3>(a, pa.N, node, pa.st0, pa.e0, out, plane); break;
+      }
+    }
+    __syncthreads();
+    count_units(a.units, pb.due);
+    int sys = -1;
+    unsigned long long res = 0;
+    if (pb.due) {
+      const double *in = sm + (t & 3) * pitch + (t >> 2);
+      const double idt = a.idt, cd = c < 3 ? damp : 0.0;
+      if (MODE != 1) {
+        double row[11];
+#pragma unroll
+        for (int d = 0; d < 11; ++d) row[d] = in[d * plane];
+        if (c < 3) row[0] += cd;
+        row[0] += m * idt * idt;
+#pragma unroll
+        for (int d = 1; d < 11; ++d)
+          if ((fixed & 1u) || pb.r < d || ((fixed >> d) & 1u)) row[d] = 0.0;
+        if (fixed & 1u) row[0] = 1.0;
+#pragma unroll
+        for (int d = 0; d < 11; ++d) a.band[(size_t)d * a.nd + i] = row[d];
+      }
+      if (MODE != 2) {
+        double G = in[11 * plane];
+        if (c < 3) {
+          G = fma(-m, a.g[c], G);
+          G = fma(cd, dq, G);
+        }
+        if (a.fc) G -= fc;
+        double f = m * idt * idt * dq - m * idt * vn + G;
+        if (fixed & 1u) f = 0.0;
+        a.f[i] = f;
+        sys = pb.sys;
+        res = (unsigned long long)__double_as_longlong(fabs(f) * rscale);
+      }
+    }
+    if (MODE != 2) max_residual(a.sys_res, sys, res);
+    __syncthreads();
   }
 }
-__global__ void __launch_bounds__(256) k_rows_rod_res(RowArgs a) {
-  for (int b0 = blockIdx.x * blockDim.x; b0 < a.nd; b0 += gridDim.x * blockDim.x) {
-    int sys;
-    const unsigned long long r = k_rows_rod_one<1>(a, b0 + threadIdx.x, sys);
-    max_residual(a.sys_res, sys, r);
-  }
+
+__global__ void __launch_bounds__(kRowThreads, 4) k_rows_rod(RowArgs a) {
+  __shared__ double sm[12 * 4 * (kRowThreads / 4 + 4)];
+  rows_rod<0>(a, sm);
 }
-__global__ void __launch_bounds__(256) k_rows_rod_band(RowArgs a) {
-  for (int b0 = blockIdx.x * blockDim.x; b0 < a.nd; b0 += gridDim.x * blockDim.x) {
-    int sys;
-    k_rows_rod_one<2>(a, b0 + threadIdx.x, sys);
-  }
+__global__ void __launch_bounds__(kRowThreads) k_rows_rod_res(RowArgs a) {
+  __shared__ double sm[12 * 4 * (kRowThreads / 4 + 4)];
+  rows_rod<1>(a, sm);
+}
+__global__ void __launch_bounds__(kRowThreads, 4) k_rows_rod_band(RowArgs a) {
+  __shared__ double sm[12 * 4 * (kRowThreads / 4 + 4)];
+  rows_rod<2>(a, sm);
 }
 
 // Line search (optional): Armijo test on the 2-norm of the scaled residual
