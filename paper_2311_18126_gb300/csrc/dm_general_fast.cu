@@ -49,9 +49,16 @@ static_assert(kLimbExtra == 11 * kRow + kLBlk * kLRec + 12 + kSmall && kLimbExtr
 static_assert(kFastMaxRows <= 32 * 2 * kLBlk * kLRec, "a bit per row fits the records");
 constexpr unsigned kFull = 0xffffffffu;
 
-// Pivots of the border system's elimination in order smaller than this
-// fraction of their original diagonal entry send it to partial pivoting.
-constexpr double kTinyPivotB = 1e-13;
+// Pivots of an elimination in order smaller than 2^-43 of their starting
+// diagonal entry, or not finite, send it to partial pivoting; the test compares
+// the upper words (exponent and 20 mantissa bits), off the FP64 pipe.
+__device__ __forceinline__ int pivot_floor(double d) {
+  return max((__double2hiint(d) & 0x7FFFFFFF) - (43 << 20), 1 << 20);
+}
+__device__ __forceinline__ bool pivot_ok(double v, int floor) {
+  const int h = __double2hiint(v) & 0x7FFFFFFF;
+  return h >= floor && h < 0x7FF00000;
+}
 
 __device__ __forceinline__ double limb_recip(double d) { return rcp_any(d); }
 
@@ -188,13 +195,13 @@ __device__ __forceinline__ void limb_column(const LimbLane &ln, const int t, con
     }
   __syncwarp();
   v[0] = fma(-lsm(ln.lo[t][0]), uq[0], dv[0]);
+  v[1] = fma(-lsm(ln.lo[t][1]), uq[1], dv[1]);
   RcpChain ch;
   ch.seed(__shfl_sync(kFull, v[0], 0));
-  v[1] = fma(-lsm(ln.lo[t][1]), after(uq[1], ch.S, zero), dv[1]);
+  if (NK > 2) v[2] = fma(-lsm(ln.lo[t][2]), after(uq[2], ch.S, zero), dv[2]);
   ch.residual();
-  if (NK > 2) v[2] = fma(-lsm(ln.lo[t][2]), after(uq[2], (unsigned)ch.t, zero), dv[2]);
+  if (NK > 3) v[3] = fma(-lsm(ln.lo[t][3]), after(uq[3], (unsigned)ch.t, zero), dv[3]);
   rj = ch.result();
-  if (NK > 3) v[3] = fma(-lsm(ln.lo[t][3]), after(uq[3], (unsigned)__double2loint(rj), zero), dv[3]);
   if (act) {
 #pragma unroll
     for (int h = 0; h < 4; ++h)
@@ -371,14 +378,12 @@ __global__ void __launch_bounds__(128) k_gen_limb_factor(SolveGenArgs a) {
       const int r = e / (nbc + 1);
       M[(m + r) * ldm + m + e - r * (nbc + 1)] = 0.0;
     }
-    // the test in the upper words: exponent and 20 mantissa bits
-    const int thr = lane < m ? max((__double2hiint(A[(ne + lane) * kRow + 10]) & 0x7FFFFFFF) - (43 << 20), 1 << 20) : 0;
+    const int thr = lane < m ? pivot_floor(A[(ne + lane) * kRow + 10]) : 0;
     __syncwarp();
     bool ok = true;
     for (int c = 0; c < m; ++c) {
       const double pv = M[c * ldm + c];
-      const int ph = __double2hiint(pv) & 0x7FFFFFFF;
-      if (ph < __shfl_sync(kFull, thr, c) || ph >= 0x7FF00000) {
+      if (!pivot_ok(pv, __shfl_sync(kFull, thr, c))) {
         ok = false;  // uniform
         break;
       }
@@ -459,7 +464,7 @@ __global__ void __launch_bounds__(128) k_gen_limb_factor(SolveGenArgs a) {
 // elimination in order, the trailing update spread over all threads (one
 // matrix entry per thread and step) and the next pivot's reciprocal taken by
 // the thread that updates it, so one barrier per column; a pivot below
-// kTinyPivotB of its original diagonal entry restarts the elimination with
+// 2^-43 of its original diagonal entry restarts the elimination with
 // partial pivoting (the pivot search, row swap and multipliers by warp 0).
 // Then a column-oriented back substitution by warp 0 with the right-hand
 // sides in registers (rows lane, lane + 32, lane + 64).
@@ -504,7 +509,8 @@ __global__ void __launch_bounds__(kGenBorderThreads) k_gen_border(SolveGenArgs a
   bool bad = flag[1] != 0;
   const int nB = a.gs_nB[w];
   const int ld = nB + 1;
-  double *S = sm, *rinv = sm + (size_t)nB * ld, *lm = rinv + nB, *dorig = lm + nB;
+  double *S = sm, *rinv = sm + (size_t)nB * ld, *lm = rinv + nB;
+  int *least = reinterpret_cast<int *>(lm + nB);  // per row: the smallest pivot taken
   const int32_t *bd = a.border_dof + a.gs_border0[w];
   double *J = a.gen + a.gs_JBB[w];
   double *acc = a.gen + a.gs_rB[w];
@@ -522,16 +528,16 @@ __global__ void __launch_bounds__(kGenBorderThreads) k_gen_border(SolveGenArgs a
   if (go && !bad && nB > 0) {
     load();
     __syncthreads();
-    for (int b = tid; b < nB; b += nt) dorig[b] = fabs(S[b * ld + b]);
+    for (int b = tid; b < nB; b += nt) least[b] = pivot_floor(S[b * ld + b]);
     if (tid == 0) flag[3] = 1;
     __syncthreads();
     // first attempt: elimination in order, without pivoting; the thread that
     // updates the next pivot takes its reciprocal (one barrier per column).
-    // A pivot below kTinyPivotB of its original diagonal entry, or not
+    // A pivot below 2^-43 of its original diagonal entry, or not
     // finite, abandons it for partial pivoting.
     if (tid == 0) {
       const double v = S[0];
-      if (!(fabs(v) > kTinyPivotB * dorig[0]) || !isfinite(v)) flag[3] = 0;
+      if (!pivot_ok(v, least[0])) flag[3] = 0;
       else rinv[0] = limb_recip(v);
     }
     __syncthreads();
@@ -545,7 +551,7 @@ __global__ void __launch_bounds__(kGenBorderThreads) k_gen_border(SolveGenArgs a
         const double v = fma(-(S[i * ld + j] * rp), S[j * ld + c], S[i * ld + c]);
         S[i * ld + c] = v;
         if (r == 0 && c == j + 1) {
-          if (!(fabs(v) > kTinyPivotB * dorig[j + 1]) || !isfinite(v)) flag[3] = 0;
+          if (!pivot_ok(v, least[j + 1])) flag[3] = 0;
           else rinv[j + 1] = limb_recip(v);
         }
       }
