@@ -133,7 +133,8 @@ typedef struct dm_params {
                            committed at q_{n+1}.  The step adjoint rejects it. */
   int32_t long_rod_dofs; /* single rods with at least this many DOFs are solved
                            by the partitioned band solve (dm_solve_band_
-                           partitioned, interiors of 502 rows) instead of the
+                           partitioned, interiors of 128 to 2048 rows by the
+                           rods' and the batch's size) instead of the
                            twisted LDL^T chain; 0 = 2048 (512 nodes),
                            negative = never */
   int32_t predictor;    /* Newton's starting guess (the paper leaves it open;
@@ -251,10 +252,10 @@ dm_status dm_solve_band(int32_t nsys, const int32_t *sys_dof0, const int32_t *sy
 /* The same solve for long systems (rods of thousands of nodes), without
  * the sequential chain over the whole system: each system is cut into
  * interiors of part_rows - 10 rows separated by 10-row separators (interiors
- * do not couple); a warp per interior factors it (band L D L^T) and forms
- * its Schur contributions to the neighbouring separators (forward solves
- * only, by symmetry), a warp per system solves the block-tridiagonal
- * separator system (10 x 10 blocks, Gauss-Jordan), and a warp per interior
+ * do not couple); a warp per interior eliminates it with the coupling to its
+ * upper separator carried along, which leaves its Schur contributions to
+ * both separators, a block of four warps per system solves the
+ * block-tridiagonal separator system (10 x 10 blocks), and a warp per interior
  * back-substitutes.  Arguments and batch rules as dm_solve_band, plus
  * part_rows (0 = 512; otherwise 21..1024).  Nothing is pivoted: interiors
  * and separator blocks are eliminated in order, like the full band, and a
@@ -400,7 +401,7 @@ dm_status dm_ws_column_stats(const float *data, int64_t rows, int32_t cols, floa
  * and its output gradients are written to its first copy (zeros in the
  * others), so that outputs can be fed back as inputs.  is_device: the
  * pointers are device (1) or host (0) memory.  Rods with edge-edge contact
- * solve J^T lambda with the transposed dense-band LU of the contact path;
+ * solve J^T lambda with the transposed tiled LU of the contact path;
  * edge-edge friction (pair_mu != 0), and networks with a limb jointed at
  * both ends, are rejected (DM_ERR_INVALID_ARG); the ground friction
  * force's dependence on x_n enters
@@ -540,7 +541,7 @@ const char *dm_kernel_name(int32_t id); /* "" for unused ids */
  * "f" (residual, DOF order), "sg"/"sh" (stencil gradients [11][Ns] and packed
  * Hessians [66][Ns]), "es" (stretch force/Hessian [9][Ne]), "ef" (edge frames
  * [13][Ne]), "nt" (node contact terms [12][Nn]), "gen" (general-path matrix
- * storage).  Synchronises the stream.  Not part of the solve. */
+ * storage; limbs of the condensation path keep no band).  Synchronises the stream.  Not part of the solve. */
 dm_status dm_debug_copy(dm_system *sys, const char *name, double *out, int64_t n);
 
 /* Measures the FP64 FMA throughput of the current device (GFLOP/s, an FMA

@@ -548,10 +548,10 @@ static dm_status create_impl(const dm_system_desc *desc, const dm_params *prm,
     for (size_t L = 0; L < T.lb_n.size(); ++L)
       if (T.gs_fast[T.lb_gsys[L]]) s->x.limb_nmax = std::max(s->x.limb_nmax, T.lb_n[L]);
     {
-      // warps per block: up to 4, within 200 KB of shared memory per block
+      // warps per block: up to 4, within a block's shared memory
       const size_t pf = gen_factor_smem(s->x.limb_nmax) * sizeof(double);
       const size_t pb = gen_back_smem() * sizeof(double);
-      s->x.wpb_factor = (int)std::max<size_t>(1, std::min<size_t>(4, (200 << 10) / pf));
+      s->x.wpb_factor = (int)std::max<size_t>(1, std::min<size_t>(4, (226 << 10) / pf));
       s->x.wpb_back = (int)std::max<size_t>(1, std::min<size_t>(4, (200 << 10) / pb));
       s->x.wpb_factor_max = s->x.wpb_factor;
       s->x.wpb_back_max = s->x.wpb_back;
