@@ -725,17 +725,20 @@ __device__ __forceinline__ bool factor_tile(double (*D)[kNB + 1], double *R) {
 }
 
 // The blocks of a system meet (all of them are resident: a cooperative launch
-// when there are several).  False: a wait ran out, or (`check`) a zero pivot.
+// when there are several): a release by thread 0 after the block's barrier, an
+// acquire before the next; work between the two calls needs nothing of the
+// other blocks.  lu_wait: false if a wait ran out, or (`check`) at a zero pivot.
 constexpr int kSpinLimit = 1 << 22;  // a few seconds
-__device__ __forceinline__ bool lu_barrier(int32_t *bar, int32_t *bad, int blocks, int &target, bool check) {
-  __shared__ int ok;
+__device__ __forceinline__ void lu_arrive(int32_t *bar, int blocks, int &target) {
   __syncthreads();
+  target += blocks;
+  if (threadIdx.x == 0 && blocks > 1) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(bar) : "memory");
+}
+__device__ __forceinline__ bool lu_wait(int32_t *bar, int32_t *bad, int blocks, int target, bool check) {
+  __shared__ int ok;
   if (threadIdx.x == 0) {
     int fine = 1;
     if (blocks > 1) {
-      target += blocks;
-      __threadfence();
-      atomicAdd(bar, 1);
       int seen = 0, spins = 0;
       do {
         asm volatile("ld.acquire.gpu.s32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
@@ -744,7 +747,6 @@ __device__ __forceinline__ bool lu_barrier(int32_t *bar, int32_t *bad, int block
         atomicExch(bad, 1);
         fine = 0;
       }
-      __threadfence();
     }
     // (a zero pivot is written before the barrier that follows its panel, and
     // none while any block is between that barrier and the next)
@@ -777,14 +779,14 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
   const int levels = lev[kLevelInts - 1];
   const auto fronts = [&](int I) { return (reach[I >> 2] >> (8 * (I & 3))) & 0xffu; };
   const int blocks = gridDim.x;
-  int target = 0;
-  for (int l = 0; l < levels; ++l) {
+  int target = 0, items = 0, vecs = 0;
+  // level l's record, its fronts' neighbours and who neighbours whom
+  const auto load_level = [&](int l) {
     if (tid < 1 + 2 * kFronts) reinterpret_cast<int *>(&lv)[tid] = lev[l * kLevelInts + tid];
     for (int e = tid; e < (nt + 3) / 4; e += kLuThreads) reach[e] = 0;
     __syncthreads();
-    const int nf = lv.nf;
-    int items = 0, vecs = 0;
-    for (int f = 0; f < nf; ++f) {
+    items = vecs = 0;
+    for (int f = 0; f < lv.nf; ++f) {
       const uint16_t *src = adj + (size_t)lv.k[f] * nt;
       for (int e = tid; e < lv.m[f]; e += kLuThreads) {
         const int I = src[e];
@@ -795,6 +797,10 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
       vecs += lv.m[f];
     }
     __syncthreads();
+  };
+  load_level(0);
+  for (int l = 0; l < levels; ++l) {
+    const int nf = lv.nf;
 
     // panel: the blocks are dealt to the fronts by their vectors (rows of L,
     // columns of U, the right-hand side: a warp each), so that a block factors
@@ -873,7 +879,8 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
       }
     }
     if (l + 1 == levels) return;  // (the last level has no neighbours left)
-    if (!lu_barrier(a.lu_bar + c, a.cbad + c, blocks, target, true)) return;
+    lu_arrive(a.lu_bar + c, blocks, target);
+    if (!lu_wait(a.lu_bar + c, a.cbad + c, blocks, target, true)) return;
 
     // update, by half a block: quarter items (16 x 16 of a tile), front by front,
     // then the right-hand side's rows; a tile or row of several fronts belongs to the
@@ -927,7 +934,9 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
       }
       if (in) *p = old - acc;
     }
-    if (!lu_barrier(a.lu_bar + c, a.cbad + c, blocks, target, false)) return;
+    lu_arrive(a.lu_bar + c, blocks, target);
+    load_level(l + 1);  // (its own shared memory only)
+    if (!lu_wait(a.lu_bar + c, a.cbad + c, blocks, target, false)) return;
   }
 }
 
