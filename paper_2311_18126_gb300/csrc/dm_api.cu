@@ -966,6 +966,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     }
     if (ls_on) {
       if (gen_on) k_line_search_loop<<<S * kLoopBlocks, kLineSearchThreads, 0, rs>>>(la, lb);
+      else if (s->x.cc.max_n > 1024) k_line_search_wide<<<S, kLineSearchWide, 0, rs>>>(la);
       else k_line_search<<<S, kLineSearchThreads, 0, rs>>>(la);
       if (ws_trial && it == 0) DM_CK(ws_inject(s, rs, s->x.ls_action, s->x.ls_trial));
     }
@@ -994,7 +995,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     }
     if (contact_on) {
       Timed t(s, K_SOLVE_CONTACT, rs);
-      k_cc_band<<<blocks(nd, 256), 256, 0, rs>>>(ca, d.f, d.dq);
+      k_cc_band<<<blocks(nd, 64), 64, 0, rs>>>(ca, d.f, d.dq);
       k_cc_decide<<<blocks(s->x.cc.n_contact, 128), 128, 0, rs>>>(ca, va);
       DM_CK(lu_solve(ca, va, s->x.sms, rs));
     }
@@ -1922,7 +1923,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     std::vector<int32_t> onec(nc, 1);
     DM_CK(cudaMemcpyAsync(ca.cgo, onec.data(), nc * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     DM_CK(cudaMemsetAsync(ca.cbad, 0, nc * sizeof(int32_t), st));
-    k_cc_band<<<blocks(nd, 256), 256, 0, st>>>(ca, nrhs, d.dq);
+    k_cc_band<<<blocks(nd, 64), 64, 0, st>>>(ca, nrhs, d.dq);
     k_cc_transpose<<<dim3(blocks(s->x.cc.max_n, kNB), nc), 256, 0, st>>>(ca);
     if (!A.ints) DM_TRY(dalloc(s, &A.ints, 6 * (size_t)S + 2 * (size_t)std::max(ngen, 1) + 8));
     int32_t *its = A.ints, *sts = its + S, *ctl = sts + S;

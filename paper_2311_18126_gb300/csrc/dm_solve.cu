@@ -201,12 +201,13 @@ __global__ void __launch_bounds__(kRowThreads, 4) k_rows_rod_band(RowArgs a) {
 // |f_i| / (D_i l_i) of each system (the Newton direction is a descent
 // direction for it); a trial point without sufficient decrease is pulled
 // halfway back to the last accepted iterate, at most 12 times.  One block
-// of kLineSearchThreads per system: the merit in a fixed summation order
-// (per-thread strided sums, then a fixed tree: deterministic), the decision
-// by thread 0, then the move (or the new accepted iterate) over the
-// system's DOFs.
-__global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchArgs a) {
-  __shared__ double part[kLineSearchThreads / 32];
+// per system: the merit in a fixed summation order (per-thread strided sums,
+// then a fixed tree: deterministic), the decision by thread 0, then the move
+// (or the new accepted iterate) over the system's DOFs.  128 threads, 512 for
+// contact systems of over 1024 DOFs (a coil of 1999: 22 us with 128, 8 with 512).
+template <int T>
+__device__ __forceinline__ void line_search(const LineSearchArgs &a) {
+  __shared__ double part[T / 32];
   __shared__ int s_action;
   __shared__ double s_alpha;
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -219,13 +220,13 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   double qv[U], qa[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int i = tid + u * kLineSearchThreads;
+    const int i = tid + u * T;
     qv[u] = i < n ? a.q[d0 + i] : 0.0;
     qa[u] = i < n ? a.qacc[d0 + i] : 0.0;
   }
   double acc = 0.0;
 #pragma unroll 4
-  for (int i = tid; i < n; i += kLineSearchThreads) {
+  for (int i = tid; i < n; i += T) {
     const double v = a.f[d0 + i] * a.rscale[d0 + i];
     acc = fma(v, v, acc);
   }
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   if (tid == 0) {
     double tot = 0.0;
 #pragma unroll
-    for (int w = 0; w < kLineSearchThreads / 32; ++w) tot += part[w];
+    for (int w = 0; w < T / 32; ++w) tot += part[w];
     const double m = sqrt(tot);
     a.merit[s] = m;
     const int action = line_search_decide(m, ls);
@@ -254,15 +255,22 @@ __global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchAr
   const double alpha = s_alpha;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int i = tid + u * kLineSearchThreads;
+    const int i = tid + u * T;
     if (i >= n) break;
     if (action == 1) a.q[d0 + i] = alpha == 0.0 ? qa[u] : 0.5 * (qv[u] + qa[u]);
     else a.qacc[d0 + i] = qv[u];
   }
-  for (int i = d0 + tid + U * kLineSearchThreads; i < d0 + n; i += kLineSearchThreads) {
+  for (int i = d0 + tid + U * T; i < d0 + n; i += T) {
     if (action == 1) a.q[i] = alpha == 0.0 ? a.qacc[i] : 0.5 * (a.q[i] + a.qacc[i]);
     else a.qacc[i] = a.q[i];
   }
+}
+
+__global__ void __launch_bounds__(kLineSearchThreads) k_line_search(LineSearchArgs a) {
+  line_search<kLineSearchThreads>(a);
+}
+__global__ void __launch_bounds__(kLineSearchWide) k_line_search_wide(LineSearchArgs a) {
+  line_search<kLineSearchWide>(a);
 }
 
 }  // namespace dm
