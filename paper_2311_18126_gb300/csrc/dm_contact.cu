@@ -551,10 +551,10 @@ __global__ void __launch_bounds__(256) k_cc_clear(ContactArgs a) {
 // neighbours) has 24, a gripper of five 60-node fingers (38) has 8.  The
 // diagonal tile's 32 dependent columns run on four warps (one per SM
 // partition).
-// Measured (GB300): a level 45 k cycles and up -- the diagonal tile 23 k, its
-// solves 7 k, the two meetings 4 k each, the update from 6 k (few tiles) to 85 k
+// Measured (GB300): a level 42 k cycles and up -- the diagonal tile 23 k, its
+// solves 7 k, the two meetings 3 k each, the update from 6 k (few tiles) to 85 k
 // (2400 quarters: the FP64 pipes' rate); factorisation and solve of the coil 2.8
-// -> 1.1 ms, of four grippers 1.8 -> 0.4 ms (before: tile columns in their
+// -> 1.0 ms, of four grippers 1.8 -> 0.4 ms (before: tile columns in their
 // order, two launches for each; before that, the full bandwidth: 9 and 21 ms).
 
 __global__ void k_cc_decide(ContactArgs a, SolveArgs v) {

@@ -25,10 +25,11 @@
 // reciprocal on the integer pipe; a pivot outside [2^-126, 2^126) (zero and
 // non-finite included) fails the system.  The back substitution keeps the
 // pending rows in lane registers: one update and one shuffle per row.
-// Measured, 1024 star robots of 3 to 8 limbs of 112 rows, a step of 63 rounds:
-// limb kernels and border 7.6 ms, assembly of the couplings 3.9 -> 1.6 ms (the
-// limbs' bands are no longer stored), back substitution 1.8 -> 1.3 ms; step
-// 22.7 -> 17.9 ms together with the residual's maximum by the warp.
+// Measured, 1024 star robots of 3 to 8 limbs of 112 rows, every robot active:
+// factor 424 -> 330 us, border 81 -> 69 us, back substitution 102 -> 60 us,
+// assembly of the couplings 352 -> 86 us (the limbs' bands are no longer
+// stored); a round of few robots: a limb 89 k cycles, 58 k of them its 104
+// columns (560 each), 12 k the coupled block, 10 k forming the rows.
 //
 // The Jacobian is that of Sec. III-C (M/dt^2 - dF/dq, with the contact and
 // friction terms of Sec. III-B), not symmetric when friction acts, hence LU.
