@@ -532,6 +532,7 @@ __global__ void __cluster_dims__(kLoopBlocks, 1, 1) __launch_bounds__(kLineSearc
   const int d0 = a.sys_dof0[s], n = a.sys_ndof[s];
   const bool small = b.rows.sys_kind[s] == SOLVE_GENERAL && n <= kLoopDofs;
   LineState ls{a.trial[s], a.nback[s], a.wstry ? a.wstry[s] : 0, a.alpha[s], a.racc[s]};
+  cluster.sync();  // every block has the state before the first block writes the new one
   const int e0 = b.edge_ptr[s], ne = b.edge_ptr[s + 1] - e0, v0 = b.node_ptr[s];
   const int nv = b.rows.nt ? b.node_ptr[s + 1] - v0 : 0, k0 = b.st_ptr[s], nk = b.st_ptr[s + 1] - k0;
   const int nk32 = (nk + 31) & ~31;
