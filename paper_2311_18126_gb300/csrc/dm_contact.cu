@@ -1063,18 +1063,23 @@ cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStre
   const int words = nt * ((nt + 31) / 32), threads = std::max(512, (nt + 31) / 32 * 32);
   k_lu_order<<<nc, threads, 4 * words, st>>>(a);
   // the chip shared among the systems; several blocks of a system wait for one
-  // another, so all of them must be resident (two per SM fit)
+  // another, so all of them must be resident (one per SM), which a cooperative
+  // launch guarantees; without such launches one block per system
+  int dev = 0, coop = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t cfg{};
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cfg.stream = st;
-  const int share = std::max(1, std::min(sms / nc, 4 * nt * nt));
+  const int share = coop ? std::max(1, std::min(sms / nc, 4 * nt * nt)) : 1;
   cfg.gridDim = dim3(share, nc);
   cfg.blockDim = dim3(kLuThreads);
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = share > 1 ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_lu, a, v.dq);
+  e = cudaLaunchKernelEx(&cfg, k_lu, a, v.dq);
   if (e != cudaSuccess) return e;
   // a cluster of up to eight blocks while the systems leave SMs idle
   int cs = 8;
