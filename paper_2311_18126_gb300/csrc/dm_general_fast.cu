@@ -150,6 +150,15 @@ namespace {
 // the lane's first.
 __host__ __device__ constexpr int limb_slots(int R) { return (R * (R + 1) + 31) / 32; }
 
+// Columns of a limb before the first one with ten rows below it: that is an x
+// (rod row 0 mod 4) of a limb eliminated from its first row, a z (2 mod 4) of
+// one eliminated from its last.  Limbs with a free end start there (rods have
+// 4 N - 1 rows); one whose border was fixed away starts at the twist angle
+// behind it, with seven rows.
+__host__ __device__ constexpr int limb_lead(int first, int n, int dir) {
+  return dir ? (first + n - 1 + 2) & 3 : (4 - (first & 3)) & 3;
+}
+
 struct LimbLane {
   int to[4][4], uo[4][4], lo[4][4];  // byte offsets by column type: target, U entry, multiplier
   int so, ro;                        // the lane's product with the reciprocal: source, destination
@@ -356,14 +365,22 @@ __global__ void __launch_bounds__(128) k_gen_limb_factor(SolveGenArgs a) {
   const int ne = n - m;  // rows eliminated inside the limb
   bool bad = false;
   double rj = rcp_any(A[10]);
-  for (int j0 = 0; j0 < ne; j0 += kLBlk) {
-#pragma unroll
-    for (int u = 0; u < kLBlk; ++u) limb_column(ln, u & 3, u, w0 + 8 * kRow * j0, rj, j0 + u < ne, a.zero);
-    const int cnt = min(kLBlk, ne - j0);
+  // after columns j0 .. j0 + cnt - 1: their pivots' range, their records
+  const auto finish = [&](int j0, int cnt) {
     if (lane < cnt && !rcp64_in_range(A[(j0 + lane) * kRow + 10])) bad = true;
     for (int e = lane; e < cnt * (kLRec / 2); e += 32)
       *reinterpret_cast<double2 *>(U + (size_t)j0 * kLRec + 2 * e) = *reinterpret_cast<const double2 *>(rec + 2 * e);
     __syncwarp();
+  };
+  // the columns before the envelope's first one of ten rows, with all ten rows
+  const int lead = min(limb_lead(f, n, dir), ne);
+#pragma unroll 1
+  for (int u = 0; u < lead; ++u) limb_column(ln, 0, u, w0, rj, true, a.zero);
+  if (lead > 0) finish(0, lead);
+  for (int j0 = lead; j0 < ne; j0 += kLBlk) {
+#pragma unroll
+    for (int u = 0; u < kLBlk; ++u) limb_column(ln, u & 3, u, w0 + 8 * kRow * j0, rj, j0 + u < ne, a.zero);
+    finish(j0, min(kLBlk, ne - j0));
   }
   bad = __any_sync(kFull, bad);
   if (!bad && m > 0) {
