@@ -26,7 +26,7 @@
 // Measured: inference of 444544 rows 233 -> 164 us (0.9 PFLOP/s; a tile 13.6 k
 // cycles, 5.1 k of them tensor work, 2.6 k waits for weights with two 32 KB
 // blocks in flight, 3.1 k for epilogues where the short first and last layers
-// meet); a training step of 16384 rows 548 -> 75 us.
+// meet); a training step of 16384 rows 548 -> 77 us.
 // Training keeps the ReLU masks in registers, forms the loss and its gradient
 // in the output epilogue, and stores the hidden activations and the gradients
 // of every layer row-major by TMA (k_mlp_wgrad reads them as they are, with
@@ -702,34 +702,45 @@ namespace {
 // batch rows per stage: both operands are [batch][width] arrays whose width is
 // the MMA's M or N, so the descriptors are MN-major (64-wide boxes with the
 // 128-byte swizzle: 8 batch rows of 128 bytes per swizzle group, the boxes
-// 8 KB apart).  The hidden biases' gradients are the same product with a
-// column of ones (N = 16, one small extra MMA).  Partials per share, summed in
+// 8 KB apart).  The tensor core truncates as it accumulates: sums of one sign
+// over 2^15 rows in one chain were off by 1e-6 to 1e-5 of their size.  So a
+// chain ends after kGSeg stages (512 rows), and eight epilogue warps add it to
+// the sums in their registers (FP32, rounded to nearest) while the next one
+// fills the other half of the tensor memory; they also sum the hidden biases'
+// gradients, the columns of dZ, from the stages (errors now 1e-7 whatever the
+// batch; a step of 16384 rows 74.5 -> 77.4 us).  Partials per share, summed in
 // a fixed order by k_mlp_update.
 constexpr int kGStages = 4;
+constexpr int kGSeg = 8;                        // stages of a chain
+constexpr int kGWarps = 8;                      // epilogue warps; then the MMA and the TMA warp
+constexpr int kGThreads = 32 * (kGWarps + 2);
 constexpr int kGBox = 64 * 128;                 // bytes of a 64 x 64 box
 constexpr int kGStageBytes = 6 * kGBox;         // 2 boxes of M, up to 4 of N
-constexpr int kGOffOnes = kGStages * kGStageBytes;
-constexpr int kGOffBar = kGOffOnes + 512;
-constexpr int kSmemGrad = kGOffBar + 8 * (2 * kGStages + 1) + 16 + 1024;
-static_assert(kSmemGrad <= 227 * 1024, "shared memory of the weight-gradient kernel");
+constexpr int kGOffBar = kGStages * kGStageBytes;
+constexpr int kGBars = 2 * kGStages + 5;
+constexpr int kSmemGrad = kGOffBar + 8 * kGBars + 16 + 1024;
+static_assert(kSmemGrad <= 224 * 1024, "shared memory of the weight-gradient kernel");
 
 struct GradMaps {
   CUtensorMap m[4], n[4];  // per layer: the operand along M, along N
 };
 
-__host__ __device__ constexpr uint32_t make_idesc_mn(int M, int N, bool b_mn) {
-  return tc::make_idesc(M, N) | (1u << 15) | (b_mn ? 1u << 16 : 0u);
+__host__ __device__ constexpr uint32_t make_idesc_mn(int M, int N) {  // both operands MN-major
+  return tc::make_idesc(M, N) | (1u << 15) | (1u << 16);
 }
 
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kGThreads, 1)
     k_mlp_wgrad(const __grid_constant__ GradMaps maps, int nkb, int s_small, int s_big, float *part, int *err) {
   using namespace tc;
   extern __shared__ char smem_raw[];
   char *smem = reinterpret_cast<char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ float bsum[4][128];  // the bias sums of each quarter of the stages' rows
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kGOffBar);
-  uint64_t *bar_full = bar, *bar_free = bar + kGStages, *bar_done = bar + 2 * kGStages;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_done + 1);
+  // stages full and free; per half of the tensor memory: chain complete, read
+  uint64_t *bar_full = bar, *bar_free = bar + kGStages, *bar_acc = bar + 2 * kGStages, *bar_read = bar_acc + 2;
+  uint64_t *bar_end = bar_acc + 4;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + kGBars);
   volatile int *fail = reinterpret_cast<volatile int *>(tmem_slot + 1);
   // block -> layer, row tile, share z of S
   int u = blockIdx.x, l = 0;
@@ -749,17 +760,25 @@ __global__ void __launch_bounds__(192, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int i = 0; i < 2 * kGStages + 1; ++i) mbar_init(&bar[i], 1);
+    for (int i = 0; i < kGStages; ++i) {
+      mbar_init(&bar_full[i], 1);
+      mbar_init(&bar_free[i], bias ? 1 + kGWarps : 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bar_acc[i], 1);
+      mbar_init(&bar_read[i], kGWarps);
+    }
+    mbar_init(bar_end, 1);
     *fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
-  if (tid < 128) reinterpret_cast<uint32_t *>(smem + kGOffOnes)[tid] = 0x3F803F80u;  // ones, bf16
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
-  if (warp == 5) {
+  float *out = part + mlp_part_offset(l, s_small, s_big) + (size_t)z * mlp_part_size(l);
+  if (warp == kGWarps + 1) {
+    // ---- TMA loads
     if (lane == 0) {
       bool ok = true;
       int g = 0;
@@ -775,57 +794,100 @@ __global__ void __launch_bounds__(192, 1)
         for (int k = g > kGStages ? g - kGStages : 0; k < g; ++k)
           mbar_wait(&bar_full[k % kGStages], (uint32_t)((k / kGStages) & 1));
     }
-  } else if (warp == 4) {
+  } else if (warp == kGWarps) {
+    // ---- MMAs, by one lane
     if (lane == 0) {
-      int g = 0;
-      for (int k = k0; k < k1; ++k, ++g) {
-        const int s = g % kGStages;
-        if (!wait_on(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail)) break;
+      bool ok = true;
+      for (int g = 0; g < k1 - k0 && ok; ++g) {
+        const int s = g % kGStages, seg = g / kGSeg, first = g % kGSeg == 0;
+        if (first && seg > 1 && !(ok = wait_on(&bar_read[seg & 1], (uint32_t)((seg / 2 - 1) & 1), fail))) break;
+        if (!(ok = wait_on(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail))) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
         const uint32_t a0 = smem_u32(smem + s * kGStageBytes), b0 = a0 + 2 * kGBox;
-        const uint32_t o0 = smem_u32(smem + kGOffOnes);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {  // 16 batch rows: two swizzle groups of 1024 bytes
-          const uint64_t ad = make_desc(a0 + 2048 * kk, kGBox, 1024, kSwizzle128B);
-          mma_bf16(tmem, ad, make_desc(b0 + 2048 * kk, kGBox, 1024, kSwizzle128B), make_idesc_mn(128, N, true),
-                   (g | kk) ? 1u : 0u);
-          if (bias) mma_bf16(tmem + 256u, ad, make_desc(o0, 128, 256), make_idesc_mn(128, 16, false), (g | kk) ? 1u : 0u);
-        }
+        for (int kk = 0; kk < 4; ++kk)  // 16 batch rows: two swizzle groups of 1024 bytes
+          mma_bf16(tmem + 256u * (uint32_t)(seg & 1), make_desc(a0 + 2048 * kk, kGBox, 1024, kSwizzle128B),
+                   make_desc(b0 + 2048 * kk, kGBox, 1024, kSwizzle128B), make_idesc_mn(128, N),
+                   first && kk == 0 ? 0u : 1u);
         mma_commit(&bar_free[s]);
+        if (g % kGSeg == kGSeg - 1 || g + 1 == k1 - k0) mma_commit(&bar_acc[seg & 1]);
       }
-      mma_commit(bar_done);
+      if (!ok || *fail) {  // every MMA issued is done before the tensor memory is freed
+        mma_commit(bar_end);
+        mbar_wait(bar_end, 0);
+      }
     }
-  }
-  __syncwarp();
-  // the end of every MMA issued (on a failure too, before the tensor memory is freed)
-  const bool done = mbar_wait(bar_done, 0);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp < 4 && done && !*fail) {
-    // partial: [256 or 64 rows][N] of the layer, then its 256 bias sums
-    float *out = part + mlp_part_offset(l, s_small, s_big) + (size_t)z * mlp_part_size(l);
-    const int row = 128 * mt + 32 * warp + lane;
-    const uint32_t t = tmem + ((uint32_t)(32 * warp) << 16);
-    for (int c = 0; c < N; c += 32) {
-      uint32_t r[32];
-      tmem_ld16_nowait(t + (uint32_t)c, r);
-      tmem_ld16_nowait(t + (uint32_t)c + 16, r + 16);
-      tmem_wait32(r);
-      float4 *o = reinterpret_cast<float4 *>(out + (size_t)row * N + c);
+  } else {
+    // ---- epilogues: warp w has accumulator lanes 32 (w % 4).. and half w / 4 of the columns
+    const int quarter = warp & 3, half = warp >> 2;
+    const uint32_t t = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(half * (N / 2));
+    float acc[4][32];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        o[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
-                           __uint_as_float(r[4 * j + 3]));
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int j = 0; j < 32; ++j) acc[c][j] = 0.0f;
+    // bias columns 2 pair, 2 pair + 1 of rows 16 rg .. 16 rg + 15 of a stage
+    // (a warp reads a row's 128 bytes: no bank conflicts)
+    const int pair = tid & 63, rg = tid >> 6;
+    const char *bcol = smem + (pair >> 5) * kGBox + 16 * rg * 128 + 4 * (pair & 3);
+    const int chunk = (pair & 31) >> 2;
+    float b0 = 0.0f, b1 = 0.0f;
+    bool ok = true;
+    for (int g0 = 0, seg = 0; g0 < k1 - k0; g0 += kGSeg, ++seg) {
+      if (bias)
+        for (int g = g0; g < min(g0 + kGSeg, k1 - k0) && ok; ++g) {
+          const int s = g % kGStages;
+          ok = __all_sync(kFullMask, wait_on(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail));
+          if (!ok) break;
+          uint32_t x[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            x[i] = *reinterpret_cast<const uint32_t *>(bcol + s * kGStageBytes + i * 128 + ((chunk ^ (i & 7)) << 4));
+          warp_arrive(&bar_free[s]);
+          float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            s0 += __uint_as_float(x[i] << 16);
+            s1 += __uint_as_float(x[i] & 0xFFFF0000u);
+          }
+          b0 += s0;
+          b1 += s1;
+        }
+      ok = ok && __all_sync(kFullMask, wait_on(&bar_acc[seg & 1], (uint32_t)((seg / 2) & 1), fail));
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (32 * c >= N / 2) break;  // uniform
+        uint32_t r[32];
+        const uint32_t tc0 = t + 256u * (uint32_t)(seg & 1) + 32u * (uint32_t)c;
+        tmem_ld16_nowait(tc0, r);
+        tmem_ld16_nowait(tc0 + 16u, r + 16);
+        tmem_wait32(r);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[c][j] += __uint_as_float(r[j]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      warp_arrive(&bar_read[seg & 1]);
     }
-    if (bias) {
-      uint32_t r[16];
-      tmem_ld16_nowait(t + 256u, r);
-      tmem_wait();
-      out[(size_t)256 * N + row] = __uint_as_float(r[0]);
+    // partial: [256 or 64 rows][N] of the layer, then its 256 bias sums
+    if (ok) {
+      float4 *o = reinterpret_cast<float4 *>(out + (size_t)(128 * mt + 32 * quarter + lane) * N + half * (N / 2));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (32 * c >= N / 2) break;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          o[8 * c + j] = make_float4(acc[c][4 * j], acc[c][4 * j + 1], acc[c][4 * j + 2], acc[c][4 * j + 3]);
+      }
     }
+    bsum[rg][2 * pair] = b0;
+    bsum[rg][2 * pair + 1] = b1;
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (tid == 0 && (*fail || !done)) atomicExch(err, 1);
+  if (bias && tid < 128) out[(size_t)256 * N + 128 * mt + tid] = (bsum[0][tid] + bsum[1][tid]) + (bsum[2][tid] + bsum[3][tid]);
+  if (tid == 0 && *fail) atomicExch(err, 1);
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
 }
@@ -928,7 +990,7 @@ cudaError_t launch_mlp_train(int M, const void *X, const float *target, int n_va
   if (e != cudaSuccess) return e;
   const TrainArgs ta{target, n_valid, (float)(M * n_valid), (double)(M * n_valid), loss, gb4};
   k_mlp_fused<<<s.ctas, kThreadsF, kSmemFused, st>>>(t, b[0], b[1], b[2], b[3], M / kTM, err, ta);
-  k_mlp_wgrad<<<4 * (s.s_small + s.s_big), 192, kSmemGrad, st>>>(g, M / 64, s.s_small, s.s_big, part, err);
+  k_mlp_wgrad<<<4 * (s.s_small + s.s_big), kGThreads, kSmemGrad, st>>>(g, M / 64, s.s_small, s.s_big, part, err);
   return cudaGetLastError();
 }
 
