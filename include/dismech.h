@@ -344,7 +344,8 @@ dm_status dm_mlp_check(dm_mlp *m);
 dm_status dm_mlp_set_fused(dm_mlp *m, int32_t enable);
 /* One Adam step (learning rate lr; lr = 0 computes gradients only) on the
  * mean squared error against Y [M][out_dim]; grads (device, optional) gets
- * the gradient in the parameter layout, loss the loss before the update. */
+ * the gradient in the parameter layout, loss the loss before the update.  A
+ * step that fails on the device (DM_ERR_CUDA) leaves the network as it was. */
 dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M, float lr,
                             float *grads, double *loss);
 

@@ -60,6 +60,7 @@ struct UpdateArgs {
   int n_gb4;               // rows of gb4
   MlpTrainShape shape;
   float *grads;            // [params], or NULL
+  const int *err;          // set: the partials are not complete, nothing is updated
   float lr, b1, b2, eps, c1, c2;
 };
 
@@ -81,6 +82,7 @@ __device__ __forceinline__ float adam(const UpdateArgs &a, float g, float *p, fl
 // each, 16 threads per column with several loads in flight).
 constexpr int kUpdateThreads = 256, kBiasBlocks = kOut / 16;
 __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
+  if (*a.err) return;
   const int bias_block = (int)blockIdx.x - ((int)gridDim.x - kBiasBlocks);
   if (bias_block >= 0) {
     __shared__ float red[16][17];
@@ -148,7 +150,10 @@ struct dm_mlp {
   uint16_t *act[3] = {}, *dz[3] = {}, *dy = nullptr;
   float *part = nullptr, *gb4 = nullptr;  // partial gradients of the batch's shares
   size_t part_n = 0, gb4_n = 0;
-  double *loss = nullptr;                 // and the error flag behind it
+  // the loss, and behind it the training step's error flag and the one of the
+  // asynchronous forward passes (err), which dm_mlp_check reads and clears
+  double *loss = nullptr;
+  int *train_err = nullptr;
   bool fused = true;  // inference: the fused 4-layer kernel (else a GEMM per layer)
   int *err = nullptr;
   int64_t step = 0;
@@ -323,7 +328,10 @@ dm_status dm_mlp_create(int32_t in_dim, int32_t out_dim, uint64_t seed, void *st
     }
   }
   if (st == DM_OK) st = mlp_alloc(m, &m->loss, 2);
-  if (st == DM_OK) m->err = reinterpret_cast<int *>(m->loss + 1);
+  if (st == DM_OK) {
+    m->train_err = reinterpret_cast<int *>(m->loss + 1);
+    m->err = m->train_err + 1;
+  }
   if (st != DM_OK) {
     dm_mlp_destroy(m);
     return st;
@@ -447,7 +455,7 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   const MlpTrainShape shape = mlp_train_shape(M);
   if (ensure_train(m, M, shape) != DM_OK) return DM_ERR_OOM;
   cudaStream_t st = m->stream;
-  cudaMemsetAsync(m->loss, 0, 16, st);
+  cudaMemsetAsync(m->loss, 0, sizeof(double) + sizeof(int), st);
   const void *W[kLayers], *Wt[kLayers];
   const float *b[kLayers];
   for (int l = 0; l < kLayers; ++l) {
@@ -456,10 +464,10 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
     b[l] = m->b[l];
   }
   void *act[3] = {m->act[0], m->act[1], m->act[2]}, *dz[3] = {m->dz[0], m->dz[1], m->dz[2]};
-  if (launch_mlp_train(M, X, Y, m->out_dim, W, Wt, b, act, dz, m->dy, m->loss, m->part, m->gb4, m->err, st) !=
+  if (launch_mlp_train(M, X, Y, m->out_dim, W, Wt, b, act, dz, m->dy, m->loss, m->part, m->gb4, m->train_err, st) !=
       cudaSuccess)
     return DM_ERR_CUDA;
-  m->step += 1;
+  const float step = (float)(m->step + 1);  // counted once it has succeeded
   UpdateArgs a{};
   for (int l = 0; l < kLayers; ++l) {
     a.W[l] = m->W[l]; a.b[l] = m->b[l]; a.mW[l] = m->mW[l]; a.vW[l] = m->vW[l];
@@ -471,25 +479,27 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   a.n_gb4 = 4 * shape.ctas;
   a.shape = shape;
   a.grads = grads_out;
+  a.err = m->train_err;
   a.lr = lr;
   a.b1 = 0.9f;
   a.b2 = 0.999f;
   a.eps = 1e-8f;
-  a.c1 = 1.0f - std::pow(a.b1, (float)m->step);
-  a.c2 = 1.0f - std::pow(a.b2, (float)m->step);
+  a.c1 = 1.0f - std::pow(a.b1, step);
+  a.c2 = 1.0f - std::pow(a.b2, step);
   size_t params = 0;
   for (int l = 0; l < kLayers; ++l) params += mlp_part_size(l);
   k_mlp_update<<<nb((int64_t)params, kUpdateThreads) + kBiasBlocks, kUpdateThreads, 0, st>>>(a);
   struct {
     double loss;
-    int err[2];
+    int err, other;
   } h = {};
-  static_assert(sizeof(h) == 16, "loss and error flag");
+  static_assert(sizeof(h) == 16, "loss and error flags");
   cudaMemcpyAsync(&h, m->loss, 16, cudaMemcpyDeviceToHost, st);
-  if (cudaStreamSynchronize(st) != cudaSuccess || h.err[0]) {
+  if (cudaStreamSynchronize(st) != cudaSuccess || h.err) {
     set_error("dm_mlp_train_step: CUDA error or tensor-core barrier timeout");
     return DM_ERR_CUDA;
   }
+  m->step += 1;
   if (loss_out) *loss_out = h.loss;
   return DM_OK;
 }
