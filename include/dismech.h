@@ -56,7 +56,8 @@ typedef enum dm_status {
                                in the rod and limb eliminations, outside
                                [2^-126, 2^126), the reciprocal's range)     */
   DM_ERR_PENETRATION = 5,   /* edge-edge distance D <= 0 (Eq. 10 undefined)  */
-  DM_ERR_CUDA = 6,          /* a CUDA runtime call failed                    */
+  DM_ERR_CUDA = 6,          /* a CUDA runtime call failed, or a bounded wait
+                               inside a kernel ran out                       */
   DM_ERR_OOM = 7            /* device allocation failed                      */
 } dm_status;
 

@@ -1192,7 +1192,8 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       DM_CK(cudaStreamSynchronize(st));
       if (stats) stats->first_failed = first;
       set_error("step " + std::to_string(step) + ": system " + std::to_string(first) +
-                " failed with status " + std::to_string(code));
+                " failed with status " + std::to_string(code) +
+                (code == DM_ERR_CUDA ? " (a wait inside its solve ran out)" : ""));
       return (dm_status)code;
     }
     DM_CK(ws_keep_velocity(s, st));
@@ -1939,8 +1940,12 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     DM_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
     DM_CK(cudaStreamSynchronize(st));
     if (h[1] > 0) {
-      set_error("dm_step_adjoint: zero or non-finite pivot in the transposed contact solve");
-      bs = DM_ERR_DEGENERATE;
+      int32_t code = 0;  // of the first system that failed
+      DM_CK(cudaMemcpyAsync(&code, sts + h[2], sizeof(code), cudaMemcpyDeviceToHost, st));
+      DM_CK(cudaStreamSynchronize(st));
+      set_error(code == DM_ERR_CUDA ? "dm_step_adjoint: a wait inside the transposed contact solve ran out"
+                                    : "dm_step_adjoint: zero or non-finite pivot in the transposed contact solve");
+      bs = (dm_status)code;
     }
   }
   // the system stays at step n whatever happened

@@ -735,6 +735,10 @@ __device__ __forceinline__ bool factor_tile(double (*D)[kNB + 1], double *R) {
   return exact || !__syncthreads_or(warp == 0 && !rcp64_in_range(D[lane][lane]));
 }
 
+// Why a system's factorisation stopped (cbad): a pivot that is zero or not
+// finite, or a wait between its blocks that ran out, which goes before.
+constexpr int kLuZeroPivot = 1, kLuTimeout = 2;
+
 // The blocks of a system meet (all of them are resident: a cooperative launch
 // when there are several): a release by thread 0 after the block's barrier, an
 // acquire before the next; work between the two calls needs nothing of the
@@ -755,7 +759,7 @@ __device__ __forceinline__ bool lu_wait(int32_t *bar, int32_t *bad, int blocks, 
         asm volatile("ld.acquire.gpu.s32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
       } while (seen < target && ++spins < kSpinLimit);
       if (seen < target) {
-        atomicExch(bad, 1);
+        atomicMax(bad, kLuTimeout);
         fine = 0;
       }
     }
@@ -843,7 +847,7 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
       if (!factor_tile<false>(D, R)) {
         load();
         factor_tile<true>(D, R);
-        if (warp == 0 && zero_or_nonfinite(D[lane][lane])) a.cbad[c] = 1;
+        if (warp == 0 && zero_or_nonfinite(D[lane][lane])) atomicMax(a.cbad + c, kLuZeroPivot);
         __syncthreads();
       }
       const double rl = R[lane];
@@ -985,7 +989,7 @@ __global__ void __launch_bounds__(32 * kSubstWarps) k_cc_subst(ContactArgs a, So
   if (!a.cgo[c]) return;
   if (a.cbad[c]) {
     if (rank == 0 && threadIdx.x == 0) {
-      v.sys_status[s] = DM_ERR_DEGENERATE;
+      v.sys_status[s] = a.cbad[c] == kLuTimeout ? DM_ERR_CUDA : DM_ERR_DEGENERATE;
       v.sys_active[s] = 0;
       atomicAdd(&v.ctrl[1], 1);
       atomicMin(&v.ctrl[2], s);

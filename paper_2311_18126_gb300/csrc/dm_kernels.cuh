@@ -350,7 +350,7 @@ struct ContactArgs {
   int32_t *pairs, *npairs;
   double *fc, *dense;
   int n_contact;
-  int32_t *cgo, *cbad;  // per contact system: solve this round, zero pivot met
+  int32_t *cgo, *cbad;  // per contact system: solve this round, why its factorisation stopped (0: it did not)
   int nn;  // nodes (ground terms of contact systems)
   unsigned long long *lu_flops;  // profiling: FP64 flops of the LU's trailing updates (or NULL)
 };
