@@ -940,7 +940,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       DM_CK(cudaMemsetAsync(c.fc, 0, nd * sizeof(double), rs));
       DM_CK(cudaMemsetAsync(c.npairs, 0, sizeof(int32_t), rs));
       DM_CK(cudaMemsetAsync(c.bucket_count, 0, c.table * sizeof(int32_t), rs));
-      k_cc_clear<<<dim3(blocks(c.max_n, kNB), c.n_contact), 256, 0, rs>>>(ca);
+      k_cc_clear<<<dim3(c.n_contact, blocks(c.max_n, kNB)), 256, 0, rs>>>(ca);
       k_cc_cells<<<blocks(ne, 256), 256, 0, rs>>>(ca);
       k_cc_scan<<<1, 1024, 0, rs>>>(ca);
       k_cc_fill<<<blocks(ne, 256), 256, 0, rs>>>(ca);
@@ -1819,7 +1819,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     DM_CK(cudaMemsetAsync(c.fc, 0, nd * sizeof(double), st));
     DM_CK(cudaMemsetAsync(c.npairs, 0, sizeof(int32_t), st));
     DM_CK(cudaMemsetAsync(c.bucket_count, 0, c.table * sizeof(int32_t), st));
-    k_cc_clear<<<dim3(blocks(c.max_n, kNB), c.n_contact), 256, 0, st>>>(ca);
+    k_cc_clear<<<dim3(c.n_contact, blocks(c.max_n, kNB)), 256, 0, st>>>(ca);
     k_cc_cells<<<blocks(ne, 256), 256, 0, st>>>(ca);
     k_cc_scan<<<1, 1024, 0, st>>>(ca);
     k_cc_fill<<<blocks(ne, 256), 256, 0, st>>>(ca);
@@ -1925,7 +1925,7 @@ dm_status dm_step_adjoint(dm_system *sys, const double *q_next, const double *gq
     DM_CK(cudaMemcpyAsync(ca.cgo, onec.data(), nc * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     DM_CK(cudaMemsetAsync(ca.cbad, 0, nc * sizeof(int32_t), st));
     k_cc_band<<<blocks(nd, 64), 64, 0, st>>>(ca, nrhs, d.dq);
-    k_cc_transpose<<<dim3(blocks(s->x.cc.max_n, kNB), nc), 256, 0, st>>>(ca);
+    k_cc_transpose<<<dim3(nc, blocks(s->x.cc.max_n, kNB)), 256, 0, st>>>(ca);
     if (!A.ints) DM_TRY(dalloc(s, &A.ints, 6 * (size_t)S + 2 * (size_t)std::max(ngen, 1) + 8));
     int32_t *its = A.ints, *sts = its + S, *ctl = sts + S;
     DM_CK(cudaMemsetAsync(its, 0, 2 * S * sizeof(int32_t), st));

@@ -506,8 +506,8 @@ __global__ void k_cc_band(ContactArgs a, const double *f, double *y) {
 // Zeroes the tiles that the last factorisation of each contact system used,
 // and their marks: a block per tile row.
 __global__ void __launch_bounds__(256) k_cc_clear(ContactArgs a) {
-  const int s = a.contact_sys[blockIdx.y];
-  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.x;
+  const int s = a.contact_sys[blockIdx.x];
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.y;
   if (I >= nt) return;
   uint8_t *nz = a.nz + a.sys_nz0[s] + (size_t)I * nt;
   double *M = a.dense + a.sys_dense0[s];
@@ -772,10 +772,11 @@ __device__ __forceinline__ bool lu_wait(int32_t *bar, int32_t *bad, int blocks, 
   return ok != 0;
 }
 
-// Factorisation of all levels: gridDim.x blocks per system.
+// Factorisation of all levels: gridDim.y blocks per system (a grid takes more
+// systems along x than along y: 65535).
 constexpr int kLuThreads = 512;
 __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yall) {
-  const int c = blockIdx.y;
+  const int c = blockIdx.x, block = blockIdx.y;
   if (!a.cgo[c]) return;
   const int s = a.contact_sys[c];
   const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB;
@@ -793,7 +794,7 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
   const int32_t *lev = a.lu_level + (size_t)c * a.max_tiles * kLevelInts;
   const int levels = lev[kLevelInts - 1];
   const auto fronts = [&](int I) { return (reach[I >> 2] >> (8 * (I & 3))) & 0xffu; };
-  const int blocks = gridDim.x;
+  const int blocks = gridDim.y;
   int target = 0, items = 0, vecs = 0;
   // level l's record, its fronts' neighbours and who neighbours whom
   const auto load_level = [&](int l) {
@@ -825,10 +826,10 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
       int part = 0, parts = 1;
       if (blocks >= nf) {
         parts += (blocks - nf) * vec / (2 * kNB * vecs + nf);
-        part = (int)blockIdx.x - start;
+        part = block - start;
         start += parts;
         if (part < 0 || part >= parts) continue;
-      } else if (f % blocks != (int)blockIdx.x) {
+      } else if (f % blocks != block) {
         continue;
       }
       const int each = min((vec + parts - 1) / parts, kLuThreads / 32);  // vectors of a block at a time
@@ -900,7 +901,7 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
     // update, by half a block: quarter items (16 x 16 of a tile), front by front,
     // then the right-hand side's rows; a tile or row of several fronts belongs to the
     // first, which takes the others' parts along
-    for (int f = 0, base = 0, it = blockIdx.x + half * blocks; it < items + vecs; it += 2 * blocks) {
+    for (int f = 0, base = 0, it = block + half * blocks; it < items + vecs; it += 2 * blocks) {
       if (it >= items) {  // right-hand side: a lane per term
         int g = it - items, fv = 0;
         while (g >= lv.m[fv]) g -= lv.m[fv++];
@@ -958,8 +959,8 @@ __global__ void __launch_bounds__(kLuThreads, 1) k_lu(ContactArgs a, double *yal
 // In-place transpose of the contact systems' matrices (for the adjoint's
 // J^T solve): a block per tile row, the tiles on and right of the diagonal.
 __global__ void __launch_bounds__(256) k_cc_transpose(ContactArgs a) {
-  const int s = a.contact_sys[blockIdx.y];
-  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.x;
+  const int s = a.contact_sys[blockIdx.x];
+  const int n = a.sys_ndof[s], nt = (n + kNB - 1) / kNB, I = blockIdx.y;
   if (I >= nt) return;
   const uint8_t *nz = a.nz + a.sys_nz0[s] + (size_t)I * nt;
   double *A = a.dense + a.sys_dense0[s];
@@ -1079,7 +1080,7 @@ cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStre
   cfg.numAttrs = 1;
   cfg.stream = st;
   const int share = coop ? std::max(1, std::min(sms / nc, 4 * nt * nt)) : 1;
-  cfg.gridDim = dim3(share, nc);
+  cfg.gridDim = dim3(nc, share);
   cfg.blockDim = dim3(kLuThreads);
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = share > 1 ? 1 : 0;
