@@ -1069,17 +1069,19 @@ cudaError_t lu_solve(const ContactArgs &a, const SolveArgs &v, int sms, cudaStre
   k_lu_order<<<nc, threads, 4 * words, st>>>(a);
   // the chip shared among the systems; several blocks of a system wait for one
   // another, so all of them must be resident (one per SM), which a cooperative
-  // launch guarantees; without such launches one block per system
-  int dev = 0, coop = 0;
+  // launch guarantees; without such launches, and under MPS, where CUDA takes
+  // none inside the round's graph, one block per system
+  int dev = 0, coop = 0, mps = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&mps, cudaDevAttrMpsEnabled, dev);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t cfg{};
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cfg.stream = st;
-  const int share = coop ? std::max(1, std::min(sms / nc, 4 * nt * nt)) : 1;
+  const int share = coop && !mps ? std::max(1, std::min(sms / nc, 4 * nt * nt)) : 1;
   cfg.gridDim = dim3(nc, share);
   cfg.blockDim = dim3(kLuThreads);
   at[0].id = cudaLaunchAttributeCooperative;
