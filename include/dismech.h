@@ -245,7 +245,8 @@ int64_t dm_num_edges(const dm_system *sys);
  * pivot D_i is small against its row; a pivot that is zero, not finite,
  * below 2^-43 |J_ii| (1.1e-13) or outside [2^-126, 2^126) returns
  * DM_ERR_DEGENERATE (the system is then numerically singular for this
- * solver) instead of an inaccurate x. */
+ * solver) instead of an inaccurate x: x of such a system is zero, the other
+ * systems are solved.  Entries of x outside every system are zero. */
 dm_status dm_solve_band(int32_t nsys, const int32_t *sys_dof0, const int32_t *sys_ndof,
                         int64_t ntot, const double *band, const double *rhs, double *x,
                         void *stream);

@@ -29,6 +29,13 @@ __global__ void k_band_prepare(int nsys, int32_t *active, int32_t *iters, int32_
   }
 }
 
+// x of the systems that failed: zero (a block per system)
+__global__ void k_band_clear_failed(const int32_t *dof0, const int32_t *ndof, const int32_t *status, double *x) {
+  if (status[blockIdx.x] == 0) return;
+  double *xs = x + dof0[blockIdx.x];
+  for (int i = threadIdx.x; i < ndof[blockIdx.x]; i += blockDim.x) xs[i] = 0.0;
+}
+
 inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -154,11 +161,14 @@ dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof,
   int32_t hc[4] = {0, 0, 0, 0};
   BS_CK(cudaMemcpyAsync(hc, ctrl, sizeof(hc), cudaMemcpyDeviceToHost, st));
   BS_CK(cudaStreamSynchronize(st));
-#undef BS_CK
   if (hc[1] > 0) {
+    k_band_clear_failed<<<nsys, 128, 0, st>>>(d_dof0, d_ndof, status, x);
+    BS_CK(cudaGetLastError());
+    BS_CK(cudaStreamSynchronize(st));
     set_error("dm_solve_band: zero or non-finite pivot in system " + std::to_string(hc[2]));
     return DM_ERR_DEGENERATE;
   }
+#undef BS_CK
   return DM_OK;
 }
 
