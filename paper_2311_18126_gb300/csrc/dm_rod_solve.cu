@@ -465,9 +465,9 @@ __global__ void __launch_bounds__(128, L == 16 ? 3 : 2) k_solve_rod(SolveArgs a)
       for (int u = 0; u < 10; ++u) column<L, ENV>(ln, 0, 0, 8 * s_buf + 96 * u, 96 * u, rj, sep, cb);
       bool sbad = false;
       if (sep) {
-        for (int u = p; u < 10; u += L) {  // zero, subnormal, infinite or NaN
+        for (int u = p; u < 10; u += L) {  // zero, subnormal, infinite, NaN, or of subnormal reciprocal
           const unsigned h = ((unsigned)__double2hiint(S[12 * u]) & 0x7FFFFFFFu) >> 20;
-          if (h == 0u || h == 2047u) sbad = true;
+          if (h - 1u >= 2044u) sbad = true;
         }
         store_records<L>(c, R, m, 10, p);
       }
