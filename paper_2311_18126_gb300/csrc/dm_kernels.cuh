@@ -216,18 +216,21 @@ __device__ __forceinline__ double rcp_any(double d) {
 
 // sqrt(x), x >= 0: where x is well inside the FP32 range, the FP32 reciprocal
 // root r of its leading 23 bits, moved between the formats by integer
-// operations as in rcp64_seed, and with h = x r, e = 1 - h r the series
-// h (1 + e/2 + 3 e^2/8) of h / sqrt(1 - e): five FP64 instructions, relative
-// error below 2 * 2^-53.
+// operations as in rcp64_seed, with h = x r, e = 1 - h r the series y = h (1 +
+// e/2 + 3 e^2/8) of h / sqrt(1 - e) (within 2 * 2^-53), and the residual's
+// correction y + r (x - y^2)/2: seven FP64 instructions, the correctly rounded
+// root but where that lies within 2^-19 of a unit in the last place of a tie.
 __device__ __forceinline__ double sqrt_any(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   if (hi - ((1023u - 100u) << 20) >= (200u << 20)) return sqrt(x);
   float sf;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(sf) : "f"(__uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29))));
   const unsigned sb = __float_as_uint(sf);
-  const double r = __hiloint2double((int)((sb >> 3) + 0x38000000u), (int)(sb << 29));
+  const int rh = (int)((sb >> 3) + 0x38000000u), rl = (int)(sb << 29);
+  const double r = __hiloint2double(rh, rl), half = __hiloint2double(rh - (1 << 20), rl);
   const double h = x * r, e = fma(-h, r, 1.0);
-  return fma(h, e * fma(0.375, e, 0.5), h);
+  const double y = fma(h, e * fma(0.375, e, 0.5), h);
+  return fma(fma(-y, y, x), half, y);
 }
 
 // Maximum of the scaled residuals (their bits) per system (-1: none), order
