@@ -76,7 +76,8 @@ __device__ __forceinline__ D1 d1_apply(const D1 &a, double f0, double f1) { retu
 // (1 - s, s, t - 1, -t): at the closest points f's derivative in a free s or t
 // is zero, so D's gradient is f_x / D and its Hessian comes from f_xx + f_xz z_x
 // + (f_xz z_x)^T + z_x^T f_zz z_x, where z_x = (s_x, t_x) are the closest
-// points' own derivatives (zero for a clamped one).  Every lane has the values;
+// points' own derivatives (zero for a clamped one); for near-parallel segments
+// f_t t_x and f_t t_xx come in.  Every lane has the values;
 // lanes 0-11 the derivatives of their own coordinate, which the lanes' second
 // derivatives fetch.  (Second-order dual numbers through the whole computation
 // took 1400 FP64 instructions a pair, 94 us a launch for 897 pairs.)
@@ -132,11 +133,15 @@ __device__ __forceinline__ Distance pair_distance(const double *x, const HLane &
   q.tx = !tfree ? 0.0 : joint ? -fma(B, fs, A * ft) * iden : fma(w1, bc, -mt * pick(d1)) * iC;
   q.sx = !sfree ? 0.0 : fma(B, q.tx, -fs) * iA;
   // (the last term vanishes but for near-parallel segments, where t is the
-  // closest point of s = 0)
+  // closest point of s = 0 and f's derivative in t, -d b, is not zero)
   q.Dx = iD * fma(-dot3(q.d, b), q.tx, w * dc);
 #pragma unroll
   for (int e = 0; e < 3; ++e) q.dx[e] = fma(a[e], q.sx, fma(-b[e], q.tx, e == c ? w : 0.0));
   const double ps = fma(0.5, fma(A, q.sx, -B * q.tx), fs), pt = fma(0.5, fma(C, q.tx, -B * q.sx), ft);
+  // t's own second derivative for those: t = E / C, E = b r and C = b b, with b
+  // = sum -mt_n x_n and r = sum rho_n x_n
+  const bool curved = parallel && tfree;  // warp-uniform
+  const double rho = m == 0 ? 1.0 : m == 2 ? -1.0 : 0.0, cx = -2.0 * mt * bc, ftC = -dot3(q.d, b) * iC;
 #pragma unroll
   for (int k = 0; k < kHP; ++k) {
     const int i = ln.i[k], j = ln.j[k];
@@ -146,6 +151,14 @@ __device__ __forceinline__ Distance pair_distance(const double *x, const HLane &
     h = fma(__shfl_sync(full, pt, i), __shfl_sync(full, q.tx, j), h);
     h = fma(__shfl_sync(full, q.sx, i), __shfl_sync(full, ps, j), h);
     h = fma(__shfl_sync(full, q.tx, i), __shfl_sync(full, pt, j), h);
+    if (curved) {
+      const double bi = -__shfl_sync(full, mt, i), bj = -__shfl_sync(full, mt, j);
+      const double ri = __shfl_sync(full, rho, i), rj = __shfl_sync(full, rho, j);
+      double tt = i % 3 == j % 3 ? fma(bi, rj, ri * bj) - 2.0 * q.t * bi * bj : 0.0;
+      tt = fma(-__shfl_sync(full, q.tx, i), __shfl_sync(full, cx, j), tt);
+      tt = fma(-__shfl_sync(full, cx, i), __shfl_sync(full, q.tx, j), tt);
+      h = fma(ftC, tt, h);
+    }
     q.gi[k] = __shfl_sync(full, q.Dx, i);
     q.gj[k] = __shfl_sync(full, q.Dx, j);
     q.h[k] = iD * fma(-q.gi[k], q.gj[k], h);
