@@ -26,7 +26,7 @@
 // Measured: inference of 444544 rows 233 -> 164 us (0.9 PFLOP/s; a tile 13.6 k
 // cycles, 5.1 k of them tensor work, 2.6 k waits for weights with two 32 KB
 // blocks in flight, 3.1 k for epilogues where the short first and last layers
-// meet); a training step of 16384 rows 548 -> 77 us.
+// meet); a training step of 16384 rows 548 -> 80 us.
 // Training keeps the ReLU masks in registers, forms the loss and its gradient
 // in the output epilogue, and stores the hidden activations and the gradients
 // of every layer row-major by TMA (k_mlp_wgrad reads them as they are, with
@@ -106,6 +106,11 @@ __device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, volatile
   }
   *fail = 1;
   return false;
+}
+// The same by a whole warp, with one answer for all its lanes: what follows
+// takes every lane (tcgen05.ld), also where only some of them gave up.
+__device__ __forceinline__ bool wait_warp(uint64_t *bar, uint32_t parity, volatile int *fail) {
+  return __all_sync(kFullMask, wait_on(bar, parity, fail));
 }
 __device__ __forceinline__ void arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
@@ -321,7 +326,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     uint32_t mask[3][2];  // ReLU masks of the hidden layers
     float gb = 0.0f;      // output column 16 part + lane's gradient sum
     auto acc_ready = [&]() -> uint32_t {
-      ok = ok && wait_on(&bar_acc[ph & 1], (uint32_t)((ph >> 1) & 1), fail);
+      ok = ok && wait_warp(&bar_acc[ph & 1], (uint32_t)((ph >> 1) & 1), fail);
       asm volatile("tcgen05.fence::after_thread_sync;");
       const uint32_t t = tmem + 256u * (uint32_t)(ph & 1) + lane_off;
       ++ph;
@@ -338,7 +343,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     auto hidden = [&](int l, bool back) {
       const uint32_t t = acc_ready();
       if (!ok) return;
-      if (stores > 0 && !(ok = wait_on(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
+      if (stores > 0 && !(ok = wait_warp(bar_stored, (uint32_t)((stores - 1) & 1), fail))) return;
       ++stores;
       uint32_t r[2][32];  // the group's K-blocks: group, group + 2
       const uint32_t tc0 = t + (uint32_t)(64 * group + 32 * half);
@@ -616,7 +621,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     uint32_t phase = 0;
     bool ok = true;
     auto acc_ready = [&]() {
-      ok = ok && wait_on(&bar_acc[t], phase & 1u, fail);
+      ok = ok && wait_warp(&bar_acc[t], phase & 1u, fail);
       ++phase;
       asm volatile("tcgen05.fence::after_thread_sync;");
     };
@@ -837,23 +842,26 @@ __global__ void __launch_bounds__(kGThreads, 1)
       if (bias)
         for (int g = g0; g < min(g0 + kGSeg, k1 - k0) && ok; ++g) {
           const int s = g % kGStages;
-          ok = __all_sync(kFullMask, wait_on(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail));
+          ok = wait_warp(&bar_full[s], (uint32_t)((g / kGStages) & 1), fail);
           if (!ok) break;
-          uint32_t x[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            x[i] = *reinterpret_cast<const uint32_t *>(bcol + s * kGStageBytes + i * 128 + ((chunk ^ (i & 7)) << 4));
-          warp_arrive(&bar_free[s]);
           float s0 = 0.0f, s1 = 0.0f;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            s0 += __uint_as_float(x[i] << 16);
-            s1 += __uint_as_float(x[i] & 0xFFFF0000u);
+          for (int i0 = 0; i0 < 16; i0 += 8) {  // (eight words in registers beside the sums)
+            uint32_t x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              x[i] = *reinterpret_cast<const uint32_t *>(bcol + s * kGStageBytes + (i0 + i) * 128 + ((chunk ^ i) << 4));
+            if (i0 == 8) warp_arrive(&bar_free[s]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              s0 += __uint_as_float(x[i] << 16);
+              s1 += __uint_as_float(x[i] & 0xFFFF0000u);
+            }
           }
           b0 += s0;
           b1 += s1;
         }
-      ok = ok && __all_sync(kFullMask, wait_on(&bar_acc[seg & 1], (uint32_t)((seg / 2) & 1), fail));
+      ok = ok && wait_warp(&bar_acc[seg & 1], (uint32_t)((seg / 2) & 1), fail);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
