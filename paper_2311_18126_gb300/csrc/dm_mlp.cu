@@ -82,7 +82,7 @@ __device__ __forceinline__ float adam(const UpdateArgs &a, float g, float *p, fl
 // each, 16 threads per column with several loads in flight).
 constexpr int kUpdateThreads = 256, kBiasBlocks = kOut / 16;
 __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
-  if (*a.err) return;
+  const int failed = *a.err;  // (looked at after the sums, whose loads hide its own)
   const int bias_block = (int)blockIdx.x - ((int)gridDim.x - kBiasBlocks);
   if (bias_block >= 0) {
     __shared__ float red[16][17];
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
     for (int k = 0; k < 16; ++k) s += red[k][col];
     size_t o = 0;
     for (int l = 0; l < kLayers; ++l) o += mlp_part_size(l);
+    if (failed) return;
     if (a.grads) a.grads[o + c] = s;
     if (a.lr > 0.0f) adam(a, s, a.b[3] + c, a.mb[3] + c, a.vb[3] + c, a.maskb[3][c]);
     return;
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(kUpdateThreads) k_mlp_update(UpdateArgs a) {
   float g = 0.0f;
 #pragma unroll 8
   for (int z = 0; z < S; ++z) g += part[(size_t)z * mlp_part_size(l)];
+  if (failed) return;
   const int in = l == 0 ? kIn : kHid, out = l == 3 ? kOut : kHid;
   if (e >= in * out) {
     const int c = e - in * out;
@@ -150,8 +152,9 @@ struct dm_mlp {
   uint16_t *act[3] = {}, *dz[3] = {}, *dy = nullptr;
   float *part = nullptr, *gb4 = nullptr;  // partial gradients of the batch's shares
   size_t part_n = 0, gb4_n = 0;
-  // the loss, and behind it the training step's error flag and the one of the
-  // asynchronous forward passes (err), which dm_mlp_check reads and clears
+  // the loss, behind it (cleared and read with it, 16 bytes) the training step's
+  // error flag, then the one of the asynchronous forward passes (err), which
+  // dm_mlp_check reads and clears
   double *loss = nullptr;
   int *train_err = nullptr;
   bool fused = true;  // inference: the fused 4-layer kernel (else a GEMM per layer)
@@ -327,10 +330,10 @@ dm_status dm_mlp_create(int32_t in_dim, int32_t out_dim, uint64_t seed, void *st
       cudaMemcpy(m->maskb[l], mb.data(), mb.size() * 4, cudaMemcpyHostToDevice);
     }
   }
-  if (st == DM_OK) st = mlp_alloc(m, &m->loss, 2);
+  if (st == DM_OK) st = mlp_alloc(m, &m->loss, 3);
   if (st == DM_OK) {
     m->train_err = reinterpret_cast<int *>(m->loss + 1);
-    m->err = m->train_err + 1;
+    m->err = reinterpret_cast<int *>(m->loss + 2);
   }
   if (st != DM_OK) {
     dm_mlp_destroy(m);
@@ -444,7 +447,7 @@ dm_status dm_mlp_forward(dm_mlp *m, const void *X, float *Y, int32_t M) {
 // batch's shares, Adam and the BF16 weights in the third.  grads_out (device,
 // optional) receives the fp32 gradients in the dm_mlp_get_params layout;
 // loss_out the loss before the update.
-// Measured (GB300): batch 16384 77 us against 548 us with a launch per layer
+// Measured (GB300): batch 16384 80 us against 548 us with a launch per layer
 // and operation (some 55 launches with transposed copies of every operand).
 dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M, float lr,
                             float *grads_out, double *loss_out) {
@@ -455,7 +458,7 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   const MlpTrainShape shape = mlp_train_shape(M);
   if (ensure_train(m, M, shape) != DM_OK) return DM_ERR_OOM;
   cudaStream_t st = m->stream;
-  cudaMemsetAsync(m->loss, 0, sizeof(double) + sizeof(int), st);
+  cudaMemsetAsync(m->loss, 0, 16, st);
   const void *W[kLayers], *Wt[kLayers];
   const float *b[kLayers];
   for (int l = 0; l < kLayers; ++l) {
@@ -491,9 +494,9 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   k_mlp_update<<<nb((int64_t)params, kUpdateThreads) + kBiasBlocks, kUpdateThreads, 0, st>>>(a);
   struct {
     double loss;
-    int err, other;
+    int err, none;
   } h = {};
-  static_assert(sizeof(h) == 16, "loss and error flags");
+  static_assert(sizeof(h) == 16, "loss and error flag");
   cudaMemcpyAsync(&h, m->loss, 16, cudaMemcpyDeviceToHost, st);
   if (cudaStreamSynchronize(st) != cudaSuccess || h.err) {
     set_error("dm_mlp_train_step: CUDA error or tensor-core barrier timeout");
