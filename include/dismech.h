@@ -280,13 +280,13 @@ dm_status dm_solve_band_partitioned(int32_t nsys, const int32_t *sys_dof0,
  * the same arguments and returns the same result as dm_solve_band, but keeps
  * all of its scratch in one fixed device array inside the library, sized for
  * DM_NOALLOC_MAX_SYSTEMS systems and DM_NOALLOC_MAX_DOFS DOFs in total
- * (about 3.3 MiB).  Larger batches are rejected with DM_ERR_INVALID_ARG and
+ * (about 3.1 MiB).  Larger batches are rejected with DM_ERR_INVALID_ARG and
  * a message naming the limit.  It calls no allocating CUDA routine itself.
  *  - The array belongs to the library's module: the CUDA driver reserves it
  *    on a device when it loads that module there, and keeps it until the
  *    process exits.  Under CUDA's default lazy module loading that happens
  *    inside the first call of this entry point on the device, which can
- *    then fail with DM_ERR_CUDA if the device has no 3.3 MiB left; make one
+ *    then fail with DM_ERR_CUDA if the device has no 3.1 MiB left; make one
  *    call at set-up, while memory is still free and before any stream
  *    capture, to take that reservation early.
  *  - Each call looks the array's address up in the current context, with

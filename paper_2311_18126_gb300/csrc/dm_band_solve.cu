@@ -64,8 +64,8 @@ bool check_band_batch(int32_t nsys, const int32_t *dof0, const int32_t *ndof, in
       set_error("dm_solve_band: system " + std::to_string(k) + " outside [0, ntot)");
       return false;
     }
-  // the kernel updates each system's rows in place and accumulates into x:
-  // systems may not share rows
+  // the kernel writes x (and its records) row by row of each system: systems
+  // may not share rows
   std::vector<int32_t> by_start(nsys);
   for (int k = 0; k < nsys; ++k) by_start[k] = k;
   std::sort(by_start.begin(), by_start.end(),
@@ -92,7 +92,7 @@ bool check_band_batch(int32_t nsys, const int32_t *dof0, const int32_t *ndof, in
 }
 
 // Runs the banded solve with all scratch inside `scr` (band_scratch_bytes
-// bytes, 256-byte aligned) and waits for it.  h_ctrl: 4 host ints.
+// bytes, 256-byte aligned) and waits for it.  band and rhs are only read.
 dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof, int64_t ntot,
                          const double *band, const double *rhs, double *x, char *scr,
                          cudaStream_t st) {

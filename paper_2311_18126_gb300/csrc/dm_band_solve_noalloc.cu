@@ -17,14 +17,14 @@ dm_status run_band_solve(int32_t nsys, const int32_t *dof0, const int32_t *ndof,
 namespace {
 
 // Scratch for DM_NOALLOC_MAX_SYSTEMS systems and DM_NOALLOC_MAX_DOFS DOFs:
-// band copy, right-hand side and substitution vectors (13 doubles per DOF),
-// six ints and one residual word per system, four counters.  About 3.3 MiB.
+// the solver's column records (12 doubles per DOF), six ints and one residual
+// word per system, four counters.  About 3.1 MiB.
 // The driver allocates it on a device when it loads this file's module
 // there: at the first call of this entry point on that device under CUDA's
 // default lazy module loading, at context creation under eager loading.
 // It is then held until the process exits.
 constexpr size_t kScratchBytes =
-    13 * (size_t)DM_NOALLOC_MAX_DOFS * sizeof(double) +
+    12 * (size_t)DM_NOALLOC_MAX_DOFS * sizeof(double) +
     ((6 * (size_t)DM_NOALLOC_MAX_SYSTEMS * sizeof(int32_t) + 255) & ~(size_t)255) +
     ((DM_NOALLOC_MAX_SYSTEMS * sizeof(unsigned long long) + 255) & ~(size_t)255) + 256;
 
@@ -70,7 +70,7 @@ extern "C" dm_status dm_solve_band_noalloc(int32_t nsys, const int32_t *sys_dof0
   char *scr = nullptr;
   dm_status st = scratch_for_current_context(&scr);
   if (st != DM_OK) return st;
-  // run_band_solve clears every part of the scratch the kernel reads
-  // before it reads it (band copy, right-hand side, counters, flags).
+  // nothing of an earlier call is read: run_band_solve writes the ints, flags
+  // and counters first, and the kernel stores every record before it fetches it
   return run_band_solve(nsys, sys_dof0, sys_ndof, ntot, band, rhs, x, scr, (cudaStream_t)stream);
 }

@@ -138,10 +138,6 @@ __device__ __forceinline__ double sgnmul(unsigned sw, double x) {
   return __hiloint2double(__double2hiint(x) ^ (int)sw, __double2loint(x));
 }
 __device__ __forceinline__ unsigned sign_word(int s) { return s < 0 ? 0x80000000u : 0u; }
-__device__ __forceinline__ v3 sgn3(int s, v3 v) {
-  const unsigned sw = sign_word(s);
-  return mk(sgnmul(sw, v.x), sgnmul(sw, v.y), sgnmul(sw, v.z));
-}
 
 // An edge's material frame (m1, m2, t), right-handed and orthonormal, in the
 // stencil's orientation (a reversed edge: t and m2 flipped), and its 1/l.

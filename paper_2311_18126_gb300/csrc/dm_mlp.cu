@@ -468,8 +468,10 @@ dm_status dm_mlp_train_step(dm_mlp *m, const void *X, const float *Y, int32_t M,
   }
   void *act[3] = {m->act[0], m->act[1], m->act[2]}, *dz[3] = {m->dz[0], m->dz[1], m->dz[2]};
   if (launch_mlp_train(M, X, Y, m->out_dim, W, Wt, b, act, dz, m->dy, m->loss, m->part, m->gb4, m->train_err, st) !=
-      cudaSuccess)
+      cudaSuccess) {
+    set_error("dm_mlp_train_step: launch failed");
     return DM_ERR_CUDA;
+  }
   const float step = (float)(m->step + 1);  // counted once it has succeeded
   UpdateArgs a{};
   for (int l = 0; l < kLayers; ++l) {
