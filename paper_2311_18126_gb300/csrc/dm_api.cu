@@ -1072,8 +1072,12 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
       s->x.launches[k] = before[k];
     }
     s->x.round_launches[K_BEGIN] += 1;  // k_round_continue
-    if (rst == DM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&s->x.round_graph, g, 0);
-    cudaGraphDestroy(g);
+    // (a graph whose body's capture was invalidated, by a launch that failed in
+    // it, is left behind: destroying it ends the process)
+    const bool captured = e == cudaSuccess;
+    if (rst == DM_OK && captured) e = cudaGraphInstantiate(&s->x.round_graph, g, 0);
+    if (captured) cudaGraphDestroy(g);
+    if (rst != DM_OK || e != cudaSuccess) (void)cudaGetLastError();  // reported here, not by the next call
     if (rst != DM_OK) return rst;
     if (e != cudaSuccess) {
       s->x.round_graph = nullptr;
@@ -1101,6 +1105,7 @@ dm_status dm_step(dm_system *sys, int32_t nsteps, dm_step_stats *stats) {
     s->x.first_launches[K_BEGIN] += 1;  // k_round_count
     if (rst == DM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&s->x.first_graph, g, 0);
     if (g) cudaGraphDestroy(g);
+    if (rst != DM_OK || e != cudaSuccess) (void)cudaGetLastError();
     if (rst != DM_OK) return rst;
     if (e != cudaSuccess) {
       s->x.first_graph = nullptr;
