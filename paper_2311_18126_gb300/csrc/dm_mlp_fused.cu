@@ -708,13 +708,16 @@ namespace {
 // the MMA's M or N, so the descriptors are MN-major (64-wide boxes with the
 // 128-byte swizzle: 8 batch rows of 128 bytes per swizzle group, the boxes
 // 8 KB apart).  The tensor core truncates as it accumulates: sums of one sign
-// over 2^15 rows in one chain were off by 1e-6 to 1e-5 of their size.  So a
-// chain ends after kGSeg stages (512 rows), and eight epilogue warps add it to
+// over 2700 rows in one chain were off by 4e-7 of their size, over 11000 by
+// 5e-6.  So a chain ends after kGSeg stages (512 rows), and eight epilogue warps add it to
 // the sums in their registers (FP32, rounded to nearest) while the next one
 // fills the other half of the tensor memory; they also sum the hidden biases'
 // gradients, the columns of dZ, from the stages (errors now 1e-7 whatever the
-// batch; a step of 16384 rows 74.5 -> 77.4 us).  Partials per share, summed in
-// a fixed order by k_mlp_update.
+// batch).  Bound by the loads and the chain of a share (ten stages at 16384 rows,
+// 19 us against 17 in one chain: the bias sums read the stages beside the MMAs;
+// chains of 12 stages take the same time, and draining a chain in quarters
+// between the stages spilled registers and took 21).  Partials per share, summed
+// in a fixed order by k_mlp_update.
 constexpr int kGStages = 4;
 constexpr int kGSeg = 8;                        // stages of a chain
 constexpr int kGWarps = 8;                      // epilogue warps; then the MMA and the TMA warp
